@@ -22,6 +22,7 @@
 #include <algorithm>
 #include <cfloat>
 #include <climits>
+#include <cstring>
 #include <mutex>
 #include <string>
 #include <type_traits>
@@ -624,6 +625,7 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 
 constexpr int kSpmvThreads = 256;
 constexpr int kSpmvWarps = kSpmvThreads / 32;
+constexpr int64_t kMaxBlockSmem = 227 * 1024;  // dynamic shared memory a block can have
 
 // Shared memory per warp for the gather schemes (k <= 16): the lanes' tile
 // words and tile columns (lane-private, so the flat bit walk can index them),
@@ -881,8 +883,9 @@ __device__ __forceinline__ void load_lane_tiles(const SpmvGeom& g, int32_t tl, u
 }
 
 // ---------------------------------------------------------------------------
-// chunk kernel for the bit-vector schemes (all k) and for the value schemes
-// at k = 32: registers hold the accumulators (static row indices)
+// chunk kernel for the bit-vector schemes at k = 16 and 32 and for the value
+// schemes that neither the small-tile kernel nor the staged one takes:
+// registers hold the accumulators (static row indices)
 // ---------------------------------------------------------------------------
 template <int K, class SEM>
 __global__ void __launch_bounds__(kSpmvThreads) spmv_chunks_kernel(SpmvGeom g, SEM sem,
@@ -979,176 +982,367 @@ __global__ void __launch_bounds__(kSpmvThreads) spmv_chunks_kernel(SpmvGeom g, S
 }
 
 // ---------------------------------------------------------------------------
-// tile_dim-4 chunk kernel for the bit-vector schemes (Boolean and count
-// SpMVs) and the unweighted 4-byte value schemes (plus-times, label min, fp32
-// max: one gather per set bit).  At k = 4 a tile is 4 bytes, so the tile
-// stream is tiny per tile and the kernel is shaped by per-tile latency:
+// small-tile chunk kernel: the bit-vector schemes (Boolean and count SpMVs) at
+// k = 4 and 8, and at k = 4 the unweighted value schemes with 4- and 8-byte
+// values (plus-times, label min, fp32 max, 32- and 64-lane OR).  A tile is one
+// 32- or 64-bit word there, 256 tiles a chunk, so the kernel is bound by
+// instructions and by the input gathers, not by the tile stream:
 //   * persistent warps: warp gw takes chunks gw, gw + W, ... and loads the
-//     next chunk's tile stream (8 tile words and 8 tile columns a lane, one
-//     32-byte load each, marked not to be kept in L1, plus the chunk's row
-//     pointers) into registers before it works on the current one, so every
-//     warp keeps a chunk in flight;
-//   * a chunk inside one tile-row (most chunks of a power-law graph) needs no
-//     row search, walk or segmented scan: one fixed-order butterfly joins the
-//     lanes; other chunks take the chunk kernel's walk and joins.
+//     next chunk's tile stream into registers before it works on the current
+//     one, so every warp keeps a chunk in flight;
+//   * a value scheme loads the whole 4-value input segment under a tile in
+//     one 16- or 32-byte load (a gather costs a 32-byte sector whatever its
+//     width) and adds it under the tile's 16 bits, with no loop over set bits:
+//     nothing diverges, and every load of a lane is in flight at once;
+//   * the chunk's row ends become a 256-bit mask and a table of row numbers in
+//     shared memory, made from one coalesced load of row pointers, so the walk
+//     tests one bit per tile and loads no row pointers;
+//   * a chunk inside one tile-row (more than half of them on a power-law
+//     graph) needs no walk: one fixed-order tree joins the lanes.
+// What bounds the value schemes is the L1 data pipe: a gather takes one
+// wavefront per distinct 128-byte line, 32 a warp for scattered columns (79%
+// of the pipe, 27.2M wavefronts an SpMV on R-MAT 20).  R-MAT 20, k = 4, direct
+// schedule, SpMV call in us before / after (one gather per set bit, a row
+// search and a row-pointer walk per lane before): plus-times 173 / 126
+// (permuted ids 148 / 139), label min 183 / 135 (154 / 144), 64-lane OR
+// 238 / 177; Boolean 86 / 68 at k = 4 and 99 / 72 at k = 8.  Warp
+// instructions of the plus-times kernel: 98M / 59M.
 // ---------------------------------------------------------------------------
-// resident 256-thread blocks the registers are budgeted for (every lane holds
-// two chunks' tile words and columns)
-constexpr int kK4MinBlocks = 4;
+// min and max schemes
+template <class S>
+struct MinMax : std::false_type {};
+template <int K>
+struct MinMax<SemMinI32<K>> : std::true_type {};
+template <int K>
+struct MinMax<SemMaxF32<K>> : std::true_type {};
 
+// How a scheme reads its input: bits from global memory, bits from the
+// block's copy of the whole bitset in shared memory, whole aligned segments of
+// values, or one value per set column (an input that is not aligned to a
+// segment, or whose last segment is ragged).
+enum { kSmBits = 0, kSmBitsShared = 1, kSmSegs = 2, kSmVals = 3 };
+// Threads a block, and the resident blocks the registers are budgeted for
+// (every lane holds two chunks' tile words and columns).  R-MAT 20, k = 4, in
+// us with 4 / 3 blocks an SM: plus-times 126 / 128, label min 145 / 135 (four
+// blocks spill there), 16-source BFS 1,265 / 1,330.  The shared bitset leaves
+// room for one block: k = 8 with 512 / 640 / 768 threads 83 / 74 / 72.5.
+template <int K, int MODE>
+constexpr int small_threads() {
+    return MODE != kSmBitsShared ? kSpmvThreads : (K == 8 ? 768 : 1024);
+}
+template <int K, class SEM, int MODE>
+constexpr int small_min_blocks() {
+    if (MODE == kSmBitsShared) return 1;
+    return K == 8 || sizeof(typename SEM::V) == 8 || MinMax<SEM>::value ? 3 : 4;
+}
 
-// The tile stream of one chunk as a lane holds it: the chunk's first and last
-// tile-rows and their row pointers (lane j: rowptr[ra + j]), whether every
-// output row of it is masked out (then no tiles are read and the words are
-// zero: the walk still stores its rows and partials, all the identity), and
-// the lane's 8 tile words and columns.
-struct K4Tiles {
+// The tile stream of one chunk as a lane holds it: the chunk's first tile-row
+// and that of the next chunk, their row pointers (lane j: rowptr[ra + j]),
+// and the lane's 8 tiles and columns.  Words are zero where every output row
+// of the chunk is masked out (no tiles are read then; the walk still stores
+// its rows and partials, all the identity).
+template <int K>
+struct SmallTiles {
+    static constexpr int TW = ChunkShape<K>::TW;
     int32_t ra, rb;
     int32_t win;
-    bool sat;
-    uint32_t w[8], cu[8];
+    uint32_t w[8 * TW], cu[8];
 };
 
-template <class SEM>
-__device__ __forceinline__ void k4_load(const SpmvGeom& g, const SEM& sem, int32_t c, int lane, K4Tiles& t) {
+template <int K, class SEM>
+__device__ __forceinline__ void small_load(const SpmvGeom& g, const SEM& sem, int32_t c, int lane, SmallTiles<K>& t) {
+    constexpr int TW = SmallTiles<K>::TW;
     t.ra = __ldg(g.chunk_row + c);
     t.rb = __ldg(g.chunk_row + c + 1);
     t.win = row_window(g, t.ra, t.rb - t.ra, lane);
-    t.sat = sem.saturated((int64_t)t.ra * 4, ((int64_t)t.rb + 1) * 4);
-    if (!t.sat) {
-        // the arrays are padded to whole chunks, so every lane's 32 bytes exist
-        const int64_t tl = (int64_t)c * chunk_tiles(4) + lane * 8;
-        ld32_stream(reinterpret_cast<const uint32_t*>(g.tiles) + tl, t.w);
+    if (!sem.saturated((int64_t)t.ra * K, ((int64_t)t.rb + 1) * K)) {
+        // the arrays are padded to whole chunks, so every lane's bytes exist
+        const int64_t tl = (int64_t)c * chunk_tiles(K) + lane * 8;
+        const uint32_t* src = reinterpret_cast<const uint32_t*>(g.tiles) + tl * TW;
+#pragma unroll
+        for (int q = 0; q < TW; ++q) {
+            uint32_t v[8];
+            ld32_stream(src + 8 * q, v);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) t.w[8 * q + i] = v[i];
+        }
         ld32_stream(g.colind + tl, t.cu);
     } else {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) { t.w[i] = 0u; t.cu[i] = 0u; }
+        for (int i = 0; i < 8 * TW; ++i) t.w[i] = 0u;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) t.cu[i] = 0u;
     }
 }
 
-// The set bits of one k = 4 tile (row r in byte r) gather their inputs and
-// add them to the lane's row accumulators (value schemes).
+// Row ends of a chunk, per warp: bit t of `mask` is set iff tile cs + t is the
+// last of its tile-row; row[j] is the tile-row of the j-th such tile.
+struct ChunkRows {
+    uint32_t mask[8];
+    int32_t row[256];
+};
+
+// Fills s from the chunk's row pointers, 31 rows a step (lane j of a step: the
+// row starting at its pointer, ending at lane j + 1's); stores the identity
+// for the empty tile-rows between ra and rb, which hold the first tiles of
+// this and the next chunk, so that each is stored by one chunk.
 template <class SEM, class Acc>
-__device__ __forceinline__ void k4_gather_tile(const SEM& sem, Acc& acc, uint32_t w, int32_t J) {
-    using G = typename SEM::G;
-    using V = typename SEM::V;
-    const G* xt = sem.src() + (int64_t)J * 4;
-    while (w) {
-        const int bit = __ffs(w) - 1;
-        w &= w - 1;
-        const int r = bit >> 3;
-        const G xv = __ldg(xt + (bit & 7));
-        if constexpr (sizeof(V) == 8) {
-#pragma unroll
-            for (int v = 0; v < 4; ++v)
-                if (v == r) acc.set(v, sem.apply(acc.get(v), xv, 1.0f));
-        } else {
-            acc.set(r, sem.apply(acc.get(r), xv, 1.0f));
+__device__ __forceinline__ void chunk_ends(const SpmvGeom& g, const SEM& sem, int32_t ra, int32_t rb, int32_t win,
+                                           int32_t cs, int32_t ce, int lane, const Acc& idv, ChunkRows& s) {
+    constexpr unsigned FULL = 0xffffffffu;
+    __syncwarp();  // the previous chunk's readers are done
+    if (lane < 8) s.mask[lane] = 0u;
+    __syncwarp();
+    const int32_t span = rb - ra;
+    int found = 0;
+    for (int32_t j0 = 0; j0 <= span; j0 += 31) {
+        const int32_t j = j0 + lane;
+        const int32_t a = j0 == 0 ? win : (j <= span + 1 ? __ldg(g.rowptr + ra + j) : INT32_MAX);
+        const int32_t b = __shfl_down_sync(FULL, a, 1);
+        const bool row = lane < 31 && j <= span;
+        const bool end = row && b > a && b > cs && b <= ce;
+        const unsigned ends = __ballot_sync(FULL, end);
+        if (end) {
+            s.row[found + __popc(ends & ((1u << lane) - 1u))] = ra + j;
+            atomicOr(&s.mask[(b - 1 - cs) >> 5], 1u << ((b - 1 - cs) & 31));
+        } else if (row && a == b) {
+            sem.store(ra + j, idv);
         }
+        found += __popc(ends);
+    }
+    __syncwarp();
+}
+
+// The four input values under a k = 4 tile.
+template <class G, int MODE>
+__device__ __forceinline__ void load_seg(const G* __restrict__ x, uint32_t J, uint32_t w, G (&v)[4]) {
+    if constexpr (MODE == kSmSegs) {
+        if constexpr (sizeof(G) == 4) {
+            const uint4 q = __ldg(reinterpret_cast<const uint4*>(x) + J);
+            const uint32_t u[4] = {q.x, q.y, q.z, q.w};
+            memcpy(v, u, sizeof(v));
+        } else {
+            uint32_t u[8];
+            asm("ld.global.nc.v8.u32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
+                : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]), "=r"(u[7])
+                : "l"(x + 4 * (int64_t)J));
+            memcpy(v, u, sizeof(v));
+        }
+    } else {
+        const uint32_t cols = w | (w >> 8) | (w >> 16) | (w >> 24);
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            if ((cols >> c) & 1u) v[c] = __ldg(x + 4 * (int64_t)J + c);
+            else v[c] = G();
+    }
+}
+
+// Adds the tile's rows (row r in byte r of w) to the row accumulators, columns
+// in increasing order.
+template <class SEM, class G, class Acc>
+__device__ __forceinline__ void seg_add(const SEM& sem, Acc& acc, uint32_t w, const G (&v)[4]) {
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            if (w & (1u << (8 * r + c))) acc.set(r, sem.apply(acc.get(r), v[c], 1.0f));
+    }
+}
+
+// Joins the lanes' NV values with the tree of a butterfly (lane pairs, then
+// pairs of pairs, ...: the order of the segmented scan's last lane).  Four
+// values: the first two levels halve the values a lane carries, so lane l < 4
+// ends with value (l >> 1) | (l & 1) << 1; otherwise every lane ends with all.
+template <class SEM, class Acc>
+__device__ __forceinline__ void join_lanes(const SEM& sem, Acc& acc, int lane) {
+    using V = typename SEM::V;
+    constexpr int NV = SEM::NV;
+    constexpr unsigned FULL = 0xffffffffu;
+    if constexpr (!SEM::kGather) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v)
+            acc.set(v, std::is_signed<V>::value ? (V)__reduce_add_sync(FULL, (int)acc.get(v))
+                                                : (V)__reduce_or_sync(FULL, (unsigned)acc.get(v)));
+    } else {
+        static_assert(NV == 4, "value schemes at k = 4");
+        V a = acc.get(0), b = acc.get(1);
+        {
+            const bool hi = lane & 1;
+            const V sa = hi ? acc.get(0) : acc.get(2), sb = hi ? acc.get(1) : acc.get(3);
+            const V ka = hi ? acc.get(2) : acc.get(0), kb = hi ? acc.get(3) : acc.get(1);
+            const V oa = shfl_xor(sa, 1), ob = shfl_xor(sb, 1);
+            a = hi ? sem.comb(oa, ka) : sem.comb(ka, oa);
+            b = hi ? sem.comb(ob, kb) : sem.comb(kb, ob);
+        }
+        {
+            const bool hi = lane & 2;
+            const V s = hi ? a : b, k = hi ? b : a;
+            const V o = shfl_xor(s, 2);
+            a = hi ? sem.comb(o, k) : sem.comb(k, o);
+        }
+#pragma unroll
+        for (int d = 4; d < 32; d <<= 1) {
+            const V o = shfl_xor(a, d);
+            a = (lane & d) ? sem.comb(o, a) : sem.comb(a, o);
+        }
+        acc.set(0, a);
     }
 }
 
 // One chunk from its loaded tile stream.
-template <class SEM>
-__device__ __forceinline__ void k4_chunk(const SpmvGeom& g, const SEM& sem, Partials<typename SEM::V> part, int32_t c,
-                                         int lane, const K4Tiles& t) {
-    using S = ChunkShape<4>;
+template <int K, class SEM, int MODE>
+__device__ __forceinline__ void small_chunk(const SpmvGeom& g, const SEM& sem, Partials<typename SEM::V> part,
+                                            int32_t c, int lane, const SmallTiles<K>& t, ChunkRows& s,
+                                            const uint8_t* sx) {
+    using Sh = ChunkShape<K>;
     using V = typename SEM::V;
     constexpr int NV = SEM::NV;
-    constexpr int P = S::P;
-    static_assert(P == 8 && S::TW == 1, "eight one-word tiles a lane");
-    LaneSpan ls;
-    ls.cs = c * S::CT;
-    ls.ce = min(ls.cs + S::CT, (int32_t)g.T);
-    ls.tl = ls.cs + lane * P;
-    ls.cnt = max(0, min(P, ls.ce - ls.tl));
-    const int32_t ra = t.ra, rb = t.rb;
-    // the 4-bit input segment under each tile (bit-vector schemes)
-    uint32_t xs[SEM::kGather ? 1 : P];
-    if constexpr (!SEM::kGather) {
-#pragma unroll
-        for (int i = 0; i < P; ++i) {
-            const bool ok = i < ls.cnt && t.w[i] != 0u;
-            xs[i] = ok ? sem.xseg((int32_t)t.cu[i]) : 0u;
-        }
-    }
+    constexpr int TW = Sh::TW;
+    static_assert(Sh::P == 8 && TW <= 2, "eight tiles of one or two words a lane");
+    const int32_t cs = c * Sh::CT;
+    const int32_t ce = min(cs + Sh::CT, (int32_t)g.T);
     RegAcc<V, NV> acc, F, idv;
 #pragma unroll
     for (int v = 0; v < NV; ++v) { acc.set(v, sem.ident()); F.set(v, sem.ident()); idv.set(v, sem.ident()); }
-
-    if (ra == rb) {
-        // The whole chunk lies in tile-row ra (warp-uniform): every lane's
-        // tiles add to the same k rows, so no row search, walk or segmented
-        // scan is needed -- one fixed-order butterfly joins the lanes.
-        const int32_t row_start = __shfl_sync(0xffffffffu, t.win, 0);
+    const bool one_row = t.ra == t.rb;  // warp-uniform: the whole chunk lies in tile-row ra
+    uint32_t ends = 0u;
+    int rank = 0;
+    if (!one_row) {
+        chunk_ends(g, sem, t.ra, t.rb, t.win, cs, ce, lane, idv, s);
+        ends = reinterpret_cast<const uint8_t*>(s.mask)[lane];
+        rank = __popc(ends);
 #pragma unroll
-        for (int i = 0; i < P; ++i) {
-            if (i < ls.cnt) {
-                if constexpr (SEM::kGather) k4_gather_tile(sem, acc, t.w[i], (int32_t)t.cu[i]);
-                else sem.tile(acc, t.w + i, xs[i]);
-            }
+        for (int d = 1; d < 32; d <<= 1) {
+            const int o = __shfl_up_sync(0xffffffffu, rank, d);
+            if (lane >= d) rank += o;
+        }
+        rank -= __popc(ends);  // row ends before the lane's tiles
+    }
+    const int rank0 = rank;
+    bool has_end = false;
+    auto end_tile = [&](int i) {
+        if (!((ends >> i) & 1u)) return;
+        if (!has_end) {  // the lane's first row: joined with earlier lanes below
+#pragma unroll
+            for (int v = 0; v < NV; ++v) F.set(v, acc.get(v));
+            has_end = true;
+        } else {
+            sem.store(s.row[rank], acc);
         }
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
+        for (int v = 0; v < NV; ++v) acc.set(v, sem.ident());
+        ++rank;
+    };
+    if constexpr (SEM::kGather) {
+        // tiles whose segments are loaded together (plus-times on R-MAT 20: 1, 2,
+        // 4 tiles 127, 126, 130 us; the loads of more cost registers)
+        constexpr int GRP = 2;
+        using G = typename SEM::G;
 #pragma unroll
-            for (int v = 0; v < NV; ++v) {
-                const V other = shfl_xor(acc.get(v), o);
-                acc.set(v, (lane & o) ? sem.comb(other, acc.get(v)) : sem.comb(acc.get(v), other));
+        for (int i0 = 0; i0 < 8; i0 += GRP) {
+            G x[GRP][4];
+#pragma unroll
+            for (int i = 0; i < GRP; ++i) load_seg<G, MODE>(sem.src(), t.cu[i0 + i], t.w[i0 + i], x[i]);
+#pragma unroll
+            for (int i = 0; i < GRP; ++i) {
+                seg_add(sem, acc, t.w[i0 + i], x[i]);
+                if (!one_row) end_tile(i0 + i);
             }
         }
-        if (lane == 0) {
-            const bool head = row_start == ls.cs;  // the row begins with this chunk
-            if (head && ls.cs > 0)                 // empty tile-rows just before it
-                for (int32_t R = ra - 1; R >= 0 && __ldg(g.rowptr + R) == ls.cs; --R) sem.store(R, idv);
-            if (head && c + 1 == g.nchunks) {
-                sem.store(ra, acc);  // begins and ends in this chunk (the matrix's last)
-            } else {
-                // continued by later chunks (head) or begun in earlier ones
-                V* dst = (head ? part.val_last : part.val_first) + (int64_t)c * NV;
+    } else {
+        uint32_t xs[8];
 #pragma unroll
-                for (int v = 0; v < NV; ++v) dst[v] = acc.get(v);
+        for (int i = 0; i < 8; ++i) {
+            if constexpr (MODE == kSmBitsShared)
+                xs[i] = K == 8 ? sx[t.cu[i]] : (sx[t.cu[i] >> 1] >> (4 * (t.cu[i] & 1u))) & 0xFu;
+            else
+                xs[i] = sem.xseg((int32_t)t.cu[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            sem.tile(acc, t.w + i * TW, xs[i]);
+            if (!one_row) end_tile(i);
+        }
+    }
+    if (one_row) {
+        const bool head = __shfl_sync(0xffffffffu, t.win, 0) == cs;  // the row begins with this chunk
+        join_lanes(sem, acc, lane);
+        if (head && c + 1 == g.nchunks) {  // begins and ends in this chunk (the matrix's last)
+            if constexpr (SEM::kGather) {
+                if (lane < 4) sem.store_row(t.ra, (lane >> 1) | ((lane & 1) << 1), acc.get(0));
+            } else if (lane == 0) {
+                sem.store(t.ra, acc);
             }
+            return;
+        }
+        // continued by later chunks (head) or begun in earlier ones
+        V* dst = (head ? part.val_last : part.val_first) + (int64_t)c * NV;
+        if constexpr (SEM::kGather) {
+            if (lane < 4) dst[(lane >> 1) | ((lane & 1) << 1)] = acc.get(0);
+        } else if (lane == 0) {
+#pragma unroll
+            for (int v = 0; v < NV; ++v) dst[v] = acc.get(v);
         }
         return;
     }
-    const RowCursor rc = locate_row_win(g, ra, rb - ra, t.win, ls, lane);
-    Walk<SEM, RegAcc<V, NV>> wk;
-    wk.row = rc.row;
-    wk.next = rc.next;
-    if (ls.cnt > 0) {
-        // empty tile-rows just before a row that starts at this lane's first tile
-        if (ls.tl > 0 && rc.row_start == ls.tl)
-            for (int32_t R = rc.row - 1; R >= 0 && __ldg(g.rowptr + R) == ls.tl; --R) sem.store(R, idv);
-#pragma unroll
-        for (int i = 0; i < P; ++i) {
-            if (i < ls.cnt) {
-                if constexpr (SEM::kGather) k4_gather_tile(sem, acc, t.w[i], (int32_t)t.cu[i]);
-                else sem.tile(acc, t.w + i, xs[i]);
-                wk.end_tile(g, sem, acc, F, ls.tl + i, i, ls.cnt, idv);
-            }
-        }
-    }
-    close_chunk(sem, part, c, ls, lane, rc.head_cs, rc.row, wk.has_end, wk.open, acc, F, P);
+    LaneSpan ls;
+    ls.cs = cs;
+    ls.ce = ce;
+    const bool head_cs = __shfl_sync(0xffffffffu, t.win, 0) == cs;
+    // a tail after the chunk's last row end is continued by the next chunk
+    const bool open = !((s.mask[(ce - 1 - cs) >> 5] >> ((ce - 1 - cs) & 31)) & 1u);
+    const int32_t first_row = has_end ? s.row[rank0] : 0;
+    close_chunk(sem, part, c, ls, lane, head_cs, first_row, has_end, open, acc, F, Sh::P);
 }
 
-template <class SEM>
-__global__ void __launch_bounds__(kSpmvThreads, kK4MinBlocks)
-    spmv_k4_kernel(SpmvGeom g, SEM sem, Partials<typename SEM::V> part) {
+// Dynamic shared memory: a ChunkRows per warp, then (kSmBitsShared) the input bitset.
+template <int K, class SEM, int MODE>
+__device__ __forceinline__ void small_body(const SpmvGeom& g, const SEM& sem, Partials<typename SEM::V> part) {
+    constexpr int WARPS = small_threads<K, MODE>() / 32;
+    extern __shared__ __align__(16) uint8_t small_smem[];
+    if (gated_off(g.gate)) return;
+    ChunkRows* rows = reinterpret_cast<ChunkRows*>(small_smem) + (threadIdx.x >> 5);
+    const uint8_t* sx = small_smem + WARPS * sizeof(ChunkRows);
     const int lane = (int)lane_id();
-    const int32_t W = (int32_t)gridDim.x * kSpmvWarps;
-    int32_t c = (int32_t)blockIdx.x * kSpmvWarps + (threadIdx.x >> 5);
-    if (c >= g.nchunks || gated_off(g.gate)) return;  // whole warps leave together
-    K4Tiles cur, nxt;
-    k4_load(g, sem, c, lane, cur);
+    const int32_t W = (int32_t)gridDim.x * WARPS;
+    int32_t c = (int32_t)blockIdx.x * WARPS + (threadIdx.x >> 5);
+    SmallTiles<K> cur, nxt;
+    if (c < g.nchunks) small_load<K>(g, sem, c, lane, cur);
+    if constexpr (MODE == kSmBitsShared) {
+        uint32_t* dst = reinterpret_cast<uint32_t*>(small_smem + WARPS * sizeof(ChunkRows));
+        const int words = (sem.n + 31) / 32;
+        int at = 0;
+        if (reinterpret_cast<uintptr_t>(sem.x) % 16 == 0) {
+            const uint4* src = reinterpret_cast<const uint4*>(sem.x);
+            for (int i = threadIdx.x; i < words / 4; i += WARPS * 32) reinterpret_cast<uint4*>(dst)[i] = __ldg(src + i);
+            at = words & ~3;
+        }
+        for (int i = at + threadIdx.x; i < words; i += WARPS * 32) dst[i] = __ldg(sem.x + i);
+        __syncthreads();
+    }
+    if (c >= g.nchunks) return;  // whole warps leave together
     for (;;) {
         const int32_t cn = c + W;
         const bool more = cn < g.nchunks;
-        if (more) k4_load(g, sem, cn, lane, nxt);
-        k4_chunk(g, sem, part, c, lane, cur);
+        if (more) small_load<K>(g, sem, cn, lane, nxt);
+        small_chunk<K, SEM, MODE>(g, sem, part, c, lane, cur, *rows, sx);
         if (!more) break;
         c = cn;
         cur = nxt;
     }
+}
+
+// k = 4 with the bit-vector schemes and 4-byte values; the other small-tile
+// cases (k = 8, 8-byte values).
+template <class SEM, int MODE>
+__global__ void __launch_bounds__((small_threads<4, MODE>()), (small_min_blocks<4, SEM, MODE>()))
+    spmv_k4_kernel(SpmvGeom g, SEM sem, Partials<typename SEM::V> part) {
+    small_body<4, SEM, MODE>(g, sem, part);
+}
+template <int K, class SEM, int MODE>
+__global__ void __launch_bounds__((small_threads<K, MODE>()), (small_min_blocks<K, SEM, MODE>()))
+    spmv_chunks_kernel(SpmvGeom g, SEM sem, Partials<typename SEM::V> part) {
+    small_body<K, SEM, MODE>(g, sem, part);
 }
 
 // ---------------------------------------------------------------------------
@@ -1580,28 +1774,56 @@ static double spmv_bytes(const b2sr_matrix* h, double vec_bytes) {
     return 4.0 * ((double)h->ntr + 1.0) + (double)h->T * (4.0 + tile_bytes(h->k)) + vec_bytes;
 }
 
-// The tile_dim-4 kernel serves, at k = 4, the bit-vector schemes and the
-// unweighted value schemes with 4-byte values (plus-times, the label min, fp32
-// max); 8-byte values would not fit its registers without spilling.
+// The small-tile kernel serves the bit-vector schemes at k = 4 and 8 and the
+// unweighted value schemes with 4- and 8-byte values at k = 4.
 template <int K, class SEM>
-constexpr bool use_k4() {
-    if constexpr (!SEM::kGather) return K == 4;
-    else return K == 4 && !SEM::kMayWeight && sizeof(typename SEM::V) == 4;
+constexpr bool use_small() {
+    if constexpr (!SEM::kGather) return K <= 8;
+    else return K == 4 && !SEM::kMayWeight && sizeof(typename SEM::V) <= 8;
 }
 
-// The direct chunk kernel: the tile_dim-4 one where it serves, else the
+template <int K, class SEM, int MODE>
+static b2sr_status launch_small(const b2sr_matrix* h, const SEM& sem, Partials<typename SEM::V> part, cudaStream_t s,
+                                const SpmvGeom& g) {
+    // persistent: the resident blocks, each warp looping over chunks
+    constexpr int threads = small_threads<K, MODE>();
+    const unsigned grid = (unsigned)std::min<int64_t>(ceil_div(h->nchunks, threads / 32),
+                                                      (int64_t)sm_count() * small_min_blocks<K, SEM, MODE>());
+    const int smem = threads / 32 * (int)sizeof(ChunkRows) + (MODE == kSmBitsShared ? (int)ceil_div(h->n, 32) * 4 : 0);
+    void (*kernel)(SpmvGeom, SEM, Partials<typename SEM::V>);
+    if constexpr (K == 4 && sizeof(typename SEM::V) == 4) kernel = spmv_k4_kernel<SEM, MODE>;
+    else kernel = spmv_chunks_kernel<K, SEM, MODE>;
+    if (smem > 48 * 1024)
+        B2SR_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    kernel<<<grid, threads, smem, s>>>(g, sem, part);
+    B2SR_LAUNCH_CHECK("small-tile SpMV kernel");
+    return B2SR_OK;
+}
+
+// The direct chunk kernel: the small-tile one where it serves, else the
 // general one.
 template <int K, class SEM>
 static b2sr_status launch_direct(const b2sr_matrix* h, const SEM& sem, Partials<typename SEM::V> part,
                                  cudaStream_t s, const SpmvGeom& g) {
-    const unsigned blocks = (unsigned)ceil_div(h->nchunks, kSpmvWarps);
-    if constexpr (use_k4<K, SEM>()) {
-        // persistent: the resident blocks, each warp looping over chunks
-        const unsigned grid = (unsigned)std::min<int64_t>(blocks, (int64_t)sm_count() * kK4MinBlocks);
-        spmv_k4_kernel<SEM><<<grid, kSpmvThreads, 0, s>>>(g, sem, part);
-        B2SR_LAUNCH_CHECK("spmv_k4_kernel");
+    if constexpr (use_small<K, SEM>()) {
+        if constexpr (!SEM::kGather) {
+            // The bitset of x in shared memory (x gathers at one distinct 128-byte
+            // line a cycle were what bound the kernel) when it fits and a warp has a
+            // few chunks to spread the copy over: R-MAT 20, k = 4 / k = 8, Boolean:
+            // 75 / 74.7 us without, 68 / 72.5 with it; permuted ids 76 / 89 and 67 / 82.
+            constexpr int threads = small_threads<K, kSmBitsShared>();
+            if (h->nchunks >= (int64_t)sm_count() * (threads / 32) * 4 &&
+                ceil_div(h->n, 32) * 4 + threads / 32 * (int64_t)sizeof(ChunkRows) <= kMaxBlockSmem)
+                return launch_small<K, SEM, kSmBitsShared>(h, sem, part, s, g);
+            return launch_small<K, SEM, kSmBits>(h, sem, part, s, g);
+        } else {
+            // whole segments need an aligned input without a ragged last one
+            const bool segs = h->n % 4 == 0 && reinterpret_cast<uintptr_t>(sem.x) % (4 * sizeof(typename SEM::G)) == 0;
+            if (segs) return launch_small<K, SEM, kSmSegs>(h, sem, part, s, g);
+            return launch_small<K, SEM, kSmVals>(h, sem, part, s, g);
+        }
     } else {
-        spmv_chunks_kernel<K, SEM><<<blocks, kSpmvThreads, 0, s>>>(g, sem, part);
+        spmv_chunks_kernel<K, SEM><<<(unsigned)ceil_div(h->nchunks, kSpmvWarps), kSpmvThreads, 0, s>>>(g, sem, part);
         B2SR_LAUNCH_CHECK("spmv_chunks_kernel");
     }
     return B2SR_OK;
