@@ -253,9 +253,8 @@ def b2sr_autotune(n: int, rowptr: torch.Tensor, colind: torch.Tensor, sample, se
 def b2sr_to_csr(m: Matrix, stream=None):
     dev = torch.device("cuda", torch.cuda.current_device())
     rowptr = torch.empty(m.n + 1, dtype=torch.int32, device=dev)
+    colind = torch.empty(max(m.nnz, 1), dtype=torch.int32, device=dev)
     nnz = ctypes.c_int64()
-    _check(lib.b2sr_to_csr(m.handle, _ptr(rowptr), None, ctypes.byref(nnz), _stream(stream)))
-    colind = torch.empty(max(nnz.value, 1), dtype=torch.int32, device=dev)
     _check(lib.b2sr_to_csr(m.handle, _ptr(rowptr), _ptr(colind), ctypes.byref(nnz), _stream(stream)))
     return rowptr, colind[: nnz.value]
 

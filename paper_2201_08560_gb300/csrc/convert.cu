@@ -20,6 +20,7 @@
 #include "b2sr_internal.cuh"
 
 namespace b2sr {
+b2sr_status row_counts(const b2sr_matrix* h, int32_t* cnt, int32_t* first, int32_t* last, cudaStream_t s);
 
 // ---------------------------------------------------------------------------
 // input validation
@@ -865,40 +866,123 @@ b2sr_status ensure_outdeg(b2sr_matrix* h, cudaStream_t s) {
 // ---------------------------------------------------------------------------
 // B2SR -> CSR
 // ---------------------------------------------------------------------------
+// Ones per row come from the row-count SpMV (spmv.cu), which also leaves the
+// partial counts of the tile-rows that cross chunks; a scan makes them row
+// pointers.  The columns are then written by a warp per chunk of tiles, 32
+// tiles a step: an entry's place is its row's pointer, plus the row's ones in
+// earlier chunks (the partials), plus those in earlier steps (a carry), plus
+// those in earlier tiles of the step (a scan over the lanes that restarts at
+// every tile-row).  The work is balanced over tiles, so a hub's row of 10^5
+// tiles is shared by many warps (a thread a row walked it alone).
 template <int K>
-__global__ void row_nnz_kernel(const int32_t* __restrict__ trp, const uint8_t* __restrict__ tiles,
-                               int32_t n, int32_t* __restrict__ cnt) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        int64_t I = i / K;
-        int r = (int)(i % K);
-        int c = 0;
-        for (int64_t t = trp[I]; t < trp[I + 1]; ++t) c += __popc(tile_word<K>(tiles, t, r));
-        cnt[i] = c;
+__global__ void __launch_bounds__(256) csr_fill_kernel(const int32_t* __restrict__ trp,
+                                                       const int32_t* __restrict__ tci,
+                                                       const uint8_t* __restrict__ tiles, int64_t T, int64_t nchunks,
+                                                       const int32_t* __restrict__ chunk_row,
+                                                       const int64_t* __restrict__ off,
+                                                       const int32_t* __restrict__ first,
+                                                       const int32_t* __restrict__ last,
+                                                       int32_t* __restrict__ colind) {
+    constexpr unsigned FULL = 0xffffffffu;
+    constexpr int CT = chunk_tiles(K);
+    constexpr int H = K / 2;  // 16-bit counters, two a word (a chunk holds at most 2,048 ones of a row)
+    __shared__ int32_t s_base[8][K];
+    const int lane = (int)lane_id(), warp = threadIdx.x >> 5;
+    const int64_t c = (int64_t)blockIdx.x * 8 + warp;
+    if (c >= nchunks) return;  // whole warps leave together
+    const int32_t cs = (int32_t)(c * CT), ce = (int32_t)min((int64_t)cs + CT, T);
+    const int32_t ra = __ldg(chunk_row + c), rb = __ldg(chunk_row + c + 1);
+    // ones of tile-row ra in earlier chunks
+    const int32_t rs = __ldg(trp + ra);
+    {
+        constexpr int L = 32 / K;  // lanes a row: lane l takes row l % K of every L-th chunk
+        const int64_t ca = rs / CT;
+        int32_t v = 0;
+        if (rs < cs)
+            for (int64_t q = ca + lane / K; q < c; q += L) v += __ldg((q == ca ? last : first) + q * K + lane % K);
+#pragma unroll
+        for (int o = K; o < 32; o <<= 1) v += __shfl_xor_sync(FULL, v, o);
+        if (lane < K) s_base[warp][lane] = v;
+    }
+    __syncwarp();
+    uint32_t carry[H];  // ones of tile-row crow in earlier steps
+    int32_t crow = ra;
+#pragma unroll
+    for (int h = 0; h < H; ++h) carry[h] = 0u;
+    for (int32_t g0 = cs; g0 < ce; g0 += 32) {
+        const int32_t t = g0 + lane;
+        const bool live = t < ce;
+        int32_t lo = ra, hi = rb;  // the tile's row: the last one starting at or before t
+        while (lo < hi) {
+            const int32_t mid = lo + ((hi - lo + 1) >> 1);
+            if (__ldg(trp + mid) <= t) lo = mid; else hi = mid - 1;
+        }
+        const int32_t I = lo;
+        uint32_t row[K], inc[H];
+#pragma unroll
+        for (int r = 0; r < K; ++r) row[r] = live ? tile_word<K>(tiles, t, r) : 0u;
+#pragma unroll
+        for (int h = 0; h < H; ++h) inc[h] = __popc(row[2 * h]) | (__popc(row[2 * h + 1]) << 16);
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int32_t Io = __shfl_up_sync(FULL, I, d);
+            const bool same = lane >= d && Io == I;
+#pragma unroll
+            for (int h = 0; h < H; ++h) {
+                const uint32_t o = __shfl_up_sync(FULL, inc[h], d);
+                if (same) inc[h] += o;
+            }
+        }
+        if (I == crow) {
+#pragma unroll
+            for (int h = 0; h < H; ++h) inc[h] += carry[h];
+        }
+        if (live) {
+            const int32_t j0 = __ldg(tci + t) * K;
+#pragma unroll
+            for (int r = 0; r < K; ++r) {
+                uint32_t b = row[r];
+                if (!b) continue;
+                const int32_t before = (int32_t)((inc[r / 2] >> (16 * (r & 1))) & 0xFFFFu) - __popc(b);
+                int64_t at = __ldg(off + (int64_t)I * K + r) + before + (I == ra ? s_base[warp][r] : 0);
+                do {
+                    colind[at++] = j0 + __ffs(b) - 1;
+                    b &= b - 1;
+                } while (b);
+            }
+        }
+        crow = __shfl_sync(FULL, I, 31);
+#pragma unroll
+        for (int h = 0; h < H; ++h) carry[h] = __shfl_sync(FULL, inc[h], 31);
     }
 }
 
-template <int K>
-__global__ void row_fill_kernel(const int32_t* __restrict__ trp, const int32_t* __restrict__ tci,
-                                const uint8_t* __restrict__ tiles, int32_t n,
-                                const int64_t* __restrict__ off, int32_t* __restrict__ rowptr,
-                                int32_t* __restrict__ colind) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i <= n;
-         i += (int64_t)gridDim.x * blockDim.x) {
+__global__ void rowptr_out_kernel(const int64_t* __restrict__ off, int64_t len, int32_t* __restrict__ rowptr) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < len; i += (int64_t)gridDim.x * blockDim.x)
         rowptr[i] = (int32_t)off[i];
-        if (i == n || colind == nullptr) continue;
-        int64_t I = i / K;
-        int r = (int)(i % K);
-        int64_t w = off[i];
-        for (int64_t t = trp[I]; t < trp[I + 1]; ++t) {
-            uint32_t bits = tile_word<K>(tiles, t, r);
-            while (bits) {
-                int c = __ffs(bits) - 1;
-                bits &= bits - 1;
-                colind[w++] = tci[t] * K + c;
-            }
-        }
-    }
+}
+
+b2sr_status extract_csr(const b2sr_matrix* h, int64_t* off, int32_t* rowptr, int32_t* colind, cudaStream_t s) {
+    const int32_t n = h->n;
+    DevBuf cnt(s), part(s);
+    B2SR_TRY(cnt.alloc(((size_t)n + 1) * sizeof(int32_t)));
+    const size_t np = (size_t)h->nchunks * h->k;
+    B2SR_TRY(part.alloc(std::max<size_t>(2 * np, 1) * sizeof(int32_t)));
+    int32_t* first = part.as<int32_t>();
+    int32_t* last = first + np;
+    B2SR_CUDA_TRY(cudaMemsetAsync(cnt.as<int32_t>() + n, 0, sizeof(int32_t), s));
+    B2SR_TRY(row_counts(h, cnt.as<int32_t>(), first, last, s));
+    B2SR_TRY(exclusive_scan_i32_to_i64(cnt.as<int32_t>(), off, (int64_t)n + 1, s));
+    rowptr_out_kernel<<<grid_wide((int64_t)n + 1), 256, 0, s>>>(off, (int64_t)n + 1, rowptr);
+    B2SR_LAUNCH_CHECK("rowptr_out_kernel");
+    if (!colind || h->nchunks == 0) return B2SR_OK;
+    return with_tile(h->k, [&](auto kc) -> b2sr_status {
+        constexpr int K = decltype(kc)::value;
+        csr_fill_kernel<K><<<(unsigned)ceil_div(h->nchunks, 8), 256, 0, s>>>(
+            h->rowptr, h->colind, h->tiles, h->T, h->nchunks, h->chunk_row, off, first, last, colind);
+        B2SR_LAUNCH_CHECK("csr_fill_kernel");
+        return B2SR_OK;
+    });
 }
 
 // ---------------------------------------------------------------------------
@@ -1150,23 +1234,11 @@ extern "C" b2sr_status b2sr_to_csr(b2sr_handle h, int32_t* rowptr, int32_t* coli
     B2SR_TRY(check_handle(h));
     if (!rowptr) return fail(B2SR_ERR_INVALID_ARG, "rowptr is NULL");
     cudaStream_t s = to_stream(stream);
-    const int32_t n = h->n;
-    DevBuf cnt(s), off(s);
-    B2SR_TRY(cnt.alloc(((size_t)n + 1) * sizeof(int32_t)));
-    B2SR_TRY(off.alloc(((size_t)n + 1) * sizeof(int64_t)));
-    B2SR_CUDA_TRY(cudaMemsetAsync(cnt.as<int32_t>() + n, 0, sizeof(int32_t), s));
-    B2SR_TRY(with_tile(h->k, [&](auto kc) -> b2sr_status {
-        constexpr int K = decltype(kc)::value;
-        if (n > 0) row_nnz_kernel<K><<<grid_wide(n), 256, 0, s>>>(h->rowptr, h->tiles, n, cnt.as<int32_t>());
-        B2SR_LAUNCH_CHECK("row_nnz_kernel");
-        B2SR_TRY(exclusive_scan_i32_to_i64(cnt.as<int32_t>(), off.as<int64_t>(), (int64_t)n + 1, s));
-        row_fill_kernel<K><<<grid_wide((int64_t)n + 1), 256, 0, s>>>(h->rowptr, h->colind, h->tiles, n,
-                                                                   off.as<int64_t>(), rowptr, colind);
-        B2SR_LAUNCH_CHECK("row_fill_kernel");
-        return B2SR_OK;
-    }));
+    DevBuf off(s);
+    B2SR_TRY(off.alloc(((size_t)h->n + 1) * sizeof(int64_t)));
+    B2SR_TRY(extract_csr(h, off.as<int64_t>(), rowptr, colind, s));
     int64_t nnz = 0;
-    B2SR_CUDA_TRY(cudaMemcpyAsync(&nnz, off.as<int64_t>() + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    B2SR_CUDA_TRY(cudaMemcpyAsync(&nnz, off.as<int64_t>() + h->n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     B2SR_CUDA_TRY(cudaStreamSynchronize(s));
     if (nnz_host) *nnz_host = nnz;
     return B2SR_OK;

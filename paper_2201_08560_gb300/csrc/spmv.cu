@@ -303,6 +303,13 @@ struct SemCount {
     }
 };
 
+// ones per row: the count of a vector of ones, which needs no input
+template <int K>
+struct SemOnes : SemCount<K> {
+    static constexpr bool kNoInput = true;
+    __device__ uint32_t xseg(int32_t) const { return K == 32 ? 0xFFFFFFFFu : (1u << (K & 31)) - 1u; }
+};
+
 // bmv_bin_full_full over plus-times: float in, float out; partials of rows
 // that cross chunks are joined with a compensated fp32 sum (CSum)
 template <int K>
@@ -1707,6 +1714,12 @@ struct HasSelfTerm : std::false_type {};
 template <class S>
 struct HasSelfTerm<S, std::void_t<decltype(S::kSelfTerm)>> : std::bool_constant<S::kSelfTerm> {};
 
+// schemes that read no input vector
+template <class S, class = void>
+struct NoInput : std::false_type {};
+template <class S>
+struct NoInput<S, std::void_t<decltype(S::kNoInput)>> : std::bool_constant<S::kNoInput> {};
+
 template <class T>
 __device__ __forceinline__ T min_self(T a, T b) {
     if constexpr (std::is_same<T, float>::value) return fminf(a, b);
@@ -1812,9 +1825,10 @@ static b2sr_status launch_direct(const b2sr_matrix* h, const SEM& sem, Partials<
             // few chunks to spread the copy over: R-MAT 20, k = 4 / k = 8, Boolean:
             // 75 / 74.7 us without, 68 / 72.5 with it; permuted ids 76 / 89 and 67 / 82.
             constexpr int threads = small_threads<K, kSmBitsShared>();
-            if (h->nchunks >= (int64_t)sm_count() * (threads / 32) * 4 &&
-                ceil_div(h->n, 32) * 4 + threads / 32 * (int64_t)sizeof(ChunkRows) <= kMaxBlockSmem)
-                return launch_small<K, SEM, kSmBitsShared>(h, sem, part, s, g);
+            if constexpr (!NoInput<SEM>::value)
+                if (h->nchunks >= (int64_t)sm_count() * (threads / 32) * 4 &&
+                    ceil_div(h->n, 32) * 4 + threads / 32 * (int64_t)sizeof(ChunkRows) <= kMaxBlockSmem)
+                    return launch_small<K, SEM, kSmBitsShared>(h, sem, part, s, g);
             return launch_small<K, SEM, kSmBits>(h, sem, part, s, g);
         } else {
             // whole segments need an aligned input without a ragged last one
@@ -1873,6 +1887,28 @@ static b2sr_status run_spmv(const b2sr_matrix* h, const SEM& sem, uint32_t* bits
     return B2SR_OK;
 }
 
+
+// Ones per row, and the partial counts of the tile-rows that cross chunks
+// (first, last: nchunks * k each): last[c] holds what chunk c has of a row
+// continued from it, first[c] what it has of a row begun before it.
+b2sr_status row_counts(const b2sr_matrix* h, int32_t* cnt, int32_t* first, int32_t* last, cudaStream_t s) {
+    return with_tile(h->k, [&](auto kc) -> b2sr_status {
+        constexpr int K = decltype(kc)::value;
+        using SEM = SemOnes<K>;
+        SEM sem;
+        sem.x = nullptr;
+        sem.y = cnt;
+        sem.mask = nullptr;
+        sem.comp = 0;
+        sem.n = h->n;
+        SpmvGeom g{h->rowptr, h->colind, h->tiles, h->chunk_row, h->T, h->nchunks, h->ntr, nullptr};
+        B2SR_TRY((launch_edges<K, SEM>(h, sem, s, nullptr)));
+        if (h->nchunks == 0) return B2SR_OK;
+        const Partials<int32_t> part{first, last};
+        B2SR_TRY((launch_direct<K, SEM>(h, sem, part, s, g)));
+        return launch_fixup<K, SEM>(h, sem, part, s, nullptr);
+    });
+}
 
 b2sr_status spmv_dispatch(b2sr_matrix* h, b2sr_semiring sr, b2sr_vec in_kind, const void* x, b2sr_vec out_kind,
                           void* y, const uint32_t* mask, int comp, const float* weights, cudaStream_t s,
