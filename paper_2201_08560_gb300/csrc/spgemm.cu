@@ -146,6 +146,138 @@ __global__ void masked_count_kernel(MatView A, MatView B, MatView M, unsigned lo
 }
 
 // ---------------------------------------------------------------------------
+// masked count over rows
+// ---------------------------------------------------------------------------
+// For every mask entry (i, j): the columns common to row i of A and row j of
+// B.  The three operands' rows are extracted as column lists first (one
+// balanced pass over their tiles); then a block takes kRunEntries consecutive
+// mask entries, row by row:
+//   * a row of A with more than 32 columns becomes a bitmap in the block's
+//     shared memory; the row's mask entries are dealt to the warps, and the
+//     lanes of a warp walk row j of B, testing each column in the bitmap: a
+//     coalesced load and one shared load per column, no searches;
+//   * a shorter row of A stays a list: the warps take such rows one by one,
+//     a group of lanes (as wide as the row) per mask entry, each lane
+//     searching its column in row j of B.
+// Where a bitmap of n bits does not fit in shared memory every row takes the
+// second form.
+constexpr int kRunEntries = 256;
+constexpr int64_t kMaxBitmapBytes = 200 * 1024;
+
+struct RowLists {
+    const int32_t* rowptr;
+    const int32_t* colind;
+};
+
+// Ones of the short row list a[0..d) in row j of B, over mask entries
+// [e0, e1), by one warp.
+__device__ __forceinline__ uint32_t count_listed(const int32_t* __restrict__ acol, int32_t d, RowLists B,
+                                                 const int32_t* __restrict__ mcol, int32_t e0, int32_t e1, int lane) {
+    int width = 32;  // lanes a mask entry: the least power of two holding the row
+    while (width > 1 && width / 2 >= d) width >>= 1;
+    const int sub = lane & (width - 1);
+    uint32_t acc = 0;
+    for (int32_t e = e0 + lane / width; e < e1; e += 32 / width) {
+        const int32_t j = __ldg(mcol + e);
+        const int32_t b0 = __ldg(B.rowptr + j), b1 = __ldg(B.rowptr + j + 1);
+        for (int32_t p = sub; p < d; p += width) {
+            const int32_t v = __ldg(acol + p);
+            const int32_t q = lower_bound_i32(B.colind, b0, b1, v);
+            acc += q < b1 && __ldg(B.colind + q) == v;
+        }
+    }
+    return acc;
+}
+
+__global__ void __launch_bounds__(256) masked_rows_kernel(int32_t n, RowLists A, RowLists B, RowLists M,
+                                                          int32_t mnnz, int use_bitmap, int bitmap_words,
+                                                          unsigned long long* __restrict__ out) {
+    extern __shared__ __align__(16) uint32_t bitmap[];
+    __shared__ unsigned long long warp_sum[8];
+    __shared__ int32_t long_row[kRunEntries];  // at least one mask entry of the run in each
+    __shared__ int nlong;
+    const int lane = (int)lane_id(), warp = threadIdx.x >> 5;
+    const int32_t e0 = (int32_t)blockIdx.x * kRunEntries;
+    const int32_t e1 = min(e0 + kRunEntries, mnnz);
+    // rows of the first and the last mask entry of the run
+    auto row_of_entry = [&](int32_t e) {
+        int32_t lo = 0, hi = n - 1;  // the last row starting at or before e
+        while (lo < hi) {
+            const int32_t mid = lo + ((hi - lo + 1) >> 1);
+            if (__ldg(M.rowptr + mid) <= e) lo = mid; else hi = mid - 1;
+        }
+        return lo;
+    };
+    const int32_t i0 = row_of_entry(e0), i1 = row_of_entry(e1 - 1);
+    if (use_bitmap)
+        for (int w = threadIdx.x; w < bitmap_words; w += 256) bitmap[w] = 0u;
+    if (threadIdx.x == 0) nlong = 0;
+    __syncthreads();
+    uint32_t acc = 0;
+    const int32_t listed = use_bitmap ? 32 : INT32_MAX;  // longest row taken as a list
+    for (int32_t base = i0; base <= i1; base += 256) {
+        const int32_t i = base + 8 * lane + warp;  // neighbouring rows go to different warps
+        int32_t a0 = 0, d = 0, m0 = 0, m1 = 0;
+        if (i <= i1) {
+            a0 = __ldg(A.rowptr + i);
+            d = __ldg(A.rowptr + i + 1) - a0;
+            m0 = max(e0, __ldg(M.rowptr + i));
+            m1 = min(e1, __ldg(M.rowptr + i + 1));
+        }
+        const bool live = d > 0 && m0 < m1;
+        if (live && d > listed) long_row[atomicAdd(&nlong, 1)] = i;
+        for (unsigned todo = __ballot_sync(0xffffffffu, live && d <= listed); todo; todo &= todo - 1) {
+            const int src = __ffs(todo) - 1;
+            acc += count_listed(A.colind + __shfl_sync(0xffffffffu, a0, src), __shfl_sync(0xffffffffu, d, src), B,
+                                M.colind, __shfl_sync(0xffffffffu, m0, src), __shfl_sync(0xffffffffu, m1, src), lane);
+        }
+    }
+    if (use_bitmap) {
+        __syncthreads();
+        for (int r = 0; r < nlong; ++r) {
+            const int32_t i = long_row[r];
+            const int32_t a0 = __ldg(A.rowptr + i), a1 = __ldg(A.rowptr + i + 1);
+            const int32_t m0 = max(e0, __ldg(M.rowptr + i)), m1 = min(e1, __ldg(M.rowptr + i + 1));
+            for (int32_t p = a0 + threadIdx.x; p < a1; p += 256) {
+                const int32_t v = __ldg(A.colind + p);
+                atomicOr(bitmap + (v >> 5), 1u << (v & 31));
+            }
+            __syncthreads();
+            // lane l of warp w holds mask entry m0 + 8 l + w (at most 256 entries a run)
+            const int32_t e = m0 + 8 * lane + warp;
+            int32_t b0 = 0, b1 = 0;
+            if (e < m1) {
+                const int32_t j = __ldg(M.colind + e);
+                b0 = __ldg(B.rowptr + j);
+                b1 = __ldg(B.rowptr + j + 1);
+            }
+            const int cnt = m1 - m0 > warp ? (m1 - m0 - warp + 7) / 8 : 0;
+            for (int q = 0; q < cnt; ++q) {
+                const int32_t s0 = __shfl_sync(0xffffffffu, b0, q), s1 = __shfl_sync(0xffffffffu, b1, q);
+#pragma unroll 4
+                for (int32_t p = s0 + lane; p < s1; p += 32) {
+                    const int32_t v = __ldg(B.colind + p);
+                    acc += (bitmap[v >> 5] >> (v & 31)) & 1u;
+                }
+            }
+            __syncthreads();
+            for (int32_t p = a0 + threadIdx.x; p < a1; p += 256) bitmap[__ldg(A.colind + p) >> 5] = 0u;
+            __syncthreads();
+        }
+    }
+    unsigned long long sum = acc;
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (lane == 0) warp_sum[warp] = sum;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned long long total = 0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) total += warp_sum[w];
+        if (total) atomicAdd(out, total);
+    }
+}
+
+// ---------------------------------------------------------------------------
 // Boolean SpGEMM (expand, sort, merge)
 // ---------------------------------------------------------------------------
 __global__ void row_of_tiles_kernel(const int32_t* __restrict__ rowptr, int32_t ntr, int64_t T,
@@ -246,8 +378,42 @@ __global__ void build_rowptr_from_rows(const int32_t* __restrict__ tilerow, int6
 
 static MatView view(const b2sr_matrix* h) { return MatView{h->rowptr, h->colind, h->tiles, h->T, h->ntr}; }
 
+// Row lists of a handle, owned by `buf`.
+static b2sr_status row_lists(const b2sr_matrix* h, DevBuf& buf, RowLists* out, cudaStream_t s) {
+    DevBuf off(s);
+    const size_t rp = round_up(((int64_t)h->n + 1) * sizeof(int32_t), 256);
+    B2SR_TRY(off.alloc(((size_t)h->n + 1) * sizeof(int64_t)));
+    B2SR_TRY(buf.alloc(rp + (size_t)h->nnz * sizeof(int32_t) + 4));
+    int32_t* rowptr = buf.as<int32_t>();
+    int32_t* colind = reinterpret_cast<int32_t*>(buf.as<char>() + rp);
+    B2SR_TRY(extract_csr(h, off.as<int64_t>(), rowptr, colind, s));
+    *out = RowLists{rowptr, colind};
+    return B2SR_OK;
+}
+
+static b2sr_status masked_count_rows(const b2sr_matrix* A, const b2sr_matrix* B, const b2sr_matrix* M,
+                                     unsigned long long* out, cudaStream_t s, double bytes) {
+    DevBuf abuf(s), bbuf(s), mbuf(s);
+    RowLists a, b, m;
+    B2SR_TRY(row_lists(A, abuf, &a, s));
+    if (B == A) b = a; else B2SR_TRY(row_lists(B, bbuf, &b, s));
+    if (M == A) m = a; else if (M == B) m = b; else B2SR_TRY(row_lists(M, mbuf, &m, s));
+    const int64_t words = ceil_div(A->n, 32);
+    const int use_bitmap = words * 4 <= kMaxBitmapBytes;
+    const int smem = use_bitmap ? (int)words * 4 : 0;
+    B2SR_CUDA_TRY(cudaFuncSetAttribute(masked_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    void* tok = timing_begin(s);
+    masked_rows_kernel<<<(unsigned)ceil_div(M->nnz, kRunEntries), 256, smem, s>>>(A->n, a, b, m, (int32_t)M->nnz,
+                                                                                use_bitmap, (int)words, out);
+    timing_end(tok, "spgemm_masked", bytes, s);
+    B2SR_LAUNCH_CHECK("masked_rows_kernel");
+    return B2SR_OK;
+}
+
 // The masked count; `pairs` (device int64, optional) receives the number of
-// AND-popc word operations done (one per mask bit per common tile-column).
+// AND-popc word operations of the tile form (one per mask bit per common
+// tile-column).  The row form extracts all of A's and B's rows, so a mask of
+// far fewer tiles than they have takes the tile form.
 b2sr_status masked_count(const b2sr_matrix* A, const b2sr_matrix* B, const b2sr_matrix* M, int64_t* count,
                          cudaStream_t s, int64_t* pairs) {
     B2SR_CUDA_TRY(cudaMemsetAsync(count, 0, sizeof(int64_t), s));
@@ -256,6 +422,9 @@ b2sr_status masked_count(const b2sr_matrix* A, const b2sr_matrix* B, const b2sr_
     auto* out = reinterpret_cast<unsigned long long*>(count);
     auto* prs = reinterpret_cast<unsigned long long*>(pairs);
     const double bytes = 3.0 * (4.0 * ((double)A->ntr + 1.0)) + ((double)A->T + B->T + M->T) * (4.0 + tile_bytes(A->k));
+    const int64_t most = std::max(A->nnz, std::max(B->nnz, M->nnz));
+    if (!pairs && most < (int64_t(1) << 31) - kRunEntries && 16 * M->T >= A->T + B->T)
+        return masked_count_rows(A, B, M, out, s, bytes);
     return with_tile(A->k, [&](auto kc) -> b2sr_status {
         constexpr int K = decltype(kc)::value;
         // runs of eight mask tiles a warp; the blocks are scheduled as SMs free
