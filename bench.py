@@ -667,14 +667,16 @@ def roofline_of(fam, ms_total, peak, peak_src, tile, schedule, graph):
 def spmv_kernel_name(family, tile, schedule):
     """The SpMV kernel a family runs at this tile_dim and schedule (the
     library's dispatch: at k = 4 the tile_dim-4 kernel for the bit-vector
-    schemes and, under the direct schedule, for the unweighted 4-byte value
-    schemes; the staged gather kernel for the value schemes under the staged
-    schedule at k <= 16; the chunk kernel otherwise)."""
+    schemes and, unless the schedule is the staged one, for the unweighted
+    4-byte value schemes; the staged gather kernel for the value schemes at
+    k <= 16 under the staged schedule and, from k = 8, the default one; the
+    chunk kernels otherwise)."""
     bits = family in ("spmv_bool", "spmv_count")
     k4_values = family in ("spmv_plus", "spmv_min_i32", "spmv_max", "spmm_or32")
-    if tile == 4 and (bits or (k4_values and schedule == 2)):
+    direct = schedule == 2 or (schedule == 0 and tile == 4 and family != "spmv_minplus")
+    if tile == 4 and (bits or (k4_values and direct)):
         return "spmv_k4_kernel"
-    if not bits and tile <= 16 and schedule != 2:
+    if not bits and tile <= 16 and not direct:
         return "spmv_gather_kernel"
     return "spmv_chunks_kernel"
 

@@ -771,10 +771,10 @@ struct Walk {
 // Warp segmented scan of (reset = has_end, value = acc), then: lanes that end
 // their first tile-row store it (or leave it as the chunk's first partial if
 // it began in an earlier chunk); lane 31 leaves the still-open tail.
-template <class SEM, class Acc>
+template <class SEM, class Acc, class First>
 __device__ __forceinline__ void close_chunk(const SEM& sem, Partials<typename SEM::V> part, int64_t c,
                                             const LaneSpan& ls, int lane, bool head_cs, int32_t first_row,
-                                            bool has_end, bool open, Acc& acc, Acc& F, int P) {
+                                            bool has_end, bool open, Acc& acc, First& F, int P) {
     using V = typename SEM::V;
     constexpr int NV = SEM::NV;
     constexpr unsigned FULL = 0xffffffffu;
@@ -1008,11 +1008,12 @@ __global__ void __launch_bounds__(kSpmvThreads) spmv_chunks_kernel(SpmvGeom g, S
 //     graph) needs no walk: one fixed-order tree joins the lanes.
 // What bounds the value schemes is the L1 data pipe: a gather takes one
 // wavefront per distinct 128-byte line, 32 a warp for scattered columns (79%
-// of the pipe, 27.2M wavefronts an SpMV on R-MAT 20).  R-MAT 20, k = 4, direct
-// schedule, SpMV call in us before / after (one gather per set bit, a row
-// search and a row-pointer walk per lane before): plus-times 173 / 126
-// (permuted ids 148 / 139), label min 183 / 135 (154 / 144), 64-lane OR
-// 238 / 177; Boolean 86 / 68 at k = 4 and 99 / 72 at k = 8.  Warp
+// of the pipe, 27.2M wavefronts an SpMV on R-MAT 20 before the tiles of
+// one-row chunks were dealt out).  R-MAT 20, k = 4, direct schedule, SpMV call
+// in us before / after (one gather per set bit, a row search and a row-pointer
+// walk per lane before): plus-times 173 / 118 (permuted ids 148 / 138), label
+// min 183 / 129 (154 / 144), 64-lane OR 238 / 176, four fp32 columns 312 / 224
+// (236 / 194); Boolean 86 / 64 at k = 4 and 99 / 64 at k = 8.  Warp
 // instructions of the plus-times kernel: 98M / 59M.
 // ---------------------------------------------------------------------------
 // min and max schemes
@@ -1025,21 +1026,28 @@ struct MinMax<SemMaxF32<K>> : std::true_type {};
 
 // How a scheme reads its input: bits from global memory, bits from the
 // block's copy of the whole bitset in shared memory, whole aligned segments of
-// values, or one value per set column (an input that is not aligned to a
-// segment, or whose last segment is ragged).
-enum { kSmBits = 0, kSmBitsShared = 1, kSmSegs = 2, kSmVals = 3 };
+// values, one value per set column (an input that is not aligned to a segment,
+// or whose last segment is ragged; 16-byte values, whose segment would be two
+// sectors), or one value per set bit in a loop (16-byte values where tiles
+// hold hardly more than one: the 16 predicated updates are 64 then).
+enum { kSmBits = 0, kSmBitsShared = 1, kSmSegs = 2, kSmVals = 3, kSmEach = 4 };
 // Threads a block, and the resident blocks the registers are budgeted for
-// (every lane holds two chunks' tile words and columns).  R-MAT 20, k = 4, in
+// (every lane holds two chunks' tile words and columns; with 16-byte values
+// one).  R-MAT 20, k = 4, in
 // us with 4 / 3 blocks an SM: plus-times 126 / 128, label min 145 / 135 (four
-// blocks spill there), 16-source BFS 1,265 / 1,330.  The shared bitset leaves
+// blocks spill there), 16-source BFS 1,265 / 1,330; four columns by bit with 4
+// / 3 / 2 blocks 237 / 269 / 385.  The shared bitset leaves
 // room for one block: k = 8 with 512 / 640 / 768 threads 83 / 74 / 72.5.
-template <int K, int MODE>
+template <int K, class SEM, int MODE>
 constexpr int small_threads() {
-    return MODE != kSmBitsShared ? kSpmvThreads : (K == 8 ? 768 : 1024);
+    if (MODE != kSmBitsShared) return kSpmvThreads;
+    return K == 4 ? 1024 : (SEM::NV == 8 ? 640 : 768);  // eight counts a row need the registers
 }
 template <int K, class SEM, int MODE>
 constexpr int small_min_blocks() {
     if (MODE == kSmBitsShared) return 1;
+    if (sizeof(typename SEM::V) == 16) return MODE == kSmEach ? 4 : 3;
+    if (SEM::NV == 8) return 2;
     return K == 8 || sizeof(typename SEM::V) == 8 || MinMax<SEM>::value ? 3 : 4;
 }
 
@@ -1056,29 +1064,52 @@ struct SmallTiles {
     uint32_t w[8 * TW], cu[8];
 };
 
+__device__ __forceinline__ uint32_t ld4_stream(const void* p) {
+    uint32_t v;
+    asm volatile("ld.global.nc.L1::no_allocate.u32 %0, [%1];\n" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ void ld8_stream(const void* p, uint32_t& a, uint32_t& b) {
+    asm volatile("ld.global.nc.L1::no_allocate.v2.u32 {%0,%1}, [%2];\n" : "=r"(a), "=r"(b) : "l"(p));
+}
+
+// ra, rb: chunk_row[c], chunk_row[c + 1]
 template <int K, class SEM>
-__device__ __forceinline__ void small_load(const SpmvGeom& g, const SEM& sem, int32_t c, int lane, SmallTiles<K>& t) {
+__device__ __forceinline__ void small_load(const SpmvGeom& g, const SEM& sem, int32_t c, int lane, int32_t ra,
+                                           int32_t rb, SmallTiles<K>& t) {
     constexpr int TW = SmallTiles<K>::TW;
-    t.ra = __ldg(g.chunk_row + c);
-    t.rb = __ldg(g.chunk_row + c + 1);
-    t.win = row_window(g, t.ra, t.rb - t.ra, lane);
-    if (!sem.saturated((int64_t)t.ra * K, ((int64_t)t.rb + 1) * K)) {
-        // the arrays are padded to whole chunks, so every lane's bytes exist
-        const int64_t tl = (int64_t)c * chunk_tiles(K) + lane * 8;
-        const uint32_t* src = reinterpret_cast<const uint32_t*>(g.tiles) + tl * TW;
-#pragma unroll
-        for (int q = 0; q < TW; ++q) {
-            uint32_t v[8];
-            ld32_stream(src + 8 * q, v);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) t.w[8 * q + i] = v[i];
-        }
-        ld32_stream(g.colind + tl, t.cu);
-    } else {
+    t.ra = ra;
+    t.rb = rb;
+    t.win = row_window(g, ra, rb - ra, lane);
+    const int64_t c0 = (int64_t)c * chunk_tiles(K);
+    const uint32_t* tiles = reinterpret_cast<const uint32_t*>(g.tiles);
+    // the arrays are padded to whole chunks, so every lane's bytes exist
+    if (sem.saturated((int64_t)ra * K, ((int64_t)rb + 1) * K)) {
 #pragma unroll
         for (int i = 0; i < 8 * TW; ++i) t.w[i] = 0u;
 #pragma unroll
         for (int i = 0; i < 8; ++i) t.cu[i] = 0u;
+    } else if (ra == rb) {
+        // inside one tile-row the tiles are dealt to the lanes (lane l: tiles l,
+        // l + 32, ...): a gather's 32 lanes then have neighbouring columns and
+        // share lines (R-MAT 20: 23 distinct 128-byte lines instead of 32)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int64_t tl = c0 + 32 * i + lane;
+            if constexpr (TW == 1) t.w[i] = ld4_stream(tiles + tl);
+            else ld8_stream(tiles + 2 * tl, t.w[2 * i], t.w[2 * i + 1]);
+            t.cu[i] = ld4_stream(g.colind + tl);
+        }
+    } else {
+        const int64_t tl = c0 + lane * 8;
+#pragma unroll
+        for (int q = 0; q < TW; ++q) {
+            uint32_t v[8];
+            ld32_stream(tiles + tl * TW + 8 * q, v);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) t.w[8 * q + i] = v[i];
+        }
+        ld32_stream(g.colind + tl, t.cu);
     }
 }
 
@@ -1156,10 +1187,39 @@ __device__ __forceinline__ void seg_add(const SEM& sem, Acc& acc, uint32_t w, co
     }
 }
 
+// One value per set bit; the first bit's (most tiles have no other) is loaded
+// beforehand, so that those of several tiles are in flight together.
+template <class G>
+__device__ __forceinline__ G first_value(const G* __restrict__ x, uint32_t J, uint32_t w) {
+    return w ? __ldg(x + 4 * (int64_t)J + ((__ffs(w) - 1) & 7)) : G();
+}
+template <class SEM, class G, class Acc>
+__device__ __forceinline__ void each_add(const SEM& sem, Acc& acc, uint32_t J, uint32_t w, G v) {
+    while (w) {
+        const int r = (__ffs(w) - 1) >> 3;
+        w &= w - 1;
+        G more = G();
+        if (w) more = first_value(sem.src(), J, w);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)  // constant indices keep the accumulators in registers
+            if (u == r) acc.set(u, sem.apply(acc.get(u), v, 1.0f));
+        v = more;
+    }
+}
+
 // Joins the lanes' NV values with the tree of a butterfly (lane pairs, then
-// pairs of pairs, ...: the order of the segmented scan's last lane).  Four
-// values: the first two levels halve the values a lane carries, so lane l < 4
-// ends with value (l >> 1) | (l & 1) << 1; otherwise every lane ends with all.
+// pairs of pairs, ...: the order of the segmented scan's last lane).  Value
+// schemes: the first levels halve the values a lane carries, so lane l < NV
+// ends with value joined_value<NV>(l) in slot 0; bit schemes: every lane ends
+// with all.
+template <int NV>
+__device__ __forceinline__ int joined_value(int lane) {
+    int v = 0;
+#pragma unroll
+    for (int d = 1, half = NV / 2; half >= 1; d <<= 1, half >>= 1) v += (lane & d) ? half : 0;
+    return v;
+}
+
 template <class SEM, class Acc>
 __device__ __forceinline__ void join_lanes(const SEM& sem, Acc& acc, int lane) {
     using V = typename SEM::V;
@@ -1171,28 +1231,21 @@ __device__ __forceinline__ void join_lanes(const SEM& sem, Acc& acc, int lane) {
             acc.set(v, std::is_signed<V>::value ? (V)__reduce_add_sync(FULL, (int)acc.get(v))
                                                 : (V)__reduce_or_sync(FULL, (unsigned)acc.get(v)));
     } else {
-        static_assert(NV == 4, "value schemes at k = 4");
-        V a = acc.get(0), b = acc.get(1);
-        {
-            const bool hi = lane & 1;
-            const V sa = hi ? acc.get(0) : acc.get(2), sb = hi ? acc.get(1) : acc.get(3);
-            const V ka = hi ? acc.get(2) : acc.get(0), kb = hi ? acc.get(3) : acc.get(1);
-            const V oa = shfl_xor(sa, 1), ob = shfl_xor(sb, 1);
-            a = hi ? sem.comb(oa, ka) : sem.comb(ka, oa);
-            b = hi ? sem.comb(ob, kb) : sem.comb(kb, ob);
-        }
-        {
-            const bool hi = lane & 2;
-            const V s = hi ? a : b, k = hi ? b : a;
-            const V o = shfl_xor(s, 2);
-            a = hi ? sem.comb(o, k) : sem.comb(k, o);
-        }
 #pragma unroll
-        for (int d = 4; d < 32; d <<= 1) {
-            const V o = shfl_xor(a, d);
-            a = (lane & d) ? sem.comb(o, a) : sem.comb(a, o);
+        for (int d = 1, half = NV / 2; d < 32; d <<= 1, half = half > 1 ? half / 2 : 0) {
+            const bool hi = lane & d;
+            if (half >= 1) {
+#pragma unroll
+                for (int v = 0; v < half; ++v) {
+                    const V send = hi ? acc.get(v) : acc.get(v + half), keep = hi ? acc.get(v + half) : acc.get(v);
+                    const V o = shfl_xor(send, d);
+                    acc.set(v, hi ? sem.comb(o, keep) : sem.comb(keep, o));
+                }
+            } else {
+                const V o = shfl_xor(acc.get(0), d);
+                acc.set(0, hi ? sem.comb(o, acc.get(0)) : sem.comb(acc.get(0), o));
+            }
         }
-        acc.set(0, a);
     }
 }
 
@@ -1200,7 +1253,7 @@ __device__ __forceinline__ void join_lanes(const SEM& sem, Acc& acc, int lane) {
 template <int K, class SEM, int MODE>
 __device__ __forceinline__ void small_chunk(const SpmvGeom& g, const SEM& sem, Partials<typename SEM::V> part,
                                             int32_t c, int lane, const SmallTiles<K>& t, ChunkRows& s,
-                                            const uint8_t* sx) {
+                                            const uint8_t* sx, typename SEM::V* first) {
     using Sh = ChunkShape<K>;
     using V = typename SEM::V;
     constexpr int NV = SEM::NV;
@@ -1208,7 +1261,10 @@ __device__ __forceinline__ void small_chunk(const SpmvGeom& g, const SEM& sem, P
     static_assert(Sh::P == 8 && TW <= 2, "eight tiles of one or two words a lane");
     const int32_t cs = c * Sh::CT;
     const int32_t ce = min(cs + Sh::CT, (int32_t)g.T);
-    RegAcc<V, NV> acc, F, idv;
+    RegAcc<V, NV> acc, idv;
+    // the values of the lane's first tile-row: in shared memory where they are wide
+    typename std::conditional<sizeof(V) == 16, SmemAcc<V, NV>, RegAcc<V, NV>>::type F;
+    if constexpr (sizeof(V) == 16) F.p = first + lane;
 #pragma unroll
     for (int v = 0; v < NV; ++v) { acc.set(v, sem.ident()); F.set(v, sem.ident()); idv.set(v, sem.ident()); }
     const bool one_row = t.ra == t.rb;  // warp-uniform: the whole chunk lies in tile-row ra
@@ -1243,17 +1299,29 @@ __device__ __forceinline__ void small_chunk(const SpmvGeom& g, const SEM& sem, P
     if constexpr (SEM::kGather) {
         // tiles whose segments are loaded together (plus-times on R-MAT 20: 1, 2,
         // 4 tiles 127, 126, 130 us; the loads of more cost registers)
-        constexpr int GRP = 2;
+        constexpr int GRP = MODE == kSmVals && sizeof(V) == 16 ? 1 : 2;
         using G = typename SEM::G;
 #pragma unroll
         for (int i0 = 0; i0 < 8; i0 += GRP) {
-            G x[GRP][4];
+            if constexpr (MODE == kSmEach) {
+                G x[GRP];
 #pragma unroll
-            for (int i = 0; i < GRP; ++i) load_seg<G, MODE>(sem.src(), t.cu[i0 + i], t.w[i0 + i], x[i]);
+                for (int i = 0; i < GRP; ++i) x[i] = first_value(sem.src(), t.cu[i0 + i], t.w[i0 + i]);
 #pragma unroll
-            for (int i = 0; i < GRP; ++i) {
-                seg_add(sem, acc, t.w[i0 + i], x[i]);
-                if (!one_row) end_tile(i0 + i);
+                for (int i = 0; i < GRP; ++i) {
+                    each_add(sem, acc, t.cu[i0 + i], t.w[i0 + i], x[i]);
+                    if (!one_row) end_tile(i0 + i);
+                }
+            } else {
+                G x[GRP][4];
+#pragma unroll
+                for (int i = 0; i < GRP; ++i)
+                    load_seg<G, MODE>(sem.src(), t.cu[i0 + i], t.w[i0 + i], x[i]);
+#pragma unroll
+                for (int i = 0; i < GRP; ++i) {
+                    seg_add(sem, acc, t.w[i0 + i], x[i]);
+                    if (!one_row) end_tile(i0 + i);
+                }
             }
         }
     } else {
@@ -1276,7 +1344,7 @@ __device__ __forceinline__ void small_chunk(const SpmvGeom& g, const SEM& sem, P
         join_lanes(sem, acc, lane);
         if (head && c + 1 == g.nchunks) {  // begins and ends in this chunk (the matrix's last)
             if constexpr (SEM::kGather) {
-                if (lane < 4) sem.store_row(t.ra, (lane >> 1) | ((lane & 1) << 1), acc.get(0));
+                if (lane < NV) sem.store_row(t.ra, joined_value<NV>(lane), acc.get(0));
             } else if (lane == 0) {
                 sem.store(t.ra, acc);
             }
@@ -1285,7 +1353,7 @@ __device__ __forceinline__ void small_chunk(const SpmvGeom& g, const SEM& sem, P
         // continued by later chunks (head) or begun in earlier ones
         V* dst = (head ? part.val_last : part.val_first) + (int64_t)c * NV;
         if constexpr (SEM::kGather) {
-            if (lane < 4) dst[(lane >> 1) | ((lane & 1) << 1)] = acc.get(0);
+            if (lane < NV) dst[joined_value<NV>(lane)] = acc.get(0);
         } else if (lane == 0) {
 #pragma unroll
             for (int v = 0; v < NV; ++v) dst[v] = acc.get(v);
@@ -1302,21 +1370,38 @@ __device__ __forceinline__ void small_chunk(const SpmvGeom& g, const SEM& sem, P
     close_chunk(sem, part, c, ls, lane, head_cs, first_row, has_end, open, acc, F, Sh::P);
 }
 
-// Dynamic shared memory: a ChunkRows per warp, then (kSmBitsShared) the input bitset.
+// Dynamic shared memory a warp: its ChunkRows, and for 16-byte values the
+// lanes' first rows.
+template <class SEM>
+constexpr int small_warp_smem() {
+    return (int)sizeof(ChunkRows) + (sizeof(typename SEM::V) == 16 ? 32 * SEM::NV * 16 : 0);
+}
+
+// Dynamic shared memory: that for every warp, then (kSmBitsShared) the input bitset.
 template <int K, class SEM, int MODE>
 __device__ __forceinline__ void small_body(const SpmvGeom& g, const SEM& sem, Partials<typename SEM::V> part) {
-    constexpr int WARPS = small_threads<K, MODE>() / 32;
+    constexpr int WARPS = small_threads<K, SEM, MODE>() / 32;
     extern __shared__ __align__(16) uint8_t small_smem[];
     if (gated_off(g.gate)) return;
-    ChunkRows* rows = reinterpret_cast<ChunkRows*>(small_smem) + (threadIdx.x >> 5);
-    const uint8_t* sx = small_smem + WARPS * sizeof(ChunkRows);
+    uint8_t* mine = small_smem + (threadIdx.x >> 5) * small_warp_smem<SEM>();
+    ChunkRows* rows = reinterpret_cast<ChunkRows*>(mine);
+    typename SEM::V* first = reinterpret_cast<typename SEM::V*>(mine + sizeof(ChunkRows));  // 16-byte values only
+    const uint8_t* sx = small_smem + WARPS * small_warp_smem<SEM>();
     const int lane = (int)lane_id();
     const int32_t W = (int32_t)gridDim.x * WARPS;
     int32_t c = (int32_t)blockIdx.x * WARPS + (threadIdx.x >> 5);
     SmallTiles<K> cur, nxt;
-    if (c < g.nchunks) small_load<K>(g, sem, c, lane, cur);
+    // tile-rows of the chunk after the loaded one: its loads depend on them
+    int32_t na = 0, nb = 0;
+    if (c < g.nchunks) {
+        small_load<K>(g, sem, c, lane, __ldg(g.chunk_row + c), __ldg(g.chunk_row + c + 1), cur);
+        if (c + W < g.nchunks) {
+            na = __ldg(g.chunk_row + c + W);
+            nb = __ldg(g.chunk_row + c + W + 1);
+        }
+    }
     if constexpr (MODE == kSmBitsShared) {
-        uint32_t* dst = reinterpret_cast<uint32_t*>(small_smem + WARPS * sizeof(ChunkRows));
+        uint32_t* dst = reinterpret_cast<uint32_t*>(small_smem + WARPS * small_warp_smem<SEM>());
         const int words = (sem.n + 31) / 32;
         int at = 0;
         if (reinterpret_cast<uintptr_t>(sem.x) % 16 == 0) {
@@ -1328,11 +1413,29 @@ __device__ __forceinline__ void small_body(const SpmvGeom& g, const SEM& sem, Pa
         __syncthreads();
     }
     if (c >= g.nchunks) return;  // whole warps leave together
+    if constexpr (sizeof(typename SEM::V) == 16) {
+        // one chunk at a time: more warps hide its loads better than the
+        // registers of a second chunk would (R-MAT 20: 225 and 270 us)
+        for (;;) {
+            small_chunk<K, SEM, MODE>(g, sem, part, c, lane, cur, *rows, sx, first);
+            c += W;
+            if (c >= g.nchunks) return;
+            small_load<K>(g, sem, c, lane, na, nb, cur);
+            if (c + W < g.nchunks) {
+                na = __ldg(g.chunk_row + c + W);
+                nb = __ldg(g.chunk_row + c + W + 1);
+            }
+        }
+    }
     for (;;) {
         const int32_t cn = c + W;
         const bool more = cn < g.nchunks;
-        if (more) small_load<K>(g, sem, cn, lane, nxt);
-        small_chunk<K, SEM, MODE>(g, sem, part, c, lane, cur, *rows, sx);
+        if (more) small_load<K>(g, sem, cn, lane, na, nb, nxt);
+        if (cn + W < g.nchunks) {
+            na = __ldg(g.chunk_row + cn + W);
+            nb = __ldg(g.chunk_row + cn + W + 1);
+        }
+        small_chunk<K, SEM, MODE>(g, sem, part, c, lane, cur, *rows, sx, first);
         if (!more) break;
         c = cn;
         cur = nxt;
@@ -1342,12 +1445,12 @@ __device__ __forceinline__ void small_body(const SpmvGeom& g, const SEM& sem, Pa
 // k = 4 with the bit-vector schemes and 4-byte values; the other small-tile
 // cases (k = 8, 8-byte values).
 template <class SEM, int MODE>
-__global__ void __launch_bounds__((small_threads<4, MODE>()), (small_min_blocks<4, SEM, MODE>()))
+__global__ void __launch_bounds__((small_threads<4, SEM, MODE>()), (small_min_blocks<4, SEM, MODE>()))
     spmv_k4_kernel(SpmvGeom g, SEM sem, Partials<typename SEM::V> part) {
     small_body<4, SEM, MODE>(g, sem, part);
 }
 template <int K, class SEM, int MODE>
-__global__ void __launch_bounds__((small_threads<K, MODE>()), (small_min_blocks<K, SEM, MODE>()))
+__global__ void __launch_bounds__((small_threads<K, SEM, MODE>()), (small_min_blocks<K, SEM, MODE>()))
     spmv_chunks_kernel(SpmvGeom g, SEM sem, Partials<typename SEM::V> part) {
     small_body<K, SEM, MODE>(g, sem, part);
 }
@@ -1792,17 +1895,17 @@ static double spmv_bytes(const b2sr_matrix* h, double vec_bytes) {
 template <int K, class SEM>
 constexpr bool use_small() {
     if constexpr (!SEM::kGather) return K <= 8;
-    else return K == 4 && !SEM::kMayWeight && sizeof(typename SEM::V) <= 8;
+    else return K == 4 && !SEM::kMayWeight;
 }
 
 template <int K, class SEM, int MODE>
 static b2sr_status launch_small(const b2sr_matrix* h, const SEM& sem, Partials<typename SEM::V> part, cudaStream_t s,
                                 const SpmvGeom& g) {
     // persistent: the resident blocks, each warp looping over chunks
-    constexpr int threads = small_threads<K, MODE>();
+    constexpr int threads = small_threads<K, SEM, MODE>();
     const unsigned grid = (unsigned)std::min<int64_t>(ceil_div(h->nchunks, threads / 32),
                                                       (int64_t)sm_count() * small_min_blocks<K, SEM, MODE>());
-    const int smem = threads / 32 * (int)sizeof(ChunkRows) + (MODE == kSmBitsShared ? (int)ceil_div(h->n, 32) * 4 : 0);
+    const int smem = threads / 32 * small_warp_smem<SEM>() + (MODE == kSmBitsShared ? (int)ceil_div(h->n, 32) * 4 : 0);
     void (*kernel)(SpmvGeom, SEM, Partials<typename SEM::V>);
     if constexpr (K == 4 && sizeof(typename SEM::V) == 4) kernel = spmv_k4_kernel<SEM, MODE>;
     else kernel = spmv_chunks_kernel<K, SEM, MODE>;
@@ -1824,17 +1927,25 @@ static b2sr_status launch_direct(const b2sr_matrix* h, const SEM& sem, Partials<
             // line a cycle were what bound the kernel) when it fits and a warp has a
             // few chunks to spread the copy over: R-MAT 20, k = 4 / k = 8, Boolean:
             // 75 / 74.7 us without, 68 / 72.5 with it; permuted ids 76 / 89 and 67 / 82.
-            constexpr int threads = small_threads<K, kSmBitsShared>();
+            constexpr int threads = small_threads<K, SEM, kSmBitsShared>();
             if constexpr (!NoInput<SEM>::value)
                 if (h->nchunks >= (int64_t)sm_count() * (threads / 32) * 4 &&
-                    ceil_div(h->n, 32) * 4 + threads / 32 * (int64_t)sizeof(ChunkRows) <= kMaxBlockSmem)
+                    ceil_div(h->n, 32) * 4 + threads / 32 * small_warp_smem<SEM>() <= kMaxBlockSmem)
                     return launch_small<K, SEM, kSmBitsShared>(h, sem, part, s, g);
             return launch_small<K, SEM, kSmBits>(h, sem, part, s, g);
         } else {
-            // whole segments need an aligned input without a ragged last one
-            const bool segs = h->n % 4 == 0 && reinterpret_cast<uintptr_t>(sem.x) % (4 * sizeof(typename SEM::G)) == 0;
-            if (segs) return launch_small<K, SEM, kSmSegs>(h, sem, part, s, g);
-            return launch_small<K, SEM, kSmVals>(h, sem, part, s, g);
+            using G = typename SEM::G;
+            if constexpr (sizeof(G) == 16) {
+                // R-MAT 20 (1.15 set bits a tile), its permutation (1.01), R-MAT 16
+                // (1.3), us: by column 224 / 241 / 27, by bit 237 / 195 / 47
+                if (8 * h->nnz > 9 * h->T) return launch_small<K, SEM, kSmVals>(h, sem, part, s, g);
+                return launch_small<K, SEM, kSmEach>(h, sem, part, s, g);
+            } else {
+                // whole segments need an aligned input without a ragged last one
+                if (h->n % 4 == 0 && reinterpret_cast<uintptr_t>(sem.x) % (4 * sizeof(G)) == 0)
+                    return launch_small<K, SEM, kSmSegs>(h, sem, part, s, g);
+                return launch_small<K, SEM, kSmVals>(h, sem, part, s, g);
+            }
         }
     } else {
         spmv_chunks_kernel<K, SEM><<<(unsigned)ceil_div(h->nchunks, kSpmvWarps), kSpmvThreads, 0, s>>>(g, sem, part);
@@ -1853,7 +1964,10 @@ static b2sr_status run_chunks(const b2sr_matrix* h, const SEM& sem, cudaStream_t
     B2SR_TRY((alloc_partials<V, SEM::NV>(pbuf, h->nchunks, &part)));
     const unsigned blocks = (unsigned)ceil_div(h->nchunks, kSpmvWarps);
     bool staged = false;
-    if constexpr (SEM::kGather && K <= 16) staged = h->schedule != B2SR_SCHED_DIRECT;
+    // AUTO: the small-tile kernel where it serves
+    if constexpr (SEM::kGather && K <= 16)
+        staged = h->schedule == B2SR_SCHED_STAGED ||
+                 (h->schedule == B2SR_SCHED_AUTO && !use_small<K, SEM>());
     if constexpr (SEM::kGather && K <= 16) if (staged) {
         const int smem = kSpmvWarps * GatherLayout<K, SEM>::bytes;
         if (smem > 48 * 1024)
