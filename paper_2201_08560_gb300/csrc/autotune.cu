@@ -15,11 +15,6 @@
 #include "b2sr_internal.cuh"
 
 namespace b2sr {
-b2sr_status spmv_dispatch(b2sr_matrix* h, b2sr_semiring sr, b2sr_vec in_kind, const void* x, b2sr_vec out_kind,
-                          void* y, const uint32_t* mask, int comp, const float* weights, cudaStream_t s,
-                          const int32_t* gate);
-b2sr_status spmm64_dispatch(b2sr_matrix* h, const uint64_t* X, uint64_t* Y, const uint64_t* M, int comp,
-                            cudaStream_t s, const int32_t* gate);
 
 static const int kTileDims[4] = {4, 8, 16, 32};
 

@@ -174,6 +174,17 @@ b2sr_status validate_csr_async(int32_t n, const int32_t* rowptr, const int32_t* 
 b2sr_status new_handle_from_tiles(int32_t n, int k, int64_t T, int32_t* rowptr, int32_t* colind,
                                   uint8_t* tiles, int64_t cap, cudaStream_t s, b2sr_matrix** out);
 
+// SpMV and lane SpMM (spmv.cu), optionally gated on a device flag.  edges =
+// false (Boolean and OR results): the output already holds zeros where the
+// matrix has no tiles, before its first tile-row and after its last.
+b2sr_status spmv_dispatch(b2sr_matrix* h, b2sr_semiring sr, b2sr_vec in_kind, const void* x, b2sr_vec out_kind,
+                          void* y, const uint32_t* mask, int comp, const float* weights, cudaStream_t s,
+                          const int32_t* gate, bool edges = true);
+b2sr_status spmm64_dispatch(b2sr_matrix* h, const uint64_t* X, uint64_t* Y, const uint64_t* M, int comp,
+                            cudaStream_t s, const int32_t* gate, bool edges = true);
+b2sr_status spmm32_dispatch(b2sr_matrix* h, const uint32_t* X, uint32_t* Y, const uint32_t* M, int comp,
+                            cudaStream_t s, const int32_t* gate, bool edges = true);
+
 // primitives (primitives.cu)
 b2sr_status exclusive_scan_i32_to_i64(const int32_t* in, int64_t* out, int64_t n, cudaStream_t s);
 b2sr_status exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, cudaStream_t s);

@@ -25,16 +25,57 @@ inline b2sr_status read_flag(const int32_t* dev, HostFlag& hf, cudaStream_t s, i
 __device__ __forceinline__ bool gate_closed(const int32_t* gate) { return gate && *gate == 0; }
 
 // ---------------------------------------------------------------------------
-// captured round loop
+// end of a round, inside the round's last kernel
 // ---------------------------------------------------------------------------
-// Enqueues `per_graph` rounds (body(stream, r)) into one CUDA graph on a
-// private stream, then replays it until *active reads 0.  Every round must be
-// gated on *active.  Returns in *rounds the rounds replayed; B2SR_ERR_NOT_CONVERGED
-// if *active is still set after max_rounds.
+struct LoopFlags {  // device
+    int32_t active;  // 1 while rounds have work
+    int32_t found;   // this round found something
+    int32_t level;   // rounds run
+    uint32_t ticket;
+};
+
+// Called by every thread of every block of a gated kernel; `any`: the thread
+// found something.  The last block to arrive moves the loop on: active <-
+// found, one more level.
+__device__ __forceinline__ void finish_round(LoopFlags* f, int any) {
+    const int found = __syncthreads_or(any);
+    if (threadIdx.x != 0) return;
+    if (found) atomicOr(&f->found, 1);
+    __threadfence();
+    if (atomicAdd(&f->ticket, 1u) != gridDim.x - 1u) return;
+    __threadfence();
+    f->ticket = 0u;
+    f->active = atomicExch(&f->found, 0);
+    f->level += 1;
+}
+
+// ---------------------------------------------------------------------------
+// round loop
+// ---------------------------------------------------------------------------
+// Runs rounds (body(stream, r) enqueues one; r counts from 0 within a batch of
+// `per_graph`) until *active reads 0, reading it after every batch.  Every
+// round must be gated on *active.  The first kEagerBatches batches are
+// enqueued on the caller's stream; a loop that goes on longer captures a batch
+// into a CUDA graph on a private stream and replays it.  (Capture,
+// instantiation, the private stream and its pinned flag cost 200 to 250 us a
+// call, more than all launches of a search that ends in a few batches:
+// single-source BFS on R-MAT 12 took 312 us.)  Returns in *rounds the rounds
+// enqueued; B2SR_ERR_NOT_CONVERGED if *active is still set after max_rounds.
+constexpr int kEagerBatches = 4;
+
 template <class Body>
 b2sr_status run_captured(cudaStream_t user, int per_graph, int64_t max_rounds, const int32_t* active,
                                 Body&& body, int64_t* rounds) {
     *rounds = 0;
+    for (int batch = 0; batch < kEagerBatches; ++batch) {
+        for (int r = 0; r < per_graph; ++r) B2SR_TRY(body(user, r));
+        *rounds += per_graph;
+        int32_t got = 0;
+        B2SR_CUDA_TRY(cudaMemcpyAsync(&got, active, sizeof(int32_t), cudaMemcpyDeviceToHost, user));
+        B2SR_CUDA_TRY(cudaStreamSynchronize(user));
+        if (!got) return B2SR_OK;
+        if (*rounds >= max_rounds) return fail(B2SR_ERR_NOT_CONVERGED, "exceeded max_iters rounds");
+    }
     cudaStream_t cs = nullptr;
     cudaEvent_t ev = nullptr;
     cudaGraph_t graph = nullptr;

@@ -18,49 +18,48 @@
 #include "captured.cuh"
 
 namespace b2sr {
-b2sr_status spmv_dispatch(b2sr_matrix* h, b2sr_semiring sr, b2sr_vec in_kind, const void* x, b2sr_vec out_kind,
-                          void* y, const uint32_t* mask, int comp, const float* weights, cudaStream_t s,
-                          const int32_t* gate);
-b2sr_status spmm64_dispatch(b2sr_matrix* h, const uint64_t* X, uint64_t* Y, const uint64_t* M, int comp,
-                            cudaStream_t s, const int32_t* gate);
 b2sr_status masked_count(const b2sr_matrix* A, const b2sr_matrix* B, const b2sr_matrix* M, int64_t* count,
                          cudaStream_t s, int64_t* pairs);
-
-// active <- found (only while active); level counter advances with it
-__global__ void advance_kernel(int32_t* active, const int32_t* found, int32_t* level) {
-    if (threadIdx.x == 0 && blockIdx.x == 0 && *active) {
-        *active = *found;
-        *level += 1;
-    }
-}
 
 // ---------------------------------------------------------------------------
 // BFS from a set of sources (all at level 0)
 // ---------------------------------------------------------------------------
-__global__ void bfs_init_kernel(int32_t* levels, int32_t n, uint32_t* frontier, uint32_t* visited, int64_t words) {
+__global__ void bfs_init_kernel(int32_t* levels, int32_t n, uint32_t* fa, uint32_t* fb, uint32_t* visited,
+                                int64_t words, LoopFlags* flags) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n || i < words;
          i += (int64_t)gridDim.x * blockDim.x) {
         if (i < n) levels[i] = -1;
-        if (i < words) { frontier[i] = 0u; visited[i] = 0u; }
+        if (i < words) { fa[i] = 0u; fb[i] = 0u; visited[i] = 0u; }
     }
+    if (blockIdx.x == 0 && threadIdx.x == 0) *flags = LoopFlags{1, 0, 0, 0u};
 }
 
-__global__ void bfs_seed_kernel(const int32_t* srcs, int nsrc, int32_t* levels, uint32_t* frontier,
+// Up to kParamSources sources travel as a kernel argument.
+constexpr int kParamSources = 64;
+struct SourceList {
+    int32_t v[kParamSources];
+};
+static SourceList source_list(const int32_t* srcs, int nsrc) {
+    SourceList l = {};
+    for (int i = 0; i < nsrc && i < kParamSources; ++i) l.v[i] = srcs[i];
+    return l;
+}
+
+__global__ void bfs_seed_kernel(const int32_t* srcs, SourceList few, int nsrc, int32_t* levels, uint32_t* frontier,
                                 uint32_t* visited) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nsrc; i += gridDim.x * blockDim.x) {
-        const int32_t v = srcs[i];
+        const int32_t v = srcs ? srcs[i] : few.v[i];
         levels[v] = 0;
         atomicOr(frontier + (v >> 5), 1u << (v & 31));
         atomicOr(visited + (v >> 5), 1u << (v & 31));
     }
 }
 
-// visited |= next; levels[v] = level+1 for every new vertex; found if any
+// visited |= next; levels[v] = level+1 for every new vertex; ends the round
 __global__ void bfs_update_kernel(const uint32_t* __restrict__ next, uint32_t* __restrict__ visited,
-                                  int32_t* __restrict__ levels, int64_t words, const int32_t* level,
-                                  const int32_t* gate, int32_t* found) {
-    if (gate_closed(gate)) return;
-    const int32_t lv = *level + 1;
+                                  int32_t* __restrict__ levels, int64_t words, LoopFlags* flags) {
+    if (gate_closed(&flags->active)) return;
+    const int32_t lv = *reinterpret_cast<const volatile int32_t*>(&flags->level) + 1;
     int any = 0;
     for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < words;
          w += (int64_t)gridDim.x * blockDim.x) {
@@ -74,7 +73,7 @@ __global__ void bfs_update_kernel(const uint32_t* __restrict__ next, uint32_t* _
             levels[w * 32 + c] = lv;
         }
     }
-    if (__syncthreads_or(any) && threadIdx.x == 0) atomicOr(found, 1);
+    finish_round(flags, any);
 }
 
 b2sr_status bfs_sources(b2sr_matrix* h, const int32_t* srcs_host, int nsrc, int32_t* levels, int max_iters,
@@ -82,36 +81,33 @@ b2sr_status bfs_sources(b2sr_matrix* h, const int32_t* srcs_host, int nsrc, int3
     const int32_t n = h->n;
     const int64_t words = ceil_div(n, 32);
     DevBuf buf(s);
-    B2SR_TRY(buf.alloc(3 * words * sizeof(uint32_t) + (size_t)(nsrc + 8) * sizeof(int32_t)));
-    uint32_t* fa = buf.as<uint32_t>();
+    B2SR_TRY(buf.alloc(sizeof(LoopFlags) + 3 * words * sizeof(uint32_t) + (size_t)nsrc * sizeof(int32_t)));
+    LoopFlags* flags = buf.as<LoopFlags>();
+    uint32_t* fa = reinterpret_cast<uint32_t*>(flags + 1);
     uint32_t* fb = fa + words;
     uint32_t* vis = fb + words;
-    int32_t* flags = reinterpret_cast<int32_t*>(vis + words);  // active, found, level
-    int32_t* dsrc = flags + 8;
-    B2SR_CUDA_TRY(cudaMemcpyAsync(dsrc, srcs_host, nsrc * sizeof(int32_t), cudaMemcpyHostToDevice, s));
-    bfs_init_kernel<<<grid_for(std::max<int64_t>(n, words)), 256, 0, s>>>(levels, n, fa, vis, words);
+    int32_t* dsrc = nullptr;
+    if (nsrc > kParamSources) {
+        dsrc = reinterpret_cast<int32_t*>(vis + words);
+        B2SR_CUDA_TRY(cudaMemcpyAsync(dsrc, srcs_host, nsrc * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+    }
+    bfs_init_kernel<<<grid_for(std::max<int64_t>(n, words)), 256, 0, s>>>(levels, n, fa, fb, vis, words, flags);
     B2SR_LAUNCH_CHECK("bfs_init_kernel");
-    bfs_seed_kernel<<<(unsigned)ceil_div(nsrc, 256), 256, 0, s>>>(dsrc, nsrc, levels, fa, vis);
+    bfs_seed_kernel<<<(unsigned)ceil_div(nsrc, 256), 256, 0, s>>>(dsrc, source_list(srcs_host, nsrc), nsrc, levels, fa,
+                                                                vis);
     B2SR_LAUNCH_CHECK("bfs_seed_kernel");
-    const int32_t init[3] = {1, 0, 0};
-    B2SR_CUDA_TRY(cudaMemcpyAsync(flags, init, sizeof(init), cudaMemcpyHostToDevice, s));
-    int32_t* active = flags;
-    int32_t* found = flags + 1;
-    int32_t* level = flags + 2;
     const int64_t cap = max_iters > 0 ? max_iters : (int64_t)n + 1;
     int64_t rounds = 0;
-    return run_captured(s, 4, cap + 1, active,
+    return run_captured(s, 4, cap + 1, &flags->active,
                         [&](cudaStream_t cs, int r) -> b2sr_status {
                             uint32_t* f = (r & 1) ? fb : fa;
                             uint32_t* nx = (r & 1) ? fa : fb;
+                            // rows without tiles are zero in fb from the start, and in fa (which may
+                            // have sources there) once a round has written it
                             B2SR_TRY(spmv_dispatch(h, B2SR_BOOL_OR_AND, B2SR_VEC_BITS, f, B2SR_VEC_BITS, nx, vis, 1,
-                                                   nullptr, cs, active));
-                            B2SR_CUDA_TRY(cudaMemsetAsync(found, 0, sizeof(int32_t), cs));
-                            bfs_update_kernel<<<grid_for(words), 256, 0, cs>>>(nx, vis, levels, words, level, active,
-                                                                               found);
+                                                   nullptr, cs, &flags->active, r == 1));
+                            bfs_update_kernel<<<grid_for(words), 256, 0, cs>>>(nx, vis, levels, words, flags);
                             B2SR_LAUNCH_CHECK("bfs_update_kernel");
-                            advance_kernel<<<1, 32, 0, cs>>>(active, found, level);
-                            B2SR_LAUNCH_CHECK("advance_kernel");
                             return B2SR_OK;
                         },
                         &rounds);
@@ -122,64 +118,74 @@ b2sr_status bfs_sources(b2sr_matrix* h, const int32_t* srcs_host, int nsrc, int3
 // ---------------------------------------------------------------------------
 // The lane word: 64 frontiers (uint64) or, for at most 32 sources, 32 (uint32:
 // half the bytes per gather, and the SpMV takes the tile_dim-4 kernel).
-__device__ __forceinline__ int lowest_lane(unsigned long long b) { return __ffsll((long long)b) - 1; }
-__device__ __forceinline__ int lowest_lane(uint32_t b) { return __ffs(b) - 1; }
-
 template <class W>
-__global__ void msbfs_init_kernel(int32_t* levels, int32_t n, int nsrc, W* X, W* vis) {
+__global__ void msbfs_init_kernel(int32_t* levels, int32_t n, int nsrc, W* X, W* Y, W* vis, LoopFlags* flags) {
     constexpr int BITS = 8 * (int)sizeof(W);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (int64_t)n * nsrc || i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
         if (i < (int64_t)n * nsrc) levels[i] = -1;
         // unused lanes count as visited, so a vertex every source has reached is
         // all ones in the mask and the SpMM can skip its rows
-        if (i < n) { X[i] = (W)0; vis[i] = nsrc < BITS ? (W)~(((W)1 << nsrc) - (W)1) : (W)0; }
+        if (i < n) {
+            X[i] = (W)0;
+            Y[i] = (W)0;
+            vis[i] = nsrc < BITS ? (W)~(((W)1 << nsrc) - (W)1) : (W)0;
+        }
     }
+    if (blockIdx.x == 0 && threadIdx.x == 0) *flags = LoopFlags{1, 0, 0, 0u};
 }
 
 template <class W>
-__global__ void msbfs_seed_kernel(const int32_t* srcs, int nsrc, int32_t n, int32_t* levels, W* X, W* vis) {
+__global__ void msbfs_seed_kernel(SourceList srcs, int nsrc, int32_t n, int32_t* levels, W* X, W* vis) {
     int s = threadIdx.x;
     if (s < nsrc) {
-        int32_t v = srcs[s];
+        int32_t v = srcs.v[s];
         levels[(int64_t)s * n + v] = 0;
         atomicOr(X + v, (W)1 << s);
         atomicOr(vis + v, (W)1 << s);
     }
 }
 
+// visited |= next, and the level of every (lane, vertex) pair found.  A warp
+// takes 32 consecutive vertices and goes through the lanes that any of them
+// has, so a store writes one lane's levels of neighbouring vertices (a thread
+// that walked its own vertex's lanes wrote 32 different lines a store:
+// R-MAT 22, 64 sources: 260 us a level).
 template <class W>
 __global__ void msbfs_update_kernel(const W* __restrict__ Y, W* __restrict__ vis, int32_t* __restrict__ levels,
-                                    int32_t n, const int32_t* level, const int32_t* gate, int32_t* found) {
-    if (gate_closed(gate)) return;
-    const int32_t lv = *level + 1;
+                                    int32_t n, LoopFlags* flags) {
+    if (gate_closed(&flags->active)) return;
+    const int32_t lv = *reinterpret_cast<const volatile int32_t*>(&flags->level) + 1;
     int any = 0;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
-         v += (int64_t)gridDim.x * blockDim.x) {
-        W b = Y[v];
-        if (!b) continue;
-        any = 1;
-        vis[v] |= b;
-        while (b) {
-            int s = lowest_lane(b);
-            b &= b - 1;
-            levels[(int64_t)s * n + v] = lv;
+    const int lane = (int)lane_id();
+    for (int64_t v0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) - lane; v0 < n;
+         v0 += (int64_t)gridDim.x * blockDim.x) {  // warp-uniform
+        const int64_t v = v0 + lane;
+        const W b = v < n ? Y[v] : (W)0;
+        if (b) vis[v] |= b;
+#pragma unroll
+        for (int half = 0; half < (int)sizeof(W) / 4; ++half) {
+            const uint32_t mine = (uint32_t)(b >> (32 * half * (int)(sizeof(W) > 4)));
+            uint32_t lanes = __reduce_or_sync(0xffffffffu, mine);
+            any |= lanes != 0u;
+            for (; lanes; lanes &= lanes - 1u) {
+                const int s = __ffs(lanes) - 1;
+                if ((mine >> s) & 1u) levels[(int64_t)(32 * half + s) * n + v] = lv;
+            }
         }
     }
-    if (__syncthreads_or(any) && threadIdx.x == 0) atomicOr(found, 1);
+    finish_round(flags, any);
 }
 
-b2sr_status spmm32_dispatch(b2sr_matrix* h, const uint32_t* X, uint32_t* Y, const uint32_t* M, int comp,
-                            cudaStream_t s, const int32_t* gate);
 
 static b2sr_status spmm_lanes(b2sr_matrix* h, const unsigned long long* X, unsigned long long* Y,
-                              const unsigned long long* M, cudaStream_t s, const int32_t* gate) {
+                              const unsigned long long* M, cudaStream_t s, const int32_t* gate, bool edges) {
     return spmm64_dispatch(h, reinterpret_cast<const uint64_t*>(X), reinterpret_cast<uint64_t*>(Y),
-                           reinterpret_cast<const uint64_t*>(M), 1, s, gate);
+                           reinterpret_cast<const uint64_t*>(M), 1, s, gate, edges);
 }
 static b2sr_status spmm_lanes(b2sr_matrix* h, const uint32_t* X, uint32_t* Y, const uint32_t* M, cudaStream_t s,
-                              const int32_t* gate) {
-    return spmm32_dispatch(h, X, Y, M, 1, s, gate);
+                              const int32_t* gate, bool edges) {
+    return spmm32_dispatch(h, X, Y, M, 1, s, gate, edges);
 }
 
 template <class W>
@@ -187,35 +193,26 @@ static b2sr_status bfs_multi_lanes(b2sr_matrix* h, const int32_t* srcs_host, int
                                    int max_iters, cudaStream_t s) {
     const int32_t n = h->n;
     DevBuf buf(s);
-    B2SR_TRY(buf.alloc(3 * round_up((size_t)n * sizeof(W), 256) + 72 * sizeof(int32_t)));
+    const size_t vb = round_up((size_t)n * sizeof(W), 256);
+    B2SR_TRY(buf.alloc(3 * vb + sizeof(LoopFlags)));
     W* X = buf.as<W>();
-    W* Yb = reinterpret_cast<W*>(buf.as<char>() + round_up((size_t)n * sizeof(W), 256));
-    W* vis = reinterpret_cast<W*>(buf.as<char>() + 2 * round_up((size_t)n * sizeof(W), 256));
-    int32_t* dsrc = reinterpret_cast<int32_t*>(buf.as<char>() + 3 * round_up((size_t)n * sizeof(W), 256));
-    int32_t* flags = dsrc + 64;  // active, found, level
-    B2SR_CUDA_TRY(cudaMemcpyAsync(dsrc, srcs_host, nsrc * sizeof(int32_t), cudaMemcpyHostToDevice, s));
-    msbfs_init_kernel<W><<<grid_for((int64_t)n * nsrc), 256, 0, s>>>(levels, n, nsrc, X, vis);
+    W* Yb = reinterpret_cast<W*>(buf.as<char>() + vb);
+    W* vis = reinterpret_cast<W*>(buf.as<char>() + 2 * vb);
+    LoopFlags* flags = reinterpret_cast<LoopFlags*>(buf.as<char>() + 3 * vb);
+    msbfs_init_kernel<W><<<grid_for((int64_t)n * nsrc), 256, 0, s>>>(levels, n, nsrc, X, Yb, vis, flags);
     B2SR_LAUNCH_CHECK("msbfs_init_kernel");
-    msbfs_seed_kernel<W><<<1, 64, 0, s>>>(dsrc, nsrc, n, levels, X, vis);
+    msbfs_seed_kernel<W><<<1, 64, 0, s>>>(source_list(srcs_host, nsrc), nsrc, n, levels, X, vis);
     B2SR_LAUNCH_CHECK("msbfs_seed_kernel");
-    const int32_t init[3] = {1, 0, 0};
-    B2SR_CUDA_TRY(cudaMemcpyAsync(flags, init, sizeof(init), cudaMemcpyHostToDevice, s));
-    int32_t* active = flags;
-    int32_t* found = flags + 1;
-    int32_t* level = flags + 2;
     const int64_t cap = max_iters > 0 ? max_iters : (int64_t)n + 1;
     int64_t rounds = 0;
-    return run_captured(s, 4, cap + 1, active,
+    return run_captured(s, 4, cap + 1, &flags->active,
                         [&](cudaStream_t cs, int r) -> b2sr_status {
                             W* cur = (r & 1) ? Yb : X;
                             W* nxt = (r & 1) ? X : Yb;
-                            B2SR_TRY(spmm_lanes(h, cur, nxt, vis, cs, active));
-                            B2SR_CUDA_TRY(cudaMemsetAsync(found, 0, sizeof(int32_t), cs));
-                            msbfs_update_kernel<W><<<grid_for(n), 256, 0, cs>>>(nxt, vis, levels, n, level, active,
-                                                                               found);
+                            // as in bfs_sources: rows without tiles need zeros in X once
+                            B2SR_TRY(spmm_lanes(h, cur, nxt, vis, cs, &flags->active, r == 1));
+                            msbfs_update_kernel<W><<<grid_for(n), 256, 0, cs>>>(nxt, vis, levels, n, flags);
                             B2SR_LAUNCH_CHECK("msbfs_update_kernel");
-                            advance_kernel<<<1, 32, 0, cs>>>(active, found, level);
-                            B2SR_LAUNCH_CHECK("advance_kernel");
                             return B2SR_OK;
                         },
                         &rounds);
@@ -230,48 +227,41 @@ b2sr_status bfs_multi(b2sr_matrix* h, const int32_t* srcs_host, int nsrc, int32_
 // ---------------------------------------------------------------------------
 // SSSP: d <- min(d, A min.+ d) until no distance changes
 // ---------------------------------------------------------------------------
-__global__ void sssp_init_kernel(float* d, int32_t n, int32_t src) {
+__global__ void sssp_init_kernel(float* d, int32_t n, int32_t src, LoopFlags* flags) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         d[i] = (i == src) ? 0.0f : INFINITY;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *flags = LoopFlags{1, 0, 0, 0u};
 }
 
 // found if a distance changed; the round's result becomes the current vector
 __global__ void sssp_update_kernel(const float* __restrict__ nxt, float* __restrict__ cur, int32_t n,
-                                   const int32_t* gate, int32_t* found) {
-    if (gate_closed(gate)) return;
+                                   LoopFlags* flags) {
+    if (gate_closed(&flags->active)) return;
     int diff = 0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const float v = nxt[i];
         if (v != cur[i]) { diff = 1; cur[i] = v; }
     }
-    if (__syncthreads_or(diff) && threadIdx.x == 0) atomicOr(found, 1);
+    finish_round(flags, diff);
 }
 
 b2sr_status sssp(b2sr_matrix* h, const float* w, int32_t src, float* dist, int max_iters, cudaStream_t s) {
     const int32_t n = h->n;
     if (w) B2SR_TRY(ensure_voff(h, s));  // built before capture: capture must not allocate for the handle
     DevBuf buf(s);
-    B2SR_TRY(buf.alloc((size_t)n * sizeof(float) + 16));
-    float* tmp = buf.as<float>();
-    int32_t* flags = reinterpret_cast<int32_t*>(tmp + n);
-    sssp_init_kernel<<<grid_for(n), 256, 0, s>>>(dist, n, src);
+    B2SR_TRY(buf.alloc(sizeof(LoopFlags) + (size_t)n * sizeof(float)));
+    LoopFlags* flags = buf.as<LoopFlags>();
+    float* tmp = reinterpret_cast<float*>(flags + 1);
+    sssp_init_kernel<<<grid_for(n), 256, 0, s>>>(dist, n, src, flags);
     B2SR_LAUNCH_CHECK("sssp_init_kernel");
-    const int32_t init[3] = {1, 0, 0};
-    B2SR_CUDA_TRY(cudaMemcpyAsync(flags, init, sizeof(init), cudaMemcpyHostToDevice, s));
-    int32_t* active = flags;
-    int32_t* found = flags + 1;
-    int32_t* level = flags + 2;
     const int64_t cap = max_iters > 0 ? max_iters : (int64_t)n + 1;
     int64_t rounds = 0;
-    return run_captured(s, 16, cap + 1, active,
+    return run_captured(s, 16, cap + 1, &flags->active,
                         [&](cudaStream_t cs, int) -> b2sr_status {
                             B2SR_TRY(spmv_dispatch(h, B2SR_MIN_PLUS, B2SR_VEC_F32, dist, B2SR_VEC_F32, tmp, nullptr, 0, w,
-                                                   cs, active));
-                            B2SR_CUDA_TRY(cudaMemsetAsync(found, 0, sizeof(int32_t), cs));
-                            sssp_update_kernel<<<grid_for(n), 256, 0, cs>>>(tmp, dist, n, active, found);
+                                                   cs, &flags->active));
+                            sssp_update_kernel<<<grid_for(n), 256, 0, cs>>>(tmp, dist, n, flags);
                             B2SR_LAUNCH_CHECK("sssp_update_kernel");
-                            advance_kernel<<<1, 32, 0, cs>>>(active, found, level);
-                            B2SR_LAUNCH_CHECK("advance_kernel");
                             return B2SR_OK;
                         },
                         &rounds);

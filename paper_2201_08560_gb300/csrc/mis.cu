@@ -36,9 +36,6 @@
 #include "tile_bits.cuh"
 
 namespace b2sr {
-b2sr_status spmv_dispatch(b2sr_matrix* h, b2sr_semiring sr, b2sr_vec in_kind, const void* x, b2sr_vec out_kind,
-                          void* y, const uint32_t* mask, int comp, const float* weights, cudaStream_t s,
-                          const int32_t* gate);
 b2sr_status spmv_maxkey_dispatch(b2sr_matrix* h, const uint64_t* x, uint64_t* y, const uint32_t* mask, int comp,
                                  cudaStream_t s, const int32_t* gate);
 

@@ -39,8 +39,6 @@
 #include "b2sr_internal.cuh"
 
 namespace b2sr {
-b2sr_status spmm64_dispatch(b2sr_matrix* h, const uint64_t* X, uint64_t* Y, const uint64_t* M, int comp,
-                            cudaStream_t s, const int32_t* gate);
 b2sr_status spmm4_dispatch(b2sr_matrix* h, const float* X, float* Y, const uint32_t* M, int comp, cudaStream_t s,
                            const int32_t* gate);
 

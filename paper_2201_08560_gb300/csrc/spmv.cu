@@ -1972,13 +1972,13 @@ static b2sr_status run_chunks(const b2sr_matrix* h, const SEM& sem, cudaStream_t
         const int smem = kSpmvWarps * GatherLayout<K, SEM>::bytes;
         if (smem > 48 * 1024)
             B2SR_CUDA_TRY(cudaFuncSetAttribute(spmv_gather_kernel<K, SEM>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        void* tok = timing_begin(s);
+        void* tok = gate ? nullptr : timing_begin(s);  // a gated launch may do nothing
         spmv_gather_kernel<K, SEM><<<blocks, kSpmvThreads, smem, s>>>(g, sem, part);
         timing_end(tok, family, spmv_bytes(h, vec_bytes), s);
         B2SR_LAUNCH_CHECK("spmv_gather_kernel");
     }
     if (!staged) {
-        void* tok = timing_begin(s);
+        void* tok = gate ? nullptr : timing_begin(s);  // a gated launch may do nothing
         const b2sr_status st = launch_direct<K, SEM>(h, sem, part, s, g);
         timing_end(tok, family, spmv_bytes(h, vec_bytes), s);
         B2SR_TRY(st);
@@ -1988,10 +1988,12 @@ static b2sr_status run_chunks(const b2sr_matrix* h, const SEM& sem, cudaStream_t
 
 template <int K, class SEM>
 static b2sr_status run_spmv(const b2sr_matrix* h, const SEM& sem, uint32_t* bits_out, cudaStream_t s,
-                            const char* family, double vec_bytes, const int32_t* gate) {
+                            const char* family, double vec_bytes, const int32_t* gate, bool edges = true) {
     SpmvGeom g{h->rowptr, h->colind, h->tiles, h->chunk_row, h->T, h->nchunks, h->ntr, gate};
-    if (bits_out) B2SR_TRY(clear_bitset_tail<K>(h, bits_out, s, gate));
-    B2SR_TRY((launch_edges<K, SEM>(h, sem, s, gate)));
+    if (edges) {
+        if (bits_out) B2SR_TRY(clear_bitset_tail<K>(h, bits_out, s, gate));
+        B2SR_TRY((launch_edges<K, SEM>(h, sem, s, gate)));
+    }
     if (h->nchunks > 0) B2SR_TRY((run_chunks<K, SEM>(h, sem, s, family, vec_bytes, gate, g)));
     if constexpr (HasSelfTerm<SEM>::value) {
         const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(h->n, 256), (int64_t)sm_count() * 8));
@@ -2026,14 +2028,15 @@ b2sr_status row_counts(const b2sr_matrix* h, int32_t* cnt, int32_t* first, int32
 
 b2sr_status spmv_dispatch(b2sr_matrix* h, b2sr_semiring sr, b2sr_vec in_kind, const void* x, b2sr_vec out_kind,
                           void* y, const uint32_t* mask, int comp, const float* weights, cudaStream_t s,
-                          const int32_t* gate) {
+                          const int32_t* gate, bool edges) {
     comp = comp ? 1 : 0;
     if (sr == B2SR_BOOL_OR_AND && in_kind == B2SR_VEC_BITS && out_kind == B2SR_VEC_BITS) {
         if (weights) return fail(B2SR_ERR_INVALID_ARG, "weights apply to MIN_PLUS only");
         return with_tile(h->k, [&](auto kc) -> b2sr_status {
             constexpr int K = decltype(kc)::value;
             SemBool<K> sem{static_cast<const uint32_t*>(x), static_cast<uint32_t*>(y), mask, comp, h->n};
-            return run_spmv<K>(h, sem, static_cast<uint32_t*>(y), s, "spmv_bool", (mask ? 3.0 : 2.0) * h->n / 8.0, gate);
+            return run_spmv<K>(h, sem, static_cast<uint32_t*>(y), s, "spmv_bool", (mask ? 3.0 : 2.0) * h->n / 8.0, gate,
+                               edges);
         });
     }
     if (sr == B2SR_PLUS_TIMES && in_kind == B2SR_VEC_BITS && out_kind == B2SR_VEC_I32) {
@@ -2083,23 +2086,23 @@ b2sr_status spmv_dispatch(b2sr_matrix* h, b2sr_semiring sr, b2sr_vec in_kind, co
 }
 
 b2sr_status spmm64_dispatch(b2sr_matrix* h, const uint64_t* X, uint64_t* Y, const uint64_t* M, int comp,
-                            cudaStream_t s, const int32_t* gate) {
+                            cudaStream_t s, const int32_t* gate, bool edges) {
     return with_tile(h->k, [&](auto kc) -> b2sr_status {
         constexpr int K = decltype(kc)::value;
         SemOr64<K> sem{reinterpret_cast<const unsigned long long*>(X), reinterpret_cast<unsigned long long*>(Y),
                        reinterpret_cast<const unsigned long long*>(M), comp ? 1 : 0, h->n};
-        return run_spmv<K>(h, sem, nullptr, s, "spmm_or64", (M ? 24.0 : 16.0) * h->n, gate);
+        return run_spmv<K>(h, sem, nullptr, s, "spmm_or64", (M ? 24.0 : 16.0) * h->n, gate, edges);
     });
 }
 
 // The same over 32-lane words (at most 32 frontiers): half the bytes per
 // gather and 4-byte accumulators, which the tile_dim-4 kernel takes.
 b2sr_status spmm32_dispatch(b2sr_matrix* h, const uint32_t* X, uint32_t* Y, const uint32_t* M, int comp,
-                            cudaStream_t s, const int32_t* gate) {
+                            cudaStream_t s, const int32_t* gate, bool edges) {
     return with_tile(h->k, [&](auto kc) -> b2sr_status {
         constexpr int K = decltype(kc)::value;
         SemOr32<K> sem{X, Y, M, comp ? 1 : 0, h->n};
-        return run_spmv<K>(h, sem, nullptr, s, "spmm_or32", (M ? 12.0 : 8.0) * h->n, gate);
+        return run_spmv<K>(h, sem, nullptr, s, "spmm_or32", (M ? 12.0 : 8.0) * h->n, gate, edges);
     });
 }
 
