@@ -146,8 +146,9 @@ struct b2sr_matrix {
     int64_t nchunks = 0;
     int32_t first_row = 0;       // tile-row of tile 0 (ntr if T == 0)
     int32_t last_row = -1;       // tile-row of tile T-1 (-1 if T == 0)
-    // tile-rows that span SpMV chunks: (row, first chunk, last chunk) triples,
-    // rows spanning at most kSplitShort chunks first, then the longer ones
+    // tile-rows that span SpMV chunks: (row, first chunk, last chunk) triples;
+    // nchunks of them, rows spanning at most kSplitShort chunks from the front,
+    // the longer ones from the back
     int32_t* split = nullptr;
     int64_t nsplit_short = 0;
     int64_t nsplit_long = 0;
@@ -172,7 +173,8 @@ b2sr_status extract_csr(const b2sr_matrix* h, int64_t* off, int32_t* rowptr, int
 b2sr_status validate_csr_async(int32_t n, const int32_t* rowptr, const int32_t* colind, int64_t nnz, int* bad,
                                cudaStream_t s);
 b2sr_status new_handle_from_tiles(int32_t n, int k, int64_t T, int32_t* rowptr, int32_t* colind,
-                                  uint8_t* tiles, int64_t cap, cudaStream_t s, b2sr_matrix** out);
+                                  uint8_t* tiles, int64_t cap, cudaStream_t s, b2sr_matrix** out,
+                                  int64_t known_nnz = -1);  // set bits, if the caller knows
 
 // SpMV and lane SpMM (spmv.cu), optionally gated on a device flag.  edges =
 // false (Boolean and OR results): the output already holds zeros where the

@@ -8,11 +8,12 @@
 // with S the bit width of a tile index.  Once the keys are in order, equal
 // tiles are runs in (tile-row, tile-column) order, run heads become the tiles,
 // and each entry ORs its bit into its tile.  When every CSR row is already in
-// column order (the usual case) the k rows of a tile-row are k sorted runs and
-// the keys are put in order by ranking each entry among its tile-row's rows
-// (binary searches) and, at k = 16 and 32, merging groups of eight rows
-// pairwise; otherwise a radix sort on the tile part orders them.  Both replace
-// the paper's cusparseXcsr2bsrNnz / cusparseScsr2bsr + packing kernels
+// column order (the usual case) the k rows of a tile-row are k sorted runs.  At
+// k = 4 and 8, without repeated entries, blocks merge them and build the tiles
+// in shared memory, piece by piece; otherwise the keys are put in order by
+// ranking each entry among its tile-row's rows (binary searches) and, at k =
+// 16 and 32, merging groups of eight rows pairwise.  Rows in no order go
+// through a radix sort on the tile part.  All replace the paper's cusparseXcsr2bsrNnz / cusparseScsr2bsr + packing kernels
 // (Sec. III-B) and give the same three arrays.
 #include <algorithm>
 #include <mutex>
@@ -55,14 +56,14 @@ __global__ void validate_rows_kernel(int32_t n, const int32_t* __restrict__ rowp
 }
 
 // Entry pass, four entries a step: every column in [0, n) (else bit 4 of
-// *bad), and *unsorted set if an entry that does not begin a row has a
-// smaller column than the entry before it.
+// *bad); bit 1 of *unsorted set if an entry that does not begin a row has a
+// smaller column than the entry before it, bit 2 if it has the same.
 __global__ void validate_entries_kernel(int32_t n, const int32_t* __restrict__ colind, int64_t nnz,
                                         const uint32_t* __restrict__ starts, int* __restrict__ bad,
                                         int* __restrict__ unsorted) {
     const int64_t groups = (nnz + 3) / 4;
     const bool vec = (reinterpret_cast<uintptr_t>(colind) & 15u) == 0;
-    bool out = false, down = false;
+    bool out = false, down = false, same = false;
     for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < groups;
          g += (int64_t)gridDim.x * blockDim.x) {
         const int64_t e0 = g * 4;
@@ -80,12 +81,15 @@ __global__ void validate_entries_kernel(int32_t n, const int32_t* __restrict__ c
         for (int q = 0; q < 4; ++q) {
             if (e0 + q >= nnz) break;
             out |= c[q] < 0 || c[q] >= n;
-            down |= e0 + q > 0 && !((sw >> q) & 1u) && prev > c[q];
+            const bool inner = e0 + q > 0 && !((sw >> q) & 1u);
+            down |= inner && prev > c[q];
+            same |= inner && prev == c[q];
             prev = c[q];
         }
     }
     if (out) atomicOr(bad, 4);
     if (down) atomicOr(unsorted, 1);
+    if (same) atomicOr(unsorted, 2);
 }
 
 // Sets *bad (device) non-zero if the CSR is malformed; stream-ordered, no sync.
@@ -346,8 +350,9 @@ __device__ __forceinline__ uint32_t run_heads(const uint64_t (&key)[kFillItems],
 
 // Sum of v over the block; every thread gets it.  Also returns, in *excl,
 // the sum over the threads before this one.
+template <int THREADS>
 __device__ __forceinline__ int block_scan(int v, int* excl) {
-    __shared__ int warp_tot[kFillThreads / 32];
+    __shared__ int warp_tot[THREADS / 32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int inc = v;
 #pragma unroll
@@ -359,7 +364,7 @@ __device__ __forceinline__ int block_scan(int v, int* excl) {
     __syncthreads();
     int before = 0, total = 0;
 #pragma unroll
-    for (int w = 0; w < kFillThreads / 32; ++w) {
+    for (int w = 0; w < THREADS / 32; ++w) {
         const int x = warp_tot[w];
         before += w < wid ? x : 0;
         total += x;
@@ -374,7 +379,7 @@ __global__ void __launch_bounds__(kFillThreads) count_heads_kernel(const uint64_
     uint64_t key[kFillItems], before;
     load_run(keys, N, base, key, before);
     int excl;
-    const int total = block_scan(__popc(run_heads(key, before, base, N)), &excl);
+    const int total = block_scan<kFillThreads>(__popc(run_heads(key, before, base, N)), &excl);
     if (threadIdx.x == 0) sums[blockIdx.x] = total;
 }
 
@@ -418,7 +423,7 @@ __global__ void __launch_bounds__(kFillThreads) fill_small_tiles_kernel(const ui
     const uint64_t before = threadIdx.x > 0 ? s_key[fill_slot(q0 - 1)] : (b0 > 0 ? __ldg(keys + b0 - 1) : 0ull);
     const uint32_t h = run_heads(key, before, b0 + q0, N);
     int excl;
-    const int heads = block_scan(__popc(h), &excl);
+    const int heads = block_scan<kFillThreads>(__popc(h), &excl);
     const int64_t boff = block_off[blockIdx.x];
     const uint64_t jmask = (1ull << sbits) - 1ull;
     const bool wide = k == 8;
@@ -498,7 +503,7 @@ __global__ void __launch_bounds__(kFillThreads, 4) fill_tiles_kernel(const uint6
     load_run(keys, N, base, key, before);
     const uint32_t h = run_heads(key, before, base, N);
     int excl;
-    block_scan(__popc(h), &excl);
+    block_scan<kFillThreads>(__popc(h), &excl);
     const int wb = word_bytes(k);
     const uint64_t jmask = (1ull << sbits) - 1ull;
     int64_t t = block_off[blockIdx.x] + excl - 1;  // the tile of the run in progress
@@ -566,82 +571,470 @@ __global__ void __launch_bounds__(kFillThreads, 4) fill_tiles_kernel(const uint6
 }
 
 // ---------------------------------------------------------------------------
-// schedule: tile-row of the first tile of every SpMV chunk
+// rows in column order without repeats, k = 4 and 8: pieces merged in shared
+// memory
 // ---------------------------------------------------------------------------
-__global__ void chunk_rows_kernel(const int32_t* __restrict__ rowptr, int32_t ntr, int64_t T, int64_t CT,
-                                  int64_t nchunks, int32_t* __restrict__ chunk_row) {
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c <= nchunks;
-         c += (int64_t)gridDim.x * blockDim.x) {
-        int64_t t = min(c * CT, T - 1);
-        chunk_row[c] = row_of(rowptr, 0, ntr - 1, t);
+// A piece is at most kPieceCap entries of whole tile-rows, or of one long
+// tile-row's range of tile-columns.  The CSR entries are cut into windows of
+// kWindow; a window's pieces are the tile-rows that begin in it, and if the
+// last of those is longer than kWindow (a long tile-row; its end lies past the
+// window, so it is the last), its slices of about kSliceTarget entries.  A
+// block loads a piece, merges the k rows of each of its tile-rows pairwise in
+// shared memory (log2 k levels; a thread finds where its eight outputs begin
+// in the two runs by a binary search along their diagonal and merges from
+// there), counts the run heads, and builds the tiles and their column indices
+// there.  They leave in coalesced stores to the piece's place
+// among the entries (a piece has at most as many tiles as entries); once the
+// counts are scanned a second kernel moves them together.  Ranking every entry
+// in global memory instead cost 393M warp instructions and 504 us on R-MAT 20
+// at k = 4, and the 8-byte keys it wrote were read twice to build the tiles
+// (187 us).  Merging and building takes 470 us there (300M instructions; the
+// block's barriers and the merge's dependent shared loads bound it: 48 warps
+// an SM, of which a piece of 1,100 entries keeps five in eight busy), finding
+// the pieces 90 and moving the tiles together 80.
+constexpr int kWindow = 1024;
+constexpr int kPieceCap = 2048;
+constexpr int kSliceTarget = 1920;  // a slice is cut at a tile-column: up to k * k <= 64 entries more
+constexpr int kPieceThreads = 256;
+constexpr int kPieceItems = kPieceCap / kPieceThreads;
+
+// First tile-row beginning at entry e or later (ntr if none).
+__device__ __forceinline__ int32_t tile_row_from(const int32_t* __restrict__ rowptr, int32_t n, int32_t ntr, int k,
+                                                 int64_t e) {
+    int32_t lo = 0, hi = ntr;
+    while (lo < hi) {
+        const int32_t mid = lo + ((hi - lo) >> 1);
+        if ((int64_t)__ldg(rowptr + min((int64_t)mid * k, (int64_t)n)) < e) lo = mid + 1; else hi = mid;
+    }
+    return lo;
+}
+
+// Window b: first[b] = its first tile-row, slices[b] = the slices of its long
+// tile-row (0: none), cnt[b] = its pieces.  Runs beside the validation: a malformed rowptr gives meaningless numbers, never an
+// access out of range.
+__global__ void windows_kernel(const int32_t* __restrict__ rowptr, int32_t n, int32_t ntr, int k, int64_t nwin,
+                               int32_t* __restrict__ first, int32_t* __restrict__ slices,
+                               int32_t* __restrict__ cnt) {
+    for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b <= nwin;
+         b += (int64_t)gridDim.x * blockDim.x) {
+        if (b == nwin) {
+            first[b] = ntr;
+            slices[b] = 0;
+            cnt[b] = 0;
+            continue;
+        }
+        const int32_t f = tile_row_from(rowptr, n, ntr, k, b * kWindow);
+        const int32_t g = b + 1 == nwin ? ntr : tile_row_from(rowptr, n, ntr, k, (b + 1) * kWindow);
+        int32_t parts = 0;
+        if (g > f) {
+            const int64_t last = (int64_t)(g - 1) * k;
+            const int32_t len = __ldg(rowptr + min(last + k, (int64_t)n)) - __ldg(rowptr + last);
+            if (len > kWindow) parts = (len + kSliceTarget - 1) / kSliceTarget;
+        }
+        first[b] = f;
+        slices[b] = parts;
+        cnt[b] = parts + (g - (parts > 0 ? 1 : 0) > f ? 1 : 0);
     }
 }
 
-// Tile-rows that span chunks: the row R that chunk c begins inside, when R
-// started in an earlier chunk and ends in c.  kind[c] = 1 (at most
-// kSplitShort chunks), 2 (more), 0 (none).
-__global__ void split_kind_kernel(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ chunk_row,
-                                  int64_t T, int64_t CT, int64_t nchunks, int32_t* __restrict__ kshort,
-                                  int32_t* __restrict__ klong) {
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < nchunks;
-         c += (int64_t)gridDim.x * blockDim.x) {
-        int32_t ks = 0, kl = 0;
-        if (c > 0) {
-            const int64_t cs = c * CT, ce = min(cs + CT, T);
-            const int32_t R = chunk_row[c];
-            const int64_t rs = rowptr[R], re = rowptr[R + 1];
-            if (rs < cs && re <= ce) {
-                const int64_t np = c - rs / CT + 1;
-                if (np <= kSplitShort) ks = 1; else kl = 1;
+// What a block needs of piece p: its window, and for a slice the position in
+// each of the k rows where it begins (the next slice's, or the rows' ends, are
+// where it ends).
+__global__ void pieces_kernel(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ colind, int32_t n,
+                              int32_t ntr, int k, int64_t nwin, const int32_t* __restrict__ first,
+                              const int32_t* __restrict__ parts, const int64_t* __restrict__ poff, int64_t npieces, int32_t* __restrict__ window,
+                              int32_t* __restrict__ cut) {
+    const int lane = (int)lane_id();
+    const int q = lane & (k - 1);  // a group of k lanes a piece, lane q for row q
+    const unsigned group = ((k == 32 ? 0u : 1u << k) - 1u) << (lane - q);
+    const int64_t stride = ((int64_t)gridDim.x * blockDim.x) / k;
+    for (int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / k; p < npieces; p += stride) {
+        int64_t lo = 0, hi = nwin - 1;  // the last window whose pieces begin at or before p
+        while (lo < hi) {
+            const int64_t mid = (lo + hi + 1) >> 1;
+            if (__ldg(poff + mid) <= p) lo = mid; else hi = mid - 1;
+        }
+        if (q == 0) window[p] = (int32_t)lo;
+        const int64_t slices = __ldg(parts + lo);
+        const int64_t slice = p - (__ldg(poff + lo + 1) - slices);
+        if (slice < 0) continue;
+        const int64_t row0 = (int64_t)(__ldg(first + lo + 1) - 1) * k;
+        int32_t plo = __ldg(rowptr + min(row0 + q, (int64_t)n));
+        if (slice > 0) {
+            const int32_t start = __ldg(rowptr + row0);
+            const int64_t len = __ldg(rowptr + min(row0 + k, (int64_t)n)) - start;
+            const int64_t target = slice * len / slices;
+            const int32_t r0 = plo;
+            int32_t phi = __ldg(rowptr + min(row0 + q + 1, (int64_t)n));
+            // the tile-column J with at most `target` entries before it, at most k * k short of it
+            int32_t jlo = 0, jhi = ntr;
+            while (jhi - jlo > 1) {
+                const int32_t mid = jlo + ((jhi - jlo) >> 1);
+                int32_t a = plo, b = phi;
+                while (a < b) {
+                    const int32_t m = a + ((b - a) >> 1);
+                    if ((int64_t)__ldg(colind + m) < (int64_t)mid * k) a = m + 1; else b = m;
+                }
+                int32_t before = a - r0;
+                for (int o = 1; o < k; o <<= 1) before += __shfl_xor_sync(group, before, o);
+                if (before <= target) {
+                    jlo = mid;
+                    plo = a;
+                    if (before >= target - k * k) break;
+                } else {
+                    jhi = mid;
+                    phi = a;
+                }
             }
         }
-        kshort[c] = ks;
-        klong[c] = kl;
+        cut[p * k + q] = plo;
     }
 }
 
-__global__ void split_fill_kernel(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ chunk_row,
-                                  int64_t CT, int64_t nchunks, const int32_t* __restrict__ kshort,
-                                  const int32_t* __restrict__ klong, const int64_t* __restrict__ pshort,
-                                  const int64_t* __restrict__ plong, int64_t nshort, int32_t* __restrict__ split) {
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < nchunks;
+template <int K>
+struct PieceTile {
+    using type = typename std::conditional<K == 4, uint32_t, unsigned long long>::type;
+};
+
+template <int K>
+__global__ void __launch_bounds__(kPieceThreads, K == 4 ? 6 : 5) merge_piece_kernel(
+    const int32_t* __restrict__ rowptr, const int32_t* __restrict__ colind, int32_t n, const int32_t* __restrict__ first,
+    const int32_t* __restrict__ parts, const int64_t* __restrict__ poff, const int32_t* __restrict__ window,
+    const int32_t* __restrict__ cut,
+    int32_t* __restrict__ trow_at, int32_t* __restrict__ count, int32_t* __restrict__ place, int32_t* __restrict__ col,
+    typename PieceTile<K>::type* __restrict__ tile) {
+    using Tile = typename PieceTile<K>::type;
+    constexpr int LK = K == 4 ? 2 : 3;
+    __shared__ __align__(16) uint32_t s_key[2][kPieceCap];  // column * K + row in tile
+    __shared__ __align__(16) int32_t s_row[kPieceCap];      // row at the position, from the piece's first
+    __shared__ __align__(16) Tile s_tile[kPieceCap];
+    __shared__ int32_t s_off[K + 1];  // a slice's rows
+    const int lane = (int)lane_id(), warp = threadIdx.x >> 5;
+    const int64_t p = blockIdx.x;
+    const int32_t b = __ldg(window + p);
+    const int32_t slices = __ldg(parts + b);
+    const int64_t p0 = __ldg(poff + b + 1) - slices;  // the first slice
+    const bool slice = p >= p0;
+    const int32_t I0 = slice ? __ldg(first + b + 1) - 1 : __ldg(first + b);
+    const int32_t I1 = slice ? I0 + 1 : __ldg(first + b + 1) - (slices > 0 ? 1 : 0);
+    const int64_t row0 = (int64_t)I0 * K;
+    const int32_t nrows = (int32_t)(min((int64_t)I1 * K, (int64_t)n) - row0);
+    int32_t e0, cnt;
+    if (slice) {
+        if (threadIdx.x == 0) {
+            const bool final = p == p0 + slices - 1;
+            int32_t at = 0;
+            int64_t before = 0;
+            for (int q = 0; q < K; ++q) {
+                const int32_t lo = __ldg(cut + p * K + q);
+                const int32_t hi = final ? __ldg(rowptr + min(row0 + q + 1, (int64_t)n)) : __ldg(cut + (p + 1) * K + q);
+                before += lo - __ldg(rowptr + min(row0 + q, (int64_t)n));
+                s_off[q] = at;
+                at += hi - lo;
+            }
+            s_off[K] = at;
+            place[p] = __ldg(rowptr + row0) + (int32_t)before;
+        }
+        __syncthreads();
+        cnt = s_off[K];
+        e0 = 0;
+#pragma unroll
+        for (int q = 0; q < K; ++q) {
+            const int32_t lo = __ldg(cut + p * K + q), at = s_off[q], len = s_off[q + 1] - at;
+            for (int32_t i = threadIdx.x; i < len; i += kPieceThreads) {
+                s_key[0][at + i] = (uint32_t)__ldg(colind + lo + i) * K + q;
+                s_row[at + i] = q;
+            }
+        }
+    } else {
+        e0 = __ldg(rowptr + min(row0, (int64_t)n));
+        cnt = __ldg(rowptr + row0 + nrows) - e0;
+        if (threadIdx.x == 0) place[p] = e0;
+        uint32_t v[kPieceItems];  // all loads in flight before the rows are known
+#pragma unroll
+        for (int i = 0; i < kPieceItems; ++i) {
+            const int32_t at = i * kPieceThreads + threadIdx.x;
+            v[i] = at < cnt ? (uint32_t)__ldg(colind + e0 + at) * K : 0u;
+        }
+        constexpr int W = kPieceThreads / 32;  // neighbouring rows go to different warps
+        for (int32_t r0 = warp; r0 < nrows; r0 += kPieceThreads) {
+            const int32_t r = r0 + W * lane;
+            int32_t a = 0, z = 0;
+            if (r < nrows) {
+                a = __ldg(rowptr + row0 + r) - e0;
+                z = __ldg(rowptr + row0 + r + 1) - e0;
+            }
+            for (unsigned todo = __ballot_sync(0xffffffffu, z > a); todo; todo &= todo - 1) {
+                const int src = __ffs(todo) - 1;
+                const int32_t ra = __shfl_sync(0xffffffffu, a, src), rz = __shfl_sync(0xffffffffu, z, src);
+                for (int32_t i = ra + lane; i < rz; i += 32) s_row[i] = r0 + W * src;
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kPieceItems; ++i) {
+            const int32_t at = i * kPieceThreads + threadIdx.x;
+            if (at < cnt) s_key[0][at] = v[i] + (uint32_t)(s_row[at] & (K - 1));
+        }
+    }
+    for (int i = threadIdx.x; i < cnt; i += kPieceThreads) s_tile[i] = 0;
+    __syncthreads();
+    // merge level l: runs of 2^l rows, two by two; a thread makes the eight
+    // outputs at its positions.  A position stays inside its tile-row (and its
+    // pair of runs), so s_row says which pair it belongs to.
+    const int32_t q0 = threadIdx.x * kPieceItems;
+#pragma unroll
+    for (int l = 0; l < LK; ++l) {
+        const uint32_t* src = s_key[l & 1];
+        uint32_t* dst = s_key[(l & 1) ^ 1];
+        const int32_t q1 = min(q0 + kPieceItems, cnt);
+        // the pair of runs [st, m) and [m, e) that holds position `at`
+        int32_t st = 0, m = 0, e = 0;
+        auto pair_of = [&](int32_t at) {
+            const int32_t r = (s_row[at] >> (l + 1)) << (l + 1);
+            if (slice) {
+                st = s_off[r];
+                m = s_off[r + (1 << l)];
+                e = s_off[r + (2 << l)];
+            } else {
+                st = __ldg(rowptr + row0 + r) - e0;
+                m = __ldg(rowptr + min(row0 + r + (1 << l), (int64_t)n)) - e0;
+                e = __ldg(rowptr + min(row0 + r + (2 << l), (int64_t)n)) - e0;
+            }
+        };
+        int32_t ia = 0, ib = 0;
+        uint32_t ka = 0u, kb = 0u;
+        auto heads_of = [&]() {
+            ka = ia < m ? src[ia] : 0xFFFFFFFFu;  // above every key
+            kb = ib < e ? src[ib] : 0xFFFFFFFFu;
+        };
+        if (q0 < q1) {
+            pair_of(q0);
+            const int32_t d = q0 - st;  // outputs before: how many of them from the first run?
+            int32_t lo = max(0, d - (e - m)), hi = min(d, m - st);
+            while (lo < hi) {
+                const int32_t mid = (lo + hi) >> 1;
+                if (src[st + mid] < src[m + d - 1 - mid]) lo = mid + 1; else hi = mid;
+            }
+            ia = st + lo;
+            ib = m + d - lo;
+            heads_of();
+        }
+#pragma unroll
+        for (int i = 0; i < kPieceItems; ++i) {
+            const int32_t at = q0 + i;
+            if (at < q1) {
+                if (at == e) {  // the next pair begins here
+                    pair_of(at);
+                    ia = st;
+                    ib = m;
+                    heads_of();
+                }
+                const bool first_run = ka < kb;
+                dst[at] = first_run ? ka : kb;
+                const int32_t next = first_run ? ++ia : ++ib;
+                const uint32_t k2 = next < (first_run ? m : e) ? src[next] : 0xFFFFFFFFu;
+                if (first_run) ka = k2; else kb = k2;
+            }
+        }
+        __syncthreads();
+    }
+    const uint32_t* keys = s_key[LK & 1];
+    int32_t* s_col = reinterpret_cast<int32_t*>(s_key[(LK & 1) ^ 1]);
+    // run heads, then tiles
+    uint32_t key[kPieceItems];
+    int32_t trow[kPieceItems];
+    {
+        const uint4 a = *reinterpret_cast<const uint4*>(keys + q0), c = *reinterpret_cast<const uint4*>(keys + q0 + 4);
+        key[0] = a.x; key[1] = a.y; key[2] = a.z; key[3] = a.w;
+        key[4] = c.x; key[5] = c.y; key[6] = c.z; key[7] = c.w;
+        const int4 r = *reinterpret_cast<const int4*>(s_row + q0), t = *reinterpret_cast<const int4*>(s_row + q0 + 4);
+        trow[0] = r.x >> LK; trow[1] = r.y >> LK; trow[2] = r.z >> LK; trow[3] = r.w >> LK;
+        trow[4] = t.x >> LK; trow[5] = t.y >> LK; trow[6] = t.z >> LK; trow[7] = t.w >> LK;
+    }
+    const uint32_t key_before = q0 > 0 ? keys[q0 - 1] : 0u;
+    const int32_t trow_before = q0 > 0 ? s_row[q0 - 1] >> LK : -1;
+    uint32_t h = 0u;
+#pragma unroll
+    for (int q = 0; q < kPieceItems; ++q) {
+        const uint32_t kp = q == 0 ? key_before : key[q - 1];
+        const int32_t rp = q == 0 ? trow_before : trow[q - 1];
+        if (q0 + q < cnt && (rp != trow[q] || (kp >> (2 * LK)) != (key[q] >> (2 * LK)))) h |= 1u << q;
+    }
+    int excl;
+    const int heads = block_scan<kPieceThreads>(__popc(h), &excl);
+    {
+        int t = excl - 1;  // tile of the run in progress
+        Tile acc = 0;
+        bool owned = false;  // the run began in this thread
+        auto flush = [&](bool ended) {
+            if (!acc) return;
+            if (owned && ended) s_tile[t] = acc;
+            else atomicOr(&s_tile[t], acc);
+            acc = 0;
+        };
+#pragma unroll
+        for (int q = 0; q < kPieceItems; ++q) {
+            if (q0 + q < cnt) {
+                if ((h >> q) & 1u) {
+                    flush(true);
+                    ++t;
+                    owned = true;
+                    s_col[t] = (int32_t)(key[q] >> (2 * LK));
+                    const int32_t rp = q == 0 ? trow_before : trow[q - 1];
+                    if (!slice)
+                        for (int32_t r = rp + 1; r <= trow[q]; ++r) trow_at[I0 + r] = t;
+                }
+                acc |= (Tile)1 << ((key[q] & (K - 1)) * 8 + ((key[q] >> LK) & (K - 1)));
+            }
+        }
+        flush(false);
+    }
+    __syncthreads();
+    if (!slice) {  // tile-rows after the last entry, or all of an empty piece
+        const int32_t from = cnt > 0 ? (s_row[cnt - 1] >> LK) + 1 : 0;
+        for (int32_t r = from + threadIdx.x; r < I1 - I0; r += kPieceThreads) trow_at[I0 + r] = heads;
+    } else if (threadIdx.x == 0 && p == p0) {
+        trow_at[I0] = 0;
+    }
+    if (threadIdx.x == 0) count[p] = heads;
+    const int64_t to = slice ? place[p] : e0;
+    for (int i = threadIdx.x; i < heads; i += kPieceThreads) {
+        col[to + i] = s_col[i];
+        tile[to + i] = s_tile[i];
+    }
+}
+
+// Moves every piece's tiles to their final place and completes TileRowPtr
+// (trow_at holds a tile-row's first tile counted from its piece's first).
+template <int K>
+__global__ void __launch_bounds__(kPieceThreads) gather_pieces_kernel(
+    int32_t ntr, int64_t npieces, const int32_t* __restrict__ first, const int32_t* __restrict__ parts,
+    const int64_t* __restrict__ poff, const int32_t* __restrict__ window, const int32_t* __restrict__ place, const int64_t* __restrict__ toff,
+    const int32_t* __restrict__ col, const typename PieceTile<K>::type* __restrict__ tile, int32_t* __restrict__ rowptr,
+    int32_t* __restrict__ colind, typename PieceTile<K>::type* __restrict__ tiles) {
+    const int64_t p = blockIdx.x;
+    const int32_t b = __ldg(window + p);
+    const int32_t slices = __ldg(parts + b);
+    const int64_t p0 = __ldg(poff + b + 1) - slices;  // the first slice
+    const int64_t t0 = __ldg(toff + p);
+    const int64_t cnt = __ldg(toff + p + 1) - t0, from = __ldg(place + p);
+    const int32_t f1 = __ldg(first + b + 1);
+    if (p < p0) {
+        for (int32_t I = __ldg(first + b) + threadIdx.x; I < f1 - (slices > 0 ? 1 : 0); I += kPieceThreads)
+            rowptr[I] += (int32_t)t0;
+    } else if (p == p0 && threadIdx.x == 0) {
+        rowptr[f1 - 1] += (int32_t)t0;
+    }
+    if (p == npieces - 1 && threadIdx.x == 0) rowptr[ntr] = (int32_t)(t0 + cnt);
+    // four tiles a thread and step, all loads before the stores
+    for (int64_t i0 = threadIdx.x; i0 < cnt; i0 += 4 * kPieceThreads) {
+        int32_t c[4];
+        typename PieceTile<K>::type w[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int64_t i = i0 + q * kPieceThreads;
+            if (i < cnt) {
+                c[q] = __ldg(col + from + i);
+                w[q] = __ldg(tile + from + i);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int64_t i = i0 + q * kPieceThreads;
+            if (i < cnt) {
+                colind[t0 + i] = c[q];
+                tiles[t0 + i] = w[q];
+            }
+        }
+    }
+}
+
+// Output arrays for T tiles; the padding after T is zeroed.
+struct TileArrays {
+    int32_t* rowptr = nullptr;
+    int32_t* colind = nullptr;
+    uint8_t* tiles = nullptr;
+    int64_t cap = 0;
+};
+
+static b2sr_status merge_pieces(int32_t n, const int32_t* rowptr, const int32_t* colind, int64_t nnz, int k,
+                                int32_t ntr, int64_t nwin, const int32_t* first, const int32_t* parts,
+                                const int64_t* poff, int64_t npieces, cudaStream_t s, TileArrays* out, int64_t* T) {
+    const int tb = tile_bytes(k);
+    DevBuf info(s), tmp(s), toff(s);
+    B2SR_TRY(info.alloc((size_t)npieces * (3 + k) * sizeof(int32_t) + sizeof(int32_t)));
+    int32_t* window = info.as<int32_t>();
+    int32_t* place = window + npieces;
+    int32_t* count = place + npieces;           // npieces + 1
+    int32_t* cut = count + npieces + 1;         // npieces * k
+    B2SR_TRY(tmp.alloc((size_t)nnz * (tb + sizeof(int32_t))));
+    uint8_t* tile = tmp.as<uint8_t>();          // 8-byte tiles first: aligned
+    int32_t* col = reinterpret_cast<int32_t*>(tile + (size_t)nnz * tb);
+    B2SR_TRY(toff.alloc((size_t)(npieces + 1) * sizeof(int64_t)));
+    B2SR_TRY(dalloc(&out->rowptr, (size_t)ntr + 1, s));
+    pieces_kernel<<<grid_wide(npieces * k), 256, 0, s>>>(rowptr, colind, n, ntr, k, nwin, first, parts, poff, npieces, window,
+                                                        cut);
+    B2SR_LAUNCH_CHECK("pieces_kernel");
+    B2SR_CUDA_TRY(cudaMemsetAsync(count + npieces, 0, sizeof(int32_t), s));
+    if (k == 4)
+        merge_piece_kernel<4><<<(unsigned)npieces, kPieceThreads, 0, s>>>(rowptr, colind, n, first, parts, poff, window, cut,
+                                                                        out->rowptr, count, place, col,
+                                                                        reinterpret_cast<uint32_t*>(tile));
+    else
+        merge_piece_kernel<8><<<(unsigned)npieces, kPieceThreads, 0, s>>>(rowptr, colind, n, first, parts, poff, window, cut,
+                                                                        out->rowptr, count, place, col,
+                                                                        reinterpret_cast<unsigned long long*>(tile));
+    B2SR_LAUNCH_CHECK("merge_piece_kernel");
+    B2SR_TRY(exclusive_scan_i32_to_i64(count, toff.as<int64_t>(), npieces + 1, s));
+    B2SR_CUDA_TRY(cudaMemcpyAsync(T, toff.as<int64_t>() + npieces, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    B2SR_CUDA_TRY(cudaStreamSynchronize(s));
+    out->cap = std::max<int64_t>(round_up(*T, kTilePad), kTilePad);
+    B2SR_TRY(dalloc(&out->colind, (size_t)out->cap, s));
+    B2SR_TRY(dalloc(&out->tiles, (size_t)out->cap * tb, s));
+    B2SR_CUDA_TRY(cudaMemsetAsync(out->colind + *T, 0, (size_t)(out->cap - *T) * sizeof(int32_t), s));
+    B2SR_CUDA_TRY(cudaMemsetAsync(out->tiles + *T * tb, 0, (size_t)(out->cap - *T) * tb, s));
+    if (k == 4)
+        gather_pieces_kernel<4><<<(unsigned)npieces, kPieceThreads, 0, s>>>(
+            ntr, npieces, first, parts, poff, window, place, toff.as<int64_t>(), col, reinterpret_cast<const uint32_t*>(tile),
+            out->rowptr, out->colind, reinterpret_cast<uint32_t*>(out->tiles));
+    else
+        gather_pieces_kernel<8><<<(unsigned)npieces, kPieceThreads, 0, s>>>(
+            ntr, npieces, first, parts, poff, window, place, toff.as<int64_t>(), col,
+            reinterpret_cast<const unsigned long long*>(tile), out->rowptr, out->colind,
+            reinterpret_cast<unsigned long long*>(out->tiles));
+    B2SR_LAUNCH_CHECK("gather_pieces_kernel");
+    return B2SR_OK;
+}
+
+// ---------------------------------------------------------------------------
+// schedule: tile-row of the first tile of every SpMV chunk, and the tile-rows
+// that cross chunks
+// ---------------------------------------------------------------------------
+// The row R that chunk c begins inside, when R started in an earlier chunk
+// and ends in c, goes to the split list: rows over at most kSplitShort chunks
+// from the front, longer ones from the back (in no order: each is joined by
+// itself).  meta: first and last tile-row with tiles, short and long rows.
+__global__ void schedule_kernel(const int32_t* __restrict__ rowptr, int32_t ntr, int64_t T, int64_t CT,
+                                int64_t nchunks, int32_t* __restrict__ chunk_row, int32_t* __restrict__ split,
+                                int32_t* __restrict__ meta) {
+    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c <= nchunks;
          c += (int64_t)gridDim.x * blockDim.x) {
-        if (!kshort[c] && !klong[c]) continue;
-        const int32_t R = chunk_row[c];
-        const int64_t at = kshort[c] ? pshort[c] : nshort + plong[c];
+        const int64_t cs = min(c * CT, T - 1);
+        const int32_t R = row_of(rowptr, 0, ntr - 1, cs);
+        chunk_row[c] = R;
+        if (c == 0) meta[0] = R;
+        if (c == nchunks) meta[1] = R;
+        if (c == 0 || c == nchunks) continue;
+        const int64_t ce = min(cs + CT, T);
+        const int64_t rs = rowptr[R], re = rowptr[R + 1];
+        if (rs >= cs || re > ce) continue;
+        const int64_t ca = rs / CT;
+        const int64_t at = c - ca + 1 <= kSplitShort ? atomicAdd(meta + 2, 1) : nchunks - 1 - atomicAdd(meta + 3, 1);
         split[3 * at] = R;
-        split[3 * at + 1] = (int32_t)(rowptr[R] / CT);
+        split[3 * at + 1] = (int32_t)ca;
         split[3 * at + 2] = (int32_t)c;
     }
-}
-
-static b2sr_status build_split_list(b2sr_matrix* h, cudaStream_t s) {
-    const int64_t CT = chunk_tiles(h->k);
-    const int64_t nc = h->nchunks;
-    DevBuf ks(s), kl(s), ps(s), pl(s);
-    B2SR_TRY(ks.alloc((nc + 1) * sizeof(int32_t)));
-    B2SR_TRY(kl.alloc((nc + 1) * sizeof(int32_t)));
-    B2SR_TRY(ps.alloc((nc + 1) * sizeof(int64_t)));
-    B2SR_TRY(pl.alloc((nc + 1) * sizeof(int64_t)));
-    int grid = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(nc, 256), (int64_t)sm_count() * 8));
-    split_kind_kernel<<<grid, 256, 0, s>>>(h->rowptr, h->chunk_row, h->T, CT, nc, ks.as<int32_t>(), kl.as<int32_t>());
-    B2SR_LAUNCH_CHECK("split_kind_kernel");
-    B2SR_CUDA_TRY(cudaMemsetAsync(ks.as<int32_t>() + nc, 0, sizeof(int32_t), s));
-    B2SR_CUDA_TRY(cudaMemsetAsync(kl.as<int32_t>() + nc, 0, sizeof(int32_t), s));
-    B2SR_TRY(exclusive_scan_i32_to_i64(ks.as<int32_t>(), ps.as<int64_t>(), nc + 1, s));
-    B2SR_TRY(exclusive_scan_i32_to_i64(kl.as<int32_t>(), pl.as<int64_t>(), nc + 1, s));
-    int64_t ns = 0, nl = 0;
-    B2SR_CUDA_TRY(cudaMemcpyAsync(&ns, ps.as<int64_t>() + nc, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    B2SR_CUDA_TRY(cudaMemcpyAsync(&nl, pl.as<int64_t>() + nc, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    B2SR_CUDA_TRY(cudaStreamSynchronize(s));
-    B2SR_TRY(dalloc(&h->split, (size_t)std::max<int64_t>(3 * (ns + nl), 3), s));
-    split_fill_kernel<<<grid, 256, 0, s>>>(h->rowptr, h->chunk_row, CT, nc, ks.as<int32_t>(), kl.as<int32_t>(),
-                                           ps.as<int64_t>(), pl.as<int64_t>(), ns, h->split);
-    B2SR_LAUNCH_CHECK("split_fill_kernel");
-    B2SR_CUDA_TRY(cudaStreamSynchronize(s));
-    h->nsplit_short = ns;
-    h->nsplit_long = nl;
-    return B2SR_OK;
 }
 
 b2sr_status build_schedule(b2sr_matrix* h, cudaStream_t s) {
@@ -651,23 +1044,28 @@ b2sr_status build_schedule(b2sr_matrix* h, cudaStream_t s) {
         h->last_row = -1;
         return B2SR_OK;
     }
-    int64_t CT = chunk_tiles(h->k);
+    const int64_t CT = chunk_tiles(h->k);
     h->nchunks = ceil_div(h->T, CT);
     B2SR_TRY(dalloc(&h->chunk_row, h->nchunks + 1, s));
-    int grid = (int)std::min<int64_t>(ceil_div(h->nchunks + 1, 256), (int64_t)sm_count() * 8);
-    chunk_rows_kernel<<<grid, 256, 0, s>>>(h->rowptr, h->ntr, h->T, CT, h->nchunks, h->chunk_row);
-    B2SR_LAUNCH_CHECK("chunk_rows_kernel");
-    int32_t fr = 0, lr = 0;
-    B2SR_CUDA_TRY(cudaMemcpyAsync(&fr, h->chunk_row, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-    B2SR_CUDA_TRY(cudaMemcpyAsync(&lr, h->chunk_row + h->nchunks, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    B2SR_TRY(dalloc(&h->split, 3 * h->nchunks, s));
+    DevBuf meta(s);
+    B2SR_TRY(meta.alloc(4 * sizeof(int32_t)));
+    B2SR_CUDA_TRY(cudaMemsetAsync(meta.p, 0, 4 * sizeof(int32_t), s));
+    schedule_kernel<<<grid_for(h->nchunks + 1), 256, 0, s>>>(h->rowptr, h->ntr, h->T, CT, h->nchunks, h->chunk_row,
+                                                            h->split, meta.as<int32_t>());
+    B2SR_LAUNCH_CHECK("schedule_kernel");
+    int32_t got[4] = {0, 0, 0, 0};
+    B2SR_CUDA_TRY(cudaMemcpyAsync(got, meta.p, sizeof(got), cudaMemcpyDeviceToHost, s));
     B2SR_CUDA_TRY(cudaStreamSynchronize(s));
-    h->first_row = fr;
-    h->last_row = lr;
-    return build_split_list(h, s);
+    h->first_row = got[0];
+    h->last_row = got[1];
+    h->nsplit_short = got[2];
+    h->nsplit_long = got[3];
+    return B2SR_OK;
 }
 
 b2sr_status new_handle_from_tiles(int32_t n, int k, int64_t T, int32_t* rowptr, int32_t* colind,
-                                  uint8_t* tiles, int64_t cap, cudaStream_t s, b2sr_matrix** out) {
+                                  uint8_t* tiles, int64_t cap, cudaStream_t s, b2sr_matrix** out, int64_t known_nnz) {
     b2sr_matrix* h = new b2sr_matrix();
     h->n = n;
     h->k = k;
@@ -686,14 +1084,21 @@ b2sr_status new_handle_from_tiles(int32_t n, int k, int64_t T, int32_t* rowptr, 
     // the SpMV and driver kernels index tiles with int32
     if (T >= (int64_t(1) << 31)) return cleanup(fail(B2SR_ERR_OOM, "more than 2^31 - 1 tiles"));
     DevBuf cnt(s);
-    b2sr_status st = cnt.alloc(sizeof(int64_t));
-    if (st != B2SR_OK) return cleanup(st);
-    st = popcount_bytes(tiles, cap * tile_bytes(k), cnt.as<int64_t>(), s);
-    if (st != B2SR_OK) return cleanup(st);
-    int64_t nnz = 0;
-    cudaError_t e = cudaMemcpyAsync(&nnz, cnt.p, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
-    if (e != cudaSuccess) return cleanup(cuda_fail(e, "copy nnz"));
-    st = build_schedule(h, s);  // synchronises s
+    b2sr_status st = B2SR_OK;
+    int64_t nnz = known_nnz;
+    if (known_nnz < 0) {
+        st = cnt.alloc(sizeof(int64_t));
+        if (st != B2SR_OK) return cleanup(st);
+        st = popcount_bytes(tiles, cap * tile_bytes(k), cnt.as<int64_t>(), s);
+        if (st != B2SR_OK) return cleanup(st);
+        cudaError_t e = cudaMemcpyAsync(&nnz, cnt.p, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
+        if (e != cudaSuccess) return cleanup(cuda_fail(e, "copy nnz"));
+        if (T == 0) {  // build_schedule does not wait for the copy then
+            e = cudaStreamSynchronize(s);
+            if (e != cudaSuccess) return cleanup(cuda_fail(e, "copy nnz"));
+        }
+    }
+    st = build_schedule(h, s);  // synchronises s when there are tiles
     if (st != B2SR_OK) return cleanup(st);
     h->nnz = nnz;
     *out = h;
@@ -1113,9 +1518,13 @@ extern "C" b2sr_status b2sr_from_csr(int32_t n, const int32_t* rowptr, const int
     if (2 * sbits + 10 > 64) return fail(B2SR_ERR_INVALID_ARG, "matrix too large");
 
     // validate; note whether every row is in column order
-    bool sorted_rows = false;
+    bool sorted_rows = false, repeats = false;
     const int64_t blocks = ceil_div(nnz, kRankEntries);
-    DevBuf brow(s);
+    // rows in column order without repeats at k <= 8: pieces (32-bit keys)
+    const bool small = k <= 8 && nnz > 0 && (int64_t)n * k < (int64_t(1) << 32);
+    const int64_t nwin = ceil_div(std::max<int64_t>(nnz, 1), kWindow);
+    int64_t npieces = 0;
+    DevBuf brow(s), wbuf(s), poff(s);
     {
         DevBuf bad(s), starts(s);
         const size_t start_words = (size_t)ceil_div(std::max<int64_t>(nnz, 1), 32);
@@ -1131,11 +1540,37 @@ extern "C" b2sr_status b2sr_from_csr(int32_t n, const int32_t* rowptr, const int
                 n, colind, nnz, starts.as<uint32_t>(), bad.as<int>(), bad.as<int>() + 1);
             B2SR_LAUNCH_CHECK("validate_entries_kernel");
         }
+        if (small) {
+            B2SR_TRY(wbuf.alloc(3 * (size_t)(nwin + 1) * sizeof(int32_t)));
+            B2SR_TRY(poff.alloc((size_t)(nwin + 1) * sizeof(int64_t)));
+            int32_t* first = wbuf.as<int32_t>();
+            int32_t* counts = first + 2 * (nwin + 1);
+            windows_kernel<<<grid_wide(nwin + 1), 256, 0, s>>>(rowptr, n, ntr, k, nwin, first, first + nwin + 1, counts);
+            B2SR_LAUNCH_CHECK("windows_kernel");
+            B2SR_TRY(exclusive_scan_i32_to_i64(counts, poff.as<int64_t>(), nwin + 1, s));
+            B2SR_CUDA_TRY(cudaMemcpyAsync(&npieces, poff.as<int64_t>() + nwin, sizeof(int64_t), cudaMemcpyDeviceToHost,
+                                          s));
+        }
         int hbad[2] = {0, 0};
         B2SR_CUDA_TRY(cudaMemcpyAsync(hbad, bad.p, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
         B2SR_CUDA_TRY(cudaStreamSynchronize(s));
         if (hbad[0]) return fail(B2SR_ERR_INVALID_ARG, "malformed CSR (rowptr/colind/nnz inconsistent)");
-        sorted_rows = hbad[1] == 0;
+        sorted_rows = (hbad[1] & 1) == 0;
+        repeats = (hbad[1] & 2) != 0;
+    }
+    if (small && sorted_rows && !repeats) {
+        TileArrays a;
+        int64_t tiles = 0;
+        const b2sr_status st = merge_pieces(n, rowptr, colind, nnz, k, ntr, nwin, wbuf.as<int32_t>(),
+                                            wbuf.as<int32_t>() + nwin + 1, poff.as<int64_t>(), npieces, s, &a, &tiles);
+        if (st != B2SR_OK) {
+            dfree(a.rowptr, s); dfree(a.colind, s); dfree(a.tiles, s);
+            return st;
+        }
+        b2sr_matrix* h = nullptr;
+        B2SR_TRY(new_handle_from_tiles(n, k, tiles, a.rowptr, a.colind, a.tiles, a.cap, s, &h, nnz));
+        *out = h;
+        return B2SR_OK;
     }
     if (nnz > 0) {
         B2SR_TRY(brow.alloc((size_t)(blocks + 1) * sizeof(int32_t)));

@@ -1717,8 +1717,8 @@ __global__ void __launch_bounds__(kSpmvThreads, (gather_min_blocks<K, SEM>())) s
 // remaining blocks give a warp to each longer row (lane l folds every 32nd
 // partial in order, then a fixed butterfly joins the lanes).
 template <int K, class SEM>
-__global__ void spmv_fixup_kernel(const int32_t* __restrict__ split, int64_t nshort, int64_t nlong,
-                                  int64_t short_blocks, SEM sem, Partials<typename SEM::V> part,
+__global__ void spmv_fixup_kernel(const int32_t* __restrict__ split, const int32_t* __restrict__ split_long,
+                                  int64_t nshort, int64_t nlong, int64_t short_blocks, SEM sem, Partials<typename SEM::V> part,
                                   const int32_t* gate) {
     using V = typename SEM::V;
     using J = typename SEM::J;
@@ -1755,9 +1755,9 @@ __global__ void spmv_fixup_kernel(const int32_t* __restrict__ split, int64_t nsh
         return;
     }
     const int lane = (int)lane_id();
-    const int64_t e = nshort + ((int64_t)(blockIdx.x - short_blocks) * blockDim.x + threadIdx.x) / 32;
-    if (e >= nshort + nlong) return;  // whole warps leave together
-    const int32_t R = split[3 * e], ca = split[3 * e + 1], cb = split[3 * e + 2];
+    const int64_t e = ((int64_t)(blockIdx.x - short_blocks) * blockDim.x + threadIdx.x) / 32;
+    if (e >= nlong) return;  // whole warps leave together
+    const int32_t R = split_long[3 * e], ca = split_long[3 * e + 1], cb = split_long[3 * e + 2];
     const int64_t np = (int64_t)cb - ca + 1;
     J acc[NV];
 #pragma unroll
@@ -1790,7 +1790,8 @@ static b2sr_status launch_fixup(const b2sr_matrix* h, const SEM& sem, Partials<t
     const int64_t short_blocks = ceil_div(h->nsplit_short * (SEM::kGather ? SEM::NV : 1), 256);
     const int64_t long_blocks = ceil_div(h->nsplit_long, 8);
     spmv_fixup_kernel<K, SEM><<<(unsigned)(short_blocks + long_blocks), 256, 0, s>>>(
-        h->split, h->nsplit_short, h->nsplit_long, short_blocks, sem, part, gate);
+        h->split, h->split + 3 * (h->nchunks - h->nsplit_long), h->nsplit_short, h->nsplit_long, short_blocks, sem, part,
+        gate);
     B2SR_LAUNCH_CHECK("spmv_fixup_kernel");
     return B2SR_OK;
 }
