@@ -150,36 +150,48 @@ __global__ void masked_count_kernel(MatView A, MatView B, MatView M, unsigned lo
 // ---------------------------------------------------------------------------
 // For every mask entry (i, j): the columns common to row i of A and row j of
 // B.  The three operands' rows are extracted as column lists first (one
-// balanced pass over their tiles); then a block takes kRunEntries consecutive
-// mask entries, row by row:
-//   * a row of A with more than 32 columns becomes a bitmap in the block's
-//     shared memory; the row's mask entries are dealt to the warps, and the
-//     lanes of a warp walk row j of B, testing each column in the bitmap: a
+// balanced pass over their tiles).  The shorter of the two rows is walked and
+// tested in the longer one: a first launch takes the entries whose row of A is
+// at least as long, by rows of the mask, a second one the others, by columns
+// (walking row j of B always: 3.5 G columns for the triangles of R-MAT 18, ef
+// 32; the shorter row: 1.2 G).  A block takes kRunEntries consecutive mask
+// entries, row by row:
+//   * a row with more than 32 columns becomes a bitmap in the block's shared
+//     memory; the warps fetch the row's mask entries one by one, and the lanes
+//     walk the entry's other row, testing each column in the bitmap: a
 //     coalesced load and one shared load per column, no searches;
-//   * a shorter row of A stays a list: the warps take such rows one by one,
-//     a group of lanes (as wide as the row) per mask entry, each lane
-//     searching its column in row j of B.
+//   * a shorter row stays a list: the warps take such rows one by one, a group
+//     of lanes (as wide as the row) per mask entry, each lane searching its
+//     column in the entry's other row.
 // Where a bitmap of n bits does not fit in shared memory every row takes the
 // second form.
 constexpr int kRunEntries = 256;
 constexpr int64_t kMaxBitmapBytes = 200 * 1024;
+// Fewer mask entries than this take one launch: grouping the others by column
+// (three launches and a scan) costs more than the shorter walks save.
+constexpr int64_t kSplitEntries = 1 << 17;
 
+// Row i: colind[begin[i] .. end[i]) (end = begin + 1 for a plain CSR).  Rows
+// lie one after another, with gaps where end[i] < begin[i + 1].
 struct RowLists {
-    const int32_t* rowptr;
+    const int32_t* begin;
+    const int32_t* end;
     const int32_t* colind;
 };
 
 // Ones of the short row list a[0..d) in row j of B, over mask entries
-// [e0, e1), by one warp.
+// [e0, e1), by one warp; with `longer` only where row j is not longer than d.
 __device__ __forceinline__ uint32_t count_listed(const int32_t* __restrict__ acol, int32_t d, RowLists B,
-                                                 const int32_t* __restrict__ mcol, int32_t e0, int32_t e1, int lane) {
+                                                 const int32_t* __restrict__ mcol, int32_t e0, int32_t e1, bool longer,
+                                                 int lane) {
     int width = 32;  // lanes a mask entry: the least power of two holding the row
     while (width > 1 && width / 2 >= d) width >>= 1;
     const int sub = lane & (width - 1);
     uint32_t acc = 0;
     for (int32_t e = e0 + lane / width; e < e1; e += 32 / width) {
         const int32_t j = __ldg(mcol + e);
-        const int32_t b0 = __ldg(B.rowptr + j), b1 = __ldg(B.rowptr + j + 1);
+        const int32_t b0 = __ldg(B.begin + j), b1 = __ldg(B.end + j);
+        if (longer && b1 - b0 > d) continue;
         for (int32_t p = sub; p < d; p += width) {
             const int32_t v = __ldg(acol + p);
             const int32_t q = lower_bound_i32(B.colind, b0, b1, v);
@@ -189,76 +201,122 @@ __device__ __forceinline__ uint32_t count_listed(const int32_t* __restrict__ aco
     return acc;
 }
 
-__global__ void __launch_bounds__(256) masked_rows_kernel(int32_t n, RowLists A, RowLists B, RowLists M,
-                                                          int32_t mnnz, int use_bitmap, int bitmap_words,
-                                                          unsigned long long* __restrict__ out) {
-    extern __shared__ __align__(16) uint32_t bitmap[];
-    __shared__ unsigned long long warp_sum[8];
-    __shared__ int32_t long_row[kRunEntries];  // at least one mask entry of the run in each
-    __shared__ int nlong;
-    const int lane = (int)lane_id(), warp = threadIdx.x >> 5;
-    const int32_t e0 = (int32_t)blockIdx.x * kRunEntries;
-    const int32_t e1 = min(e0 + kRunEntries, mnnz);
-    // rows of the first and the last mask entry of the run
-    auto row_of_entry = [&](int32_t e) {
+__global__ void column_starts_kernel(const int64_t* __restrict__ off, int64_t len, int32_t* __restrict__ colptr,
+                                     int32_t* __restrict__ cursor) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < len; i += (int64_t)gridDim.x * blockDim.x)
+        colptr[i] = cursor[i] = (int32_t)off[i];
+}
+
+// Mask entries whose row of B is longer than their row of A.  First pass: the
+// entry's row in row_of (-1 for the others), counted by column; second: the
+// rows written by column.  A thread an entry, so that a hub's row is shared
+// (a warp a row took 520 us a pass on R-MAT 18, ef 32).
+__global__ void count_by_column_kernel(int32_t n, RowLists A, RowLists B, RowLists M, int32_t mnnz,
+                                       int32_t* __restrict__ row_of, int32_t* __restrict__ count) {
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < mnnz; e += (int64_t)gridDim.x * blockDim.x) {
         int32_t lo = 0, hi = n - 1;  // the last row starting at or before e
         while (lo < hi) {
             const int32_t mid = lo + ((hi - lo + 1) >> 1);
-            if (__ldg(M.rowptr + mid) <= e) lo = mid; else hi = mid - 1;
+            if (__ldg(M.begin + mid) <= e) lo = mid; else hi = mid - 1;
         }
-        return lo;
-    };
-    const int32_t i0 = row_of_entry(e0), i1 = row_of_entry(e1 - 1);
-    if (use_bitmap)
-        for (int w = threadIdx.x; w < bitmap_words; w += 256) bitmap[w] = 0u;
-    if (threadIdx.x == 0) nlong = 0;
+        const int32_t d = __ldg(A.end + lo) - __ldg(A.begin + lo);
+        const int32_t j = __ldg(M.colind + e);
+        const bool other = d > 0 && e < __ldg(M.end + lo) && __ldg(B.end + j) - __ldg(B.begin + j) > d;
+        row_of[e] = other ? lo : -1;
+        if (other) atomicAdd(count + j, 1);
+    }
+}
+
+__global__ void place_by_column_kernel(const int32_t* __restrict__ row_of, const int32_t* __restrict__ mcol,
+                                       int32_t mnnz, int32_t* __restrict__ cursor, int32_t* __restrict__ rows) {
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < mnnz; e += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t i = __ldg(row_of + e);
+        if (i >= 0) rows[atomicAdd(cursor + __ldg(mcol + e), 1)] = i;
+    }
+}
+
+__global__ void __launch_bounds__(256) masked_rows_kernel(int32_t n, RowLists A, RowLists B, RowLists M,
+                                                          const int32_t* mnnz, int longer, int use_bitmap,
+                                                          int bitmap_words, unsigned long long* __restrict__ out) {
+    extern __shared__ __align__(16) uint32_t bitmap[];
+    __shared__ unsigned long long warp_sum[8];
+    __shared__ int32_t long_row[kRunEntries];  // at least one mask entry of the run in each
+    __shared__ int nlong, nother[2];
+    __shared__ int2 other[kRunEntries];  // the other rows of a long row's mask entries
+    const int lane = (int)lane_id(), warp = threadIdx.x >> 5;
+    const int32_t e0 = (int32_t)blockIdx.x * kRunEntries;
+    const int32_t e1 = min(e0 + kRunEntries, __ldg(mnnz));
+    if (e0 >= e1) return;
+    // rows of the first and the last mask entry of the run: warps 0 and 1
+    __shared__ int32_t row_range[2];
+    if (warp < 2) {
+        const int32_t e = warp == 0 ? e0 : e1 - 1;
+        int32_t lo = 0, hi = n - 1;  // the last row starting at or before e
+        while (lo < hi) {
+            const int32_t mid = lo + ((hi - lo + 1) >> 1);
+            if (__ldg(M.begin + mid) <= e) lo = mid; else hi = mid - 1;
+        }
+        if (lane == 0) row_range[warp] = lo;
+    }
+    if (use_bitmap) {
+        const uint4 zero = make_uint4(0u, 0u, 0u, 0u);  // the bitmap is padded to whole 16 bytes
+        for (int w = threadIdx.x; w < (bitmap_words + 3) / 4; w += 256) reinterpret_cast<uint4*>(bitmap)[w] = zero;
+    }
+    if (threadIdx.x == 0) nlong = nother[0] = 0;
     __syncthreads();
+    const int32_t i0 = row_range[0], i1 = row_range[1];
+    if (i0 == i1 && __ldg(M.end + i0) <= e0) return;  // the run lies in a gap
     uint32_t acc = 0;
     const int32_t listed = use_bitmap ? 32 : INT32_MAX;  // longest row taken as a list
     for (int32_t base = i0; base <= i1; base += 256) {
         const int32_t i = base + 8 * lane + warp;  // neighbouring rows go to different warps
         int32_t a0 = 0, d = 0, m0 = 0, m1 = 0;
         if (i <= i1) {
-            a0 = __ldg(A.rowptr + i);
-            d = __ldg(A.rowptr + i + 1) - a0;
-            m0 = max(e0, __ldg(M.rowptr + i));
-            m1 = min(e1, __ldg(M.rowptr + i + 1));
+            a0 = __ldg(A.begin + i);
+            d = __ldg(A.end + i) - a0;
+            m0 = max(e0, __ldg(M.begin + i));
+            m1 = min(e1, __ldg(M.end + i));
         }
         const bool live = d > 0 && m0 < m1;
         if (live && d > listed) long_row[atomicAdd(&nlong, 1)] = i;
         for (unsigned todo = __ballot_sync(0xffffffffu, live && d <= listed); todo; todo &= todo - 1) {
             const int src = __ffs(todo) - 1;
             acc += count_listed(A.colind + __shfl_sync(0xffffffffu, a0, src), __shfl_sync(0xffffffffu, d, src), B,
-                                M.colind, __shfl_sync(0xffffffffu, m0, src), __shfl_sync(0xffffffffu, m1, src), lane);
+                                M.colind, __shfl_sync(0xffffffffu, m0, src), __shfl_sync(0xffffffffu, m1, src), longer,
+                                lane);
         }
     }
     if (use_bitmap) {
         __syncthreads();
         for (int r = 0; r < nlong; ++r) {
             const int32_t i = long_row[r];
-            const int32_t a0 = __ldg(A.rowptr + i), a1 = __ldg(A.rowptr + i + 1);
-            const int32_t m0 = max(e0, __ldg(M.rowptr + i)), m1 = min(e1, __ldg(M.rowptr + i + 1));
+            const int32_t a0 = __ldg(A.begin + i), a1 = __ldg(A.end + i);
+            const int32_t m0 = max(e0, __ldg(M.begin + i)), m1 = min(e1, __ldg(M.end + i));
+            // the entries' other rows (at most 256 entries a run)
+            if (threadIdx.x < m1 - m0) {
+                const int32_t j = __ldg(M.colind + m0 + threadIdx.x);
+                const int32_t b0 = __ldg(B.begin + j), b1 = __ldg(B.end + j);
+                if (b1 > b0 && !(longer && b1 - b0 > a1 - a0)) other[atomicAdd(&nother[r & 1], 1)] = make_int2(b0, b1);
+            }
             for (int32_t p = a0 + threadIdx.x; p < a1; p += 256) {
                 const int32_t v = __ldg(A.colind + p);
                 atomicOr(bitmap + (v >> 5), 1u << (v & 31));
             }
+            if (threadIdx.x == 0) nother[(r + 1) & 1] = 0;
             __syncthreads();
-            // lane l of warp w holds mask entry m0 + 8 l + w (at most 256 entries a run)
-            const int32_t e = m0 + 8 * lane + warp;
-            int32_t b0 = 0, b1 = 0;
-            if (e < m1) {
-                const int32_t j = __ldg(M.colind + e);
-                b0 = __ldg(B.rowptr + j);
-                b1 = __ldg(B.rowptr + j + 1);
-            }
-            const int cnt = m1 - m0 > warp ? (m1 - m0 - warp + 7) / 8 : 0;
-            for (int q = 0; q < cnt; ++q) {
-                const int32_t s0 = __shfl_sync(0xffffffffu, b0, q), s1 = __shfl_sync(0xffffffffu, b1, q);
+            const int todo = nother[r & 1];
+            // the next entry's first columns are loaded before this one's are used
+            auto test = [&](int32_t v) { return (bitmap[v >> 5] >> (v & 31)) & 1u; };
+            int2 o = warp < todo ? other[warp] : make_int2(0, 0);
+            int32_t v = o.x + lane < o.y ? __ldg(B.colind + o.x + lane) : -1;
+            for (int q = warp; q < todo; q += 8) {
+                const int2 o2 = q + 8 < todo ? other[q + 8] : make_int2(0, 0);
+                const int32_t v2 = o2.x + lane < o2.y ? __ldg(B.colind + o2.x + lane) : -1;
+                if (v >= 0) acc += test(v);
 #pragma unroll 4
-                for (int32_t p = s0 + lane; p < s1; p += 32) {
-                    const int32_t v = __ldg(B.colind + p);
-                    acc += (bitmap[v >> 5] >> (v & 31)) & 1u;
-                }
+                for (int32_t p = o.x + 32 + lane; p < o.y; p += 32) acc += test(__ldg(B.colind + p));
+                o = o2;
+                v = v2;
             }
             __syncthreads();
             for (int32_t p = a0 + threadIdx.x; p < a1; p += 256) bitmap[__ldg(A.colind + p) >> 5] = 0u;
@@ -387,7 +445,47 @@ static b2sr_status row_lists(const b2sr_matrix* h, DevBuf& buf, RowLists* out, c
     int32_t* rowptr = buf.as<int32_t>();
     int32_t* colind = reinterpret_cast<int32_t*>(buf.as<char>() + rp);
     B2SR_TRY(extract_csr(h, off.as<int64_t>(), rowptr, colind, s));
-    *out = RowLists{rowptr, colind};
+    *out = RowLists{rowptr, rowptr + 1, colind};
+    return B2SR_OK;
+}
+
+// The count over extracted rows; `slots` entries of m.colind, gaps included,
+// hold the mask.
+static b2sr_status count_rows(int32_t n, RowLists a, RowLists b, RowLists m, int64_t slots, unsigned long long* out,
+                              cudaStream_t s, double bytes) {
+    const int64_t words = ceil_div(n, 32);
+    const int use_bitmap = words * 4 <= kMaxBitmapBytes;
+    const int smem = use_bitmap ? (int)round_up(words, 4) * 4 : 0;
+    const int64_t runs = ceil_div(slots, kRunEntries);
+    B2SR_CUDA_TRY(cudaFuncSetAttribute(masked_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    const bool split = slots >= kSplitEntries;
+    void* tok = timing_begin(s);
+    // m.begin[n] (the row pointer of a CSR) ends the slots
+    masked_rows_kernel<<<(unsigned)runs, 256, smem, s>>>(n, a, b, m, m.begin + n, split, use_bitmap, (int)words, out);
+    B2SR_LAUNCH_CHECK("masked_rows_kernel");
+    if (split) {
+        DevBuf cnt(s), off(s), cur(s), rows(s);
+        B2SR_TRY(cnt.alloc(((size_t)n + 1) * sizeof(int32_t)));
+        B2SR_TRY(off.alloc(((size_t)n + 1) * sizeof(int64_t)));
+        B2SR_TRY(cur.alloc(2 * ((size_t)n + 1) * sizeof(int32_t)));
+        B2SR_TRY(rows.alloc(2 * (size_t)slots * sizeof(int32_t)));
+        int32_t* colptr = cur.as<int32_t>();
+        int32_t* cursor = colptr + n + 1;
+        int32_t* row_of = rows.as<int32_t>() + slots;
+        B2SR_CUDA_TRY(cudaMemsetAsync(cnt.p, 0, ((size_t)n + 1) * sizeof(int32_t), s));
+        count_by_column_kernel<<<grid_wide(slots), 256, 0, s>>>(n, a, b, m, (int32_t)slots, row_of, cnt.as<int32_t>());
+        B2SR_LAUNCH_CHECK("count_by_column_kernel");
+        B2SR_TRY(exclusive_scan_i32_to_i64(cnt.as<int32_t>(), off.as<int64_t>(), (int64_t)n + 1, s));
+        column_starts_kernel<<<grid_wide((int64_t)n + 1), 256, 0, s>>>(off.as<int64_t>(), (int64_t)n + 1, colptr, cursor);
+        B2SR_LAUNCH_CHECK("column_starts_kernel");
+        place_by_column_kernel<<<grid_wide(slots), 256, 0, s>>>(row_of, m.colind, (int32_t)slots, cursor,
+                                                               rows.as<int32_t>());
+        B2SR_LAUNCH_CHECK("place_by_column_kernel");
+        const RowLists mt{colptr, colptr + 1, rows.as<int32_t>()};
+        masked_rows_kernel<<<(unsigned)runs, 256, smem, s>>>(n, b, a, mt, colptr + n, 0, use_bitmap, (int)words, out);
+        B2SR_LAUNCH_CHECK("masked_rows_kernel");
+    }
+    timing_end(tok, "spgemm_masked", bytes, s);
     return B2SR_OK;
 }
 
@@ -398,16 +496,30 @@ static b2sr_status masked_count_rows(const b2sr_matrix* A, const b2sr_matrix* B,
     B2SR_TRY(row_lists(A, abuf, &a, s));
     if (B == A) b = a; else B2SR_TRY(row_lists(B, bbuf, &b, s));
     if (M == A) m = a; else if (M == B) m = b; else B2SR_TRY(row_lists(M, mbuf, &m, s));
-    const int64_t words = ceil_div(A->n, 32);
-    const int use_bitmap = words * 4 <= kMaxBitmapBytes;
-    const int smem = use_bitmap ? (int)words * 4 : 0;
-    B2SR_CUDA_TRY(cudaFuncSetAttribute(masked_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    void* tok = timing_begin(s);
-    masked_rows_kernel<<<(unsigned)ceil_div(M->nnz, kRunEntries), 256, smem, s>>>(A->n, a, b, m, (int32_t)M->nnz,
-                                                                                use_bitmap, (int)words, out);
-    timing_end(tok, "spgemm_masked", bytes, s);
-    B2SR_LAUNCH_CHECK("masked_rows_kernel");
-    return B2SR_OK;
+    return count_rows(A->n, a, b, m, M->nnz, out, s, bytes);
+}
+
+// Row i's columns below i are a prefix of the row.
+__global__ void lower_ends_kernel(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ colind, int32_t n,
+                                  int32_t* __restrict__ end) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        end[i] = lower_bound_i32(colind, rowptr[i], rowptr[i + 1], (int32_t)i);
+}
+
+// Triangles: L the strictly lower triangle of h, sum over its entries (i, j)
+// of the columns common to rows i and j of L, without building L.
+b2sr_status lower_count(const b2sr_matrix* h, int64_t* count, cudaStream_t s) {
+    B2SR_CUDA_TRY(cudaMemsetAsync(count, 0, sizeof(int64_t), s));
+    if (h->T == 0) return B2SR_OK;
+    DevBuf buf(s), ends(s);
+    RowLists a;
+    B2SR_TRY(row_lists(h, buf, &a, s));
+    B2SR_TRY(ends.alloc((size_t)h->n * sizeof(int32_t)));
+    lower_ends_kernel<<<grid_wide(h->n), 256, 0, s>>>(a.begin, a.colind, h->n, ends.as<int32_t>());
+    B2SR_LAUNCH_CHECK("lower_ends_kernel");
+    a.end = ends.as<int32_t>();
+    const double bytes = 4.0 * ((double)h->ntr + 1.0) + (double)h->T * (4.0 + tile_bytes(h->k));
+    return count_rows(h->n, a, a, a, h->nnz, reinterpret_cast<unsigned long long*>(count), s, bytes);
 }
 
 // The masked count; `pairs` (device int64, optional) receives the number of
