@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "b2sr_internal.cuh"
+#include "bfs_cluster.cuh"
 #include "captured.cuh"
 
 namespace b2sr {
@@ -36,10 +37,6 @@ __global__ void bfs_init_kernel(int32_t* levels, int32_t n, uint32_t* fa, uint32
 }
 
 // Up to kParamSources sources travel as a kernel argument.
-constexpr int kParamSources = 64;
-struct SourceList {
-    int32_t v[kParamSources];
-};
 static SourceList source_list(const int32_t* srcs, int nsrc) {
     SourceList l = {};
     for (int i = 0; i < nsrc && i < kParamSources; ++i) l.v[i] = srcs[i];
@@ -81,6 +78,11 @@ b2sr_status bfs_sources(b2sr_matrix* h, const int32_t* srcs_host, int nsrc, int3
                         cudaStream_t s) {
     const int32_t n = h->n;
     const int64_t words = ceil_div(n, 32);
+    const int64_t cap = max_iters > 0 ? max_iters : (int64_t)n + 1;
+    bool done = false;
+    // the same round limit as below: whole batches of four
+    const b2sr_status small = bfs_cluster(h, source_list(srcs_host, nsrc), nsrc, levels, round_up(cap + 1, 4), s, &done);
+    if (done || small != B2SR_OK) return small;
     DevBuf buf(s);
     B2SR_TRY(buf.alloc(sizeof(LoopFlags) + 3 * words * sizeof(uint32_t) + (size_t)nsrc * sizeof(int32_t)));
     LoopFlags* flags = buf.as<LoopFlags>();
@@ -97,7 +99,6 @@ b2sr_status bfs_sources(b2sr_matrix* h, const int32_t* srcs_host, int nsrc, int3
     bfs_seed_kernel<<<(unsigned)ceil_div(nsrc, 256), 256, 0, s>>>(dsrc, source_list(srcs_host, nsrc), nsrc, levels, fa,
                                                                 vis);
     B2SR_LAUNCH_CHECK("bfs_seed_kernel");
-    const int64_t cap = max_iters > 0 ? max_iters : (int64_t)n + 1;
     int64_t rounds = 0;
     return run_captured(s, 4, cap + 1, &flags->active,
                         [&](cudaStream_t cs, int r) -> b2sr_status {
