@@ -1028,8 +1028,9 @@ struct MinMax<SemMaxF32<K>> : std::true_type {};
 // block's copy of the whole bitset in shared memory, whole aligned segments of
 // values, one value per set column (an input that is not aligned to a segment,
 // or whose last segment is ragged; 16-byte values, whose segment would be two
-// sectors), or one value per set bit in a loop (16-byte values where tiles
-// hold hardly more than one: the 16 predicated updates are 64 then).
+// sectors), or one value per set bit in a loop (8- and 16-byte values where
+// tiles hold hardly more than one: the 16 predicated updates are 32 and 64
+// instructions then).
 enum { kSmBits = 0, kSmBitsShared = 1, kSmSegs = 2, kSmVals = 3, kSmEach = 4 };
 // Threads a block, and the resident blocks the registers are budgeted for
 // (every lane holds two chunks' tile words and columns; with 16-byte values
@@ -1942,6 +1943,11 @@ static b2sr_status launch_direct(const b2sr_matrix* h, const SEM& sem, Partials<
                 if (8 * h->nnz > 9 * h->T) return launch_small<K, SEM, kSmVals>(h, sem, part, s, g);
                 return launch_small<K, SEM, kSmEach>(h, sem, part, s, g);
             } else {
+                // 8-byte values where hardly a tile holds two bits: by bit (64-lane OR,
+                // us, segment / bit: permuted R-MAT 20, 1.006 bits a tile, 199 / 182;
+                // R-MAT 22, 1.08 bits, 665 / 816)
+                if constexpr (sizeof(G) == 8)
+                    if (32 * h->nnz <= 33 * h->T) return launch_small<K, SEM, kSmEach>(h, sem, part, s, g);
                 // whole segments need an aligned input without a ragged last one
                 if (h->n % 4 == 0 && reinterpret_cast<uintptr_t>(sem.x) % (4 * sizeof(G)) == 0)
                     return launch_small<K, SEM, kSmSegs>(h, sem, part, s, g);
