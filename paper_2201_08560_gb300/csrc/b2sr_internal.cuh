@@ -176,14 +176,21 @@ b2sr_status new_handle_from_tiles(int32_t n, int k, int64_t T, int32_t* rowptr, 
                                   uint8_t* tiles, int64_t cap, cudaStream_t s, b2sr_matrix** out,
                                   int64_t known_nnz = -1);  // set bits, if the caller knows
 
-// SpMV and lane SpMM (spmv.cu), optionally gated on a device flag.  edges =
-// false (Boolean and OR results): the output already holds zeros where the
-// matrix has no tiles, before its first tile-row and after its last.
+// SpMV and SpMM (spmv.cu), optionally gated on a device flag.  edges = false
+// (Boolean, OR and plus-times results): the output already holds zeros where
+// the matrix has no tiles, before its first tile-row and after its last.
+// scratch: spmm_scratch_bytes(h, bytes of a value) bytes, 16-byte aligned, for
+// the partial rows (NULL: allocated and freed on the stream).
 b2sr_status spmv_dispatch(b2sr_matrix* h, b2sr_semiring sr, b2sr_vec in_kind, const void* x, b2sr_vec out_kind,
                           void* y, const uint32_t* mask, int comp, const float* weights, cudaStream_t s,
                           const int32_t* gate, bool edges = true);
 b2sr_status spmm64_dispatch(b2sr_matrix* h, const uint64_t* X, uint64_t* Y, const uint64_t* M, int comp,
-                            cudaStream_t s, const int32_t* gate, bool edges = true);
+                            cudaStream_t s, const int32_t* gate, bool edges = true, void* scratch = nullptr);
+b2sr_status spmm4_dispatch(b2sr_matrix* h, const float* X, float* Y, const uint32_t* M, int comp, cudaStream_t s,
+                           const int32_t* gate, bool edges = true, void* scratch = nullptr);
+inline size_t spmm_scratch_bytes(const b2sr_matrix* h, int value_bytes) {
+    return 2 * (size_t)round_up(h->nchunks * h->k * value_bytes, 16);
+}
 b2sr_status spmm32_dispatch(b2sr_matrix* h, const uint32_t* X, uint32_t* Y, const uint32_t* M, int comp,
                             cudaStream_t s, const int32_t* gate, bool edges = true);
 

@@ -39,8 +39,6 @@
 #include "b2sr_internal.cuh"
 
 namespace b2sr {
-b2sr_status spmm4_dispatch(b2sr_matrix* h, const float* X, float* Y, const uint32_t* M, int comp, cudaStream_t s,
-                           const int32_t* gate);
 
 using Clock = std::chrono::steady_clock;
 
@@ -74,24 +72,44 @@ __global__ void lane_init_kernel(unsigned long long* X, unsigned long long* V, i
     }
 }
 
-// visited |= next; new vertices of lane s get level depth[s] + 1; found = OR of next
+// A batch's reply to the host: the OR of the lanes that found a vertex.
+struct LaneReply {  // device, zero between steps
+    unsigned long long found;
+    uint32_t ticket;
+};
+
+// visited |= next; new vertices of lane s get level depth[s] + 1.  A warp takes
+// 32 vertices and goes through the lanes that any of them has, so a store
+// writes one lane's levels of neighbouring vertices.  The last block writes
+// the lanes that found a vertex to pinned host memory.
 __global__ void lane_update_kernel(const unsigned long long* __restrict__ Y, unsigned long long* __restrict__ V,
-                                   int32_t n, LaneArgs a, unsigned long long* found) {
+                                   int32_t n, LaneArgs a, LaneReply* reply, unsigned long long* found_host) {
     unsigned long long any = 0ull;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
-        unsigned long long b = Y[v];
-        if (!b) continue;
-        any |= b;
-        V[v] |= b;
-        while (b) {
-            const int s = __ffsll((long long)b) - 1;
-            b &= b - 1;
-            a.out[s][v] = a.depth[s] + 1;
+    const int lane = (int)lane_id();
+    for (int64_t v0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) - lane; v0 < n;
+         v0 += (int64_t)gridDim.x * blockDim.x) {  // warp-uniform
+        const int64_t v = v0 + lane;
+        const unsigned long long b = v < n ? Y[v] : 0ull;
+        if (b) V[v] |= b;
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            const uint32_t mine = (uint32_t)(b >> (32 * half));
+            uint32_t lanes = __reduce_or_sync(0xffffffffu, mine);
+            any |= (unsigned long long)lanes << (32 * half);
+            for (; lanes; lanes &= lanes - 1u) {
+                const int s = 32 * half + __ffs(lanes) - 1;
+                if ((b >> s) & 1ull) a.out[s][v] = a.depth[s] + 1;
+            }
         }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) any |= __shfl_xor_sync(0xffffffffu, any, o);
-    if ((threadIdx.x & 31) == 0 && any) atomicOr(found, any);
+    if (lane == 0 && any) atomicOr(&reply->found, any);
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    __threadfence();
+    if (atomicAdd(&reply->ticket, 1u) != gridDim.x - 1u) return;
+    __threadfence();
+    reply->ticket = 0u;
+    *found_host = atomicExch(&reply->found, 0ull);
 }
 
 struct ColArgs {
@@ -159,6 +177,7 @@ struct PRBlock {
     float* Pr = nullptr;
     float* C = nullptr;
     float* Y = nullptr;
+    void* part = nullptr;           // the SpMM's partial rows
     QueryRec* col[4] = {nullptr, nullptr, nullptr, nullptr};
     int done_it[4] = {0, 0, 0, 0};  // iterations issued
     bool fresh[4] = {false, false, false, false};
@@ -174,8 +193,10 @@ struct GraphSlot {
     bool in_flight = false;
     std::deque<QueryRec*> pend_bfs, pend_pr;
     // BFS batch
-    void* bfs_mem = nullptr;  // the allocation holding X, Y, V, found (X and Y swap every level)
-    unsigned long long *X = nullptr, *Y = nullptr, *V = nullptr, *found = nullptr;
+    void* bfs_mem = nullptr;  // the allocation holding X, Y, V, reply, part (X and Y swap every level)
+    unsigned long long *X = nullptr, *Y = nullptr, *V = nullptr;
+    LaneReply* reply = nullptr;
+    void* part = nullptr;     // the SpMM's partial rows
     int64_t bfs_bytes = 0;
     QueryRec* lane[64] = {};
     int32_t depth[64] = {};
@@ -271,15 +292,17 @@ static b2sr_status admit(b2sr_server* S, GraphSlot& g) {
         if (!g.X) {
             if (!reserve(S, g.bfs_bytes)) break;
             DevBuf tmp(g.st);
-            b2sr_status st = tmp.alloc(3 * (size_t)n * 8 + 256);
+            const size_t vb = round_up(3 * (size_t)n * 8, 256);
+            b2sr_status st = tmp.alloc(vb + 256 + spmm_scratch_bytes(g.h, 8));
             if (st != B2SR_OK) { release(S, g.bfs_bytes); return st; }
             g.bfs_mem = tmp.p;
             g.X = tmp.as<unsigned long long>();
             g.Y = g.X + n;
             g.V = g.Y + n;
-            g.found = g.V + n;
+            g.reply = reinterpret_cast<LaneReply*>(tmp.as<char>() + vb);
+            g.part = tmp.as<char>() + vb + 256;
             tmp.p = nullptr;  // owned by the slot now
-            B2SR_CUDA_TRY(cudaMemsetAsync(g.X, 0, 3 * (size_t)n * 8 + 8, g.st));
+            B2SR_CUDA_TRY(cudaMemsetAsync(g.X, 0, vb + sizeof(LaneReply), g.st));
         }
         const unsigned long long busy = g.active | g.fresh;
         if (__builtin_popcountll(busy) >= S->max_lanes) break;
@@ -303,12 +326,13 @@ static b2sr_status admit(b2sr_server* S, GraphSlot& g) {
             if ((int)g.blocks.size() >= S->max_blocks || !reserve(S, g.block_bytes)) break;
             DevBuf tmp(g.st);
             const size_t vb = round_up((size_t)n * 16, 256);
-            b2sr_status st = tmp.alloc(3 * vb);
+            b2sr_status st = tmp.alloc(3 * vb + spmm_scratch_bytes(g.h, 16));
             if (st != B2SR_OK) { release(S, g.block_bytes); return st; }
             PRBlock b;
             b.Pr = tmp.as<float>();
             b.C = reinterpret_cast<float*>(tmp.as<char>() + vb);
             b.Y = reinterpret_cast<float*>(tmp.as<char>() + 2 * vb);
+            b.part = tmp.as<char>() + 3 * vb;
             tmp.p = nullptr;
             B2SR_CUDA_TRY(cudaMemsetAsync(b.Pr, 0, 3 * vb, g.st));
             g.blocks.push_back(b);
@@ -330,7 +354,9 @@ static void trim(b2sr_server* S, GraphSlot& g) {
     if (g.X && !g.active && !g.fresh && g.pend_bfs.empty()) {
         dfree(g.bfs_mem, g.st);
         g.bfs_mem = nullptr;
-        g.X = g.Y = g.V = g.found = nullptr;
+        g.X = g.Y = g.V = nullptr;
+        g.reply = nullptr;
+        g.part = nullptr;
         release(S, g.bfs_bytes);
     }
     for (size_t i = g.blocks.size(); i-- > 0;) {
@@ -362,12 +388,10 @@ static b2sr_status launch_step(GraphSlot& g) {
             g.fresh = 0ull;
         }
         B2SR_TRY(spmm64_dispatch(g.h, reinterpret_cast<uint64_t*>(g.X), reinterpret_cast<uint64_t*>(g.Y),
-                                 reinterpret_cast<uint64_t*>(g.V), 1, g.st, nullptr));
-        B2SR_CUDA_TRY(cudaMemsetAsync(g.found, 0, 8, g.st));
-        lane_update_kernel<<<grid_for(n), 256, 0, g.st>>>(g.Y, g.V, n, la, g.found);
+                                 reinterpret_cast<uint64_t*>(g.V), 1, g.st, nullptr, true, g.part));
+        lane_update_kernel<<<grid_for(n), 256, 0, g.st>>>(g.Y, g.V, n, la, g.reply, g.found_host);
         B2SR_LAUNCH_CHECK("lane_update_kernel");
         std::swap(g.X, g.Y);
-        B2SR_CUDA_TRY(cudaMemcpyAsync(g.found_host, g.found, 8, cudaMemcpyDeviceToHost, g.st));
         g.bfs_stepped = true;
     }
     for (auto& b : g.blocks) {
@@ -387,7 +411,8 @@ static b2sr_status launch_step(GraphSlot& g) {
             col_init_kernel<<<grid_for(n), 256, 0, g.st>>>(b.Pr, b.C, g.h->outdeg, n, ca);
             B2SR_LAUNCH_CHECK("col_init_kernel");
         }
-        if (ca.step) B2SR_TRY(spmm4_dispatch(g.h, b.C, b.Y, nullptr, 0, g.st, nullptr));
+        // Y was cleared with the block: its rows without tiles stay zero
+        if (ca.step) B2SR_TRY(spmm4_dispatch(g.h, b.C, b.Y, nullptr, 0, g.st, nullptr, false, b.part));
         col_step_kernel<<<grid_for(n), 256, 0, g.st>>>(b.Y, b.Pr, b.C, g.h->outdeg, n, ca);
         B2SR_LAUNCH_CHECK("col_step_kernel");
         for (int c = 0; c < 4; ++c) {

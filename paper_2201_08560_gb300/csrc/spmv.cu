@@ -1877,10 +1877,10 @@ static b2sr_status launch_edges(const b2sr_matrix* h, const SEM& sem, cudaStream
 }
 
 template <class V, int NV>
-static b2sr_status alloc_partials(DevBuf& pbuf, int64_t nchunks, Partials<V>* part) {
+static b2sr_status alloc_partials(DevBuf& pbuf, int64_t nchunks, void* scratch, Partials<V>* part) {
     const size_t vbytes = round_up((size_t)nchunks * NV * sizeof(V), 16);
-    B2SR_TRY(pbuf.alloc(2 * vbytes));
-    uint8_t* base = pbuf.as<uint8_t>();
+    if (!scratch) B2SR_TRY(pbuf.alloc(2 * vbytes));
+    uint8_t* base = scratch ? static_cast<uint8_t*>(scratch) : pbuf.as<uint8_t>();
     part->val_first = reinterpret_cast<V*>(base);
     part->val_last = reinterpret_cast<V*>(base + vbytes);
     return B2SR_OK;
@@ -1964,11 +1964,11 @@ static b2sr_status launch_direct(const b2sr_matrix* h, const SEM& sem, Partials<
 // the chunk kernel (staged or direct) and the cross-chunk join
 template <int K, class SEM>
 static b2sr_status run_chunks(const b2sr_matrix* h, const SEM& sem, cudaStream_t s, const char* family,
-                              double vec_bytes, const int32_t* gate, const SpmvGeom& g) {
+                              double vec_bytes, const int32_t* gate, const SpmvGeom& g, void* scratch) {
     using V = typename SEM::V;
     DevBuf pbuf(s);
     Partials<V> part;
-    B2SR_TRY((alloc_partials<V, SEM::NV>(pbuf, h->nchunks, &part)));
+    B2SR_TRY((alloc_partials<V, SEM::NV>(pbuf, h->nchunks, scratch, &part)));
     const unsigned blocks = (unsigned)ceil_div(h->nchunks, kSpmvWarps);
     bool staged = false;
     // AUTO: the small-tile kernel where it serves
@@ -1995,13 +1995,14 @@ static b2sr_status run_chunks(const b2sr_matrix* h, const SEM& sem, cudaStream_t
 
 template <int K, class SEM>
 static b2sr_status run_spmv(const b2sr_matrix* h, const SEM& sem, uint32_t* bits_out, cudaStream_t s,
-                            const char* family, double vec_bytes, const int32_t* gate, bool edges = true) {
+                            const char* family, double vec_bytes, const int32_t* gate, bool edges = true,
+                            void* scratch = nullptr) {
     SpmvGeom g{h->rowptr, h->colind, h->tiles, h->chunk_row, h->T, h->nchunks, h->ntr, gate};
     if (edges) {
         if (bits_out) B2SR_TRY(clear_bitset_tail<K>(h, bits_out, s, gate));
         B2SR_TRY((launch_edges<K, SEM>(h, sem, s, gate)));
     }
-    if (h->nchunks > 0) B2SR_TRY((run_chunks<K, SEM>(h, sem, s, family, vec_bytes, gate, g)));
+    if (h->nchunks > 0) B2SR_TRY((run_chunks<K, SEM>(h, sem, s, family, vec_bytes, gate, g, scratch)));
     if constexpr (HasSelfTerm<SEM>::value) {
         const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(h->n, 256), (int64_t)sm_count() * 8));
         spmv_self_kernel<SEM><<<grid, 256, 0, s>>>(sem, gate);
@@ -2093,12 +2094,12 @@ b2sr_status spmv_dispatch(b2sr_matrix* h, b2sr_semiring sr, b2sr_vec in_kind, co
 }
 
 b2sr_status spmm64_dispatch(b2sr_matrix* h, const uint64_t* X, uint64_t* Y, const uint64_t* M, int comp,
-                            cudaStream_t s, const int32_t* gate, bool edges) {
+                            cudaStream_t s, const int32_t* gate, bool edges, void* scratch) {
     return with_tile(h->k, [&](auto kc) -> b2sr_status {
         constexpr int K = decltype(kc)::value;
         SemOr64<K> sem{reinterpret_cast<const unsigned long long*>(X), reinterpret_cast<unsigned long long*>(Y),
                        reinterpret_cast<const unsigned long long*>(M), comp ? 1 : 0, h->n};
-        return run_spmv<K>(h, sem, nullptr, s, "spmm_or64", (M ? 24.0 : 16.0) * h->n, gate, edges);
+        return run_spmv<K>(h, sem, nullptr, s, "spmm_or64", (M ? 24.0 : 16.0) * h->n, gate, edges, scratch);
     });
 }
 
@@ -2124,11 +2125,12 @@ b2sr_status spmv_maxkey_dispatch(b2sr_matrix* h, const uint64_t* x, uint64_t* y,
 }
 
 b2sr_status spmm4_dispatch(b2sr_matrix* h, const float* X, float* Y, const uint32_t* M, int comp, cudaStream_t s,
-                           const int32_t* gate) {
+                           const int32_t* gate, bool edges, void* scratch) {
     return with_tile(h->k, [&](auto kc) -> b2sr_status {
         constexpr int K = decltype(kc)::value;
         SemPlus4<K> sem{reinterpret_cast<const float4*>(X), reinterpret_cast<float4*>(Y), M, comp ? 1 : 0, h->n};
-        return run_spmv<K>(h, sem, nullptr, s, "spmm_plus4", 32.0 * h->n + (M ? h->n / 8.0 : 0.0), gate);
+        return run_spmv<K>(h, sem, nullptr, s, "spmm_plus4", 32.0 * h->n + (M ? h->n / 8.0 : 0.0), gate, edges,
+                           scratch);
     });
 }
 
