@@ -160,16 +160,16 @@ __global__ void masked_count_kernel(MatView A, MatView B, MatView M, unsigned lo
 //     memory; the warps fetch the row's mask entries one by one, and the lanes
 //     walk the entry's other row, testing each column in the bitmap: a
 //     coalesced load and one shared load per column, no searches;
-//   * a shorter row stays a list: the warps take such rows one by one, a group
-//     of lanes (as wide as the row) per mask entry, each lane searching its
-//     column in the entry's other row.
+//   * a shorter row stays a list: eight lanes a mask entry search its columns
+//     in the entry's other row.
 // Where a bitmap of n bits does not fit in shared memory every row takes the
-// second form.
+// second form, the longer ones with a warp an entry.
 constexpr int kRunEntries = 256;
 constexpr int64_t kMaxBitmapBytes = 200 * 1024;
 // Fewer mask entries than this take one launch: grouping the others by column
-// (three launches and a scan) costs more than the shorter walks save.
-constexpr int64_t kSplitEntries = 1 << 17;
+// (five launches and a scan, 60 us) costs more than the shorter walks save
+// (R-MAT 16, 1.8M entries, half of them below the diagonal: about as much).
+constexpr int64_t kSplitEntries = 1 << 21;
 
 // Row i: colind[begin[i] .. end[i]) (end = begin + 1 for a plain CSR).  Rows
 // lie one after another, with gaps where end[i] < begin[i + 1].
@@ -179,24 +179,16 @@ struct RowLists {
     const int32_t* colind;
 };
 
-// Ones of the short row list a[0..d) in row j of B, over mask entries
-// [e0, e1), by one warp; with `longer` only where row j is not longer than d.
-__device__ __forceinline__ uint32_t count_listed(const int32_t* __restrict__ acol, int32_t d, RowLists B,
-                                                 const int32_t* __restrict__ mcol, int32_t e0, int32_t e1, bool longer,
-                                                 int lane) {
-    int width = 32;  // lanes a mask entry: the least power of two holding the row
-    while (width > 1 && width / 2 >= d) width >>= 1;
-    const int sub = lane & (width - 1);
+// Columns of the list acol[0..d) in the row [b0, b1) of B, by a group of WIDTH
+// lanes.
+template <int WIDTH>
+__device__ __forceinline__ uint32_t count_listed(const int32_t* __restrict__ acol, int32_t d,
+                                                 const int32_t* __restrict__ bcol, int32_t b0, int32_t b1, int sub) {
     uint32_t acc = 0;
-    for (int32_t e = e0 + lane / width; e < e1; e += 32 / width) {
-        const int32_t j = __ldg(mcol + e);
-        const int32_t b0 = __ldg(B.begin + j), b1 = __ldg(B.end + j);
-        if (longer && b1 - b0 > d) continue;
-        for (int32_t p = sub; p < d; p += width) {
-            const int32_t v = __ldg(acol + p);
-            const int32_t q = lower_bound_i32(B.colind, b0, b1, v);
-            acc += q < b1 && __ldg(B.colind + q) == v;
-        }
+    for (int32_t p = sub; p < d; p += WIDTH) {
+        const int32_t v = __ldg(acol + p);
+        const int32_t q = lower_bound_i32(bcol, b0, b1, v);
+        acc += q < b1 && __ldg(bcol + q) == v;
     }
     return acc;
 }
@@ -240,63 +232,85 @@ __global__ void __launch_bounds__(256) masked_rows_kernel(int32_t n, RowLists A,
                                                           int bitmap_words, unsigned long long* __restrict__ out) {
     extern __shared__ __align__(16) uint32_t bitmap[];
     __shared__ unsigned long long warp_sum[8];
-    __shared__ int32_t long_row[kRunEntries];  // at least one mask entry of the run in each
-    __shared__ int nlong, nother[2];
-    __shared__ int2 other[kRunEntries];  // the other rows of a long row's mask entries
+    // the run's entries: where row i of A begins, row j of B as a range (compact:
+    // six blocks an SM beside bitmaps of 2^18 bits)
+    __shared__ int32_t row_a[kRunEntries];
+    __shared__ int2 row_b[kRunEntries];
+    __shared__ int32_t long_row[kRunEntries];  // rows taken as bitmaps; without bitmaps, row i's length
+    __shared__ uint8_t short_len[kRunEntries];  // row i's length, up to 32
+    __shared__ uint8_t listed[kRunEntries];    // entries of rows with up to 32 columns
+    __shared__ uint8_t other[kRunEntries];     // entries of one long row; without bitmaps, of all
+    __shared__ int nlong, nlisted, nother[2];
+    __shared__ int32_t row_range[2];
     const int lane = (int)lane_id(), warp = threadIdx.x >> 5;
     const int32_t e0 = (int32_t)blockIdx.x * kRunEntries;
     const int32_t e1 = min(e0 + kRunEntries, __ldg(mnnz));
     if (e0 >= e1) return;
-    // rows of the first and the last mask entry of the run: warps 0 and 1
-    __shared__ int32_t row_range[2];
-    if (warp < 2) {
-        const int32_t e = warp == 0 ? e0 : e1 - 1;
-        int32_t lo = 0, hi = n - 1;  // the last row starting at or before e
+    // the last row starting at or before entry e, between lo and hi
+    auto row_at = [&](int32_t e, int32_t lo, int32_t hi) {
         while (lo < hi) {
             const int32_t mid = lo + ((hi - lo + 1) >> 1);
             if (__ldg(M.begin + mid) <= e) lo = mid; else hi = mid - 1;
         }
-        if (lane == 0) row_range[warp] = lo;
+        return lo;
+    };
+    if (warp < 2) {  // rows of the first and the last entry of the run
+        const int32_t i = row_at(warp == 0 ? e0 : e1 - 1, 0, n - 1);
+        if (lane == 0) row_range[warp] = i;
     }
     if (use_bitmap) {
         const uint4 zero = make_uint4(0u, 0u, 0u, 0u);  // the bitmap is padded to whole 16 bytes
         for (int w = threadIdx.x; w < (bitmap_words + 3) / 4; w += 256) reinterpret_cast<uint4*>(bitmap)[w] = zero;
     }
-    if (threadIdx.x == 0) nlong = nother[0] = 0;
+    if (threadIdx.x == 0) nlong = nlisted = nother[0] = 0;
     __syncthreads();
     const int32_t i0 = row_range[0], i1 = row_range[1];
     if (i0 == i1 && __ldg(M.end + i0) <= e0) return;  // the run lies in a gap
-    uint32_t acc = 0;
-    const int32_t listed = use_bitmap ? 32 : INT32_MAX;  // longest row taken as a list
-    for (int32_t base = i0; base <= i1; base += 256) {
-        const int32_t i = base + 8 * lane + warp;  // neighbouring rows go to different warps
-        int32_t a0 = 0, d = 0, m0 = 0, m1 = 0;
-        if (i <= i1) {
-            a0 = __ldg(A.begin + i);
-            d = __ldg(A.end + i) - a0;
-            m0 = max(e0, __ldg(M.begin + i));
-            m1 = min(e1, __ldg(M.end + i));
+    {
+        const int t = threadIdx.x;
+        const int32_t e = e0 + t;
+        int2 rb = make_int2(0, 0);
+        if (e < e1) {
+            const int32_t i = row_at(e, i0, i1);
+            if (e < __ldg(M.end + i)) {
+                const int32_t j = __ldg(M.colind + e);
+                const int32_t a0 = __ldg(A.begin + i), d = __ldg(A.end + i) - a0;
+                rb = make_int2(__ldg(B.begin + j), __ldg(B.end + j));
+                if (use_bitmap && d > 32 && (t == 0 || e == __ldg(M.begin + i))) long_row[atomicAdd(&nlong, 1)] = i;
+                if (d <= 0 || rb.y <= rb.x || (longer && rb.y - rb.x > d)) {
+                    rb.y = rb.x;  // nothing to count here
+                } else if (d <= 32) {
+                    row_a[t] = a0;
+                    short_len[t] = (uint8_t)d;
+                    listed[atomicAdd(&nlisted, 1)] = (uint8_t)t;
+                } else if (!use_bitmap) {
+                    row_a[t] = a0;
+                    long_row[t] = d;
+                    other[atomicAdd(&nother[0], 1)] = (uint8_t)t;
+                }
+            }
         }
-        const bool live = d > 0 && m0 < m1;
-        if (live && d > listed) long_row[atomicAdd(&nlong, 1)] = i;
-        for (unsigned todo = __ballot_sync(0xffffffffu, live && d <= listed); todo; todo &= todo - 1) {
-            const int src = __ffs(todo) - 1;
-            acc += count_listed(A.colind + __shfl_sync(0xffffffffu, a0, src), __shfl_sync(0xffffffffu, d, src), B,
-                                M.colind, __shfl_sync(0xffffffffu, m0, src), __shfl_sync(0xffffffffu, m1, src), longer,
-                                lane);
-        }
+        row_b[t] = rb;
     }
-    if (use_bitmap) {
-        __syncthreads();
+    __syncthreads();
+    uint32_t acc = 0;
+    for (int q = threadIdx.x >> 3; q < nlisted; q += 32) {
+        const int t = listed[q];
+        acc += count_listed<8>(A.colind + row_a[t], short_len[t], B.colind, row_b[t].x, row_b[t].y, lane & 7);
+    }
+    if (!use_bitmap) {
+        for (int q = warp; q < nother[0]; q += 8) {
+            const int t = other[q];
+            acc += count_listed<32>(A.colind + row_a[t], long_row[t], B.colind, row_b[t].x, row_b[t].y, lane);
+        }
+    } else {
         for (int r = 0; r < nlong; ++r) {
             const int32_t i = long_row[r];
             const int32_t a0 = __ldg(A.begin + i), a1 = __ldg(A.end + i);
             const int32_t m0 = max(e0, __ldg(M.begin + i)), m1 = min(e1, __ldg(M.end + i));
-            // the entries' other rows (at most 256 entries a run)
             if (threadIdx.x < m1 - m0) {
-                const int32_t j = __ldg(M.colind + m0 + threadIdx.x);
-                const int32_t b0 = __ldg(B.begin + j), b1 = __ldg(B.end + j);
-                if (b1 > b0 && !(longer && b1 - b0 > a1 - a0)) other[atomicAdd(&nother[r & 1], 1)] = make_int2(b0, b1);
+                const int t = m0 - e0 + threadIdx.x;
+                if (row_b[t].y > row_b[t].x) other[atomicAdd(&nother[r & 1], 1)] = (uint8_t)t;
             }
             for (int32_t p = a0 + threadIdx.x; p < a1; p += 256) {
                 const int32_t v = __ldg(A.colind + p);
@@ -307,10 +321,10 @@ __global__ void __launch_bounds__(256) masked_rows_kernel(int32_t n, RowLists A,
             const int todo = nother[r & 1];
             // the next entry's first columns are loaded before this one's are used
             auto test = [&](int32_t v) { return (bitmap[v >> 5] >> (v & 31)) & 1u; };
-            int2 o = warp < todo ? other[warp] : make_int2(0, 0);
+            int2 o = warp < todo ? row_b[other[warp]] : make_int2(0, 0);
             int32_t v = o.x + lane < o.y ? __ldg(B.colind + o.x + lane) : -1;
             for (int q = warp; q < todo; q += 8) {
-                const int2 o2 = q + 8 < todo ? other[q + 8] : make_int2(0, 0);
+                const int2 o2 = q + 8 < todo ? row_b[other[q + 8]] : make_int2(0, 0);
                 const int32_t v2 = o2.x + lane < o2.y ? __ldg(B.colind + o2.x + lane) : -1;
                 if (v >= 0) acc += test(v);
 #pragma unroll 4
