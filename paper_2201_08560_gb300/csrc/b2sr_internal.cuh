@@ -184,15 +184,23 @@ b2sr_status new_handle_from_tiles(int32_t n, int k, int64_t T, int32_t* rowptr, 
 b2sr_status spmv_dispatch(b2sr_matrix* h, b2sr_semiring sr, b2sr_vec in_kind, const void* x, b2sr_vec out_kind,
                           void* y, const uint32_t* mask, int comp, const float* weights, cudaStream_t s,
                           const int32_t* gate, bool edges = true);
+// live: for a lane SpMM at k = 4, which groups of four input words are not
+// all zero (one bit each; device), and a device flag, not zero where most are.
+struct LiveColumns {
+    const uint32_t* bits = nullptr;
+    const int32_t* dense = nullptr;
+};
 b2sr_status spmm64_dispatch(b2sr_matrix* h, const uint64_t* X, uint64_t* Y, const uint64_t* M, int comp,
-                            cudaStream_t s, const int32_t* gate, bool edges = true, void* scratch = nullptr);
+                            cudaStream_t s, const int32_t* gate, bool edges = true, void* scratch = nullptr,
+                            LiveColumns live = LiveColumns());
 b2sr_status spmm4_dispatch(b2sr_matrix* h, const float* X, float* Y, const uint32_t* M, int comp, cudaStream_t s,
                            const int32_t* gate, bool edges = true, void* scratch = nullptr);
 inline size_t spmm_scratch_bytes(const b2sr_matrix* h, int value_bytes) {
     return 2 * (size_t)round_up(h->nchunks * h->k * value_bytes, 16);
 }
 b2sr_status spmm32_dispatch(b2sr_matrix* h, const uint32_t* X, uint32_t* Y, const uint32_t* M, int comp,
-                            cudaStream_t s, const int32_t* gate, bool edges = true);
+                            cudaStream_t s, const int32_t* gate, bool edges = true,
+                            LiveColumns live = LiveColumns());
 
 // primitives (primitives.cu)
 b2sr_status exclusive_scan_i32_to_i64(const int32_t* in, int64_t* out, int64_t n, cudaStream_t s);

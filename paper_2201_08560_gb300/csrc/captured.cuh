@@ -36,17 +36,18 @@ struct LoopFlags {  // device
 
 // Called by every thread of every block of a gated kernel; `any`: the thread
 // found something.  The last block to arrive moves the loop on: active <-
-// found, one more level.
-__device__ __forceinline__ void finish_round(LoopFlags* f, int any) {
+// found, one more level; true for its thread 0.
+__device__ __forceinline__ bool finish_round(LoopFlags* f, int any) {
     const int found = __syncthreads_or(any);
-    if (threadIdx.x != 0) return;
+    if (threadIdx.x != 0) return false;
     if (found) atomicOr(&f->found, 1);
     __threadfence();
-    if (atomicAdd(&f->ticket, 1u) != gridDim.x - 1u) return;
+    if (atomicAdd(&f->ticket, 1u) != gridDim.x - 1u) return false;
     __threadfence();
     f->ticket = 0u;
     f->active = atomicExch(&f->found, 0);
     f->level += 1;
+    return true;
 }
 
 // ---------------------------------------------------------------------------

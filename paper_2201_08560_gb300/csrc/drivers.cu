@@ -120,10 +120,19 @@ b2sr_status bfs_sources(b2sr_matrix* h, const int32_t* srcs_host, int nsrc, int3
 // ---------------------------------------------------------------------------
 // The lane word: 64 frontiers (uint64) or, for at most 32 sources, 32 (uint32:
 // half the bytes per gather, and the SpMV takes the tile_dim-4 kernel).
+// The frontier's live tile-columns at k = 4: a bit for every four vertices of
+// which one is in some lane's frontier, how many are set, and whether that is
+// more than half (the SpMM does not look then).
+struct LiveState {
+    uint32_t count;
+    int32_t dense;
+};
+
 template <class W>
-__global__ void msbfs_init_kernel(int32_t* levels, int32_t n, int nsrc, W* X, W* Y, W* vis, LoopFlags* flags) {
+__global__ void msbfs_init_kernel(int32_t* levels, int32_t n, int nsrc, W* X, W* Y, W* vis, uint8_t* live,
+                                  int64_t live_bytes, LiveState* state, LoopFlags* flags) {
     constexpr int BITS = 8 * (int)sizeof(W);
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (int64_t)n * nsrc || i < n;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (int64_t)n * nsrc || i < live_bytes;
          i += (int64_t)gridDim.x * blockDim.x) {
         if (i < (int64_t)n * nsrc) levels[i] = -1;
         // unused lanes count as visited, so a vertex every source has reached is
@@ -133,18 +142,24 @@ __global__ void msbfs_init_kernel(int32_t* levels, int32_t n, int nsrc, W* X, W*
             Y[i] = (W)0;
             vis[i] = nsrc < BITS ? (W)~(((W)1 << nsrc) - (W)1) : (W)0;
         }
+        if (i < live_bytes) live[i] = 0;
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) *flags = LoopFlags{1, 0, 0, 0u};
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *flags = LoopFlags{1, 0, 0, 0u};
+        *state = LiveState{0u, 0};
+    }
 }
 
 template <class W>
-__global__ void msbfs_seed_kernel(SourceList srcs, int nsrc, int32_t n, int32_t* levels, W* X, W* vis) {
+__global__ void msbfs_seed_kernel(SourceList srcs, int nsrc, int32_t n, int32_t* levels, W* X, W* vis,
+                                  uint32_t* live) {
     int s = threadIdx.x;
     if (s < nsrc) {
         int32_t v = srcs.v[s];
         levels[(int64_t)s * n + v] = 0;
         atomicOr(X + v, (W)1 << s);
         atomicOr(vis + v, (W)1 << s);
+        atomicOr(live + (v >> 7), 1u << ((v >> 2) & 31));
     }
 }
 
@@ -152,19 +167,32 @@ __global__ void msbfs_seed_kernel(SourceList srcs, int nsrc, int32_t n, int32_t*
 // takes 32 consecutive vertices and goes through the lanes that any of them
 // has, so a store writes one lane's levels of neighbouring vertices (a thread
 // that walked its own vertex's lanes wrote 32 different lines a store:
-// R-MAT 22, 64 sources: 260 us a level).
+// R-MAT 22, 64 sources: 260 us a level).  The 32 vertices' live bits, one for
+// each four, are a byte.
 template <class W>
 __global__ void msbfs_update_kernel(const W* __restrict__ Y, W* __restrict__ vis, int32_t* __restrict__ levels,
-                                    int32_t n, LoopFlags* flags) {
+                                    int32_t n, uint8_t* __restrict__ live, LiveState* state, LoopFlags* flags) {
     if (gate_closed(&flags->active)) return;
+    __shared__ uint32_t block_live;
+    if (threadIdx.x == 0) block_live = 0u;
+    __syncthreads();
     const int32_t lv = *reinterpret_cast<const volatile int32_t*>(&flags->level) + 1;
     int any = 0;
+    uint32_t nlive = 0;
     const int lane = (int)lane_id();
     for (int64_t v0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) - lane; v0 < n;
          v0 += (int64_t)gridDim.x * blockDim.x) {  // warp-uniform
         const int64_t v = v0 + lane;
         const W b = v < n ? Y[v] : (W)0;
         if (b) vis[v] |= b;
+        uint32_t four = __ballot_sync(0xffffffffu, b != 0);
+        four |= four >> 1;
+        four = (four | (four >> 2)) & 0x11111111u;
+        uint32_t byte = 0u;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) byte |= ((four >> (4 * q)) & 1u) << q;
+        if (lane == 0) live[v0 >> 5] = (uint8_t)byte;
+        nlive += __popc(byte);
 #pragma unroll
         for (int half = 0; half < (int)sizeof(W) / 4; ++half) {
             const uint32_t mine = (uint32_t)(b >> (32 * half * (int)(sizeof(W) > 4)));
@@ -176,18 +204,25 @@ __global__ void msbfs_update_kernel(const W* __restrict__ Y, W* __restrict__ vis
             }
         }
     }
-    finish_round(flags, any);
+    if (lane == 0 && nlive) atomicAdd(&block_live, nlive);
+    __syncthreads();
+    if (threadIdx.x == 0 && block_live) atomicAdd(&state->count, block_live);
+    if (finish_round(flags, any)) {
+        const uint32_t total = atomicExch(&state->count, 0u);
+        state->dense = 8 * (int64_t)total > n ? 1 : 0;
+    }
 }
 
 
 static b2sr_status spmm_lanes(b2sr_matrix* h, const unsigned long long* X, unsigned long long* Y,
-                              const unsigned long long* M, cudaStream_t s, const int32_t* gate, bool edges) {
+                              const unsigned long long* M, cudaStream_t s, const int32_t* gate, bool edges,
+                              LiveColumns live) {
     return spmm64_dispatch(h, reinterpret_cast<const uint64_t*>(X), reinterpret_cast<uint64_t*>(Y),
-                           reinterpret_cast<const uint64_t*>(M), 1, s, gate, edges);
+                           reinterpret_cast<const uint64_t*>(M), 1, s, gate, edges, nullptr, live);
 }
 static b2sr_status spmm_lanes(b2sr_matrix* h, const uint32_t* X, uint32_t* Y, const uint32_t* M, cudaStream_t s,
-                              const int32_t* gate, bool edges) {
-    return spmm32_dispatch(h, X, Y, M, 1, s, gate, edges);
+                              const int32_t* gate, bool edges, LiveColumns live) {
+    return spmm32_dispatch(h, X, Y, M, 1, s, gate, edges, live);
 }
 
 template <class W>
@@ -196,14 +231,20 @@ static b2sr_status bfs_multi_lanes(b2sr_matrix* h, const int32_t* srcs_host, int
     const int32_t n = h->n;
     DevBuf buf(s);
     const size_t vb = round_up((size_t)n * sizeof(W), 256);
-    B2SR_TRY(buf.alloc(3 * vb + sizeof(LoopFlags)));
+    const size_t lb = round_up(ceil_div(n, 32), 16);
+    B2SR_TRY(buf.alloc(3 * vb + lb + sizeof(LoopFlags) + sizeof(LiveState)));
     W* X = buf.as<W>();
     W* Yb = reinterpret_cast<W*>(buf.as<char>() + vb);
     W* vis = reinterpret_cast<W*>(buf.as<char>() + 2 * vb);
-    LoopFlags* flags = reinterpret_cast<LoopFlags*>(buf.as<char>() + 3 * vb);
-    msbfs_init_kernel<W><<<grid_for((int64_t)n * nsrc), 256, 0, s>>>(levels, n, nsrc, X, Yb, vis, flags);
+    uint8_t* live = reinterpret_cast<uint8_t*>(buf.as<char>() + 3 * vb);
+    LoopFlags* flags = reinterpret_cast<LoopFlags*>(live + lb);
+    LiveState* state = reinterpret_cast<LiveState*>(flags + 1);
+    const LiveColumns columns{reinterpret_cast<const uint32_t*>(live), &state->dense};
+    msbfs_init_kernel<W><<<grid_for(std::max<int64_t>((int64_t)n * nsrc, lb)), 256, 0, s>>>(
+        levels, n, nsrc, X, Yb, vis, live, (int64_t)lb, state, flags);
     B2SR_LAUNCH_CHECK("msbfs_init_kernel");
-    msbfs_seed_kernel<W><<<1, 64, 0, s>>>(source_list(srcs_host, nsrc), nsrc, n, levels, X, vis);
+    msbfs_seed_kernel<W><<<1, 64, 0, s>>>(source_list(srcs_host, nsrc), nsrc, n, levels, X, vis,
+                                          reinterpret_cast<uint32_t*>(live));
     B2SR_LAUNCH_CHECK("msbfs_seed_kernel");
     const int64_t cap = max_iters > 0 ? max_iters : (int64_t)n + 1;
     int64_t rounds = 0;
@@ -212,8 +253,8 @@ static b2sr_status bfs_multi_lanes(b2sr_matrix* h, const int32_t* srcs_host, int
                             W* cur = (r & 1) ? Yb : X;
                             W* nxt = (r & 1) ? X : Yb;
                             // as in bfs_sources: rows without tiles need zeros in X once
-                            B2SR_TRY(spmm_lanes(h, cur, nxt, vis, cs, &flags->active, r == 1));
-                            msbfs_update_kernel<W><<<grid_for(n), 256, 0, cs>>>(nxt, vis, levels, n, flags);
+                            B2SR_TRY(spmm_lanes(h, cur, nxt, vis, cs, &flags->active, r == 1, columns));
+                            msbfs_update_kernel<W><<<grid_for(n), 256, 0, cs>>>(nxt, vis, levels, n, live, state, flags);
                             B2SR_LAUNCH_CHECK("msbfs_update_kernel");
                             return B2SR_OK;
                         },

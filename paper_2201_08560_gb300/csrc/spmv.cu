@@ -560,6 +560,10 @@ struct SemOrLanes {
     const W* mask;
     int comp;
     int32_t n;
+    // optional: bit J set where one of x[4J .. 4J+3] is not zero, and a flag
+    // that says not to look (most are set)
+    const uint32_t* live = nullptr;
+    const int32_t* dense = nullptr;
     __device__ const W* src() const { return x; }
     __device__ const float* wts() const { return nullptr; }
     __device__ const int32_t* voffs() const { return nullptr; }
@@ -1016,6 +1020,12 @@ __global__ void __launch_bounds__(kSpmvThreads) spmv_chunks_kernel(SpmvGeom g, S
 // (236 / 194); Boolean 86 / 64 at k = 4 and 99 / 64 at k = 8.  Warp
 // instructions of the plus-times kernel: 98M / 59M.
 // ---------------------------------------------------------------------------
+// lane-word schemes
+template <class S>
+struct LaneWords : std::false_type {};
+template <int K, class W>
+struct LaneWords<SemOrLanes<K, W>> : std::true_type {};
+
 // min and max schemes
 template <class S>
 struct MinMax : std::false_type {};
@@ -1030,8 +1040,9 @@ struct MinMax<SemMaxF32<K>> : std::true_type {};
 // or whose last segment is ragged; 16-byte values, whose segment would be two
 // sectors), or one value per set bit in a loop (8- and 16-byte values where
 // tiles hold hardly more than one: the 16 predicated updates are 32 and 64
-// instructions then).
-enum { kSmBits = 0, kSmBitsShared = 1, kSmSegs = 2, kSmVals = 3, kSmEach = 4 };
+// instructions then), or segments where the block's copy of `live` says that
+// they are not all zero (the sparse levels of a batched BFS).
+enum { kSmBits = 0, kSmBitsShared = 1, kSmSegs = 2, kSmVals = 3, kSmEach = 4, kSmSegsLive = 5 };
 // Threads a block, and the resident blocks the registers are budgeted for
 // (every lane holds two chunks' tile words and columns; with 16-byte values
 // one).  R-MAT 20, k = 4, in
@@ -1041,12 +1052,13 @@ enum { kSmBits = 0, kSmBitsShared = 1, kSmSegs = 2, kSmVals = 3, kSmEach = 4 };
 // room for one block: k = 8 with 512 / 640 / 768 threads 83 / 74 / 72.5.
 template <int K, class SEM, int MODE>
 constexpr int small_threads() {
+    if (MODE == kSmSegsLive) return sizeof(typename SEM::V) == 8 ? 768 : 1024;
     if (MODE != kSmBitsShared) return kSpmvThreads;
     return K == 4 ? 1024 : (SEM::NV == 8 ? 640 : 768);  // eight counts a row need the registers
 }
 template <int K, class SEM, int MODE>
 constexpr int small_min_blocks() {
-    if (MODE == kSmBitsShared) return 1;
+    if (MODE == kSmBitsShared || MODE == kSmSegsLive) return 1;
     if (sizeof(typename SEM::V) == 16) return MODE == kSmEach ? 4 : 3;
     if (SEM::NV == 8) return 2;
     return K == 8 || sizeof(typename SEM::V) == 8 || MinMax<SEM>::value ? 3 : 4;
@@ -1155,7 +1167,7 @@ __device__ __forceinline__ void chunk_ends(const SpmvGeom& g, const SEM& sem, in
 // The four input values under a k = 4 tile.
 template <class G, int MODE>
 __device__ __forceinline__ void load_seg(const G* __restrict__ x, uint32_t J, uint32_t w, G (&v)[4]) {
-    if constexpr (MODE == kSmSegs) {
+    if constexpr (MODE == kSmSegs || MODE == kSmSegsLive) {
         if constexpr (sizeof(G) == 4) {
             const uint4 q = __ldg(reinterpret_cast<const uint4*>(x) + J);
             const uint32_t u[4] = {q.x, q.y, q.z, q.w};
@@ -1254,7 +1266,7 @@ __device__ __forceinline__ void join_lanes(const SEM& sem, Acc& acc, int lane) {
 template <int K, class SEM, int MODE>
 __device__ __forceinline__ void small_chunk(const SpmvGeom& g, const SEM& sem, Partials<typename SEM::V> part,
                                             int32_t c, int lane, const SmallTiles<K>& t, ChunkRows& s,
-                                            const uint8_t* sx, typename SEM::V* first) {
+                                            const uint8_t* sx, typename SEM::V* first, bool filter) {
     using Sh = ChunkShape<K>;
     using V = typename SEM::V;
     constexpr int NV = SEM::NV;
@@ -1315,12 +1327,36 @@ __device__ __forceinline__ void small_chunk(const SpmvGeom& g, const SEM& sem, P
                 }
             } else {
                 G x[GRP][4];
+                bool any = true;  // warp-uniform: some lane's segments are not all zero
+                if constexpr (MODE == kSmSegsLive) {
+                    bool on[GRP];
+                    bool mine = false;
 #pragma unroll
-                for (int i = 0; i < GRP; ++i)
-                    load_seg<G, MODE>(sem.src(), t.cu[i0 + i], t.w[i0 + i], x[i]);
+                    for (int i = 0; i < GRP; ++i) {
+                        const uint32_t J = t.cu[i0 + i];
+                        on[i] = !filter || ((reinterpret_cast<const uint32_t*>(sx)[J >> 5] >> (J & 31)) & 1u);
+                        mine |= on[i];
+                    }
+                    any = __any_sync(0xffffffffu, mine);
+                    if (any) {
+#pragma unroll
+                        for (int i = 0; i < GRP; ++i) {
+                            if (on[i]) {
+                                load_seg<G, MODE>(sem.src(), t.cu[i0 + i], t.w[i0 + i], x[i]);
+                            } else {
+#pragma unroll
+                                for (int c = 0; c < 4; ++c) x[i][c] = G();
+                            }
+                        }
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < GRP; ++i)
+                        load_seg<G, MODE>(sem.src(), t.cu[i0 + i], t.w[i0 + i], x[i]);
+                }
 #pragma unroll
                 for (int i = 0; i < GRP; ++i) {
-                    seg_add(sem, acc, t.w[i0 + i], x[i]);
+                    if (any) seg_add(sem, acc, t.w[i0 + i], x[i]);
                     if (!one_row) end_tile(i0 + i);
                 }
             }
@@ -1378,7 +1414,8 @@ constexpr int small_warp_smem() {
     return (int)sizeof(ChunkRows) + (sizeof(typename SEM::V) == 16 ? 32 * SEM::NV * 16 : 0);
 }
 
-// Dynamic shared memory: that for every warp, then (kSmBitsShared) the input bitset.
+// Dynamic shared memory: that for every warp, then (kSmBitsShared,
+// kSmSegsLive) the input bitset.
 template <int K, class SEM, int MODE>
 __device__ __forceinline__ void small_body(const SpmvGeom& g, const SEM& sem, Partials<typename SEM::V> part) {
     constexpr int WARPS = small_threads<K, SEM, MODE>() / 32;
@@ -1401,16 +1438,26 @@ __device__ __forceinline__ void small_body(const SpmvGeom& g, const SEM& sem, Pa
             nb = __ldg(g.chunk_row + c + W + 1);
         }
     }
-    if constexpr (MODE == kSmBitsShared) {
+    bool filter = false;
+    if constexpr (MODE == kSmSegsLive) filter = __ldg(sem.dense) == 0;
+    if (MODE == kSmBitsShared || filter) {
         uint32_t* dst = reinterpret_cast<uint32_t*>(small_smem + WARPS * small_warp_smem<SEM>());
-        const int words = (sem.n + 31) / 32;
+        const uint32_t* bits;
+        int words;
+        if constexpr (MODE == kSmSegsLive) {
+            bits = sem.live;
+            words = (g.ntr + 31) / 32;
+        } else {
+            bits = reinterpret_cast<const uint32_t*>(sem.x);
+            words = (sem.n + 31) / 32;
+        }
         int at = 0;
-        if (reinterpret_cast<uintptr_t>(sem.x) % 16 == 0) {
-            const uint4* src = reinterpret_cast<const uint4*>(sem.x);
+        if (reinterpret_cast<uintptr_t>(bits) % 16 == 0) {
+            const uint4* src = reinterpret_cast<const uint4*>(bits);
             for (int i = threadIdx.x; i < words / 4; i += WARPS * 32) reinterpret_cast<uint4*>(dst)[i] = __ldg(src + i);
             at = words & ~3;
         }
-        for (int i = at + threadIdx.x; i < words; i += WARPS * 32) dst[i] = __ldg(sem.x + i);
+        for (int i = at + threadIdx.x; i < words; i += WARPS * 32) dst[i] = __ldg(bits + i);
         __syncthreads();
     }
     if (c >= g.nchunks) return;  // whole warps leave together
@@ -1418,7 +1465,7 @@ __device__ __forceinline__ void small_body(const SpmvGeom& g, const SEM& sem, Pa
         // one chunk at a time: more warps hide its loads better than the
         // registers of a second chunk would (R-MAT 20: 225 and 270 us)
         for (;;) {
-            small_chunk<K, SEM, MODE>(g, sem, part, c, lane, cur, *rows, sx, first);
+            small_chunk<K, SEM, MODE>(g, sem, part, c, lane, cur, *rows, sx, first, filter);
             c += W;
             if (c >= g.nchunks) return;
             small_load<K>(g, sem, c, lane, na, nb, cur);
@@ -1436,7 +1483,7 @@ __device__ __forceinline__ void small_body(const SpmvGeom& g, const SEM& sem, Pa
             na = __ldg(g.chunk_row + cn + W);
             nb = __ldg(g.chunk_row + cn + W + 1);
         }
-        small_chunk<K, SEM, MODE>(g, sem, part, c, lane, cur, *rows, sx, first);
+        small_chunk<K, SEM, MODE>(g, sem, part, c, lane, cur, *rows, sx, first, filter);
         if (!more) break;
         c = cn;
         cur = nxt;
@@ -1907,7 +1954,9 @@ static b2sr_status launch_small(const b2sr_matrix* h, const SEM& sem, Partials<t
     constexpr int threads = small_threads<K, SEM, MODE>();
     const unsigned grid = (unsigned)std::min<int64_t>(ceil_div(h->nchunks, threads / 32),
                                                       (int64_t)sm_count() * small_min_blocks<K, SEM, MODE>());
-    const int smem = threads / 32 * small_warp_smem<SEM>() + (MODE == kSmBitsShared ? (int)ceil_div(h->n, 32) * 4 : 0);
+    const int smem = threads / 32 * small_warp_smem<SEM>() +
+                     (MODE == kSmBitsShared ? (int)ceil_div(h->n, 32) * 4
+                                            : (MODE == kSmSegsLive ? (int)ceil_div(h->ntr, 32) * 4 : 0));
     void (*kernel)(SpmvGeom, SEM, Partials<typename SEM::V>);
     if constexpr (K == 4 && sizeof(typename SEM::V) == 4) kernel = spmv_k4_kernel<SEM, MODE>;
     else kernel = spmv_chunks_kernel<K, SEM, MODE>;
@@ -1943,6 +1992,17 @@ static b2sr_status launch_direct(const b2sr_matrix* h, const SEM& sem, Partials<
                 if (8 * h->nnz > 9 * h->T) return launch_small<K, SEM, kSmVals>(h, sem, part, s, g);
                 return launch_small<K, SEM, kSmEach>(h, sem, part, s, g);
             } else {
+                // A batched BFS's frontier: zero segments are not loaded.  R-MAT 20, 16
+                // sources, us a level: the first 99, the last three 94 to 102, the dense
+                // ones between 134 to 154 (about 130 all with every segment loaded);
+                // R-MAT 22, 64 sources: 415, 390 to 450, and 660 to 800.
+                if constexpr (LaneWords<SEM>::value) {
+                    constexpr int threads = small_threads<K, SEM, kSmSegsLive>();
+                    if (sem.live && h->n % 4 == 0 && reinterpret_cast<uintptr_t>(sem.x) % (4 * sizeof(G)) == 0 &&
+                        h->nchunks >= (int64_t)sm_count() * (threads / 32) * 4 &&
+                        ceil_div(h->ntr, 32) * 4 + threads / 32 * small_warp_smem<SEM>() <= kMaxBlockSmem)
+                        return launch_small<K, SEM, kSmSegsLive>(h, sem, part, s, g);
+                }
                 // 8-byte values where hardly a tile holds two bits: by bit (64-lane OR,
                 // us, segment / bit: permuted R-MAT 20, 1.006 bits a tile, 199 / 182;
                 // R-MAT 22, 1.08 bits, 665 / 816)
@@ -2094,11 +2154,11 @@ b2sr_status spmv_dispatch(b2sr_matrix* h, b2sr_semiring sr, b2sr_vec in_kind, co
 }
 
 b2sr_status spmm64_dispatch(b2sr_matrix* h, const uint64_t* X, uint64_t* Y, const uint64_t* M, int comp,
-                            cudaStream_t s, const int32_t* gate, bool edges, void* scratch) {
+                            cudaStream_t s, const int32_t* gate, bool edges, void* scratch, LiveColumns live) {
     return with_tile(h->k, [&](auto kc) -> b2sr_status {
         constexpr int K = decltype(kc)::value;
         SemOr64<K> sem{reinterpret_cast<const unsigned long long*>(X), reinterpret_cast<unsigned long long*>(Y),
-                       reinterpret_cast<const unsigned long long*>(M), comp ? 1 : 0, h->n};
+                       reinterpret_cast<const unsigned long long*>(M), comp ? 1 : 0, h->n, live.bits, live.dense};
         return run_spmv<K>(h, sem, nullptr, s, "spmm_or64", (M ? 24.0 : 16.0) * h->n, gate, edges, scratch);
     });
 }
@@ -2106,10 +2166,10 @@ b2sr_status spmm64_dispatch(b2sr_matrix* h, const uint64_t* X, uint64_t* Y, cons
 // The same over 32-lane words (at most 32 frontiers): half the bytes per
 // gather and 4-byte accumulators, which the tile_dim-4 kernel takes.
 b2sr_status spmm32_dispatch(b2sr_matrix* h, const uint32_t* X, uint32_t* Y, const uint32_t* M, int comp,
-                            cudaStream_t s, const int32_t* gate, bool edges) {
+                            cudaStream_t s, const int32_t* gate, bool edges, LiveColumns live) {
     return with_tile(h->k, [&](auto kc) -> b2sr_status {
         constexpr int K = decltype(kc)::value;
-        SemOr32<K> sem{X, Y, M, comp ? 1 : 0, h->n};
+        SemOr32<K> sem{X, Y, M, comp ? 1 : 0, h->n, live.bits, live.dense};
         return run_spmv<K>(h, sem, nullptr, s, "spmm_or32", (M ? 12.0 : 8.0) * h->n, gate, edges);
     });
 }
