@@ -176,9 +176,10 @@ b2sr_status new_handle_from_tiles(int32_t n, int k, int64_t T, int32_t* rowptr, 
                                   uint8_t* tiles, int64_t cap, cudaStream_t s, b2sr_matrix** out,
                                   int64_t known_nnz = -1);  // set bits, if the caller knows
 
-// SpMV and SpMM (spmv.cu), optionally gated on a device flag.  edges = false
-// (Boolean, OR and plus-times results): the output already holds zeros where
-// the matrix has no tiles, before its first tile-row and after its last.
+// SpMV and SpMM (spmv.cu), optionally gated on a device flag.  edges = false:
+// a Boolean output is already zero; an OR or plus-times output already holds
+// zeros where the matrix has no tiles, before its first tile-row and after its
+// last.
 // scratch: spmm_scratch_bytes(h, bytes of a value) bytes, 16-byte aligned, for
 // the partial rows (NULL: allocated and freed on the stream).
 b2sr_status spmv_dispatch(b2sr_matrix* h, b2sr_semiring sr, b2sr_vec in_kind, const void* x, b2sr_vec out_kind,

@@ -53,15 +53,18 @@ __global__ void bfs_seed_kernel(const int32_t* srcs, SourceList few, int nsrc, i
     }
 }
 
-// visited |= next; levels[v] = level+1 for every new vertex; ends the round
-__global__ void bfs_update_kernel(const uint32_t* __restrict__ next, uint32_t* __restrict__ visited,
-                                  int32_t* __restrict__ levels, int64_t words, LoopFlags* flags) {
+// visited |= next; levels[v] = level+1 for every new vertex; the frontier just
+// used is cleared for the next round's output; ends the round
+__global__ void bfs_update_kernel(const uint32_t* __restrict__ next, uint32_t* __restrict__ used,
+                                  uint32_t* __restrict__ visited, int32_t* __restrict__ levels, int64_t words,
+                                  LoopFlags* flags) {
     if (gate_closed(&flags->active)) return;
     const int32_t lv = *reinterpret_cast<const volatile int32_t*>(&flags->level) + 1;
     int any = 0;
     for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < words;
          w += (int64_t)gridDim.x * blockDim.x) {
         uint32_t b = next[w];
+        used[w] = 0u;
         if (!b) continue;
         any = 1;
         visited[w] |= b;
@@ -104,11 +107,9 @@ b2sr_status bfs_sources(b2sr_matrix* h, const int32_t* srcs_host, int nsrc, int3
                         [&](cudaStream_t cs, int r) -> b2sr_status {
                             uint32_t* f = (r & 1) ? fb : fa;
                             uint32_t* nx = (r & 1) ? fa : fb;
-                            // rows without tiles are zero in fb from the start, and in fa (which may
-                            // have sources there) once a round has written it
                             B2SR_TRY(spmv_dispatch(h, B2SR_BOOL_OR_AND, B2SR_VEC_BITS, f, B2SR_VEC_BITS, nx, vis, 1,
-                                                   nullptr, cs, &flags->active, r == 1));
-                            bfs_update_kernel<<<grid_for(words), 256, 0, cs>>>(nx, vis, levels, words, flags);
+                                                   nullptr, cs, &flags->active, false));
+                            bfs_update_kernel<<<grid_for(words), 256, 0, cs>>>(nx, f, vis, levels, words, flags);
                             B2SR_LAUNCH_CHECK("bfs_update_kernel");
                             return B2SR_OK;
                         },
@@ -252,7 +253,8 @@ static b2sr_status bfs_multi_lanes(b2sr_matrix* h, const int32_t* srcs_host, int
                         [&](cudaStream_t cs, int r) -> b2sr_status {
                             W* cur = (r & 1) ? Yb : X;
                             W* nxt = (r & 1) ? X : Yb;
-                            // as in bfs_sources: rows without tiles need zeros in X once
+                            // rows without tiles are zero in Yb from the start, and in X (which may
+                            // have sources there) once a round has written it
                             B2SR_TRY(spmm_lanes(h, cur, nxt, vis, cs, &flags->active, r == 1, columns));
                             msbfs_update_kernel<W><<<grid_for(n), 256, 0, cs>>>(nxt, vis, levels, n, live, state, flags);
                             B2SR_LAUNCH_CHECK("msbfs_update_kernel");

@@ -215,12 +215,17 @@ __device__ __forceinline__ uint32_t nonzero_rows(const uint32_t* w) {
 // accumulator is the OR of the tile words ANDed with the input segment (one
 // word per four rows); OR commutes with "row is non-zero", so the row mask is
 // formed only when a row is stored.  For k >= 16 it is the k-bit row mask.
+// For k <= 8 every store ORs into a cleared output: a row that crosses chunks
+// is stored by each, so there are no partials, no join and no rows to fill in
+// (three launches, an allocation and a free before; the clear and one launch
+// now).
 template <int K>
 struct SemBool {
     using V = uint32_t;
     using J = uint32_t;
     static constexpr int NV = K <= 8 ? K / 4 : 1;
     static constexpr bool kGather = false;
+    static constexpr bool kOrsInto = K <= 8;
     const uint32_t* x;
     uint32_t* y;
     const uint32_t* mask;
@@ -256,17 +261,12 @@ struct SemBool {
             uint32_t mb = ld_bits(mask, (int64_t)R * K, K);
             v &= comp ? ~mb : mb;
         }
-        if (K == 32) {
+        if constexpr (kOrsInto) {
+            if (v) atomicOr(y + (((int64_t)R * K) >> 5), v << ((R * K) & 31));
+        } else if (K == 32) {
             y[R] = v;
-        } else if (K == 16) {
-            reinterpret_cast<uint16_t*>(y)[R] = (uint16_t)v;
-        } else if (K == 8) {
-            reinterpret_cast<uint8_t*>(y)[R] = (uint8_t)v;
         } else {
-            // two tile-rows share a byte: update this nibble atomically
-            int sh = (R & 7) * 4;
-            atomicAnd(y + (R >> 3), ~(0xFu << sh));
-            if (v & 0xFu) atomicOr(y + (R >> 3), (v & 0xFu) << sh);
+            reinterpret_cast<uint16_t*>(y)[R] = (uint16_t)v;
         }
     }
 };
@@ -602,6 +602,12 @@ using SemOr64 = SemOrLanes<K, unsigned long long>;
 template <int K>
 using SemOr32 = SemOrLanes<K, uint32_t>;
 
+// schemes whose stores OR into a cleared output
+template <class S, class = void>
+struct OrsInto : std::false_type {};
+template <class S>
+struct OrsInto<S, std::void_t<decltype(S::kOrsInto)>> : std::bool_constant<S::kOrsInto> {};
+
 // ---------------------------------------------------------------------------
 // kernel arguments and shared-memory layout
 // ---------------------------------------------------------------------------
@@ -778,7 +784,8 @@ struct Walk {
 template <class SEM, class Acc, class First>
 __device__ __forceinline__ void close_chunk(const SEM& sem, Partials<typename SEM::V> part, int64_t c,
                                             const LaneSpan& ls, int lane, bool head_cs, int32_t first_row,
-                                            bool has_end, bool open, Acc& acc, First& F, int P) {
+                                            bool has_end, bool open, Acc& acc, First& F, int P,
+                                            int32_t tail_row = 0) {
     using V = typename SEM::V;
     constexpr int NV = SEM::NV;
     constexpr unsigned FULL = 0xffffffffu;
@@ -798,7 +805,7 @@ __device__ __forceinline__ void close_chunk(const SEM& sem, Partials<typename SE
     const int la = (int)((ls.ce - 1 - ls.cs) / P);
     const bool tail_open = __shfl_sync(FULL, open, la);
     const bool tail_r = __shfl_sync(FULL, inc_r, 31);
-    const bool close_here = has_end && (ex_r || head_cs);
+    const bool close_here = has_end && (OrsInto<SEM>::value || ex_r || head_cs);
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
         V x = acc.get(v);
@@ -809,6 +816,10 @@ __device__ __forceinline__ void close_chunk(const SEM& sem, Partials<typename SE
         }
         const V ex = shfl_up(x, 1);
         if (has_end && lane > 0) F.set(v, sem.comb(ex, F.get(v)));
+        if constexpr (OrsInto<SEM>::value) {
+            acc.set(v, x);  // lane 31: the open tail
+            continue;
+        }
         if (has_end && !close_here) part.val_first[c * NV + v] = F.get(v);
         if (lane == 31 && tail_open) {
             if (tail_r || head_cs) part.val_last[c * NV + v] = x;
@@ -816,6 +827,8 @@ __device__ __forceinline__ void close_chunk(const SEM& sem, Partials<typename SE
         }
     }
     if (close_here) sem.store(first_row, F);
+    if constexpr (OrsInto<SEM>::value)
+        if (lane == 31 && tail_open) sem.store(tail_row, acc);
 }
 
 // 32 bytes from global memory in one load, not allocated in L1: each tile
@@ -1156,7 +1169,7 @@ __device__ __forceinline__ void chunk_ends(const SpmvGeom& g, const SEM& sem, in
         if (end) {
             s.row[found + __popc(ends & ((1u << lane) - 1u))] = ra + j;
             atomicOr(&s.mask[(b - 1 - cs) >> 5], 1u << ((b - 1 - cs) & 31));
-        } else if (row && a == b) {
+        } else if (!OrsInto<SEM>::value && row && a == b) {
             sem.store(ra + j, idv);
         }
         found += __popc(ends);
@@ -1379,6 +1392,10 @@ __device__ __forceinline__ void small_chunk(const SpmvGeom& g, const SEM& sem, P
     if (one_row) {
         const bool head = __shfl_sync(0xffffffffu, t.win, 0) == cs;  // the row begins with this chunk
         join_lanes(sem, acc, lane);
+        if constexpr (OrsInto<SEM>::value) {
+            if (lane == 0) sem.store(t.ra, acc);
+            return;
+        }
         if (head && c + 1 == g.nchunks) {  // begins and ends in this chunk (the matrix's last)
             if constexpr (SEM::kGather) {
                 if (lane < NV) sem.store_row(t.ra, joined_value<NV>(lane), acc.get(0));
@@ -1404,7 +1421,7 @@ __device__ __forceinline__ void small_chunk(const SpmvGeom& g, const SEM& sem, P
     // a tail after the chunk's last row end is continued by the next chunk
     const bool open = !((s.mask[(ce - 1 - cs) >> 5] >> ((ce - 1 - cs) & 31)) & 1u);
     const int32_t first_row = has_end ? s.row[rank0] : 0;
-    close_chunk(sem, part, c, ls, lane, head_cs, first_row, has_end, open, acc, F, Sh::P);
+    close_chunk(sem, part, c, ls, lane, head_cs, first_row, has_end, open, acc, F, Sh::P, t.rb);
 }
 
 // Dynamic shared memory a warp: its ChunkRows, and for 16-byte values the
@@ -1766,12 +1783,24 @@ __global__ void __launch_bounds__(kSpmvThreads, (gather_min_blocks<K, SEM>())) s
 // partial in order, then a fixed butterfly joins the lanes).
 template <int K, class SEM>
 __global__ void spmv_fixup_kernel(const int32_t* __restrict__ split, const int32_t* __restrict__ split_long,
-                                  int64_t nshort, int64_t nlong, int64_t short_blocks, SEM sem, Partials<typename SEM::V> part,
+                                  int64_t nshort, int64_t nlong, int64_t short_blocks, int64_t long_blocks,
+                                  int32_t lead_end, int32_t trail_begin, int32_t ntr, SEM sem, Partials<typename SEM::V> part,
                                   const int32_t* gate) {
     using V = typename SEM::V;
     using J = typename SEM::J;
     constexpr int NV = SEM::NV;
     if (gated_off(gate)) return;
+    if ((int64_t)blockIdx.x >= short_blocks + long_blocks) {  // rows outside the tiles: the identity
+        RegAcc<V, NV> idv;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) idv.set(v, sem.ident());
+        const int64_t first = short_blocks + long_blocks;
+        const int64_t stride = ((int64_t)gridDim.x - first) * blockDim.x;
+        const int64_t tid = ((int64_t)blockIdx.x - first) * blockDim.x + threadIdx.x;
+        for (int64_t R = tid; R < lead_end; R += stride) sem.store((int32_t)R, idv);
+        for (int64_t R = trail_begin + tid; R < ntr; R += stride) sem.store((int32_t)R, idv);
+        return;
+    }
     if ((int64_t)blockIdx.x < short_blocks) {
         if constexpr (SEM::kGather) {
             // value schemes: a thread per (row, value); the NV threads of a
@@ -1831,33 +1860,23 @@ __global__ void spmv_fixup_kernel(const int32_t* __restrict__ split, const int32
     }
 }
 
+// The join, and with `edges` the tile-rows before the first tile and after the
+// last one (every row when the matrix has no tiles), which get the identity.
 template <int K, class SEM>
 static b2sr_status launch_fixup(const b2sr_matrix* h, const SEM& sem, Partials<typename SEM::V> part,
-                                cudaStream_t s, const int32_t* gate) {
-    if (h->nsplit_short + h->nsplit_long == 0) return B2SR_OK;
+                                cudaStream_t s, const int32_t* gate, bool edges) {
+    const int32_t lead_end = h->T == 0 ? h->ntr : h->first_row;
+    const int32_t trail_begin = h->T == 0 ? h->ntr : h->last_row + 1;
+    const int64_t outside = edges ? (int64_t)lead_end + (h->ntr - trail_begin) : 0;
     const int64_t short_blocks = ceil_div(h->nsplit_short * (SEM::kGather ? SEM::NV : 1), 256);
     const int64_t long_blocks = ceil_div(h->nsplit_long, 8);
-    spmv_fixup_kernel<K, SEM><<<(unsigned)(short_blocks + long_blocks), 256, 0, s>>>(
-        h->split, h->split + 3 * (h->nchunks - h->nsplit_long), h->nsplit_short, h->nsplit_long, short_blocks, sem, part,
-        gate);
+    const int64_t edge_blocks = std::min<int64_t>(ceil_div(outside, 256), (int64_t)sm_count() * 4);
+    if (short_blocks + long_blocks + edge_blocks == 0) return B2SR_OK;
+    spmv_fixup_kernel<K, SEM><<<(unsigned)(short_blocks + long_blocks + edge_blocks), 256, 0, s>>>(
+        h->split, h->split + 3 * (h->nchunks - h->nsplit_long), h->nsplit_short, h->nsplit_long, short_blocks,
+        long_blocks, lead_end, trail_begin, h->ntr, sem, part, gate);
     B2SR_LAUNCH_CHECK("spmv_fixup_kernel");
     return B2SR_OK;
-}
-
-// Tile-rows before the first tile and after the last one (every row when the
-// matrix has no tiles) get the identity.
-template <int K, class SEM>
-__global__ void spmv_edges_kernel(SEM sem, int32_t lead_end, int32_t trail_begin, int32_t ntr,
-                                  const int32_t* gate) {
-    using V = typename SEM::V;
-    if (gated_off(gate)) return;
-    RegAcc<V, SEM::NV> idv;
-#pragma unroll
-    for (int v = 0; v < SEM::NV; ++v) idv.set(v, sem.ident());
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    for (int64_t R = tid; R < lead_end; R += stride) sem.store((int32_t)R, idv);
-    for (int64_t R = trail_begin + tid; R < ntr; R += stride) sem.store((int32_t)R, idv);
 }
 
 // semirings whose result includes the diagonal's self term (min-plus)
@@ -1888,7 +1907,8 @@ __global__ void spmv_self_kernel(SEM sem, const int32_t* gate) {
 
 __global__ void clear_words_kernel(uint32_t* w, int64_t count, const int32_t* gate) {
     if (gated_off(gate)) return;
-    for (int64_t i = threadIdx.x; i < count; i += blockDim.x) w[i] = 0u;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x)
+        w[i] = 0u;
 }
 
 // ---------------------------------------------------------------------------
@@ -1911,15 +1931,16 @@ static b2sr_status clear_bitset_tail(const b2sr_matrix* h, uint32_t* bits, cudaS
     return B2SR_OK;
 }
 
-template <int K, class SEM>
-static b2sr_status launch_edges(const b2sr_matrix* h, const SEM& sem, cudaStream_t s, const int32_t* gate) {
-    int32_t lead_end = h->T == 0 ? h->ntr : h->first_row;
-    int32_t trail_begin = h->T == 0 ? h->ntr : h->last_row + 1;
-    int64_t work = (int64_t)lead_end + (h->ntr - trail_begin);
-    if (work <= 0) return B2SR_OK;
-    int grid = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(work, 256), (int64_t)sm_count() * 4));
-    spmv_edges_kernel<K, SEM><<<grid, 256, 0, s>>>(sem, lead_end, trail_begin, h->ntr, gate);
-    B2SR_LAUNCH_CHECK("spmv_edges_kernel");
+// Clears the whole bitset (schemes that OR into it).
+static b2sr_status clear_bitset(const b2sr_matrix* h, uint32_t* bits, cudaStream_t s, const int32_t* gate) {
+    const int64_t words = ceil_div(h->n, 32);
+    if (words == 0) return B2SR_OK;
+    if (!gate) {
+        B2SR_CUDA_TRY(cudaMemsetAsync(bits, 0, words * sizeof(uint32_t), s));
+        return B2SR_OK;
+    }
+    clear_words_kernel<<<grid_for(words), 256, 0, s>>>(bits, words, gate);
+    B2SR_LAUNCH_CHECK("clear_words_kernel");
     return B2SR_OK;
 }
 
@@ -2024,11 +2045,11 @@ static b2sr_status launch_direct(const b2sr_matrix* h, const SEM& sem, Partials<
 // the chunk kernel (staged or direct) and the cross-chunk join
 template <int K, class SEM>
 static b2sr_status run_chunks(const b2sr_matrix* h, const SEM& sem, cudaStream_t s, const char* family,
-                              double vec_bytes, const int32_t* gate, const SpmvGeom& g, void* scratch) {
+                              double vec_bytes, const int32_t* gate, const SpmvGeom& g, void* scratch, bool edges) {
     using V = typename SEM::V;
     DevBuf pbuf(s);
-    Partials<V> part;
-    B2SR_TRY((alloc_partials<V, SEM::NV>(pbuf, h->nchunks, scratch, &part)));
+    Partials<V> part{nullptr, nullptr};
+    if (!OrsInto<SEM>::value) B2SR_TRY((alloc_partials<V, SEM::NV>(pbuf, h->nchunks, scratch, &part)));
     const unsigned blocks = (unsigned)ceil_div(h->nchunks, kSpmvWarps);
     bool staged = false;
     // AUTO: the small-tile kernel where it serves
@@ -2050,7 +2071,8 @@ static b2sr_status run_chunks(const b2sr_matrix* h, const SEM& sem, cudaStream_t
         timing_end(tok, family, spmv_bytes(h, vec_bytes), s);
         B2SR_TRY(st);
     }
-    return launch_fixup<K, SEM>(h, sem, part, s, gate);
+    if constexpr (OrsInto<SEM>::value) return B2SR_OK;
+    else return launch_fixup<K, SEM>(h, sem, part, s, gate, edges);
 }
 
 template <int K, class SEM>
@@ -2058,11 +2080,16 @@ static b2sr_status run_spmv(const b2sr_matrix* h, const SEM& sem, uint32_t* bits
                             const char* family, double vec_bytes, const int32_t* gate, bool edges = true,
                             void* scratch = nullptr) {
     SpmvGeom g{h->rowptr, h->colind, h->tiles, h->chunk_row, h->T, h->nchunks, h->ntr, gate};
-    if (edges) {
-        if (bits_out) B2SR_TRY(clear_bitset_tail<K>(h, bits_out, s, gate));
-        B2SR_TRY((launch_edges<K, SEM>(h, sem, s, gate)));
+    if (OrsInto<SEM>::value) {
+        if (edges) B2SR_TRY(clear_bitset(h, bits_out, s, gate));
+    } else if (edges && bits_out) {
+        B2SR_TRY(clear_bitset_tail<K>(h, bits_out, s, gate));
     }
-    if (h->nchunks > 0) B2SR_TRY((run_chunks<K, SEM>(h, sem, s, family, vec_bytes, gate, g, scratch)));
+    if (h->nchunks > 0) {
+        B2SR_TRY((run_chunks<K, SEM>(h, sem, s, family, vec_bytes, gate, g, scratch, edges)));
+    } else if constexpr (!OrsInto<SEM>::value) {
+        B2SR_TRY((launch_fixup<K, SEM>(h, sem, Partials<typename SEM::V>{nullptr, nullptr}, s, gate, edges)));
+    }
     if constexpr (HasSelfTerm<SEM>::value) {
         const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(h->n, 256), (int64_t)sm_count() * 8));
         spmv_self_kernel<SEM><<<grid, 256, 0, s>>>(sem, gate);
@@ -2086,11 +2113,9 @@ b2sr_status row_counts(const b2sr_matrix* h, int32_t* cnt, int32_t* first, int32
         sem.comp = 0;
         sem.n = h->n;
         SpmvGeom g{h->rowptr, h->colind, h->tiles, h->chunk_row, h->T, h->nchunks, h->ntr, nullptr};
-        B2SR_TRY((launch_edges<K, SEM>(h, sem, s, nullptr)));
-        if (h->nchunks == 0) return B2SR_OK;
         const Partials<int32_t> part{first, last};
-        B2SR_TRY((launch_direct<K, SEM>(h, sem, part, s, g)));
-        return launch_fixup<K, SEM>(h, sem, part, s, nullptr);
+        if (h->nchunks > 0) B2SR_TRY((launch_direct<K, SEM>(h, sem, part, s, g)));
+        return launch_fixup<K, SEM>(h, sem, part, s, nullptr, true);
     });
 }
 
@@ -2282,16 +2307,20 @@ static b2sr_status run_spmv_bool_fixed(const b2sr_matrix* h, const SemBool<K>& s
                                               std::to_string(2 * half) + " scratch bytes, the fixed array holds " +
                                               std::to_string(kNoallocScratchBytes));
     SpmvGeom g{h->rowptr, h->colind, h->tiles, h->chunk_row, h->T, h->nchunks, h->ntr, nullptr};
-    B2SR_TRY(clear_bitset_tail<K>(h, y, s, nullptr));
-    B2SR_TRY((launch_edges<K, SEM>(h, sem, s, nullptr)));
-    if (h->nchunks == 0) return B2SR_OK;
-    // every partial the fixup reads is written by the chunk kernel of the
-    // same call, so the scratch needs no clearing between calls
-    Partials<uint32_t> part;
-    part.val_first = static_cast<uint32_t*>(scratch);
-    part.val_last = reinterpret_cast<uint32_t*>(static_cast<unsigned char*>(scratch) + half);
-    B2SR_TRY((launch_direct<K, SEM>(h, sem, part, s, g)));
-    return launch_fixup<K, SEM>(h, sem, part, s, nullptr);
+    if constexpr (OrsInto<SEM>::value) {  // needs no scratch: the limit is the entry point's
+        B2SR_TRY(clear_bitset(h, y, s, nullptr));
+        if (h->nchunks == 0) return B2SR_OK;
+        return launch_direct<K, SEM>(h, sem, Partials<uint32_t>{nullptr, nullptr}, s, g);
+    } else {
+        B2SR_TRY(clear_bitset_tail<K>(h, y, s, nullptr));
+        // every partial the fixup reads is written by the chunk kernel of the
+        // same call, so the scratch needs no clearing between calls
+        Partials<uint32_t> part;
+        part.val_first = static_cast<uint32_t*>(scratch);
+        part.val_last = reinterpret_cast<uint32_t*>(static_cast<unsigned char*>(scratch) + half);
+        if (h->nchunks > 0) B2SR_TRY((launch_direct<K, SEM>(h, sem, part, s, g)));
+        return launch_fixup<K, SEM>(h, sem, part, s, nullptr, true);
+    }
 }
 
 }  // namespace b2sr
