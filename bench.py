@@ -669,11 +669,12 @@ def spmv_kernel_name(family, tile, schedule):
     library's dispatch: at k = 4 the tile_dim-4 kernel for the bit-vector
     schemes and, unless the schedule is the staged one, for the unweighted
     4-byte value schemes; the staged gather kernel for the value schemes at
-    k <= 16 under the staged schedule and, from k = 8, the default one; the
-    chunk kernels otherwise)."""
+    k <= 16 under the staged schedule and, under the default one, for weighted
+    min-plus and at k = 8 for all but the 64-lane OR; the chunk kernels
+    otherwise)."""
     bits = family in ("spmv_bool", "spmv_count")
     k4_values = family in ("spmv_plus", "spmv_min_i32", "spmv_max", "spmm_or32")
-    direct = schedule == 2 or (schedule == 0 and tile == 4 and family != "spmv_minplus")
+    direct = schedule == 2 or (schedule == 0 and family != "spmv_minplus" and (tile != 8 or family == "spmm_or64"))
     if tile == 4 and (bits or (k4_values and direct)):
         return "spmv_k4_kernel"
     if not bits and tile <= 16 and not direct:

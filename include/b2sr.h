@@ -95,7 +95,7 @@ typedef enum {
  * segment of a tile in shared memory (Sec. IV); STAGED is that idea for a
  * gather per set bit, DIRECT reads the vector from global memory. */
 typedef enum {
-    B2SR_SCHED_AUTO = 0,   /* DIRECT at k = 4 (except weighted min-plus), else STAGED where it exists */
+    B2SR_SCHED_AUTO = 0,   /* STAGED at k = 8 (except the 64-lane OR), for min-plus at k = 4 and, with weights, at k = 16; else DIRECT */
     B2SR_SCHED_STAGED = 1, /* set-bit gathers staged in shared memory (cp.async), then reduced */
     B2SR_SCHED_DIRECT = 2  /* each lane walks its tiles and loads x directly */
 } b2sr_schedule;

@@ -1055,7 +1055,7 @@ struct MinMax<SemMaxF32<K>> : std::true_type {};
 // tiles hold hardly more than one: the 16 predicated updates are 32 and 64
 // instructions then), or segments where the block's copy of `live` says that
 // they are not all zero (the sparse levels of a batched BFS).
-enum { kSmBits = 0, kSmBitsShared = 1, kSmSegs = 2, kSmVals = 3, kSmEach = 4, kSmSegsLive = 5 };
+enum { kSmBits = 0, kSmBitsShared = 1, kSmSegs = 2, kSmVals = 3, kSmEach = 4, kSmSegsLive = 5, kRowLanes = 6 };
 // Threads a block, and the resident blocks the registers are budgeted for
 // (every lane holds two chunks' tile words and columns; with 16-byte values
 // one).  R-MAT 20, k = 4, in
@@ -1072,6 +1072,7 @@ constexpr int small_threads() {
 template <int K, class SEM, int MODE>
 constexpr int small_min_blocks() {
     if (MODE == kSmBitsShared || MODE == kSmSegsLive) return 1;
+    if (MODE == kRowLanes) return sizeof(typename SEM::V) == 16 ? 4 : 6;
     if (sizeof(typename SEM::V) == 16) return MODE == kSmEach ? 4 : 3;
     if (SEM::NV == 8) return 2;
     return K == 8 || sizeof(typename SEM::V) == 8 || MinMax<SEM>::value ? 3 : 4;
@@ -1507,6 +1508,241 @@ __device__ __forceinline__ void small_body(const SpmvGeom& g, const SEM& sem, Pa
     }
 }
 
+// ---------------------------------------------------------------------------
+// row-lane chunk kernel: the value schemes at k = 16 and 32, the 64-lane OR at
+// k = 8.  Few of a tile's rows hold a bit there, and k accumulators a lane are
+// too many to join across lanes, so the lanes of a warp are the rows: lane l
+// takes row l % k of every (32/k)-th tile, one accumulator, and a tile-row's
+// end joins the 32/k lanes of a row by at most two shuffles and stores k
+// neighbouring values.  A step is 32/k tiles; the tiles and columns of a
+// segment (2 KB of tiles) are copied to shared memory asynchronously, where a
+// step's rows are 32 neighbouring bytes, half-words or words.  Steps go in
+// groups of four, whose first gathers are in flight together (most rows of a
+// tile hold one bit; the others loop).
+// R-MAT 20, k = 32, plus-times: 2034 us with k accumulators a lane, 661 here
+// (k = 16: 654, 439); bound by latency and instructions (2.1 an SM a cycle,
+// DRAM 37%, L1 25%), so the registers are cut to 40 for six blocks an SM (four
+// with 16-byte values, which spill then): 638 us before the sums were
+// compensated, against 738 with four blocks and groups of eight, whose gathers
+// in flight a warp are twice as many.  The compensation costs 2 to 4% (four
+// columns 10%) and takes the error below that of the k accumulators (relative
+// to a 64-bit sum, root mean square 2.0e-8 against 2.1e-8 on R-MAT 20, 2.8e-8
+// against 3.3e-8 on 3607 vertices; without it 2.2e-8 and 3.8e-8).
+// ---------------------------------------------------------------------------
+template <int K>
+struct RowLaneShape {
+    static constexpr int SUBS = 32 / K;                            // tiles a step
+    static constexpr int SEG = 2048 / ChunkShape<K>::TB;           // tiles a segment: 256, 64, 16
+    static constexpr int STEPS = SEG / SUBS;                       // 64, 32, 16
+    static constexpr int SEGS = ChunkShape<K>::CT / SEG;           // segments a chunk: 1, 2, 4
+    static constexpr int GRP = 4;                                  // steps a group
+};
+
+template <int K>
+struct RowLaneSegment {
+    __align__(16) uint8_t tiles[2048];
+    __align__(16) int32_t col[RowLaneShape<K>::SEG];
+};
+
+__device__ __forceinline__ void cp_async_stream16(void* smem, const void* gmem) {
+    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
+}
+
+// Copies the segment from tile t0 (the arrays are padded to whole chunks).
+template <int K>
+__device__ __forceinline__ void rowlane_copy(const SpmvGeom& g, int64_t t0, int lane, RowLaneSegment<K>& s) {
+    const uint8_t* src = g.tiles + t0 * ChunkShape<K>::TB;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) cp_async_stream16(s.tiles + 512 * j + 16 * lane, src + 512 * j + 16 * lane);
+    constexpr int PIECES = RowLaneShape<K>::SEG / 4;
+#pragma unroll
+    for (int j = 0; j < PIECES; j += 32)
+        if (j + lane < PIECES) cp_async_stream16(s.col + 4 * (j + lane), g.colind + t0 + 4 * (j + lane));
+    cp_async_commit();
+}
+
+// Joins the lanes of a row (lanes l, l + k, ...), earlier tiles first.
+template <int K, class SEM>
+__device__ __forceinline__ typename SEM::V rowlane_join(const SEM& sem, typename SEM::V v, int lane) {
+#pragma unroll
+    for (int d = K; d < 32; d <<= 1) {
+        const typename SEM::V o = shfl_xor(v, d);
+        v = (lane & d) ? sem.comb(o, v) : sem.comb(v, o);
+    }
+    return v;
+}
+
+// A lane's running value of its row.  fp32 sums are compensated, as a lane's
+// chain is as long as its tile-row (an infinite sum has no rounding error).
+template <class SEM, class J>
+struct RowLaneAcc {
+    typename SEM::V a;
+    __device__ __forceinline__ void clear(const SEM& sem) { a = sem.ident(); }
+    __device__ __forceinline__ void add(const SEM& sem, typename SEM::V v) { a = sem.comb(a, v); }
+    __device__ __forceinline__ typename SEM::V value() const { return a; }
+};
+__device__ __forceinline__ void csum_push(CSum& a, float v) {
+    const float t = __fadd_rn(a.s, v);
+    const float bp = __fsub_rn(t, a.s);
+    a.c = __fadd_rn(a.c, __fadd_rn(__fsub_rn(a.s, __fsub_rn(t, bp)), __fsub_rn(v, bp)));
+    a.s = t;
+}
+__device__ __forceinline__ float csum_value(CSum a) { return isfinite(a.s) ? (float)a : a.s; }
+template <class SEM>
+struct RowLaneAcc<SEM, CSum> {
+    CSum a;
+    __device__ __forceinline__ void clear(const SEM&) { a = CSum(0.0f); }
+    __device__ __forceinline__ void add(const SEM&, float v) { csum_push(a, v); }
+    __device__ __forceinline__ float value() const { return csum_value(a); }
+};
+template <class SEM>
+struct RowLaneAcc<SEM, CSum4> {
+    CSum4 a;
+    __device__ __forceinline__ void clear(const SEM& sem) { a = CSum4(sem.ident()); }
+    __device__ __forceinline__ void add(const SEM&, float4 v) {
+        csum_push(a.v[0], v.x);
+        csum_push(a.v[1], v.y);
+        csum_push(a.v[2], v.z);
+        csum_push(a.v[3], v.w);
+    }
+    __device__ __forceinline__ float4 value() const {
+        return make_float4(csum_value(a.v[0]), csum_value(a.v[1]), csum_value(a.v[2]), csum_value(a.v[3]));
+    }
+};
+
+template <int K, class SEM>
+__device__ __forceinline__ void rowlane_body(const SpmvGeom& g, const SEM& sem, Partials<typename SEM::V> part) {
+    using S = RowLaneShape<K>;
+    using V = typename SEM::V;
+    using G = typename SEM::G;
+    using Rows = typename std::conditional<K == 8, uint8_t, typename std::conditional<K == 16, uint16_t, uint32_t>::type>::type;
+    constexpr int CT = ChunkShape<K>::CT;
+    constexpr unsigned FULL = 0xffffffffu;
+    constexpr int GRP = RowLaneShape<K>::GRP;
+    static_assert(GRP == 4, "the group's tiles are added in pairs");
+    __shared__ ChunkRows rows[kSpmvWarps];
+    __shared__ RowLaneSegment<K> segs[kSpmvWarps];
+    if (gated_off(g.gate)) return;
+    ChunkRows& cr = rows[threadIdx.x >> 5];
+    RowLaneSegment<K>& seg = segs[threadIdx.x >> 5];
+    const Rows* bits = reinterpret_cast<const Rows*>(seg.tiles);
+    const int lane = (int)lane_id();
+    const int r = lane % K, sub = lane / K;
+    const int32_t W = (int32_t)gridDim.x * kSpmvWarps;
+    RegAcc<V, SEM::NV> idv;
+#pragma unroll
+    for (int v = 0; v < SEM::NV; ++v) idv.set(v, sem.ident());
+    for (int32_t c = (int32_t)blockIdx.x * kSpmvWarps + (threadIdx.x >> 5); c < g.nchunks; c += W) {
+        const int32_t ra = __ldg(g.chunk_row + c), rb = __ldg(g.chunk_row + c + 1);
+        const int32_t cs = c * CT, ce = cs + min(CT, (int32_t)g.T - cs);
+        const bool skip = sem.saturated((int64_t)ra * K, ((int64_t)rb + 1) * K);  // every row masked out
+        if (!skip) rowlane_copy<K>(g, cs, lane, seg);
+        const int32_t win = row_window(g, ra, rb - ra, lane);
+        const bool one_row = ra == rb;
+        const bool head = __shfl_sync(FULL, win, 0) == cs;  // tile-row ra begins with this chunk
+        if (!one_row) chunk_ends(g, sem, ra, rb, win, cs, ce, lane, idv, cr);
+        RowLaneAcc<SEM, typename SEM::J> acc;
+        acc.clear(sem);
+        int rank = 0;  // row ends so far
+        // the row that ends here: stored, or the chunk's first partial
+        auto end_row = [&]() {
+            const V v = rowlane_join<K>(sem, acc.value(), lane);
+            if (lane < K) {
+                if (rank > 0 || head) sem.store_row(cr.row[rank], lane, v);
+                else part.val_first[(int64_t)c * K + lane] = v;
+            }
+            ++rank;
+            acc.clear(sem);
+        };
+#pragma unroll 1
+        for (int q = 0; q < S::SEGS; ++q) {
+            if (!skip) {
+                cp_async_wait_all();
+                __syncwarp();
+            }
+#pragma unroll 1
+            for (int i0 = 0; i0 < S::STEPS; i0 += GRP) {
+                uint32_t b[GRP];
+                int32_t at[GRP];  // first input value under the tile
+                int32_t wat[GRP];
+                G x[GRP];
+                float wv[GRP];
+#pragma unroll
+                for (int i = 0; i < GRP; ++i) {
+                    const int tile = (i0 + i) * S::SUBS + sub;  // in the segment
+                    b[i] = skip ? 0u : (uint32_t)bits[(i0 + i) * 32 + lane];
+                    at[i] = (skip ? 0 : seg.col[tile]) * K;
+                    wat[i] = 0;
+                    wv[i] = 1.0f;
+                    if constexpr (SEM::kMayWeight) {
+                        if (sem.weighted) {  // the tile's bits in earlier rows, then the row's own
+                            int before = __popc(b[i]);
+#pragma unroll
+                            for (int d = 1; d < K; d <<= 1) {
+                                const int o = __shfl_up_sync(FULL, before, d, K);
+                                if (r >= d) before += o;
+                            }
+                            const int32_t t = cs + min(q * S::SEG + tile, (int32_t)g.T - 1 - cs);
+                            wat[i] = __ldg(sem.voffs() + t) + (before - __popc(b[i]));
+                        }
+                    }
+                    if (b[i]) {
+                        x[i] = __ldg(sem.src() + (at[i] + __ffs(b[i]) - 1));
+                        if constexpr (SEM::kMayWeight)
+                            if (sem.weighted) wv[i] = __ldg(sem.wts() + wat[i]);
+                    }
+                }
+                const int t0 = q * S::SEG + i0 * S::SUBS;  // the group's first tile in the chunk
+                uint32_t ends = 0u;                          // row ends among its tiles
+                if (!one_row)
+                    ends = (cr.mask[t0 >> 5] >> (t0 & 31)) & (GRP * S::SUBS == 32 ? FULL : (1u << (GRP * S::SUBS % 32)) - 1u);
+                // the lane's row of a tile: its first bit's value, then the others'
+                auto tile_sum = [&](int i) {
+                    V v = sem.ident();
+                    if (b[i] == 0u) return v;
+                    v = sem.apply(v, x[i], wv[i]);
+                    for (uint32_t more = b[i] & (b[i] - 1u); more; more &= more - 1u) {
+                        float w2 = 1.0f;
+                        if constexpr (SEM::kMayWeight)
+                            if (sem.weighted) w2 = __ldg(sem.wts() + ++wat[i]);
+                        v = sem.apply(v, __ldg(sem.src() + (at[i] + __ffs(more) - 1)), w2);
+                    }
+                    return v;
+                };
+                if (ends == 0u) {  // warp-uniform
+                    const V v = sem.comb(tile_sum(0), tile_sum(1));
+                    acc.add(sem, sem.comb(v, sem.comb(tile_sum(2), tile_sum(3))));
+                } else {
+                    // tile by tile: a lane adds its row of a tile before that
+                    // tile's end and after the ends of earlier ones
+#pragma unroll
+                    for (int i = 0; i < GRP; ++i) {
+                        const V v = tile_sum(i);
+#pragma unroll
+                        for (int u = 0; u < S::SUBS; ++u) {
+                            if (sub == u) acc.add(sem, v);
+                            if ((ends >> (i * S::SUBS + u)) & 1u) end_row();
+                        }
+                    }
+                }
+            }
+            __syncwarp();  // every lane has read the segment
+            if (q + 1 < S::SEGS && !skip) rowlane_copy<K>(g, (int64_t)cs + (q + 1) * S::SEG, lane, seg);
+        }
+        // the open row: all of a chunk inside one row, or the tail
+        const bool open = one_row || !((cr.mask[(ce - 1 - cs) >> 5] >> ((ce - 1 - cs) & 31)) & 1u);
+        if (open) {
+            const V v = rowlane_join<K>(sem, acc.value(), lane);
+            if (lane < K) {
+                if (one_row && c + 1 == g.nchunks && head) sem.store_row(ra, lane, v);
+                else if (one_row && !head) part.val_first[(int64_t)c * K + lane] = v;
+                else part.val_last[(int64_t)c * K + lane] = v;
+            }
+        }
+    }
+}
+
 // k = 4 with the bit-vector schemes and 4-byte values; the other small-tile
 // cases (k = 8, 8-byte values).
 template <class SEM, int MODE>
@@ -1517,7 +1753,8 @@ __global__ void __launch_bounds__((small_threads<4, SEM, MODE>()), (small_min_bl
 template <int K, class SEM, int MODE>
 __global__ void __launch_bounds__((small_threads<K, SEM, MODE>()), (small_min_blocks<K, SEM, MODE>()))
     spmv_chunks_kernel(SpmvGeom g, SEM sem, Partials<typename SEM::V> part) {
-    small_body<K, SEM, MODE>(g, sem, part);
+    if constexpr (MODE == kRowLanes) rowlane_body<K, SEM>(g, sem, part);
+    else small_body<K, SEM, MODE>(g, sem, part);
 }
 
 // ---------------------------------------------------------------------------
@@ -1968,6 +2205,29 @@ constexpr bool use_small() {
     else return K == 4 && !SEM::kMayWeight;
 }
 
+// The row-lane kernel serves the value schemes at k = 32, the unweighted ones
+// at k = 16 and the 64-lane OR at k = 8.  us, the better of the staged and the
+// general direct kernel / this one:
+//   R-MAT 20 and its permutation   k = 8       k = 16                k = 32
+//   plus-times               298, 230 / 285, 322   654, 622 / 439, 601     2034, 2516 / 661, 1147
+//   64-lane OR               454, 390 / 328, 355   937, 815 / 482, 641     2853, 3696 / 729, 1239
+//   four columns             650, 576 / 764, 935   1520, 1393 / 689, 911   5742, 6941 / 1257, 1968
+//   weighted min-plus        377, 294 / 592, 657   860, 748 / 895, 1250    2358, 2873 / 1360, 2459
+// The bits before a row, which a weight's place needs, cost a scan of the
+// tile; at k = 8 a step of four tiles mostly holds fewer set bits than lanes.
+enum { kRowLanesNever, kRowLanesUnweighted, kRowLanesAlways };
+template <int K, class SEM>
+constexpr int row_lanes() {
+    if constexpr (!SEM::kGather || K < 8) return kRowLanesNever;
+    else if constexpr (K == 8) return LaneWords<SEM>::value && sizeof(typename SEM::V) == 8 ? kRowLanesAlways : kRowLanesNever;
+    else return K == 16 && SEM::kMayWeight ? kRowLanesUnweighted : kRowLanesAlways;
+}
+template <int K, class SEM>
+static bool use_row_lanes(const SEM& sem) {
+    if constexpr (row_lanes<K, SEM>() == kRowLanesUnweighted) return !sem.weighted;
+    else return row_lanes<K, SEM>() == kRowLanesAlways;
+}
+
 template <int K, class SEM, int MODE>
 static b2sr_status launch_small(const b2sr_matrix* h, const SEM& sem, Partials<typename SEM::V> part, cudaStream_t s,
                                 const SpmvGeom& g) {
@@ -2036,8 +2296,20 @@ static b2sr_status launch_direct(const b2sr_matrix* h, const SEM& sem, Partials<
             }
         }
     } else {
-        spmv_chunks_kernel<K, SEM><<<(unsigned)ceil_div(h->nchunks, kSpmvWarps), kSpmvThreads, 0, s>>>(g, sem, part);
-        B2SR_LAUNCH_CHECK("spmv_chunks_kernel");
+        if constexpr (row_lanes<K, SEM>() != kRowLanesNever) {
+            if (use_row_lanes<K>(sem)) {
+                const unsigned grid =
+                    (unsigned)std::min<int64_t>(ceil_div(h->nchunks, kSpmvWarps),
+                                                (int64_t)sm_count() * small_min_blocks<K, SEM, kRowLanes>());
+                spmv_chunks_kernel<K, SEM, kRowLanes><<<grid, kSpmvThreads, 0, s>>>(g, sem, part);
+                B2SR_LAUNCH_CHECK("row-lane SpMV kernel");
+                return B2SR_OK;
+            }
+        }
+        if constexpr (row_lanes<K, SEM>() != kRowLanesAlways) {
+            spmv_chunks_kernel<K, SEM><<<(unsigned)ceil_div(h->nchunks, kSpmvWarps), kSpmvThreads, 0, s>>>(g, sem, part);
+            B2SR_LAUNCH_CHECK("spmv_chunks_kernel");
+        }
     }
     return B2SR_OK;
 }
@@ -2052,10 +2324,10 @@ static b2sr_status run_chunks(const b2sr_matrix* h, const SEM& sem, cudaStream_t
     if (!OrsInto<SEM>::value) B2SR_TRY((alloc_partials<V, SEM::NV>(pbuf, h->nchunks, scratch, &part)));
     const unsigned blocks = (unsigned)ceil_div(h->nchunks, kSpmvWarps);
     bool staged = false;
-    // AUTO: the small-tile kernel where it serves
+    // AUTO: the small-tile and row-lane kernels where they serve
     if constexpr (SEM::kGather && K <= 16)
         staged = h->schedule == B2SR_SCHED_STAGED ||
-                 (h->schedule == B2SR_SCHED_AUTO && !use_small<K, SEM>());
+                 (h->schedule == B2SR_SCHED_AUTO && !(use_small<K, SEM>() || use_row_lanes<K>(sem)));
     if constexpr (SEM::kGather && K <= 16) if (staged) {
         const int smem = kSpmvWarps * GatherLayout<K, SEM>::bytes;
         if (smem > 48 * 1024)
