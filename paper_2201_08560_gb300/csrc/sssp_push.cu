@@ -25,11 +25,16 @@
 // is read.  Distances only decrease, and every value written is the length of
 // a path, so the result is the shortest-path fixed point whatever the order of
 // the atomics: bit-exact and the same as b2sr_sssp's.
+#include <cooperative_groups.h>
+
 #include <algorithm>
+#include <atomic>
 #include <type_traits>
 
 #include "b2sr_internal.cuh"
 #include "captured.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace b2sr {
 
@@ -51,7 +56,7 @@ struct PushState {
     int32_t epoch;   // which far counters are in use
     float theta;     // threshold (infinite without buckets)
     int32_t rounds;  // rounds run
-    int32_t pad;
+    int32_t busy;    // the cluster left a round with too many rows for it
     unsigned long long worked;  // active tile-rows summed over the rounds
 };
 // Counters, each on a line of its own.  near[r & 3] is the length of the list
@@ -111,50 +116,153 @@ __device__ __forceinline__ uint32_t pushed_row(const uint8_t* __restrict__ tiles
 
 // The tile-rows a block appends to one list: kept in shared memory, appended
 // at the block's end with one global atomic (directly once the buffer is full).
-constexpr int kPushBuffer = 512;
+template <int CAP>
 struct Appends {
     int32_t n, base;
-    int32_t row[kPushBuffer];
+    int32_t row[CAP];
 };
+constexpr int kPushBuffer = 512;
 
-template <int K>
-__device__ __forceinline__ void mark_bits(const PushSet& s, int32_t* count, Appends& ap, int32_t J, uint32_t bits) {
+template <int K, int CAP>
+__device__ __forceinline__ void mark_bits(const PushSet& s, int32_t* count, Appends<CAP>& ap, int32_t J, uint32_t bits) {
     constexpr int per = 32 / K;
     constexpr uint32_t seg = K == 32 ? 0xFFFFFFFFu : (1u << (K & 31)) - 1u;
     const int sh = (J % per) * K;
     const uint32_t old = atomicOr(s.act + J / per, bits << sh);
     if (((old >> sh) & seg) != 0u) return;  // listed by whoever set the tile-row's first bit
     const int32_t at = atomicAdd(&ap.n, 1);
-    if (at < kPushBuffer) ap.row[at] = J;
+    if (at < CAP) ap.row[at] = J;
     else s.list[atomicAdd(count, 1)] = J;
 }
 
-// One round.  It is a chain of dependent memory accesses (state, list, segment
-// and row pointers, tiles, weights, two atomics, list length), so the lanes
-// take one (tile, source row) pair each and issue up to kBatch relaxations
-// side by side; a lane that walked all rows of a tile paid the chain once per
-// active row and bit.  The roles of the sets follow from the previous round:
-// its near list is this round's active set; when that is empty but far
-// vertices wait, the threshold rises by delta -- or, past a gap in the
-// distances, to the least far distance plus delta, so that the nearest waiting
-// vertex always gets in -- and the whole far set is this round's active set
-// (whatever is still past the threshold moves back); when both are empty the
-// loop is done.
-template <int K>
-__global__ void __launch_bounds__(kPushThreads) push_round_kernel(const int32_t* __restrict__ rowptr,
-                                                                  const int32_t* __restrict__ colind,
-                                                                  const uint8_t* __restrict__ tiles,
-                                                                  const int32_t* __restrict__ voff,
-                                                                  const float* __restrict__ w, PushSet s0, PushSet s1,
-                                                                  PushSet s2, PushControl* ctl, int round, float* dist,
-                                                                  int buckets, float delta) {
+struct PushGraph {  // the transpose's arrays, the edge weights (w null: 1) and the distances
+    const int32_t *rowptr, *colind;
+    const uint8_t* tiles;
+    const int32_t* voff;
+    const float* w;
+    float* dist;
+    int32_t n;
+};
+
+// When the near list has run dry: the threshold rises by delta -- or, past a
+// gap in the distances, to the least far distance plus delta, so that the
+// nearest waiting vertex always gets in -- and the far set becomes the active
+// one (whatever is still past the threshold moves back).
+__device__ __forceinline__ void raise_threshold(PushState& p, float fm, float delta) {
+    const float th = p.theta;
+    float nt = fmaxf(th + delta, fm + delta);
+    if (!(nt > fm)) nt = nextafterf(fm, INFINITY);  // delta below the spacing of floats there
+    if (!(nt > th)) nt = nextafterf(th, INFINITY);
+    p.theta = nt;
+    const int32_t t = p.cur;
+    p.cur = p.far;
+    p.far = t;
+    p.epoch = (p.epoch + 1) & 3;
+}
+
+// Relaxes the out-edges of tile-row J's active vertices; called by the `width`
+// lanes of `group`, `sub` within it.  A chain of dependent memory accesses
+// (segment, row pointers and distances; tiles; weights; two atomics), so the
+// lanes take one (tile, source row) pair each and issue up to kBatch
+// relaxations side by side; a lane that walked all rows of a tile paid the
+// chain once per active row and bit.  far_seen: the least distance sent to the
+// far set.
+template <int K, int NEAR, int FAR>
+__device__ __forceinline__ void push_row(const PushGraph& g, const PushSet& cur, const PushSet& nxt, const PushSet& far,
+                                         int32_t* near_count, int32_t* far_count, Appends<NEAR>& add_near,
+                                         Appends<FAR>& add_far, float th, int buckets, int32_t J, int width,
+                                         unsigned group, int sub, float& far_seen) {
     constexpr int per = 32 / K;
     constexpr uint32_t seg = K == 32 ? 0xFFFFFFFFu : (1u << (K & 31)) - 1u;
     constexpr int kBatch = 4;
+    const int sh = (J % per) * K;
+    uint32_t amask = (__ldcg(cur.act + J / per) >> sh) & seg;
+    const int32_t t0 = __ldg(g.rowptr + J), t1 = __ldg(g.rowptr + J + 1);
+    // the sources' distances (the bitset has no bits past n)
+    float du = 0.0f;
+    if (sub < K && (int64_t)J * K + sub < g.n) du = __ldcg(g.dist + (int64_t)J * K + sub);
+    __syncwarp(group);  // every lane has read the segment
+    if (sub == 0) atomicAnd(cur.act + J / per, ~(seg << sh));
+    if (buckets) {
+        // active vertices at or past the threshold move to the far set
+        const bool late = sub < K && ((amask >> sub) & 1u) && du >= th;
+        const uint32_t defer = __ballot_sync(group, late) >> (lane_id() - sub);
+        if (late) far_seen = fminf(far_seen, du);
+        const uint32_t mine = defer & seg;
+        if (mine && sub == 0) mark_bits<K>(far, far_count, add_far, J, mine);
+        amask &= ~mine;
+    }
+    const int na = __popc(amask);
+    if (na == 0) return;
+    const int64_t pairs = (int64_t)(t1 - t0) * na;
+    int32_t ti = sub / na;
+    int ri = sub - ti * na;
+    const int32_t dt = width / na;
+    const int dr = width - dt * na;
+    for (int64_t p = 0; p < pairs; p += width) {
+        const bool live = p + sub < pairs;
+        const int r = live ? nth_bit(amask, ri) : 0;
+        const float d = __shfl_sync(group, du, r, width);
+        if (live) {
+            const int32_t t = t0 + ti;
+            int before = 0;
+            uint32_t bits = pushed_row<K>(g.tiles, t, r, g.w != nullptr, &before);
+            const int32_t I = __ldg(g.colind + t);
+            const float* wt = g.w ? g.w + __ldg(g.voff + t) + before : nullptr;
+            while (bits) {
+                int c[kBatch];
+                float cand[kBatch];
+                int old[kBatch];
+#pragma unroll
+                for (int q = 0; q < kBatch; ++q) {
+                    c[q] = -1;
+                    if (bits) {
+                        c[q] = __ffs(bits) - 1;
+                        bits &= bits - 1;
+                        cand[q] = d + (wt ? __ldg(wt + q) : 1.0f);
+                    }
+                }
+                if (wt) wt += kBatch;
+#pragma unroll
+                for (int q = 0; q < kBatch; ++q)
+                    if (c[q] >= 0)
+                        old[q] = atomicMin(reinterpret_cast<int*>(g.dist) + (int64_t)I * K + c[q],
+                                           __float_as_int(cand[q]));
+                uint32_t near_bits = 0u, far_bits = 0u;
+#pragma unroll
+                for (int q = 0; q < kBatch; ++q)
+                    if (c[q] >= 0 && cand[q] < __int_as_float(old[q])) {
+                        if (cand[q] >= th) {
+                            far_seen = fminf(far_seen, cand[q]);
+                            far_bits |= 1u << c[q];
+                        } else {
+                            near_bits |= 1u << c[q];
+                        }
+                    }
+                if (near_bits) mark_bits<K>(nxt, near_count, add_near, I, near_bits);
+                if (far_bits) mark_bits<K>(far, far_count, add_far, I, far_bits);
+            }
+        }
+        ti += dt;
+        ri += dr;
+        if (ri >= na) {
+            ri -= na;
+            ++ti;
+        }
+    }
+}
+
+// One round over the whole chip, a warp per active tile-row.  The roles of the
+// sets follow from the previous round: its near list is this round's active
+// set; when that is empty but far vertices wait, the threshold rises; when both
+// are empty the loop is done.
+template <int K>
+__global__ void __launch_bounds__(kPushThreads) push_round_kernel(PushGraph g, PushSet s0, PushSet s1, PushSet s2,
+                                                                  PushControl* ctl, int round, int buckets, float delta) {
     constexpr unsigned FULL = 0xffffffffu;
     __shared__ PushState me;
     __shared__ int32_t ncur, block_min;
-    __shared__ Appends add_near, add_far;
+    __shared__ Appends<kPushBuffer> add_near, add_far;
     if (threadIdx.x == 0) {
         PushState p = ctl->state[round & 1];
         const int32_t nn = ctl->near[(round + 3) & 3].v;
@@ -171,15 +279,7 @@ __global__ void __launch_bounds__(kPushThreads) push_round_kernel(const int32_t*
             } else if (buckets && nf > 0) {
                 len = nf;
                 moved = true;
-                const float th = p.theta;
-                float nt = fmaxf(th + delta, fm + delta);
-                if (!(nt > fm)) nt = nextafterf(fm, INFINITY);  // delta below the spacing of floats there
-                if (!(nt > th)) nt = nextafterf(th, INFINITY);
-                p.theta = nt;
-                const int32_t t = p.cur;
-                p.cur = p.far;
-                p.far = t;
-                p.epoch = (p.epoch + 1) & 3;
+                raise_threshold(p, fm, delta);
             }
             p.active = len > 0 ? 1 : 0;
             p.rounds += len > 0 ? 1 : 0;
@@ -208,84 +308,11 @@ __global__ void __launch_bounds__(kPushThreads) push_round_kernel(const int32_t*
     const float th = me.theta;
     const int lane = (int)lane_id();
     const int64_t warps = (int64_t)gridDim.x * kPushWarps;
-    float fmin_seen = INFINITY;  // least distance this lane sent to the far set
-    for (int64_t e = (int64_t)blockIdx.x * kPushWarps + (threadIdx.x >> 5); e < ncur; e += warps) {
-        const int32_t J = cur.list[e];
-        const int sh = (J % per) * K;
-        uint32_t amask = (cur.act[J / per] >> sh) & seg;
-        const int32_t t0 = __ldg(rowptr + J), t1 = __ldg(rowptr + J + 1);
-        float du = 0.0f;  // the sources' distances (the bitset has no bits past n)
-        if (lane < K && ((amask >> lane) & 1u)) du = dist[(int64_t)J * K + lane];
-        __syncwarp();  // every lane has read the segment
-        if (lane == 0) atomicAnd(cur.act + J / per, ~(seg << sh));
-        if (buckets) {
-            // active vertices at or past the threshold move to the far set
-            const bool late = lane < K && ((amask >> lane) & 1u) && du >= th;
-            const uint32_t defer = __ballot_sync(FULL, late);
-            if (late) fmin_seen = fminf(fmin_seen, du);
-            if (defer && lane == 0) mark_bits<K>(far, far_count, add_far, J, defer);
-            amask &= ~defer;
-        }
-        const int na = __popc(amask);
-        if (na == 0) continue;
-        const int64_t pairs = (int64_t)(t1 - t0) * na;
-        int32_t ti = lane / na;
-        int ri = lane - ti * na;
-        const int32_t dt = 32 / na;
-        const int dr = 32 - dt * na;
-        for (int64_t p = 0; p < pairs; p += 32) {
-            const bool live = p + lane < pairs;
-            const int r = live ? nth_bit(amask, ri) : 0;
-            const float d = __shfl_sync(FULL, du, r);
-            if (live) {
-                const int32_t t = t0 + ti;
-                int before = 0;
-                uint32_t bits = pushed_row<K>(tiles, t, r, w != nullptr, &before);
-                const int32_t I = __ldg(colind + t);
-                const float* wt = w ? w + __ldg(voff + t) + before : nullptr;
-                while (bits) {
-                    int c[kBatch];
-                    float cand[kBatch];
-                    int old[kBatch];
-#pragma unroll
-                    for (int q = 0; q < kBatch; ++q) {
-                        c[q] = -1;
-                        if (bits) {
-                            c[q] = __ffs(bits) - 1;
-                            bits &= bits - 1;
-                            cand[q] = d + (wt ? __ldg(wt + q) : 1.0f);
-                        }
-                    }
-                    if (wt) wt += kBatch;
-#pragma unroll
-                    for (int q = 0; q < kBatch; ++q)
-                        if (c[q] >= 0)
-                            old[q] = atomicMin(reinterpret_cast<int*>(dist) + (int64_t)I * K + c[q],
-                                               __float_as_int(cand[q]));
-                    uint32_t near_bits = 0u, far_bits = 0u;
-#pragma unroll
-                    for (int q = 0; q < kBatch; ++q)
-                        if (c[q] >= 0 && cand[q] < __int_as_float(old[q])) {
-                            if (cand[q] >= th) {
-                                fmin_seen = fminf(fmin_seen, cand[q]);
-                                far_bits |= 1u << c[q];
-                            } else {
-                                near_bits |= 1u << c[q];
-                            }
-                        }
-                    if (near_bits) mark_bits<K>(nxt, near_count, add_near, I, near_bits);
-                    if (far_bits) mark_bits<K>(far, far_count, add_far, I, far_bits);
-                }
-            }
-            ti += dt;
-            ri += dr;
-            if (ri >= na) {
-                ri -= na;
-                ++ti;
-            }
-        }
-    }
-    if (fmin_seen < INFINITY) atomicMin(&block_min, __float_as_int(fmin_seen));
+    float far_seen = INFINITY;
+    for (int64_t e = (int64_t)blockIdx.x * kPushWarps + (threadIdx.x >> 5); e < ncur; e += warps)
+        push_row<K>(g, cur, nxt, far, near_count, far_count, add_near, add_far, th, buckets, cur.list[e], 32, FULL, lane,
+                    far_seen);
+    if (far_seen < INFINITY) atomicMin(&block_min, __float_as_int(far_seen));
     __syncthreads();
     const int m_near = min(add_near.n, kPushBuffer), m_far = min(add_far.n, kPushBuffer);
     if (threadIdx.x == 0 && m_near > 0) add_near.base = atomicAdd(near_count, m_near);
@@ -294,6 +321,204 @@ __global__ void __launch_bounds__(kPushThreads) push_round_kernel(const int32_t*
     __syncthreads();
     for (int i = threadIdx.x; i < m_near; i += kPushThreads) nxt.list[add_near.base + i] = add_near.row[i];
     for (int i = threadIdx.x; i < m_far; i += kPushThreads) far.list[add_far.base + i] = add_far.row[i];
+}
+
+// ---------------------------------------------------------------------------
+// rounds with few active tile-rows, many to a launch
+// ---------------------------------------------------------------------------
+// A launched round takes 6 to 7 us however few rows it has: the launch, the
+// state and the lists' way through device memory on top of the relaxations' own
+// chain.  Here one thread-block cluster runs up to kClusterRounds rounds with a
+// cluster barrier between them.  A block keeps the tile-rows it marks in shared
+// memory; the next round's work is dealt over all blocks by the prefix of their
+// counts, and a row is read from the block that holds it through distributed
+// shared memory.  Far marks are buffered until the near lists run dry.  A row
+// gets 8 to 32 lanes, by how many rows there are.  Weighted grids, us a round
+// launched / here: 31 rows a round 5.9 / 4.3, 107 rows 6.6 / 4.4, 400 rows 5.8 /
+// 5.5, 770 rows 6.4 / 7.3.  So a search starts here and, once a few hundred
+// rounds averaged more than 25 rows a block, launches the others: the rows of a
+// round go up and down with every bucket, and changing to and fro cost more
+// (115 ms against 88 on a 4096 x 4096 grid) than either.
+//
+// To the launched rounds the kernel is one round: it reads and leaves the same
+// state and lists, and it leaves a round with more than `most` rows (or one
+// whose marks did not fit) to them unrun.  Every decision is made from counts
+// that no block changes before the next barrier, so all blocks take it alike.
+constexpr int kClusterThreads = 1024;
+constexpr int kClusterWarps = kClusterThreads / 32;
+constexpr int kMaxCluster = 16;
+constexpr int kClusterRounds = 128;
+constexpr int kNearBuffer = 2048;
+constexpr int kFarBuffer = 2048;
+constexpr int kClusterAverage = 25;  // rows a block and round
+
+struct ClusterShared {
+    PushState me;
+    int32_t from[kMaxCluster + 1];  // first index of each block's rows in the round's order
+    int32_t len;                    // rows of the round
+    int32_t listed;                 // they are in the set's list in device memory
+    int32_t stop;
+    int32_t block_min;
+    Appends<kNearBuffer> near[2];  // by the parity of the round that marks
+    Appends<kFarBuffer> far;
+};
+
+static cudaLaunchConfig_t cluster_config(int blocks, cudaLaunchAttribute* at, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(kClusterThreads);
+    cfg.dynamicSmemBytes = sizeof(ClusterShared);
+    cfg.stream = s;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = blocks;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+template <int K>
+__global__ void __launch_bounds__(kClusterThreads) push_cluster_kernel(PushGraph g, PushSet s0, PushSet s1, PushSet s2,
+                                                                       PushControl* ctl, int slot, int buckets,
+                                                                       float delta, int32_t most, int64_t max_rounds) {
+    extern __shared__ __align__(16) unsigned char raw[];
+    ClusterShared& sh = *reinterpret_cast<ClusterShared*>(raw);
+    cg::cluster_group cluster = cg::this_cluster();
+    const int blocks = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    const int lane = (int)lane_id(), warp = threadIdx.x >> 5;
+    int32_t* near_count = &ctl->near[slot & 3].v;
+    auto set = [&](int i) { return i == 0 ? s0 : (i == 1 ? s1 : s2); };
+    // the buffered far marks go to the far set's list; called by all threads
+    auto flush_far = [&]() {
+        __syncthreads();
+        const int m = min(sh.far.n, kFarBuffer);
+        if (threadIdx.x == 0) {
+            if (m > 0) sh.far.base = atomicAdd(&ctl->far[sh.me.epoch].v, m);
+            if (sh.block_min < __float_as_int(INFINITY)) atomicMin(&ctl->farmin[sh.me.epoch].v, sh.block_min);
+        }
+        __syncthreads();
+        const PushSet far = set(sh.me.far);
+        for (int i = threadIdx.x; i < m; i += kClusterThreads) far.list[sh.far.base + i] = sh.far.row[i];
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            sh.far.n = 0;
+            sh.block_min = __float_as_int(INFINITY);
+        }
+    };
+    const int32_t given = __ldcg(&ctl->near[(slot + 3) & 3].v);  // rows that the round before left
+    if (threadIdx.x == 0) {
+        sh.me = ctl->state[slot & 1];
+        sh.near[0].n = sh.near[1].n = sh.far.n = 0;
+        sh.block_min = __float_as_int(INFINITY);
+        sh.listed = 1;
+        sh.len = given;
+        sh.stop = sh.me.active ? 0 : 1;
+    }
+    cluster.sync();  // every block has read the state
+    int done = 0;
+    for (;; ++done) {
+        const int q = done & 1;  // near[q] holds the rows that the last round marked
+        if (done > 0 && warp == 0) {
+            const int32_t n = lane < blocks ? cluster.map_shared_rank(&sh, lane)->near[q].n : 0;
+            int32_t end = n;
+#pragma unroll
+            for (int d = 1; d < kMaxCluster; d <<= 1) {
+                const int32_t o = __shfl_up_sync(0xffffffffu, end, d);
+                if (lane >= d) end += o;
+            }
+            const bool full = __any_sync(0xffffffffu, n > kNearBuffer);
+            if (lane < blocks) sh.from[lane + 1] = end;
+            if (lane == blocks - 1) {
+                sh.from[0] = 0;
+                sh.len = end;
+                sh.listed = 0;
+                sh.stop = full ? 1 : 0;
+            }
+            if (lane == 0) sh.near[q ^ 1].n = 0;
+        }
+        __syncthreads();
+        if (sh.stop) break;
+        if (sh.len == 0) {  // near is dry
+            flush_far();
+            cluster.sync();
+            const int32_t nf = buckets ? __ldcg(&ctl->far[sh.me.epoch].v) : 0;
+            const float fm = __int_as_float(__ldcg(&ctl->farmin[sh.me.epoch].v));
+            __syncthreads();
+            if (nf > most || (nf > 0 && (done >= kClusterRounds || sh.me.rounds >= max_rounds))) {
+                if (threadIdx.x == 0) sh.len = nf;
+                break;
+            }
+            if (threadIdx.x == 0) {
+                sh.len = nf;
+                sh.listed = 1;
+                if (nf > 0) {
+                    raise_threshold(sh.me, fm, delta);
+                    if (rank == 0) {
+                        ctl->far[(sh.me.epoch + 1) & 3].v = 0;
+                        ctl->farmin[(sh.me.epoch + 1) & 3].v = __float_as_int(INFINITY);
+                    }
+                } else {
+                    sh.me.active = 0;
+                }
+            }
+            __syncthreads();
+            if (nf == 0) break;
+        } else {
+            if (sh.len > most || done >= kClusterRounds || sh.me.rounds >= max_rounds) break;
+            if (sh.far.n > kFarBuffer / 2) flush_far();
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                const int32_t t = sh.me.cur;
+                sh.me.cur = sh.me.nxt;
+                sh.me.nxt = t;
+            }
+            __syncthreads();
+        }
+        if (threadIdx.x == 0) {
+            sh.me.rounds += 1;
+            sh.me.worked += (unsigned long long)sh.len;
+        }
+        const PushSet cur = set(sh.me.cur), nxt = set(sh.me.nxt), far = set(sh.me.far);
+        const int32_t len = sh.len;
+        const int all = blocks * kClusterWarps;
+        const int width = K == 32 || len <= all ? 32 : (K == 16 || len <= 2 * all ? 16 : 8);
+        const int sub = lane & (width - 1);
+        const unsigned group = (width == 32 ? 0xffffffffu : ((1u << width) - 1u)) << (lane - sub);
+        float far_seen = INFINITY;
+        // neighbouring rows go to different blocks
+        for (int32_t e = (lane / width) * all + warp * blocks + rank; e < len; e += all * (32 / width)) {
+            int32_t J;
+            if (sh.listed) {
+                J = __ldcg(cur.list + e);
+            } else {
+                int b = 0;
+                for (int step = kMaxCluster / 2; step; step >>= 1)
+                    if (b + step < blocks && sh.from[b + step] <= e) b += step;
+                J = cluster.map_shared_rank(&sh, b)->near[q].row[e - sh.from[b]];
+            }
+            push_row<K>(g, cur, nxt, far, near_count, &ctl->far[sh.me.epoch].v, sh.near[q ^ 1], sh.far, sh.me.theta,
+                        buckets, J, width, group, sub, far_seen);
+        }
+        if (far_seen < INFINITY) atomicMin(&sh.block_min, __float_as_int(far_seen));
+        cluster.sync();  // all marks are made
+    }
+    // what is left goes to the lists in device memory
+    flush_far();
+    const int q = done & 1;
+    if (done > 0) {
+        const int m = min(sh.near[q].n, kNearBuffer);
+        if (threadIdx.x == 0 && m > 0) sh.near[q].base = atomicAdd(near_count, m);
+        __syncthreads();
+        const PushSet nxt = set(sh.me.nxt);
+        for (int i = threadIdx.x; i < m; i += kClusterThreads) nxt.list[sh.near[q].base + i] = sh.near[q].row[i];
+    }
+    if (rank == 0 && threadIdx.x == 0) {
+        sh.me.busy = sh.me.active && sh.len > most ? 1 : 0;
+        ctl->state[(slot + 1) & 1] = sh.me;
+        ctl->near[(slot + 1) & 3].v = 0;
+        if (done == 0) *near_count = given;
+    }
+    cluster.sync();  // no block reads this one's counts any more
 }
 
 // Distances, and the loop state before round 0: the source in set 0 as the
@@ -321,6 +546,30 @@ __global__ void push_init_kernel(float* dist, int32_t n, int32_t src, int k, Pus
 thread_local int64_t g_last_push_rounds = 0;
 thread_local int64_t g_last_push_rows = 0;
 
+// Blocks of the largest cluster the device runs (0: none); looked up once per
+// device.
+template <int K>
+static int push_cluster_blocks(int device) {
+    static std::atomic<int> known[64];  // blocks + 1
+    if (device < 0 || device >= 64) return 0;
+    int got = known[device].load(std::memory_order_acquire);
+    if (got) return got - 1;
+    int blocks = 0;
+    if (cudaFuncSetAttribute(push_cluster_kernel<K>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+        cudaFuncSetAttribute(push_cluster_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sizeof(ClusterShared)) == cudaSuccess) {
+        for (int want = kMaxCluster; want >= 8 && !blocks; want /= 2) {
+            cudaLaunchAttribute at[1];
+            const cudaLaunchConfig_t cfg = cluster_config(want, at, nullptr);
+            int n = 0;
+            if (cudaOccupancyMaxActiveClusters(&n, push_cluster_kernel<K>, &cfg) == cudaSuccess && n > 0) blocks = want;
+        }
+    }
+    cudaGetLastError();  // a device without room for the cluster launches every round
+    known[device].store(blocks + 1, std::memory_order_release);
+    return blocks;
+}
+
 b2sr_status sssp_push(b2sr_matrix* hT, const float* w, int32_t src, float* dist, float delta, int max_iters,
                       cudaStream_t s) {
     g_last_push_rounds = 0;
@@ -346,25 +595,49 @@ b2sr_status sssp_push(b2sr_matrix* hT, const float* w, int32_t src, float* dist,
     // with them every raise of the threshold settles at least one vertex and
     // costs a few rounds beyond the improving ones, so 4n covers both
     const int64_t cap = max_iters > 0 ? max_iters : (buckets ? 4 * (int64_t)n + 4 : (int64_t)n + 1);
-    int64_t replayed = 0;
-    const int32_t* voff = w ? hT->voff : nullptr;
+    constexpr int kBatch = 32;  // launched rounds between two looks at the state
+    const int64_t limit = ceil_div(cap + 1, kBatch) * kBatch - 1;  // the batches' rounds, one of them finding no work
+    const PushGraph g{hT->rowptr, hT->colind, hT->tiles, w ? hT->voff : nullptr, w, dist, n};
+    PushState now = {};
+    auto look = [&]() -> b2sr_status {
+        B2SR_CUDA_TRY(cudaMemcpyAsync(&now, &ctl->state[0], sizeof(now), cudaMemcpyDeviceToHost, s));
+        B2SR_CUDA_TRY(cudaStreamSynchronize(s));
+        return B2SR_OK;
+    };
     B2SR_TRY(with_tile(hT->k, [&](auto kc) -> b2sr_status {
         constexpr int K = decltype(kc)::value;
-        return run_captured(s, 32, cap + 1, &ctl->state[0].active,
-                            [&](cudaStream_t cs, int r) -> b2sr_status {
-                                push_round_kernel<K><<<grid, kPushThreads, 0, cs>>>(hT->rowptr, hT->colind, hT->tiles,
-                                                                                   voff, w, set[0], set[1], set[2], ctl,
-                                                                                   r, dist, buckets, delta);
-                                B2SR_LAUNCH_CHECK("push_round_kernel");
-                                return B2SR_OK;
-                            },
-                            &replayed);
+        int dev = -1;
+        const int blocks = cudaGetDevice(&dev) == cudaSuccess ? push_cluster_blocks<K>(dev) : 0;
+        const int32_t most = blocks * kClusterWarps * (K <= 8 ? 4 : 32 / K) * 2;  // rows it serves in two turns
+        now.active = 1;
+        for (bool few = blocks > 0; few && now.active;) {
+            const int64_t rounds = now.rounds, worked = (int64_t)now.worked;
+            cudaLaunchAttribute at[1];
+            const cudaLaunchConfig_t cfg = cluster_config(blocks, at, s);
+            for (int slot = 0; slot < 4; ++slot) {  // four: the near counters go round once
+                B2SR_CUDA_TRY(cudaLaunchKernelEx(&cfg, push_cluster_kernel<K>, g, set[0], set[1], set[2], ctl, slot,
+                                                 buckets, delta, most, limit));
+                B2SR_LAUNCH_CHECK("push_cluster_kernel");
+            }
+            B2SR_TRY(look());
+            if (now.active && now.rounds >= limit) return fail(B2SR_ERR_NOT_CONVERGED, "exceeded max_iters rounds");
+            few = !now.busy && (int64_t)now.worked - worked <= (now.rounds - rounds) * blocks * kClusterAverage;
+        }
+        if (!now.active) return B2SR_OK;
+        int64_t replayed = 0;
+        B2SR_TRY(run_captured(s, kBatch, limit + 1 - now.rounds, &ctl->state[0].active,
+                              [&](cudaStream_t cs, int r) -> b2sr_status {
+                                  push_round_kernel<K><<<grid, kPushThreads, 0, cs>>>(g, set[0], set[1], set[2], ctl, r,
+                                                                                     buckets, delta);
+                                  B2SR_LAUNCH_CHECK("push_round_kernel");
+                                  return B2SR_OK;
+                              },
+                              &replayed));
+        B2SR_TRY(look());
+        return now.rounds > limit ? fail(B2SR_ERR_NOT_CONVERGED, "exceeded max_iters rounds") : B2SR_OK;
     }));
-    PushState end;
-    B2SR_CUDA_TRY(cudaMemcpyAsync(&end, &ctl->state[0], sizeof(end), cudaMemcpyDeviceToHost, s));
-    B2SR_CUDA_TRY(cudaStreamSynchronize(s));
-    g_last_push_rounds = end.rounds;
-    g_last_push_rows = (int64_t)end.worked;
+    g_last_push_rounds = now.rounds;
+    g_last_push_rows = (int64_t)now.worked;
     return B2SR_OK;
 }
 

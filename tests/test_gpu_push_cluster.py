@@ -1,0 +1,72 @@
+"""Push SSSP where its rounds change hands: the thread-block cluster's launches
+of 128 rounds and the launched rounds it leaves a wide round or a wide search
+to.  Distances are the same as those of the SpMV SSSP, bit for bit."""
+import numpy as np
+import pytest
+import torch
+
+from tests.gpu_util import to_dev, to_np
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    from paper_2201_08560_gb300 import binding
+    return binding
+
+
+def _csr(n, u, v):
+    rows, cols = np.concatenate([u, v]), np.concatenate([v, u])
+    order = np.lexsort((cols, rows))
+    rows, cols = rows[order], cols[order]
+    return to_dev(np.searchsorted(rows, np.arange(n + 1)).astype(np.int32)), to_dev(cols.astype(np.int32)), cols.size
+
+
+def _path(n):
+    return n, np.arange(n - 1), np.arange(1, n)
+
+
+def _broom():
+    """A path, its end joined to 60000 leaves, the leaves to a second path."""
+    a, leaves = 700, np.arange(700, 60700)
+    b = 60700
+    u = np.concatenate([np.arange(a - 1), np.full(leaves.size, a - 1), leaves, np.arange(b, b + 700)])
+    v = np.concatenate([np.arange(1, a), leaves, np.full(leaves.size, b), np.arange(b + 1, b + 701)])
+    return b + 701, u, v
+
+
+def _grid(rows, cols):
+    i = np.arange(rows * cols).reshape(rows, cols)
+    return rows * cols, np.concatenate([i[:, :-1].ravel(), i[:-1].ravel()]), np.concatenate([i[:, 1:].ravel(), i[1:].ravel()])
+
+
+SHAPES = {"path": lambda: _path(1500), "broom": _broom, "grid": lambda: _grid(400, 900)}
+
+
+@pytest.mark.parametrize("delta", [0.0, 7.0, 300.0])
+@pytest.mark.parametrize("k", [4, 8, 16, 32])
+@pytest.mark.parametrize("shape", SHAPES)
+def test_same_as_spmv_sssp(B, shape, k, delta):
+    n, u, v = SHAPES[shape]()
+    rp, ci, nnz = _csr(n, u, v)
+    rows = np.repeat(np.arange(n), np.diff(to_np(rp)))
+    lo, hi = np.minimum(rows, to_np(ci)), np.maximum(rows, to_np(ci))
+    w = (1.0 + ((lo * 7919 + hi * 104729) % 997) / 32.0).astype(np.float32)  # the same both ways
+    assert w.size == nnz
+    with B.b2sr_from_csr(n, rp, ci, k) as m:
+        wb = B.b2sr_weights_from_csr(m, rp, ci, to_dev(w))
+        for weights in (wb, None):
+            want = to_np(B.b2sr_sssp(m, 3, weights)).view(np.int32)
+            got = to_np(B.b2sr_sssp_push(m, 3, weights, delta=delta)).view(np.int32)
+            np.testing.assert_array_equal(got, want)
+
+
+@pytest.mark.parametrize("k", [4, 32])
+def test_round_limit(B, k):
+    n, u, v = _path(1000)
+    rp, ci, _ = _csr(n, u, v)
+    with B.b2sr_from_csr(n, rp, ci, k) as m:
+        with pytest.raises(Exception, match="max_iters"):
+            B.b2sr_sssp_push(m, 0, max_iters=900)
+        assert to_np(B.b2sr_sssp_push(m, 0, max_iters=1024))[-1] == 999.0
