@@ -368,7 +368,7 @@ def tc_extra(B, dev, tc):
             "edges_per_s": (ci.size // 2) / (ms / 1e3), "kernel_edges_per_s": (ci.size // 2) / (kern_ms / 1e3),
             "edges_counted": "|L|, the strictly lower triangle's entries",
             "triangles": int(cnt["t"].item()), "n": int(n),
-            "roofline": {"bound": "alu", "kernel": f"masked_count_kernel (k={EXTRA_TILE})",
+            "roofline": {"bound": "alu", "kernel": f"masked_rows_kernel (k={EXTRA_TILE})",
                          "achieved": ops / 1e12, "peak": ALU_PEAK_TOPS, "unit": "T AND-popc ops/s",
                          "frac": ops / 1e12 / ALU_PEAK_TOPS, "algorithmic_ops_per_launch": pairs,
                          "peak_source": "issue bound: 3 integer instructions (LOP3, POPC, IADD) per AND-popc "
@@ -666,7 +666,7 @@ def roofline_of(fam, ms_total, peak, peak_src, tile, schedule, graph):
 
 def spmv_kernel_name(family, tile, schedule):
     """The SpMV kernel a family runs at this tile_dim and schedule (the
-    library's dispatch: at k = 4 the tile_dim-4 kernel for the bit-vector
+    library's dispatch: at k = 4 the small-tile kernel for the bit-vector
     schemes and, unless the schedule is the staged one, for the unweighted
     4-byte value schemes; the staged gather kernel for the value schemes at
     k <= 16 under the staged schedule and, under the default one, for weighted
