@@ -591,7 +591,7 @@ __global__ void __launch_bounds__(kFillThreads, 4) fill_tiles_kernel(const uint6
 // (187 us).  Merging and building takes 470 us there (300M instructions; the
 // block's barriers and the merge's dependent shared loads bound it: 48 warps
 // an SM, of which a piece of 1,100 entries keeps five in eight busy), finding
-// the pieces 90 and moving the tiles together 80.
+// the pieces 75 and moving the tiles together 80.
 constexpr int kWindow = 1024;
 constexpr int kPieceCap = 2048;
 constexpr int kSliceTarget = 1920;  // a slice is cut at a tile-column: up to k * k <= 64 entries more
@@ -639,22 +639,24 @@ __global__ void windows_kernel(const int32_t* __restrict__ rowptr, int32_t n, in
 
 // What a block needs of piece p: its window, and for a slice the position in
 // each of the k rows where it begins (the next slice's, or the rows' ends, are
-// where it ends).
+// where it ends).  A warp a piece: the cut is a search over tile-columns with a
+// search of every row inside, a chain of loads, so 32/k tile-columns are tried
+// side by side (R-MAT 20, k = 4: 74 us with one at a time, 48 so).
 __global__ void pieces_kernel(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ colind, int32_t n,
                               int32_t ntr, int k, int64_t nwin, const int32_t* __restrict__ first,
                               const int32_t* __restrict__ parts, const int64_t* __restrict__ poff, int64_t npieces, int32_t* __restrict__ window,
                               int32_t* __restrict__ cut) {
+    constexpr unsigned FULL = 0xffffffffu;
     const int lane = (int)lane_id();
-    const int q = lane & (k - 1);  // a group of k lanes a piece, lane q for row q
-    const unsigned group = ((k == 32 ? 0u : 1u << k) - 1u) << (lane - q);
-    const int64_t stride = ((int64_t)gridDim.x * blockDim.x) / k;
-    for (int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / k; p < npieces; p += stride) {
+    const int q = lane & (k - 1), g = lane / k, tries = 32 / k;  // lane q of group g: row q, g-th tile-column
+    const int64_t stride = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; p < npieces; p += stride) {
         int64_t lo = 0, hi = nwin - 1;  // the last window whose pieces begin at or before p
         while (lo < hi) {
             const int64_t mid = (lo + hi + 1) >> 1;
             if (__ldg(poff + mid) <= p) lo = mid; else hi = mid - 1;
         }
-        if (q == 0) window[p] = (int32_t)lo;
+        if (lane == 0) window[p] = (int32_t)lo;
         const int64_t slices = __ldg(parts + lo);
         const int64_t slice = p - (__ldg(poff + lo + 1) - slices);
         if (slice < 0) continue;
@@ -669,25 +671,33 @@ __global__ void pieces_kernel(const int32_t* __restrict__ rowptr, const int32_t*
             // the tile-column J with at most `target` entries before it, at most k * k short of it
             int32_t jlo = 0, jhi = ntr;
             while (jhi - jlo > 1) {
-                const int32_t mid = jlo + ((jhi - jlo) >> 1);
+                const int32_t mid = jlo + (int32_t)((int64_t)(jhi - jlo) * (g + 1) / (tries + 1));
                 int32_t a = plo, b = phi;
                 while (a < b) {
                     const int32_t m = a + ((b - a) >> 1);
                     if ((int64_t)__ldg(colind + m) < (int64_t)mid * k) a = m + 1; else b = m;
                 }
+                __syncwarp();
                 int32_t before = a - r0;
-                for (int o = 1; o < k; o <<= 1) before += __shfl_xor_sync(group, before, o);
-                if (before <= target) {
-                    jlo = mid;
-                    plo = a;
-                    if (before >= target - k * k) break;
-                } else {
-                    jhi = mid;
-                    phi = a;
+                for (int o = 1; o < k; o <<= 1) before += __shfl_xor_sync(FULL, before, o);
+                const int below = __popc(__ballot_sync(FULL, before <= target)) / k;  // groups at or before the cut
+                const int32_t a_lo = __shfl_sync(FULL, a, max(below - 1, 0) * k + q);
+                const int32_t a_hi = __shfl_sync(FULL, a, min(below, tries - 1) * k + q);
+                const int32_t j_lo = __shfl_sync(FULL, mid, max(below - 1, 0) * k);
+                const int32_t j_hi = __shfl_sync(FULL, mid, min(below, tries - 1) * k);
+                const int32_t at = __shfl_sync(FULL, before, max(below - 1, 0) * k);
+                if (below < tries) {
+                    jhi = j_hi;
+                    phi = a_hi;
+                }
+                if (below > 0) {
+                    jlo = j_lo;
+                    plo = a_lo;
+                    if (at >= target - k * k) break;
                 }
             }
         }
-        cut[p * k + q] = plo;
+        if (g == 0) cut[p * k + q] = plo;
     }
 }
 
@@ -973,7 +983,7 @@ static b2sr_status merge_pieces(int32_t n, const int32_t* rowptr, const int32_t*
     int32_t* col = reinterpret_cast<int32_t*>(tile + (size_t)nnz * tb);
     B2SR_TRY(toff.alloc((size_t)(npieces + 1) * sizeof(int64_t)));
     B2SR_TRY(dalloc(&out->rowptr, (size_t)ntr + 1, s));
-    pieces_kernel<<<grid_wide(npieces * k), 256, 0, s>>>(rowptr, colind, n, ntr, k, nwin, first, parts, poff, npieces, window,
+    pieces_kernel<<<grid_wide(npieces * 32), 256, 0, s>>>(rowptr, colind, n, ntr, k, nwin, first, parts, poff, npieces, window,
                                                         cut);
     B2SR_LAUNCH_CHECK("pieces_kernel");
     B2SR_CUDA_TRY(cudaMemsetAsync(count + npieces, 0, sizeof(int32_t), s));
