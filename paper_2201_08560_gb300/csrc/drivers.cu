@@ -120,7 +120,7 @@ b2sr_status bfs_sources(b2sr_matrix* h, const int32_t* srcs_host, int nsrc, int3
 // multi-source BFS, 64 frontiers per vertex
 // ---------------------------------------------------------------------------
 // The lane word: 64 frontiers (uint64) or, for at most 32 sources, 32 (uint32:
-// half the bytes per gather, and the SpMV takes the tile_dim-4 kernel).
+// half the bytes per gather, and the SpMV takes the k = 4 kernel for 4-byte values).
 // The frontier's live tile-columns at k = 4: a bit for every four vertices of
 // which one is in some lane's frontier, how many are set, and whether that is
 // more than half (the SpMM does not look then).
@@ -129,91 +129,138 @@ struct LiveState {
     int32_t dense;
 };
 
+// The next frontiers of four rounds, written in turn: round r reads the one
+// before (the sources' in round 0 of all) and writes set[r & 3].
+constexpr int kFrontiers = 4;
 template <class W>
-__global__ void msbfs_init_kernel(int32_t* levels, int32_t n, int nsrc, W* X, W* Y, W* vis, uint8_t* live,
-                                  int64_t live_bytes, LiveState* state, LoopFlags* flags) {
+struct Frontiers {
+    W* set[kFrontiers];
+};
+
+// Rows without tiles are written by no SpMM: they are zero from the start.
+// Unused lanes count as visited, so a vertex every source has reached is all
+// ones in the mask and the SpMM can skip its rows.
+template <class W>
+__global__ void msbfs_init_kernel(int32_t n, int nsrc, Frontiers<W> f, W* vis, uint8_t* live, int64_t live_bytes,
+                                  LiveState* state, LoopFlags* flags) {
     constexpr int BITS = 8 * (int)sizeof(W);
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (int64_t)n * nsrc || i < live_bytes;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        if (i < (int64_t)n * nsrc) levels[i] = -1;
-        // unused lanes count as visited, so a vertex every source has reached is
-        // all ones in the mask and the SpMM can skip its rows
-        if (i < n) {
-            X[i] = (W)0;
-            Y[i] = (W)0;
-            vis[i] = nsrc < BITS ? (W)~(((W)1 << nsrc) - (W)1) : (W)0;
-        }
-        if (i < live_bytes) live[i] = 0;
+    const W unused = nsrc < BITS ? (W)~(((W)1 << nsrc) - (W)1) : (W)0;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+#pragma unroll
+        for (int q = 0; q < kFrontiers; ++q) f.set[q][i] = (W)0;
+        vis[i] = unused;
+        if (i < live_bytes) live[i] = 0;  // a byte for 32 vertices, rounded up to 16
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        *flags = LoopFlags{1, 0, 0, 0u};
-        *state = LiveState{0u, 0};
+    if (blockIdx.x == 0) {
+        for (int64_t i = n + threadIdx.x; i < live_bytes; i += blockDim.x) live[i] = 0;
+        if (threadIdx.x == 0) {
+            *flags = LoopFlags{1, 0, 0, 0u};
+            *state = LiveState{0u, 0};
+        }
     }
 }
 
 template <class W>
-__global__ void msbfs_seed_kernel(SourceList srcs, int nsrc, int32_t n, int32_t* levels, W* X, W* vis,
-                                  uint32_t* live) {
+__global__ void msbfs_seed_kernel(SourceList srcs, int nsrc, W* X, W* vis, uint32_t* live) {
     int s = threadIdx.x;
     if (s < nsrc) {
         int32_t v = srcs.v[s];
-        levels[(int64_t)s * n + v] = 0;
         atomicOr(X + v, (W)1 << s);
         atomicOr(vis + v, (W)1 << s);
         atomicOr(live + (v >> 7), 1u << ((v >> 2) & 31));
     }
 }
 
-// visited |= next, and the level of every (lane, vertex) pair found.  A warp
-// takes 32 consecutive vertices and goes through the lanes that any of them
-// has, so a store writes one lane's levels of neighbouring vertices (a thread
-// that walked its own vertex's lanes wrote 32 different lines a store:
-// R-MAT 22, 64 sources: 260 us a level).  The 32 vertices' live bits, one for
-// each four, are a byte.
+// visited |= next.  A thread takes four consecutive vertices, which share a live
+// bit, so a warp's ballot is a live word.
 template <class W>
-__global__ void msbfs_update_kernel(const W* __restrict__ Y, W* __restrict__ vis, int32_t* __restrict__ levels,
-                                    int32_t n, uint8_t* __restrict__ live, LiveState* state, LoopFlags* flags) {
+__global__ void msbfs_update_kernel(const W* __restrict__ Y, W* __restrict__ vis, int32_t n, uint32_t* __restrict__ live,
+                                    LiveState* state, LoopFlags* flags) {
     if (gate_closed(&flags->active)) return;
     __shared__ uint32_t block_live;
     if (threadIdx.x == 0) block_live = 0u;
     __syncthreads();
-    const int32_t lv = *reinterpret_cast<const volatile int32_t*>(&flags->level) + 1;
-    int any = 0;
+    struct alignas(4 * sizeof(W)) Four {
+        W w[4];
+    };
     uint32_t nlive = 0;
     const int lane = (int)lane_id();
-    for (int64_t v0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) - lane; v0 < n;
-         v0 += (int64_t)gridDim.x * blockDim.x) {  // warp-uniform
-        const int64_t v = v0 + lane;
-        const W b = v < n ? Y[v] : (W)0;
-        if (b) vis[v] |= b;
-        uint32_t four = __ballot_sync(0xffffffffu, b != 0);
-        four |= four >> 1;
-        four = (four | (four >> 2)) & 0x11111111u;
-        uint32_t byte = 0u;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) byte |= ((four >> (4 * q)) & 1u) << q;
-        if (lane == 0) live[v0 >> 5] = (uint8_t)byte;
-        nlive += __popc(byte);
-#pragma unroll
-        for (int half = 0; half < (int)sizeof(W) / 4; ++half) {
-            const uint32_t mine = (uint32_t)(b >> (32 * half * (int)(sizeof(W) > 4)));
-            uint32_t lanes = __reduce_or_sync(0xffffffffu, mine);
-            any |= lanes != 0u;
-            for (; lanes; lanes &= lanes - 1u) {
-                const int s = __ffs(lanes) - 1;
-                if ((mine >> s) & 1u) levels[(int64_t)(32 * half + s) * n + v] = lv;
-            }
+    const int64_t fours = ((int64_t)n + 3) / 4;
+    for (int64_t q0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) - lane; q0 < fours;
+         q0 += (int64_t)gridDim.x * blockDim.x) {  // warp-uniform
+        const int64_t q = q0 + lane;
+        Four b = {};
+        if (q < fours) {  // the arrays are padded to whole fours; past n nothing is set
+            b = reinterpret_cast<const Four*>(Y)[q];
+            if (4 * q + 4 > n)
+                for (int i = 0; i < 4; ++i)
+                    if (4 * q + i >= n) b.w[i] = (W)0;
         }
+        const bool some = (b.w[0] | b.w[1] | b.w[2] | b.w[3]) != 0;
+        if (some) {
+            Four o = reinterpret_cast<const Four*>(vis)[q];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) o.w[i] |= b.w[i];
+            reinterpret_cast<Four*>(vis)[q] = o;
+        }
+        const uint32_t word = __ballot_sync(0xffffffffu, some);
+        if (lane == 0) live[q0 >> 5] = word;
+        nlive += __popc(word);
     }
     if (lane == 0 && nlive) atomicAdd(&block_live, nlive);
     __syncthreads();
     if (threadIdx.x == 0 && block_live) atomicAdd(&state->count, block_live);
-    if (finish_round(flags, any)) {
+    if (finish_round(flags, nlive != 0u)) {
         const uint32_t total = atomicExch(&state->count, 0u);
         state->dense = 8 * (int64_t)total > n ? 1 : 0;
     }
 }
 
+// The levels of what the last four rounds (fewer in a search's last batch)
+// found.  After the first four every level is written, -1 where nothing was
+// found, and the sources' 0; later ones only where a round found something, a
+// warp going through the lanes that any of its 32 vertices has.  The levels are
+// most of a search's output (R-MAT 22, 64 sources: 1.07 GB): filled with -1
+// first and written round by round they took 242 us and 113 us a round; here
+// the two launches of such a search take 284 us and a round's update 20.
+template <class W>
+__global__ void msbfs_levels_kernel(Frontiers<W> f, const W* __restrict__ vis, int32_t* __restrict__ levels, int32_t n,
+                                    int nsrc, const LoopFlags* flags) {
+    const int done = flags->level;
+    const int base = (done - 1) & ~(kFrontiers - 1), run = done - base;
+    const int lane = (int)lane_id();
+    for (int64_t v0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) - lane; v0 < n;
+         v0 += (int64_t)gridDim.x * blockDim.x) {  // warp-uniform
+        const int64_t v = v0 + lane;
+        W b[kFrontiers];
+#pragma unroll
+        for (int q = 0; q < kFrontiers; ++q) b[q] = v < n && q < run ? f.set[q][v] : (W)0;
+        const W found = b[0] | b[1] | b[2] | b[3], one = b[1] | b[3], two = b[2] | b[3];
+        const W seen = base == 0 && v < n ? vis[v] : found;
+#pragma unroll
+        for (int half = 0; half < (int)sizeof(W) / 4; ++half) {
+            const int sh = 32 * half * (int)(sizeof(W) > 4);
+            const uint32_t hs = (uint32_t)(seen >> sh), hf = (uint32_t)(found >> sh), h1 = (uint32_t)(one >> sh),
+                           h2 = (uint32_t)(two >> sh);
+            int32_t* out = levels + (int64_t)sh * n + v;
+            if (base == 0) {
+                const int lanes = min(32, nsrc - sh);
+                if (v < n)
+#pragma unroll 8
+                    for (int s = 0; s < lanes; ++s)
+                        out[(int64_t)s * n] = (int32_t)((hs >> s) & 1u) + (int32_t)((hf >> s) & 1u) +
+                                              (int32_t)((h1 >> s) & 1u) + 2 * (int32_t)((h2 >> s) & 1u) - 1;
+            } else {
+                for (uint32_t lanes = __reduce_or_sync(0xffffffffu, hf); lanes; lanes &= lanes - 1u) {
+                    const int s = __ffs(lanes) - 1;
+                    if ((hf >> s) & 1u)
+                        out[(int64_t)s * n] =
+                            base + 1 + (int32_t)((h1 >> s) & 1u) + 2 * (int32_t)((h2 >> s) & 1u);
+                }
+            }
+        }
+    }
+}
 
 static b2sr_status spmm_lanes(b2sr_matrix* h, const unsigned long long* X, unsigned long long* Y,
                               const unsigned long long* M, cudaStream_t s, const int32_t* gate, bool edges,
@@ -233,31 +280,35 @@ static b2sr_status bfs_multi_lanes(b2sr_matrix* h, const int32_t* srcs_host, int
     DevBuf buf(s);
     const size_t vb = round_up((size_t)n * sizeof(W), 256);
     const size_t lb = round_up(ceil_div(n, 32), 16);
-    B2SR_TRY(buf.alloc(3 * vb + lb + sizeof(LoopFlags) + sizeof(LiveState)));
-    W* X = buf.as<W>();
-    W* Yb = reinterpret_cast<W*>(buf.as<char>() + vb);
-    W* vis = reinterpret_cast<W*>(buf.as<char>() + 2 * vb);
-    uint8_t* live = reinterpret_cast<uint8_t*>(buf.as<char>() + 3 * vb);
+    B2SR_TRY(buf.alloc((kFrontiers + 1) * vb + lb + sizeof(LoopFlags) + sizeof(LiveState)));
+    Frontiers<W> f;
+    for (int q = 0; q < kFrontiers; ++q) f.set[q] = reinterpret_cast<W*>(buf.as<char>() + q * vb);
+    W* vis = reinterpret_cast<W*>(buf.as<char>() + kFrontiers * vb);
+    uint8_t* live = reinterpret_cast<uint8_t*>(buf.as<char>() + (kFrontiers + 1) * vb);
     LoopFlags* flags = reinterpret_cast<LoopFlags*>(live + lb);
     LiveState* state = reinterpret_cast<LiveState*>(flags + 1);
     const LiveColumns columns{reinterpret_cast<const uint32_t*>(live), &state->dense};
-    msbfs_init_kernel<W><<<grid_for(std::max<int64_t>((int64_t)n * nsrc, lb)), 256, 0, s>>>(
-        levels, n, nsrc, X, Yb, vis, live, (int64_t)lb, state, flags);
+    W* sources = f.set[kFrontiers - 1];
+    msbfs_init_kernel<W><<<grid_for(n), 256, 0, s>>>(n, nsrc, f, vis, live, (int64_t)lb, state, flags);
     B2SR_LAUNCH_CHECK("msbfs_init_kernel");
-    msbfs_seed_kernel<W><<<1, 64, 0, s>>>(source_list(srcs_host, nsrc), nsrc, n, levels, X, vis,
+    msbfs_seed_kernel<W><<<1, 64, 0, s>>>(source_list(srcs_host, nsrc), nsrc, sources, vis,
                                           reinterpret_cast<uint32_t*>(live));
     B2SR_LAUNCH_CHECK("msbfs_seed_kernel");
     const int64_t cap = max_iters > 0 ? max_iters : (int64_t)n + 1;
     int64_t rounds = 0;
-    return run_captured(s, 4, cap + 1, &flags->active,
+    return run_captured(s, kFrontiers, cap + 1, &flags->active,
                         [&](cudaStream_t cs, int r) -> b2sr_status {
-                            W* cur = (r & 1) ? Yb : X;
-                            W* nxt = (r & 1) ? X : Yb;
-                            // rows without tiles are zero in Yb from the start, and in X (which may
-                            // have sources there) once a round has written it
-                            B2SR_TRY(spmm_lanes(h, cur, nxt, vis, cs, &flags->active, r == 1, columns));
-                            msbfs_update_kernel<W><<<grid_for(n), 256, 0, cs>>>(nxt, vis, levels, n, live, state, flags);
+                            W* nxt = f.set[r];
+                            // rows without tiles are zero in every set from the start, but for the
+                            // last's, which may have sources there until a round has written it
+                            B2SR_TRY(spmm_lanes(h, f.set[(r + kFrontiers - 1) % kFrontiers], nxt, vis, cs,
+                                                &flags->active, r == kFrontiers - 1, columns));
+                            msbfs_update_kernel<W><<<grid_for(ceil_div(n, 4), 4), 256, 0, cs>>>(
+                                nxt, vis, n, reinterpret_cast<uint32_t*>(live), state, flags);
                             B2SR_LAUNCH_CHECK("msbfs_update_kernel");
+                            if (r < kFrontiers - 1) return B2SR_OK;
+                            msbfs_levels_kernel<W><<<grid_for(n), 256, 0, cs>>>(f, vis, levels, n, nsrc, flags);
+                            B2SR_LAUNCH_CHECK("msbfs_levels_kernel");
                             return B2SR_OK;
                         },
                         &rounds);
