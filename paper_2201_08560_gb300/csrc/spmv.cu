@@ -1088,6 +1088,7 @@ struct SmallTiles {
     static constexpr int TW = ChunkShape<K>::TW;
     int32_t ra, rb;
     int32_t win;
+    bool dead;  // every row is masked out
     uint32_t w[8 * TW], cu[8];
 };
 
@@ -1111,7 +1112,8 @@ __device__ __forceinline__ void small_load(const SpmvGeom& g, const SEM& sem, in
     const int64_t c0 = (int64_t)c * chunk_tiles(K);
     const uint32_t* tiles = reinterpret_cast<const uint32_t*>(g.tiles);
     // the arrays are padded to whole chunks, so every lane's bytes exist
-    if (sem.saturated((int64_t)ra * K, ((int64_t)rb + 1) * K)) {
+    t.dead = sem.saturated((int64_t)ra * K, ((int64_t)rb + 1) * K);
+    if (t.dead) {
 #pragma unroll
         for (int i = 0; i < 8 * TW; ++i) t.w[i] = 0u;
 #pragma unroll
@@ -1276,11 +1278,31 @@ __device__ __forceinline__ void join_lanes(const SEM& sem, Acc& acc, int lane) {
     }
 }
 
+// A chunk (not the last) without a contribution, of a lane-word scheme: zeros
+// for the rows that end here and began here or are empty, which are neighbours,
+// and for the chunk's shares of the rows that it cuts.  Such chunks are most of
+// the first and the last levels of a batched BFS, whose walks found nothing to
+// add: the SpMMs of a search, with 16 sources on R-MAT 20, 967 to 858 us, with
+// 64 on R-MAT 22, 4,571 to 3,949 (811 and 3,755 with a loop for each case in
+// small_body).
+template <class SEM>
+__device__ __forceinline__ void zero_chunk(const SpmvGeom& g, const SEM& sem, Partials<typename SEM::V> part, int32_t c,
+                                           int32_t cs, int lane, int32_t ra, int32_t rb, int32_t start) {
+    using V = typename SEM::V;
+    constexpr int K = SEM::NV;
+    if (lane < K) {
+        part.val_first[(int64_t)c * K + lane] = V(0);
+        part.val_last[(int64_t)c * K + lane] = V(0);
+    }
+    const int64_t end = min((int64_t)rb * K, (int64_t)sem.n);  // row rb goes on after the chunk or begins there
+    for (int64_t i = ((int64_t)ra + (start == cs ? 0 : 1)) * K + lane; i < end; i += 32) sem.y[i] = V(0);
+}
+
 // One chunk from its loaded tile stream.
 template <int K, class SEM, int MODE>
 __device__ __forceinline__ void small_chunk(const SpmvGeom& g, const SEM& sem, Partials<typename SEM::V> part,
                                             int32_t c, int lane, const SmallTiles<K>& t, ChunkRows& s,
-                                            const uint8_t* sx, typename SEM::V* first, bool filter) {
+                                            const uint8_t* sx, typename SEM::V* first) {
     using Sh = ChunkShape<K>;
     using V = typename SEM::V;
     constexpr int NV = SEM::NV;
@@ -1288,6 +1310,23 @@ __device__ __forceinline__ void small_chunk(const SpmvGeom& g, const SEM& sem, P
     static_assert(Sh::P == 8 && TW <= 2, "eight tiles of one or two words a lane");
     const int32_t cs = c * Sh::CT;
     const int32_t ce = min(cs + Sh::CT, (int32_t)g.T);
+    uint32_t on = 0xFFu;  // kSmSegsLive: the lane's tiles under which a segment is not all zero
+    if constexpr (LaneWords<SEM>::value) {
+        bool dead = t.dead;
+        if constexpr (MODE == kSmSegsLive) {
+            if (!dead) {
+                on = 0u;
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    on |= ((reinterpret_cast<const uint32_t*>(sx)[t.cu[i] >> 5] >> (t.cu[i] & 31)) & 1u) << i;
+                dead = !__any_sync(0xffffffffu, on != 0u);
+            }
+        }
+        if (dead && c + 1 < g.nchunks) {
+            zero_chunk(g, sem, part, c, cs, lane, t.ra, t.rb, __shfl_sync(0xffffffffu, t.win, 0));
+            return;
+        }
+    }
     RegAcc<V, NV> acc, idv;
     // the values of the lane's first tile-row: in shared memory where they are wide
     typename std::conditional<sizeof(V) == 16, SmemAcc<V, NV>, RegAcc<V, NV>>::type F;
@@ -1343,19 +1382,11 @@ __device__ __forceinline__ void small_chunk(const SpmvGeom& g, const SEM& sem, P
                 G x[GRP][4];
                 bool any = true;  // warp-uniform: some lane's segments are not all zero
                 if constexpr (MODE == kSmSegsLive) {
-                    bool on[GRP];
-                    bool mine = false;
-#pragma unroll
-                    for (int i = 0; i < GRP; ++i) {
-                        const uint32_t J = t.cu[i0 + i];
-                        on[i] = !filter || ((reinterpret_cast<const uint32_t*>(sx)[J >> 5] >> (J & 31)) & 1u);
-                        mine |= on[i];
-                    }
-                    any = __any_sync(0xffffffffu, mine);
+                    any = __any_sync(0xffffffffu, ((on >> i0) & ((1u << GRP) - 1u)) != 0u);
                     if (any) {
 #pragma unroll
                         for (int i = 0; i < GRP; ++i) {
-                            if (on[i]) {
+                            if ((on >> (i0 + i)) & 1u) {
                                 load_seg<G, MODE>(sem.src(), t.cu[i0 + i], t.w[i0 + i], x[i]);
                             } else {
 #pragma unroll
@@ -1483,7 +1514,7 @@ __device__ __forceinline__ void small_body(const SpmvGeom& g, const SEM& sem, Pa
         // one chunk at a time: more warps hide its loads better than the
         // registers of a second chunk would (R-MAT 20: 225 and 270 us)
         for (;;) {
-            small_chunk<K, SEM, MODE>(g, sem, part, c, lane, cur, *rows, sx, first, filter);
+            small_chunk<K, SEM, MODE>(g, sem, part, c, lane, cur, *rows, sx, first);
             c += W;
             if (c >= g.nchunks) return;
             small_load<K>(g, sem, c, lane, na, nb, cur);
@@ -1493,18 +1524,26 @@ __device__ __forceinline__ void small_body(const SpmvGeom& g, const SEM& sem, Pa
             }
         }
     }
-    for (;;) {
-        const int32_t cn = c + W;
-        const bool more = cn < g.nchunks;
-        if (more) small_load<K>(g, sem, cn, lane, na, nb, nxt);
-        if (cn + W < g.nchunks) {
-            na = __ldg(g.chunk_row + cn + W);
-            nb = __ldg(g.chunk_row + cn + W + 1);
+    auto loop = [&](auto mode) {
+        for (;;) {
+            const int32_t cn = c + W;
+            const bool more = cn < g.nchunks;
+            if (more) small_load<K>(g, sem, cn, lane, na, nb, nxt);
+            if (cn + W < g.nchunks) {
+                na = __ldg(g.chunk_row + cn + W);
+                nb = __ldg(g.chunk_row + cn + W + 1);
+            }
+            small_chunk<K, SEM, decltype(mode)::value>(g, sem, part, c, lane, cur, *rows, sx, first);
+            if (!more) break;
+            c = cn;
+            cur = nxt;
         }
-        small_chunk<K, SEM, MODE>(g, sem, part, c, lane, cur, *rows, sx, first, filter);
-        if (!more) break;
-        c = cn;
-        cur = nxt;
+    };
+    if constexpr (MODE == kSmSegsLive) {  // a loop for each, so that the dense levels pay for no test
+        if (filter) loop(std::integral_constant<int, kSmSegsLive>());
+        else loop(std::integral_constant<int, kSmSegs>());
+    } else {
+        loop(std::integral_constant<int, MODE>());
     }
 }
 
@@ -2273,10 +2312,11 @@ static b2sr_status launch_direct(const b2sr_matrix* h, const SEM& sem, Partials<
                 if (8 * h->nnz > 9 * h->T) return launch_small<K, SEM, kSmVals>(h, sem, part, s, g);
                 return launch_small<K, SEM, kSmEach>(h, sem, part, s, g);
             } else {
-                // A batched BFS's frontier: zero segments are not loaded.  R-MAT 20, 16
-                // sources, us a level: the first 99, the last three 94 to 102, the dense
-                // ones between 134 to 154 (about 130 all with every segment loaded);
-                // R-MAT 22, 64 sources: 415, 390 to 450, and 660 to 800.
+                // A batched BFS's frontier: zero segments are not loaded, and chunks
+                // without a live one not walked.  R-MAT 20, 16 sources, us a level: the
+                // first 66, the dense ones 131 to 164, the last four 53 to 93 (about 130
+                // all with every segment loaded); R-MAT 22, 64 sources: 283, 703 to 865,
+                // 233 to 354.
                 if constexpr (LaneWords<SEM>::value) {
                     constexpr int threads = small_threads<K, SEM, kSmSegsLive>();
                     if (sem.live && h->n % 4 == 0 && reinterpret_cast<uintptr_t>(sem.x) % (4 * sizeof(G)) == 0 &&
