@@ -471,7 +471,10 @@ static b2sr_status count_rows(int32_t n, RowLists a, RowLists b, RowLists m, int
     const int use_bitmap = words * 4 <= kMaxBitmapBytes;
     const int smem = use_bitmap ? (int)round_up(words, 4) * 4 : 0;
     const int64_t runs = ceil_div(slots, kRunEntries);
-    B2SR_CUDA_TRY(cudaFuncSetAttribute(masked_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    // the largest bitmap, not this call's: the limit belongs to the kernel, and
+    // another thread's call with a smaller graph must not lower it before a launch
+    B2SR_CUDA_TRY(cudaFuncSetAttribute(masked_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)kMaxBitmapBytes));
     const bool split = slots >= kSplitEntries;
     void* tok = timing_begin(s);
     // m.begin[n] (the row pointer of a CSR) ends the slots
