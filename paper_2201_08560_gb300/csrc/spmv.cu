@@ -2280,8 +2280,13 @@ static b2sr_status launch_small(const b2sr_matrix* h, const SEM& sem, Partials<t
     void (*kernel)(SpmvGeom, SEM, Partials<typename SEM::V>);
     if constexpr (K == 4 && sizeof(typename SEM::V) == 4) kernel = spmv_k4_kernel<SEM, MODE>;
     else kernel = spmv_chunks_kernel<K, SEM, MODE>;
-    if (smem > 48 * 1024)
-        B2SR_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    // A size that goes with the graph is allowed up to the most a block can have,
+    // not up to this call's: the limit belongs to the kernel, and another thread's
+    // call with a smaller graph must not lower it before a launch.
+    constexpr bool sized = MODE == kSmBitsShared || MODE == kSmSegsLive;
+    if (sized || smem > 48 * 1024)
+        B2SR_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           sized ? (int)kMaxBlockSmem : smem));
     kernel<<<grid, threads, smem, s>>>(g, sem, part);
     B2SR_LAUNCH_CHECK("small-tile SpMV kernel");
     return B2SR_OK;

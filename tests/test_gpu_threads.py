@@ -59,3 +59,47 @@ def test_triangle_counts_of_two_sizes(B):
     assert [int(c.item()) for c in counts] == [0, 0]
     for m in mats:
         m.close()
+
+
+def _random(n, m, seed):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(seed)
+    u, v = torch.randint(0, n, (2, m), generator=gen, device="cuda")
+    return _csr(n, u, v)
+
+
+@pytest.mark.parametrize("k", [4, 8])
+def test_boolean_and_count_spmv_of_two_sizes(B, k):
+    """Inputs of 1.4 M and of 0.3 M bits, each copied to a block's shared memory."""
+    sizes = [(1_400_000, 4_500_000), (300_000, 4_500_000)]
+    mats = [B.b2sr_from_csr(n, *_random(n, m, 5), k) for n, m in sizes]
+    bodies, got, want = [], [], []
+    for m, (n, _) in zip(mats, sizes):
+        x = torch.randint(-2**31, 2**31 - 1, (B.bitset_words(n),), device="cuda").to(torch.int32)
+        for out, size in ((B.VEC_BITS, B.bitset_words(n)), (B.VEC_I32, n)):
+            sr = B.BOOL_OR_AND if out == B.VEC_BITS else B.PLUS_TIMES
+            want.append(B.b2sr_spmv(m, sr, B.VEC_BITS, x, out, torch.empty(size, dtype=torch.int32, device="cuda")))
+            got.append(torch.full((size,), -1, dtype=torch.int32, device="cuda"))
+            bodies.append(lambda m=m, sr=sr, x=x, out=out, y=got[-1]: B.b2sr_spmv(m, sr, B.VEC_BITS, x, out, y))
+    torch.cuda.synchronize()
+    errors = _side_by_side(bodies, 300)
+    assert not errors, errors[0]
+    for g, w in zip(got, want):
+        assert torch.equal(g, w)
+    for m in mats:
+        m.close()
+
+
+def test_batched_bfs_of_two_sizes(B):
+    """Live columns of 2^20 and of 2^18 groups of four vertices."""
+    sizes = [(1 << 22, 24_000_000), (1 << 20, 24_000_000)]
+    mats = [B.b2sr_from_csr(n, *_random(n, m, 6), 4) for n, m in sizes]
+    want = [B.b2sr_bfs_multi(m, [1, 2, 3]) for m in mats]
+    got = [torch.full_like(w, -2) for w in want]
+    torch.cuda.synchronize()
+    errors = _side_by_side([lambda m=m, g=g: B.b2sr_bfs_multi(m, [1, 2, 3], g) for m, g in zip(mats, got)], 20)
+    assert not errors, errors[0]
+    for g, w in zip(got, want):
+        assert torch.equal(g, w)
+    for m in mats:
+        m.close()
