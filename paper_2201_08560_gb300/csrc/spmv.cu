@@ -141,7 +141,8 @@ struct CSum {
     float s, c;
     CSum() = default;
     __device__ __forceinline__ CSum(float a) : s(a), c(0.0f) {}
-    __device__ __forceinline__ explicit operator float() const { return __fadd_rn(s, c); }
+    // an infinite or NaN sum has no rounding error: its c is NaN
+    __device__ __forceinline__ explicit operator float() const { return isfinite(s) ? __fadd_rn(s, c) : s; }
 };
 
 __device__ __forceinline__ CSum csum_add(CSum a, CSum b) {
@@ -1613,7 +1614,7 @@ __device__ __forceinline__ typename SEM::V rowlane_join(const SEM& sem, typename
 }
 
 // A lane's running value of its row.  fp32 sums are compensated, as a lane's
-// chain is as long as its tile-row (an infinite sum has no rounding error).
+// chain is as long as its tile-row.
 template <class SEM, class J>
 struct RowLaneAcc {
     typename SEM::V a;
@@ -1627,13 +1628,12 @@ __device__ __forceinline__ void csum_push(CSum& a, float v) {
     a.c = __fadd_rn(a.c, __fadd_rn(__fsub_rn(a.s, __fsub_rn(t, bp)), __fsub_rn(v, bp)));
     a.s = t;
 }
-__device__ __forceinline__ float csum_value(CSum a) { return isfinite(a.s) ? (float)a : a.s; }
 template <class SEM>
 struct RowLaneAcc<SEM, CSum> {
     CSum a;
     __device__ __forceinline__ void clear(const SEM&) { a = CSum(0.0f); }
     __device__ __forceinline__ void add(const SEM&, float v) { csum_push(a, v); }
-    __device__ __forceinline__ float value() const { return csum_value(a); }
+    __device__ __forceinline__ float value() const { return (float)a; }
 };
 template <class SEM>
 struct RowLaneAcc<SEM, CSum4> {
@@ -1645,9 +1645,7 @@ struct RowLaneAcc<SEM, CSum4> {
         csum_push(a.v[2], v.z);
         csum_push(a.v[3], v.w);
     }
-    __device__ __forceinline__ float4 value() const {
-        return make_float4(csum_value(a.v[0]), csum_value(a.v[1]), csum_value(a.v[2]), csum_value(a.v[3]));
-    }
+    __device__ __forceinline__ float4 value() const { return (float4)a; }
 };
 
 template <int K, class SEM>
