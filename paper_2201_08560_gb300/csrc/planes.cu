@@ -272,7 +272,7 @@ __device__ __forceinline__ A warp_sum(A v) {
 template <bool BITS>
 __device__ __forceinline__ void store_y(void* y, int64_t i, typename PlaneRows<4, BITS>::Acc v, bool kept) {
     if constexpr (BITS) static_cast<long long*>(y)[i] = kept ? v : 0ll;
-    else static_cast<float*>(y)[i] = kept ? __fadd_rn(v.s, v.c) : 0.0f;
+    else static_cast<float*>(y)[i] = kept ? (isfinite(v.s) ? __fadd_rn(v.s, v.c) : v.s) : 0.0f;  // c is NaN beside an infinite s
 }
 
 // a warp per tile-row of at most kLongRow tiles

@@ -64,3 +64,15 @@ def test_plus_times(B, graph, k, schedule):
         B.b2sr_spmm_f32x4(m, to_dev(X4), Y4)
         for c in range(4):
             np.testing.assert_array_equal(to_np(Y4)[:, c], _expect(graph, X4[:, c]))
+
+
+@pytest.mark.parametrize("k", [4, 8, 16, 32])
+def test_bit_plane_weights(B, graph, k):
+    rp, ci = csr_dev(graph)
+    w = np.random.default_rng(k).integers(1, 8, graph.nnz)
+    with B.b2sr_from_csr(N, rp, ci, k) as m:
+        planes = B.b2sr_planes_from_csr(m, rp, ci, to_dev(w.astype(np.uint32)), 3)
+        for x in _inputs():
+            y = torch.full((N,), -1.0, device="cuda")
+            B.b2sr_spmv_planes(m, planes, 3, B.VEC_F32, to_dev(x), B.VEC_F32, y)
+            np.testing.assert_array_equal(to_np(y), _expect(graph, x, w))
