@@ -596,7 +596,7 @@ b2sr_status sssp_push(b2sr_matrix* hT, const float* w, int32_t src, float* dist,
     // costs a few rounds beyond the improving ones, so 4n covers both
     const int64_t cap = max_iters > 0 ? max_iters : (buckets ? 4 * (int64_t)n + 4 : (int64_t)n + 1);
     constexpr int kBatch = 32;  // launched rounds between two looks at the state
-    const int64_t limit = ceil_div(cap + 1, kBatch) * kBatch - 1;  // the batches' rounds, one of them finding no work
+    const int64_t limit = ceil_div(cap + 1, kBatch) * kBatch;  // rounds with work: whole batches
     const PushGraph g{hT->rowptr, hT->colind, hT->tiles, w ? hT->voff : nullptr, w, dist, n};
     PushState now = {};
     auto look = [&]() -> b2sr_status {

@@ -70,3 +70,24 @@ def test_round_limit(B, k):
         with pytest.raises(Exception, match="max_iters"):
             B.b2sr_sssp_push(m, 0, max_iters=900)
         assert to_np(B.b2sr_sssp_push(m, 0, max_iters=1024))[-1] == 999.0
+
+
+def _layers(layers, width):
+    """Paths side by side, all begun by the last vertex."""
+    n = layers * width + 1
+    i = np.arange((layers - 1) * width)
+    return n, np.concatenate([i, np.full(width, n - 1)]), np.concatenate([i + width, np.arange(width)])
+
+
+@pytest.mark.parametrize("shape,k", [("path", 4), ("path", 32), ("layers", 4)])
+def test_last_allowed_round(B, shape, k):
+    """A limit of 32 m - 1 allows 32 m rounds with work, in the cluster (the
+    path) and in launched rounds (500 tile-rows a round)."""
+    (n, u, v), src, rounds = (_path(1024), 0, 1024) if shape == "path" else (_layers(639, 2000), 639 * 2000, 640)
+    rp, ci, _ = _csr(n, u, v)
+    with B.b2sr_from_csr(n, rp, ci, k) as m:
+        far = to_np(B.b2sr_sssp_push(m, src, max_iters=rounds - 1)).max()
+        assert far == rounds - 1
+        assert B.b2sr_sssp_push_rounds() == rounds
+        with pytest.raises(Exception, match="max_iters"):
+            B.b2sr_sssp_push(m, src, max_iters=rounds - 33)
