@@ -576,10 +576,11 @@ __global__ void __launch_bounds__(kFillThreads, 4) fill_tiles_kernel(const uint6
 // ---------------------------------------------------------------------------
 // A piece is at most kPieceCap entries of whole tile-rows, or of one long
 // tile-row's range of tile-columns.  The CSR entries are cut into windows of
-// kWindow; a window's pieces are the tile-rows that begin in it, and if the
-// last of those is longer than kWindow (a long tile-row; its end lies past the
-// window, so it is the last), its slices of about kSliceTarget entries.  A
-// block loads a piece, merges the k rows of each of its tile-rows pairwise in
+// kWindow; a window's pieces are the tile-rows that begin in it, at most
+// kPieceRows to a piece (a stretch of empty rows is shared by many blocks), and
+// if the last of those is longer than kWindow (a long tile-row; its end lies
+// past the window, so it is the last), its slices of about kSliceTarget entries.
+// A block loads a piece, merges the k rows of each of its tile-rows pairwise in
 // shared memory (log2 k levels; a thread finds where its eight outputs begin
 // in the two runs by a binary search along their diagonal and merges from
 // there), counts the run heads, and builds the tiles and their column indices
@@ -594,6 +595,7 @@ __global__ void __launch_bounds__(kFillThreads, 4) fill_tiles_kernel(const uint6
 // the pieces 75 and moving the tiles together 80.
 constexpr int kWindow = 1024;
 constexpr int kPieceCap = 2048;
+constexpr int kPieceRows = 1024;
 constexpr int kSliceTarget = 1920;  // a slice is cut at a tile-column: up to k * k <= 64 entries more
 constexpr int kPieceThreads = 256;
 constexpr int kPieceItems = kPieceCap / kPieceThreads;
@@ -633,7 +635,8 @@ __global__ void windows_kernel(const int32_t* __restrict__ rowptr, int32_t n, in
         }
         first[b] = f;
         slices[b] = parts;
-        cnt[b] = parts + (g - (parts > 0 ? 1 : 0) > f ? 1 : 0);
+        const int32_t rows = g - (parts > 0 ? 1 : 0) - f;
+        cnt[b] = parts + (rows > 0 ? (rows + kPieceRows - 1) / kPieceRows : 0);
     }
 }
 
@@ -725,8 +728,9 @@ __global__ void __launch_bounds__(kPieceThreads, K == 4 ? 6 : 5) merge_piece_ker
     const int32_t slices = __ldg(parts + b);
     const int64_t p0 = __ldg(poff + b + 1) - slices;  // the first slice
     const bool slice = p >= p0;
-    const int32_t I0 = slice ? __ldg(first + b + 1) - 1 : __ldg(first + b);
-    const int32_t I1 = slice ? I0 + 1 : __ldg(first + b + 1) - (slices > 0 ? 1 : 0);
+    const int32_t I0 = slice ? __ldg(first + b + 1) - 1
+                             : __ldg(first + b) + (int32_t)(p - __ldg(poff + b)) * kPieceRows;
+    const int32_t I1 = slice ? I0 + 1 : min(I0 + kPieceRows, __ldg(first + b + 1) - (slices > 0 ? 1 : 0));
     const int64_t row0 = (int64_t)I0 * K;
     const int32_t nrows = (int32_t)(min((int64_t)I1 * K, (int64_t)n) - row0);
     int32_t e0, cnt;
@@ -931,8 +935,9 @@ __global__ void __launch_bounds__(kPieceThreads) gather_pieces_kernel(
     const int64_t cnt = __ldg(toff + p + 1) - t0, from = __ldg(place + p);
     const int32_t f1 = __ldg(first + b + 1);
     if (p < p0) {
-        for (int32_t I = __ldg(first + b) + threadIdx.x; I < f1 - (slices > 0 ? 1 : 0); I += kPieceThreads)
-            rowptr[I] += (int32_t)t0;
+        const int32_t I0 = __ldg(first + b) + (int32_t)(p - __ldg(poff + b)) * kPieceRows;
+        const int32_t I1 = min(I0 + kPieceRows, f1 - (slices > 0 ? 1 : 0));
+        for (int32_t I = I0 + threadIdx.x; I < I1; I += kPieceThreads) rowptr[I] += (int32_t)t0;
     } else if (p == p0 && threadIdx.x == 0) {
         rowptr[f1 - 1] += (int32_t)t0;
     }
