@@ -21,7 +21,8 @@
 #include "b2sr_internal.cuh"
 
 namespace b2sr {
-b2sr_status row_counts(const b2sr_matrix* h, int32_t* cnt, int32_t* first, int32_t* last, cudaStream_t s);
+b2sr_status row_counts(const b2sr_matrix* h, int32_t* cnt, int32_t* first, int32_t* last, bool chunks_done,
+                       cudaStream_t s);
 
 // ---------------------------------------------------------------------------
 // input validation
@@ -1286,14 +1287,13 @@ b2sr_status ensure_outdeg(b2sr_matrix* h, cudaStream_t s) {
 // ---------------------------------------------------------------------------
 // B2SR -> CSR
 // ---------------------------------------------------------------------------
-// Ones per row come from the row-count SpMV (spmv.cu), which also leaves the
-// partial counts of the tile-rows that cross chunks; a scan makes them row
-// pointers.  The columns are then written by a warp per chunk of tiles, 32
-// tiles a step: an entry's place is its row's pointer, plus the row's ones in
-// earlier chunks (the partials), plus those in earlier steps (a carry), plus
-// those in earlier tiles of the step (a scan over the lanes that restarts at
-// every tile-row).  The work is balanced over tiles, so a hub's row of 10^5
-// tiles is shared by many warps (a thread a row walked it alone).
+// Ones per row come from the row-count SpMV (spmv.cu) or csr_rows_kernel, which also leaves the partial counts of the tile-rows that
+// cross chunks; a scan makes them row pointers.  The columns are then written by
+// a warp per chunk of tiles, so a hub's row of 10^5 tiles is shared by many
+// warps.  An entry's place is its row's pointer, plus the row's ones in earlier
+// chunks (the partials), plus those in earlier tiles of the chunk.  At k = 4 and
+// 8 (and 16) a lane takes a tile, 32 tiles a step, and those are a carry from
+// earlier steps and a scan over the lanes that restarts at every tile-row.
 template <int K>
 __global__ void __launch_bounds__(256) csr_fill_kernel(const int32_t* __restrict__ trp,
                                                        const int32_t* __restrict__ tci,
@@ -1377,6 +1377,125 @@ __global__ void __launch_bounds__(256) csr_fill_kernel(const int32_t* __restrict
     }
 }
 
+// k = 16 and 32: the lanes are the rows of a tile (two tiles a step at k = 16),
+// so that the ones in earlier tiles are a running count in a register; a lane a
+// tile scanned k counters a step over the lanes instead (16.6 M tiles of one
+// entry, k = 32: 3.97 ms a call, 1.72 so; a thread a row 2.07).  FILL: writes the
+// columns, of full tiles 32 neighbours at a time; else: counts the ones of the
+// rows that begin and end in the chunk, and the partials of the others.
+template <int K, bool FILL>
+__global__ void __launch_bounds__(256) csr_rows_kernel(const int32_t* __restrict__ trp,
+                                                       const int32_t* __restrict__ tci,
+                                                       const uint8_t* __restrict__ tiles, int32_t n, int64_t T,
+                                                       int64_t nchunks, const int32_t* __restrict__ chunk_row,
+                                                       const int64_t* __restrict__ off, int32_t* __restrict__ cnt,
+                                                       int32_t* __restrict__ first, int32_t* __restrict__ last,
+                                                       int32_t* __restrict__ colind) {
+    constexpr unsigned FULL = 0xffffffffu;
+    constexpr int CT = chunk_tiles(K);
+    constexpr int SUBS = 32 / K;  // tiles a step
+    constexpr int STEPS = 8;      // whose words are in flight together
+    static_assert(K == 16 || K == 32, "one or two tiles a step");
+    const int lane = (int)lane_id(), r = lane % K, sub = lane / K;
+    const int64_t c = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (c >= nchunks) return;  // whole warps leave together
+    const int32_t cs = (int32_t)(c * CT), ce = (int32_t)min((int64_t)cs + CT, T);
+    const int32_t ra = __ldg(chunk_row + c), rb = __ldg(chunk_row + c + 1);
+    const int32_t rs = __ldg(trp + ra);
+    const bool head = rs >= cs;  // tile-row ra begins with this chunk
+    // FILL: the rows of a tile that this warp writes (the grid's y shares them out)
+    const int row0 = (int)blockIdx.y * K / (int)gridDim.y, row1 = ((int)blockIdx.y + 1) * K / (int)gridDim.y;
+    int32_t acc = 0;             // ones of lane's row so far
+    int64_t at = 0;              // or the place of its next entry
+    if constexpr (FILL) {
+        int32_t v = 0;  // ones of the row in earlier chunks, every SUBS-th a lane
+        const int64_t ca = rs / CT;
+        if (!head)
+            for (int64_t q = ca + sub; q < c; q += SUBS) v += __ldg((q == ca ? last : first) + q * K + r);
+        if constexpr (SUBS == 2) v += __shfl_xor_sync(FULL, v, 16);
+        at = __ldg(off + min((int64_t)ra * K + r, (int64_t)n)) + v;
+    }
+    int32_t before = ra;  // tile-row of the tile before the step's
+    bool open = true;     // the last tile's row goes on in the next chunk
+    for (int32_t g0 = cs; g0 < ce; g0 += 32) {
+        const int32_t t = g0 + lane;
+        int32_t lo = ra, hi = rb;  // the tile's row: the last one starting at or before t
+        while (lo < hi) {
+            const int32_t mid = lo + ((hi - lo + 1) >> 1);
+            if (__ldg(trp + mid) <= t) lo = mid; else hi = mid - 1;
+        }
+        const int32_t I = lo;
+        int32_t Ip = __shfl_up_sync(FULL, I, 1);
+        if (lane == 0) Ip = before;
+        before = __shfl_sync(FULL, I, 31);
+        // FILL: tiles whose row is not that of the tile before; else: the last of their rows
+        const uint32_t marks = __ballot_sync(FULL, t < ce && (FILL ? I != Ip : __ldg(trp + I + 1) == t + 1));
+        int32_t j0 = 0;
+        if constexpr (FILL) j0 = t < ce ? __ldg(tci + t) * K : 0;
+        if (g0 + 32 >= ce) open = !((marks >> (ce - 1 - g0)) & 1u);
+#pragma unroll 1
+        for (int u0 = 0; u0 < min(32, ce - g0); u0 += SUBS * STEPS) {
+            uint32_t b[STEPS];
+            int64_t start[STEPS];
+#pragma unroll
+            for (int q = 0; q < STEPS; ++q) {
+                const int u = u0 + q * SUBS + sub;
+                b[q] = g0 + u < ce ? tile_word<K>(tiles, g0 + u, r) : 0u;
+                start[q] = 0;
+                if constexpr (FILL) {
+                    const int32_t Iu = __shfl_sync(FULL, I, u);
+                    if ((marks >> u) & 1u) start[q] = __ldg(off + min((int64_t)Iu * K + r, (int64_t)n));
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < STEPS; ++q) {
+                const int ua = u0 + q * SUBS;
+                if constexpr (FILL) {
+                    int64_t p = at;
+                    if constexpr (SUBS == 1) {
+                        if ((marks >> ua) & 1u) p = start[q];
+                        at = p + __popc(b[q]);
+                    } else {  // both halves follow both tiles
+                        const int mine = __popc(b[q]), theirs = __shfl_xor_sync(FULL, mine, 16);
+                        const int64_t other = __shfl_xor_sync(FULL, start[q], 16);
+                        const int64_t pa = (marks >> ua) & 1u ? (sub ? other : start[q]) : at;
+                        const int64_t pb = (marks >> (ua + 1)) & 1u ? (sub ? start[q] : other) : pa + (sub ? theirs : mine);
+                        p = sub ? pb : pa;
+                        at = pb + (sub ? mine : theirs);
+                    }
+                    const int32_t j = __shfl_sync(FULL, j0, ua + sub);
+                    if (__any_sync(FULL, __popc(b[q]) > 8)) {  // row by row, a lane a column
+                        for (int i = row0; i < row1; ++i) {
+                            const int from = sub * K + i;
+                            const uint32_t w = __shfl_sync(FULL, b[q], from);
+                            const int64_t pw = __shfl_sync(FULL, p, from);
+                            if ((w >> r) & 1u) colind[pw + __popc(w & ((1u << r) - 1u))] = j + r;
+                        }
+                    } else {
+                        for (uint32_t w = r >= row0 && r < row1 ? b[q] : 0u; w; w &= w - 1)
+                            colind[p++] = j + __ffs(w) - 1;
+                    }
+                } else {
+                    const int mine = __popc(b[q]), theirs = SUBS == 2 ? __shfl_xor_sync(FULL, mine, 16) : 0;
+#pragma unroll
+                    for (int h = 0; h < SUBS; ++h) {
+                        acc += sub == h ? mine : theirs;
+                        const int32_t Iu = __shfl_sync(FULL, I, ua + h);
+                        if ((marks >> (ua + h)) & 1u) {  // the row ends
+                            if (sub == 0) {
+                                if (Iu == ra && !head) first[c * K + r] = acc;
+                                else if ((int64_t)Iu * K + r < n) cnt[(int64_t)Iu * K + r] = acc;
+                            }
+                            acc = 0;
+                        }
+                    }
+                }
+            }
+        }
+    }
+    if (!FILL && open && sub == 0) (ra == rb && !head ? first : last)[c * K + r] = acc;
+}
+
 __global__ void rowptr_out_kernel(const int64_t* __restrict__ off, int64_t len, int32_t* __restrict__ rowptr) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < len; i += (int64_t)gridDim.x * blockDim.x)
         rowptr[i] = (int32_t)off[i];
@@ -1390,19 +1509,35 @@ b2sr_status extract_csr(const b2sr_matrix* h, int64_t* off, int32_t* rowptr, int
     B2SR_TRY(part.alloc(std::max<size_t>(2 * np, 1) * sizeof(int32_t)));
     int32_t* first = part.as<int32_t>();
     int32_t* last = first + np;
-    B2SR_CUDA_TRY(cudaMemsetAsync(cnt.as<int32_t>() + n, 0, sizeof(int32_t), s));
-    B2SR_TRY(row_counts(h, cnt.as<int32_t>(), first, last, s));
+    B2SR_CUDA_TRY(cudaMemsetAsync(cnt.p, 0, ((size_t)n + 1) * sizeof(int32_t), s));  // rows without tiles stay 0
+    // a kernel over the chunks' rows at k = 32, and at k = 16 where tiles hold more
+    // than a few entries or hardly a tile-row has one.  us, rows / tiles: 1 bit a
+    // tile 1078 / 903, 2.2 529 / 438, 9.8 104 / 104, 43 150 / 156, 171 195 / 297,
+    // 256 151 / 227; 2,000 entries in 2^26 rows 563 / 26,784.
+    auto wide_rows = [&](auto fill, const int64_t* row_start) -> b2sr_status {
+        constexpr bool FILL = decltype(fill)::value;
+        auto kernel = h->k == 16 ? csr_rows_kernel<16, FILL> : csr_rows_kernel<32, FILL>;
+        // few chunks of full tiles (64 full tiles are 65,536 entries) are shared by four warps each
+        const unsigned share = FILL && h->nchunks <= (int64_t)sm_count() * 2 ? 4 : 1;
+        kernel<<<dim3((unsigned)ceil_div(h->nchunks, 8), share), 256, 0, s>>>(h->rowptr, h->colind, h->tiles, n, h->T, h->nchunks,
+                                                                h->chunk_row, row_start, cnt.as<int32_t>(), first, last,
+                                                                colind);
+        B2SR_LAUNCH_CHECK("csr_rows_kernel");
+        return B2SR_OK;
+    };
+    const bool wide = h->nchunks > 0 && (h->k == 32 || (h->k == 16 && (h->nnz > 8 * h->T || h->ntr > 32 * h->T)));
+    if (wide) B2SR_TRY(wide_rows(std::false_type(), nullptr));
+    B2SR_TRY(row_counts(h, cnt.as<int32_t>(), first, last, wide, s));
     B2SR_TRY(exclusive_scan_i32_to_i64(cnt.as<int32_t>(), off, (int64_t)n + 1, s));
     rowptr_out_kernel<<<grid_wide((int64_t)n + 1), 256, 0, s>>>(off, (int64_t)n + 1, rowptr);
     B2SR_LAUNCH_CHECK("rowptr_out_kernel");
     if (!colind || h->nchunks == 0) return B2SR_OK;
-    return with_tile(h->k, [&](auto kc) -> b2sr_status {
-        constexpr int K = decltype(kc)::value;
-        csr_fill_kernel<K><<<(unsigned)ceil_div(h->nchunks, 8), 256, 0, s>>>(
-            h->rowptr, h->colind, h->tiles, h->T, h->nchunks, h->chunk_row, off, first, last, colind);
-        B2SR_LAUNCH_CHECK("csr_fill_kernel");
-        return B2SR_OK;
-    });
+    if (wide) return wide_rows(std::true_type(), off);
+    auto kernel = h->k == 4 ? csr_fill_kernel<4> : (h->k == 8 ? csr_fill_kernel<8> : csr_fill_kernel<16>);
+    kernel<<<(unsigned)ceil_div(h->nchunks, 8), 256, 0, s>>>(h->rowptr, h->colind, h->tiles, h->T, h->nchunks,
+                                                            h->chunk_row, off, first, last, colind);
+    B2SR_LAUNCH_CHECK("csr_fill_kernel");
+    return B2SR_OK;
 }
 
 // ---------------------------------------------------------------------------
