@@ -21,6 +21,7 @@
 namespace b2sr {
 b2sr_status masked_count(const b2sr_matrix* A, const b2sr_matrix* B, const b2sr_matrix* M, int64_t* count,
                          cudaStream_t s, int64_t* pairs);
+bool counts_by_rows(const b2sr_matrix* h);
 b2sr_status lower_count(const b2sr_matrix* h, int64_t* count, cudaStream_t s);
 
 // ---------------------------------------------------------------------------
@@ -562,8 +563,7 @@ extern "C" b2sr_status b2sr_tc(b2sr_handle h, int64_t* count, void* stream) {
     clear_error();
     B2SR_TRY(check_handle(h));
     if (!count) return fail(B2SR_ERR_INVALID_ARG, "count is NULL");
-    // rows of 2^31 entries or more keep the tile form over the lower triangle
-    if (h->nnz < (int64_t(1) << 31) - 1024) return lower_count(h, count, to_stream(stream));
+    if (counts_by_rows(h)) return lower_count(h, count, to_stream(stream));
     b2sr_handle L = nullptr;
     B2SR_TRY(b2sr_lower(h, stream, &L));
     b2sr_status st = masked_count(L, L, L, count, to_stream(stream), nullptr);

@@ -161,15 +161,29 @@ __global__ void masked_count_kernel(MatView A, MatView B, MatView M, unsigned lo
 //     walk the entry's other row, testing each column in the bitmap: a
 //     coalesced load and one shared load per column, no searches;
 //   * a shorter row stays a list: eight lanes a mask entry search its columns
-//     in the entry's other row.
-// Where a bitmap of n bits does not fit in shared memory every row takes the
-// second form, the longer ones with a warp an entry.
+//     in the entry's other row;
+//   * a long row whose entries in the run have few columns to test for the
+//     row's length, and an entry whose other row is many times longer, are
+//     searched: a warp an entry walks the shorter row and looks its columns up
+//     in the longer one.
+// Where a bitmap of n bits does not fit in shared memory every long row is
+// searched, in one launch; where it leaves an SM few blocks, rows of up to
+// kApartRow columns are.
 constexpr int kRunEntries = 256;
 constexpr int64_t kMaxBitmapBytes = 200 * 1024;
 // Fewer mask entries than this take one launch: grouping the others by column
 // (five launches and a scan, 60 us) costs more than the shorter walks save
 // (R-MAT 16, 1.8M entries, half of them below the diagonal: about as much).
 constexpr int64_t kSplitEntries = 1 << 21;
+// Up to this size a run's bitmaps are made where its lists are; larger ones
+// leave few blocks on an SM, so a second launch makes them, for the runs that
+// have rows for them, and the lists go first without.
+constexpr int kOneLaunchBitmap = 32 * 1024;
+constexpr int32_t kApartRow = 512;
+// A looked-up column costs a chain of loads where a tested one costs one, and a
+// bitmap costs two passes over its row.
+constexpr int kSearchLonger = 8;  // an entry is searched if its other row is longer by this factor
+constexpr int kSearchFewer = 4;   // a row is if it has this many columns for each one to test
 
 // Row i: colind[begin[i] .. end[i]) (end = begin + 1 for a plain CSR).  Rows
 // lie one after another, with gaps where end[i] < begin[i + 1].
@@ -227,98 +241,127 @@ __global__ void place_by_column_kernel(const int32_t* __restrict__ row_of, const
     }
 }
 
+// What a launch does of its runs: all; all but the rows that take bitmaps, and
+// lists the runs that have some; those rows, of the listed runs.
+enum { kRunsWhole, kRunsLists, kRunsBitmaps };
+
+template <int PART>
 __global__ void __launch_bounds__(256) masked_rows_kernel(int32_t n, RowLists A, RowLists B, RowLists M,
-                                                          const int32_t* mnnz, int longer, int use_bitmap,
-                                                          int bitmap_words, unsigned long long* __restrict__ out) {
+                                                          const int32_t* __restrict__ mnnz, int longer, int32_t bitmap_from,
+                                                          int bitmap_words, int32_t* __restrict__ pending,
+                                                          unsigned long long* __restrict__ out) {
     extern __shared__ __align__(16) uint32_t bitmap[];
     __shared__ unsigned long long warp_sum[8];
     // the run's entries: where row i of A begins, row j of B as a range (compact:
     // six blocks an SM beside bitmaps of 2^18 bits)
-    __shared__ int32_t row_a[kRunEntries];
+    __shared__ int32_t row_a[kRunEntries];      // at a long row's first entry: columns to test for the row
     __shared__ int2 row_b[kRunEntries];
-    __shared__ int32_t long_row[kRunEntries];  // rows taken as bitmaps; without bitmaps, row i's length
-    __shared__ uint8_t short_len[kRunEntries];  // row i's length, up to 32
-    __shared__ uint8_t listed[kRunEntries];    // entries of rows with up to 32 columns
-    __shared__ uint8_t other[kRunEntries];     // entries of one long row; without bitmaps, of all
-    __shared__ int nlong, nlisted, nother[2];
+    __shared__ int32_t long_row[kRunEntries];   // rows with more than bitmap_from columns
+    __shared__ uint8_t short_len[kRunEntries];  // row i's length, up to 32; of a longer row: 1 where the entry is searched
+    __shared__ uint8_t listed[kRunEntries];     // entries of rows with up to 32 columns; from the back, searched entries
+    __shared__ uint8_t other[kRunEntries];      // entries of one long row
+    __shared__ int nlong, nlisted, nsearched, nother;
     __shared__ int32_t row_range[2];
     const int lane = (int)lane_id(), warp = threadIdx.x >> 5;
-    const int32_t e0 = (int32_t)blockIdx.x * kRunEntries;
-    const int32_t e1 = min(e0 + kRunEntries, __ldg(mnnz));
-    if (e0 >= e1) return;
-    // the last row starting at or before entry e, between lo and hi
-    auto row_at = [&](int32_t e, int32_t lo, int32_t hi) {
-        while (lo < hi) {
-            const int32_t mid = lo + ((hi - lo + 1) >> 1);
-            if (__ldg(M.begin + mid) <= e) lo = mid; else hi = mid - 1;
-        }
-        return lo;
-    };
-    if (warp < 2) {  // rows of the first and the last entry of the run
-        const int32_t i = row_at(warp == 0 ? e0 : e1 - 1, 0, n - 1);
-        if (lane == 0) row_range[warp] = i;
-    }
-    if (use_bitmap) {
+    const int32_t nruns = PART == kRunsBitmaps ? __ldg(pending) : (int32_t)gridDim.x;  // pending[0]: how many are listed
+    unsigned long long sum = 0;
+    if (PART != kRunsLists) {
         const uint4 zero = make_uint4(0u, 0u, 0u, 0u);  // the bitmap is padded to whole 16 bytes
         for (int w = threadIdx.x; w < (bitmap_words + 3) / 4; w += 256) reinterpret_cast<uint4*>(bitmap)[w] = zero;
     }
-    if (threadIdx.x == 0) nlong = nlisted = nother[0] = 0;
-    __syncthreads();
-    const int32_t i0 = row_range[0], i1 = row_range[1];
-    if (i0 == i1 && __ldg(M.end + i0) <= e0) return;  // the run lies in a gap
-    {
-        const int t = threadIdx.x;
-        const int32_t e = e0 + t;
-        int2 rb = make_int2(0, 0);
-        if (e < e1) {
-            const int32_t i = row_at(e, i0, i1);
-            if (e < __ldg(M.end + i)) {
-                const int32_t j = __ldg(M.colind + e);
-                const int32_t a0 = __ldg(A.begin + i), d = __ldg(A.end + i) - a0;
-                rb = make_int2(__ldg(B.begin + j), __ldg(B.end + j));
-                if (use_bitmap && d > 32 && (t == 0 || e == __ldg(M.begin + i))) long_row[atomicAdd(&nlong, 1)] = i;
-                if (d <= 0 || rb.y <= rb.x || (longer && rb.y - rb.x > d)) {
-                    rb.y = rb.x;  // nothing to count here
-                } else if (d <= 32) {
-                    row_a[t] = a0;
-                    short_len[t] = (uint8_t)d;
-                    listed[atomicAdd(&nlisted, 1)] = (uint8_t)t;
-                } else if (!use_bitmap) {
-                    row_a[t] = a0;
-                    long_row[t] = d;
-                    other[atomicAdd(&nother[0], 1)] = (uint8_t)t;
+    for (int32_t run = blockIdx.x; run < nruns; run += gridDim.x) {
+        const int32_t e0 = (PART == kRunsBitmaps ? __ldg(pending + 1 + run) : run) * kRunEntries;
+        const int32_t e1 = min(e0 + kRunEntries, __ldg(mnnz));
+        if (e0 >= e1) continue;  // the same for every thread
+        // the last row starting at or before entry e, between lo and hi
+        auto row_at = [&](int32_t e, int32_t lo, int32_t hi) {
+            while (lo < hi) {
+                const int32_t mid = lo + ((hi - lo + 1) >> 1);
+                if (__ldg(M.begin + mid) <= e) lo = mid; else hi = mid - 1;
+            }
+            return lo;
+        };
+        if (PART == kRunsBitmaps) __syncthreads();  // the run before is done with
+        if (warp < 2) {  // rows of the first and the last entry of the run
+            const int32_t i = row_at(warp == 0 ? e0 : e1 - 1, 0, n - 1);
+            if (lane == 0) row_range[warp] = i;
+        }
+        if (threadIdx.x == 0) nlong = nlisted = nsearched = nother = 0;
+        row_a[threadIdx.x] = 0;
+        __syncthreads();
+        const int32_t i0 = row_range[0], i1 = row_range[1];
+        if (i0 == i1 && __ldg(M.end + i0) <= e0) continue;  // the run lies in a gap
+        {
+            const int t = threadIdx.x;
+            const int32_t e = e0 + t;
+            int2 rb = make_int2(0, 0);
+            if (e < e1) {
+                const int32_t i = row_at(e, i0, i1);
+                if (e < __ldg(M.end + i)) {
+                    const int32_t j = __ldg(M.colind + e);
+                    const int32_t a0 = __ldg(A.begin + i), d = __ldg(A.end + i) - a0;
+                    rb = make_int2(__ldg(B.begin + j), __ldg(B.end + j));
+                    if (d > bitmap_from && (t == 0 || e == __ldg(M.begin + i))) long_row[atomicAdd(&nlong, 1)] = i;
+                    const int32_t len = rb.y - rb.x;
+                    if (d <= 0 || len <= 0 || (longer && len > d)) {
+                        rb.y = rb.x;  // nothing to count here
+                    } else if (d <= 32) {
+                        row_a[t] = a0;
+                        short_len[t] = (uint8_t)d;
+                        listed[atomicAdd(&nlisted, 1)] = (uint8_t)t;
+                    } else if (d <= bitmap_from || len / kSearchLonger > d) {
+                        short_len[t] = 1;
+                        listed[kRunEntries - 1 - atomicAdd(&nsearched, 1)] = (uint8_t)t;
+                    } else {
+                        short_len[t] = 0;
+                        atomicAdd(row_a + max(__ldg(M.begin + i) - e0, 0), min(len, 1 << 22));
+                    }
                 }
             }
+            row_b[t] = rb;
         }
-        row_b[t] = rb;
-    }
-    __syncthreads();
-    uint32_t acc = 0;
-    for (int q = threadIdx.x >> 3; q < nlisted; q += 32) {
-        const int t = listed[q];
-        acc += count_listed<8>(A.colind + row_a[t], short_len[t], B.colind, row_b[t].x, row_b[t].y, lane & 7);
-    }
-    if (!use_bitmap) {
-        for (int q = warp; q < nother[0]; q += 8) {
-            const int t = other[q];
-            acc += count_listed<32>(A.colind + row_a[t], long_row[t], B.colind, row_b[t].x, row_b[t].y, lane);
+        __syncthreads();
+        uint32_t acc = 0;
+        // the columns that row i of A, [a0, a1), and row [b.x, b.y) of B share, by a warp
+        auto search = [&](int32_t a0, int32_t a1, int2 b) {
+            return b.y - b.x <= a1 - a0 ? count_listed<32>(B.colind + b.x, b.y - b.x, A.colind, a0, a1, lane)
+                                        : count_listed<32>(A.colind + a0, a1 - a0, B.colind, b.x, b.y, lane);
+        };
+        if (PART != kRunsBitmaps) {
+            for (int q = threadIdx.x >> 3; q < nlisted; q += 32) {
+                const int t = listed[q];
+                acc += count_listed<8>(A.colind + row_a[t], short_len[t], B.colind, row_b[t].x, row_b[t].y, lane & 7);
+            }
+            for (int q = warp; q < nsearched; q += 8) {
+                const int t = listed[kRunEntries - 1 - q];
+                const int32_t i = row_at(e0 + t, i0, i1);
+                acc += search(__ldg(A.begin + i), __ldg(A.end + i), row_b[t]);
+            }
         }
-    } else {
+        int bitmaps = 0;
         for (int r = 0; r < nlong; ++r) {
             const int32_t i = long_row[r];
             const int32_t a0 = __ldg(A.begin + i), a1 = __ldg(A.end + i);
             const int32_t m0 = max(e0, __ldg(M.begin + i)), m1 = min(e1, __ldg(M.end + i));
+            const int32_t tests = row_a[m0 - e0];
+            if (tests < (a1 - a0) / kSearchFewer) {  // the same for every thread
+                if (PART != kRunsBitmaps)
+                    for (int t = m0 - e0 + warp; t < m1 - e0; t += 8)
+                        if (row_b[t].y > row_b[t].x && !short_len[t]) acc += search(a0, a1, row_b[t]);
+                continue;
+            }
+            ++bitmaps;
+            if (PART == kRunsLists) continue;
             if (threadIdx.x < m1 - m0) {
                 const int t = m0 - e0 + threadIdx.x;
-                if (row_b[t].y > row_b[t].x) other[atomicAdd(&nother[r & 1], 1)] = (uint8_t)t;
+                if (row_b[t].y > row_b[t].x && !short_len[t]) other[atomicAdd(&nother, 1)] = (uint8_t)t;
             }
             for (int32_t p = a0 + threadIdx.x; p < a1; p += 256) {
                 const int32_t v = __ldg(A.colind + p);
                 atomicOr(bitmap + (v >> 5), 1u << (v & 31));
             }
-            if (threadIdx.x == 0) nother[(r + 1) & 1] = 0;
             __syncthreads();
-            const int todo = nother[r & 1];
+            const int todo = nother;
             // the next entry's first columns are loaded before this one's are used
             auto test = [&](int32_t v) { return (bitmap[v >> 5] >> (v & 31)) & 1u; };
             int2 o = warp < todo ? row_b[other[warp]] : make_int2(0, 0);
@@ -334,10 +377,12 @@ __global__ void __launch_bounds__(256) masked_rows_kernel(int32_t n, RowLists A,
             }
             __syncthreads();
             for (int32_t p = a0 + threadIdx.x; p < a1; p += 256) bitmap[__ldg(A.colind + p) >> 5] = 0u;
+            if (threadIdx.x == 0) nother = 0;
             __syncthreads();
         }
+        if (PART == kRunsLists && bitmaps > 0 && threadIdx.x == 0) pending[1 + atomicAdd(pending, 1)] = run;
+        sum += acc;
     }
-    unsigned long long sum = acc;
     for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
     if (lane == 0) warp_sum[warp] = sum;
     __syncthreads();
@@ -450,6 +495,15 @@ __global__ void build_rowptr_from_rows(const int32_t* __restrict__ tilerow, int6
 
 static MatView view(const b2sr_matrix* h) { return MatView{h->rowptr, h->colind, h->tiles, h->T, h->ntr}; }
 
+// Tiles a quarter full or more: the tile form counts such a mask faster than the
+// row form, whose work goes with the entries; at k = 32 where bitmaps leave an SM
+// few blocks.  us, tiles / rows, triangles of 64-vertex cliques, n = 2^20: k = 4
+// 1,798 / 12,817, k = 8 1,461 / 12,951, k = 16 2,327 / 12,724, k = 32 4,783 /
+// 6,948; of 256-vertex cliques, n = 2^15: k = 8 365 / 722, k = 32 1,432 / 777.
+static bool full_tiles(const b2sr_matrix* h, int64_t nnz, int64_t T) {
+    return (h->k <= 16 || ceil_div(h->n, 32) * 4 > kOneLaunchBitmap) && 4 * nnz >= (int64_t)h->k * h->k * T;
+}
+
 // Row lists of a handle, owned by `buf`.
 static b2sr_status row_lists(const b2sr_matrix* h, DevBuf& buf, RowLists* out, cudaStream_t s) {
     DevBuf off(s);
@@ -468,18 +522,40 @@ static b2sr_status row_lists(const b2sr_matrix* h, DevBuf& buf, RowLists* out, c
 static b2sr_status count_rows(int32_t n, RowLists a, RowLists b, RowLists m, int64_t slots, unsigned long long* out,
                               cudaStream_t s, double bytes) {
     const int64_t words = ceil_div(n, 32);
-    const int use_bitmap = words * 4 <= kMaxBitmapBytes;
+    const bool use_bitmap = words * 4 <= kMaxBitmapBytes;
     const int smem = use_bitmap ? (int)round_up(words, 4) * 4 : 0;
     const int64_t runs = ceil_div(slots, kRunEntries);
+    const bool split = use_bitmap && slots >= kSplitEntries;
+    const bool apart = use_bitmap && smem > kOneLaunchBitmap;
+    const int32_t bitmap_from = !use_bitmap ? INT32_MAX : (apart ? kApartRow : 32);
+    DevBuf listed(s);
+    if (apart) B2SR_TRY(listed.alloc((size_t)(runs + 1) * sizeof(int32_t)));
     // the largest bitmap, not this call's: the limit belongs to the kernel, and
     // another thread's call with a smaller graph must not lower it before a launch
-    B2SR_CUDA_TRY(cudaFuncSetAttribute(masked_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)kMaxBitmapBytes));
-    const bool split = slots >= kSplitEntries;
+    for (auto kernel : {masked_rows_kernel<kRunsWhole>, masked_rows_kernel<kRunsBitmaps>})
+        B2SR_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxBitmapBytes));
+    // the entries of mask mm, the rows of x against those of y; mm.begin[n] (the row
+    // pointer of a CSR) ends the slots
+    auto count_runs = [&](RowLists x, RowLists y, RowLists mm, int longer) -> b2sr_status {
+        if (!apart) {
+            masked_rows_kernel<kRunsWhole><<<(unsigned)runs, 256, smem, s>>>(n, x, y, mm, mm.begin + n, longer, bitmap_from,
+                                                                            use_bitmap ? (int)words : 0, nullptr, out);
+            B2SR_LAUNCH_CHECK("masked_rows_kernel");
+            return B2SR_OK;
+        }
+        int32_t* pending = listed.as<int32_t>();
+        B2SR_CUDA_TRY(cudaMemsetAsync(pending, 0, sizeof(int32_t), s));
+        masked_rows_kernel<kRunsLists><<<(unsigned)runs, 256, 0, s>>>(n, x, y, mm, mm.begin + n, longer, bitmap_from,
+                                                                     (int)words, pending, out);
+        B2SR_LAUNCH_CHECK("masked_rows_kernel");
+        const int64_t resident = (int64_t)sm_count() * std::max<int64_t>(1, kMaxBitmapBytes / smem);
+        masked_rows_kernel<kRunsBitmaps><<<(unsigned)std::min<int64_t>(runs, resident), 256, smem, s>>>(
+            n, x, y, mm, mm.begin + n, longer, bitmap_from, (int)words, pending, out);
+        B2SR_LAUNCH_CHECK("masked_rows_kernel");
+        return B2SR_OK;
+    };
     void* tok = timing_begin(s);
-    // m.begin[n] (the row pointer of a CSR) ends the slots
-    masked_rows_kernel<<<(unsigned)runs, 256, smem, s>>>(n, a, b, m, m.begin + n, split, use_bitmap, (int)words, out);
-    B2SR_LAUNCH_CHECK("masked_rows_kernel");
+    B2SR_TRY(count_runs(a, b, m, split));
     if (split) {
         DevBuf cnt(s), off(s), cur(s), rows(s);
         B2SR_TRY(cnt.alloc(((size_t)n + 1) * sizeof(int32_t)));
@@ -499,8 +575,7 @@ static b2sr_status count_rows(int32_t n, RowLists a, RowLists b, RowLists m, int
                                                                rows.as<int32_t>());
         B2SR_LAUNCH_CHECK("place_by_column_kernel");
         const RowLists mt{colptr, colptr + 1, rows.as<int32_t>()};
-        masked_rows_kernel<<<(unsigned)runs, 256, smem, s>>>(n, b, a, mt, colptr + n, 0, use_bitmap, (int)words, out);
-        B2SR_LAUNCH_CHECK("masked_rows_kernel");
+        B2SR_TRY(count_runs(b, a, mt, 0));
     }
     timing_end(tok, "spgemm_masked", bytes, s);
     return B2SR_OK;
@@ -523,6 +598,12 @@ __global__ void lower_ends_kernel(const int32_t* __restrict__ rowptr, const int3
         end[i] = lower_bound_i32(colind, rowptr[i], rowptr[i + 1], (int32_t)i);
 }
 
+// Whether lower_count is the form for the triangles of h: rows of 2^31 entries
+// or more and full tiles keep the tile form over the lower triangle.
+bool counts_by_rows(const b2sr_matrix* h) {
+    return h->nnz < (int64_t(1) << 31) - 1024 && !full_tiles(h, h->nnz, h->T);
+}
+
 // Triangles: L the strictly lower triangle of h, sum over its entries (i, j)
 // of the columns common to rows i and j of L, without building L.
 b2sr_status lower_count(const b2sr_matrix* h, int64_t* count, cudaStream_t s) {
@@ -542,7 +623,7 @@ b2sr_status lower_count(const b2sr_matrix* h, int64_t* count, cudaStream_t s) {
 // The masked count; `pairs` (device int64, optional) receives the number of
 // AND-popc word operations of the tile form (one per mask bit per common
 // tile-column).  The row form extracts all of A's and B's rows, so a mask of
-// far fewer tiles than they have takes the tile form.
+// far fewer tiles than they have takes the tile form, and so do full tiles.
 b2sr_status masked_count(const b2sr_matrix* A, const b2sr_matrix* B, const b2sr_matrix* M, int64_t* count,
                          cudaStream_t s, int64_t* pairs) {
     B2SR_CUDA_TRY(cudaMemsetAsync(count, 0, sizeof(int64_t), s));
@@ -552,7 +633,8 @@ b2sr_status masked_count(const b2sr_matrix* A, const b2sr_matrix* B, const b2sr_
     auto* prs = reinterpret_cast<unsigned long long*>(pairs);
     const double bytes = 3.0 * (4.0 * ((double)A->ntr + 1.0)) + ((double)A->T + B->T + M->T) * (4.0 + tile_bytes(A->k));
     const int64_t most = std::max(A->nnz, std::max(B->nnz, M->nnz));
-    if (!pairs && most < (int64_t(1) << 31) - kRunEntries && 16 * M->T >= A->T + B->T)
+    if (!pairs && most < (int64_t(1) << 31) - kRunEntries && 16 * M->T >= A->T + B->T &&
+        !full_tiles(A, A->nnz + B->nnz + M->nnz, A->T + B->T + M->T))
         return masked_count_rows(A, B, M, out, s, bytes);
     return with_tile(A->k, [&](auto kc) -> b2sr_status {
         constexpr int K = decltype(kc)::value;
