@@ -10,9 +10,10 @@
 // vertices kJ .. kJ+k-1 (for a symmetric matrix A^T = A and the handle serves
 // as its own transpose).
 //
-// One round: a warp per active tile-row J deals its (tile, active source row)
-// pairs to the lanes; for every set bit (r, c) of a pair's tile (J, I) the
-// target kI+c is relaxed with dist[kJ+r] + w by an integer atomicMin on the
+// One round: a warp per active tile-row J deals its tiles to the lanes, the
+// active source rows of a tile to several lanes where there are few tiles; for
+// every set bit (r, c) in an active row r of a tile (J, I) the target kI+c is
+// relaxed with dist[kJ+r] + w by an integer atomicMin on the
 // float's bits (non-negative floats order like their bit patterns).  A target
 // that improves is marked in the next set: a bitset, and a list of the
 // tile-rows that hold its bits, appended by whoever sets the first bit of a
@@ -86,32 +87,60 @@ __device__ __forceinline__ int nth_bit(uint32_t m, int i) {
     return pos;
 }
 
-// Row r of tile t, and the set bits of its earlier rows (the row's first
-// weight is that far from the tile's).
+// Row r of tile t, and the set bits of its earlier rows (the row's first weight
+// is that far from the tile's).
 template <int K>
-__device__ __forceinline__ uint32_t pushed_row(const uint8_t* __restrict__ tiles, int32_t t, int r, bool weighted,
-                                               int* before) {
+__device__ __forceinline__ uint32_t tile_row_of(const uint8_t* __restrict__ tiles, int32_t t, int r) {
+    if constexpr (K == 4) return (__ldg(reinterpret_cast<const uint32_t*>(tiles) + t) >> (8 * r)) & 0xFu;
+    else if constexpr (K == 8) return (uint32_t)(__ldg(reinterpret_cast<const unsigned long long*>(tiles) + t) >> (8 * r)) & 0xFFu;
+    else if constexpr (K == 16) return __ldg(reinterpret_cast<const uint16_t*>(tiles) + (int64_t)t * 16 + r);
+    else return __ldg(reinterpret_cast<const uint32_t*>(tiles) + (int64_t)t * 32 + r);
+}
+template <int K>
+__device__ __forceinline__ int ones_before(const uint8_t* __restrict__ tiles, int32_t t, int r) {
     if constexpr (K == 4) {
-        const uint32_t w = __ldg(reinterpret_cast<const uint32_t*>(tiles) + t);
-        *before = __popc(w & ((1u << (8 * r)) - 1u));
-        return (w >> (8 * r)) & 0xFu;
+        return __popc(__ldg(reinterpret_cast<const uint32_t*>(tiles) + t) & ((1u << (8 * r)) - 1u));
     } else if constexpr (K == 8) {
-        const unsigned long long w = __ldg(reinterpret_cast<const unsigned long long*>(tiles) + t);
-        *before = __popcll(w & ((1ull << (8 * r)) - 1ull));
-        return (uint32_t)(w >> (8 * r)) & 0xFFu;
-    } else if constexpr (K == 16) {
-        const uint16_t* p = reinterpret_cast<const uint16_t*>(tiles) + (int64_t)t * 16;
-        *before = 0;
-        if (weighted)
-            for (int q = 0; q < r; ++q) *before += __popc((uint32_t)__ldg(p + q));
-        return __ldg(p + r);
+        return __popcll(__ldg(reinterpret_cast<const unsigned long long*>(tiles) + t) & ((1ull << (8 * r)) - 1ull));
     } else {
-        const uint32_t* p = reinterpret_cast<const uint32_t*>(tiles) + (int64_t)t * 32;
-        *before = 0;
-        if (weighted)
-            for (int q = 0; q < r; ++q) *before += __popc(__ldg(p + q));
-        return __ldg(p + r);
+        constexpr int TB = K == 16 ? 32 : 128;
+        const uint4* p = reinterpret_cast<const uint4*>(tiles + (int64_t)t * TB);
+        const int bits = r * K;  // of the tile
+        int ones = 0;
+        for (int q = 0; 128 * q < bits; ++q) {
+            const uint4 v = __ldg(p + q);
+            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int left = bits - 128 * q - 32 * i;
+                if (left > 0) ones += __popc(left >= 32 ? w[i] : w[i] & ((1u << left) - 1u));
+            }
+        }
+        return ones;
     }
+}
+
+// Rows of tile t that are not empty, k = 16 and 32.
+template <int K>
+__device__ __forceinline__ uint32_t rows_with_bits(const uint8_t* __restrict__ tiles, int32_t t) {
+    constexpr int TB = K == 16 ? 32 : 128;
+    const uint4* p = reinterpret_cast<const uint4*>(tiles + (int64_t)t * TB);
+    uint32_t rows = 0u;
+#pragma unroll
+    for (int q = 0; q < TB / 16; ++q) {
+        const uint4 v = __ldg(p + q);
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if constexpr (K == 32) {
+                if (w[i]) rows |= 1u << (4 * q + i);
+            } else {
+                if (w[i] & 0xFFFFu) rows |= 1u << (8 * q + 2 * i);
+                if (w[i] >> 16) rows |= 2u << (8 * q + 2 * i);
+            }
+        }
+    }
+    return rows;
 }
 
 // The tile-rows a block appends to one list: kept in shared memory, appended
@@ -135,6 +164,11 @@ __device__ __forceinline__ void mark_bits(const PushSet& s, int32_t* count, Appe
     else s.list[atomicAdd(count, 1)] = J;
 }
 
+// Entries a tile from which lanes take single rows: R-MAT 12 and 14, k = 32 (7 and
+// 4 a tile), unit weights, us a search by pairs / by tiles: 430 / 661, 1,190 /
+// 1,448; R-MAT 14, k = 16 (2.4), is no faster by pairs.
+constexpr int64_t kPairEntries = 3;
+
 struct PushGraph {  // the transpose's arrays, the edge weights (w null: 1) and the distances
     const int32_t *rowptr, *colind;
     const uint8_t* tiles;
@@ -142,6 +176,7 @@ struct PushGraph {  // the transpose's arrays, the edge weights (w null: 1) and 
     const float* w;
     float* dist;
     int32_t n;
+    int pairs;  // tiles hold kPairEntries or more on average
 };
 
 // When the near list has run dry: the threshold rises by delta -- or, past a
@@ -161,17 +196,21 @@ __device__ __forceinline__ void raise_threshold(PushState& p, float fm, float de
 }
 
 // Relaxes the out-edges of tile-row J's active vertices; called by the `width`
-// lanes of `group`, `sub` within it.  A chain of dependent memory accesses
-// (segment, row pointers and distances; tiles; weights; two atomics), so the
-// lanes take one (tile, source row) pair each and issue up to kBatch
-// relaxations side by side; a lane that walked all rows of a tile paid the
-// chain once per active row and bit.  far_seen: the least distance sent to the
-// far set.
+// lanes of `group`, `sub` within it; du: a float for each of them in shared
+// memory.  A chain of dependent memory accesses (segment, row pointers and
+// distances; tiles; weights; two atomics), so a lane issues up to kBatch
+// relaxations side by side, and the lanes take one (tile, active row) pair each
+// where a tile-row has few of them (a mesh's has five tiles) or tiles hold
+// several entries (g.pairs).  Elsewhere most pairs are empty, and a tile goes to
+// one lane with all its active rows, or to as many as there are to a tile: one
+// lane a pair went through every tile once an active row (random graph of 2^15
+// vertices, k = 16: 6.3 ms against 1.3).  far_seen: the least distance sent to
+// the far set.
 template <int K, int NEAR, int FAR>
 __device__ __forceinline__ void push_row(const PushGraph& g, const PushSet& cur, const PushSet& nxt, const PushSet& far,
                                          int32_t* near_count, int32_t* far_count, Appends<NEAR>& add_near,
                                          Appends<FAR>& add_far, float th, int buckets, int32_t J, int width,
-                                         unsigned group, int sub, float& far_seen) {
+                                         unsigned group, int sub, float* du, float& far_seen) {
     constexpr int per = 32 / K;
     constexpr uint32_t seg = K == 32 ? 0xFFFFFFFFu : (1u << (K & 31)) - 1u;
     constexpr int kBatch = 4;
@@ -179,75 +218,129 @@ __device__ __forceinline__ void push_row(const PushGraph& g, const PushSet& cur,
     uint32_t amask = (__ldcg(cur.act + J / per) >> sh) & seg;
     const int32_t t0 = __ldg(g.rowptr + J), t1 = __ldg(g.rowptr + J + 1);
     // the sources' distances (the bitset has no bits past n)
-    float du = 0.0f;
-    if (sub < K && (int64_t)J * K + sub < g.n) du = __ldcg(g.dist + (int64_t)J * K + sub);
-    __syncwarp(group);  // every lane has read the segment
+    float mine_du = 0.0f;
+    if (sub < K && (int64_t)J * K + sub < g.n) mine_du = __ldcg(g.dist + (int64_t)J * K + sub);
+    __syncwarp(group);  // every lane has read the segment, and is done with the row before
     if (sub == 0) atomicAnd(cur.act + J / per, ~(seg << sh));
     if (buckets) {
         // active vertices at or past the threshold move to the far set
-        const bool late = sub < K && ((amask >> sub) & 1u) && du >= th;
+        const bool late = sub < K && ((amask >> sub) & 1u) && mine_du >= th;
         const uint32_t defer = __ballot_sync(group, late) >> (lane_id() - sub);
-        if (late) far_seen = fminf(far_seen, du);
+        if (late) far_seen = fminf(far_seen, mine_du);
         const uint32_t mine = defer & seg;
         if (mine && sub == 0) mark_bits<K>(far, far_count, add_far, J, mine);
         amask &= ~mine;
     }
     const int na = __popc(amask);
     if (na == 0) return;
-    const int64_t pairs = (int64_t)(t1 - t0) * na;
-    int32_t ti = sub / na;
-    int ri = sub - ti * na;
-    const int32_t dt = width / na;
-    const int dr = width - dt * na;
-    for (int64_t p = 0; p < pairs; p += width) {
-        const bool live = p + sub < pairs;
-        const int r = live ? nth_bit(amask, ri) : 0;
-        const float d = __shfl_sync(group, du, r, width);
-        if (live) {
-            const int32_t t = t0 + ti;
-            int before = 0;
-            uint32_t bits = pushed_row<K>(g.tiles, t, r, g.w != nullptr, &before);
-            const int32_t I = __ldg(g.colind + t);
-            const float* wt = g.w ? g.w + __ldg(g.voff + t) + before : nullptr;
+    const int32_t nt = t1 - t0;
+    // a batch of relaxations: targets' columns (-1: none) and distances through the tile
+    int c[kBatch];
+    float cand[kBatch];
+    auto relax = [&](int32_t I) {
+        int old[kBatch];
+#pragma unroll
+        for (int q = 0; q < kBatch; ++q)
+            if (c[q] >= 0)
+                old[q] = atomicMin(reinterpret_cast<int*>(g.dist) + (int64_t)I * K + c[q], __float_as_int(cand[q]));
+        uint32_t near_bits = 0u, far_bits = 0u;
+#pragma unroll
+        for (int q = 0; q < kBatch; ++q)
+            if (c[q] >= 0 && cand[q] < __int_as_float(old[q])) {
+                if (cand[q] >= th) {
+                    far_seen = fminf(far_seen, cand[q]);
+                    far_bits |= 1u << c[q];
+                } else {
+                    near_bits |= 1u << c[q];
+                }
+            }
+        if (near_bits) mark_bits<K>(nxt, near_count, add_near, I, near_bits);
+        if (far_bits) mark_bits<K>(far, far_count, add_far, I, far_bits);
+    };
+    // the entries of one row, from distance d; wt: the row's weights
+    auto relax_row = [&](int32_t I, uint32_t bits, float d, const float* wt) {
+        while (bits) {
+#pragma unroll
+            for (int q = 0; q < kBatch; ++q) {
+                c[q] = -1;
+                if (bits) {
+                    c[q] = __ffs(bits) - 1;
+                    bits &= bits - 1;
+                    cand[q] = d + (wt ? __ldg(wt + q) : 1.0f);
+                }
+            }
+            if (wt) wt += kBatch;
+            relax(I);
+        }
+    };
+    if (g.pairs || (int64_t)nt * na <= 2 * width) {  // the same for the group
+        const int64_t pairs = (int64_t)nt * na;
+        int32_t ti = sub / na;
+        int ri = sub - ti * na;
+        const int32_t dt = width / na;
+        const int dr = width - dt * na;
+        for (int64_t p = 0; p < pairs; p += width) {
+            const bool live = p + sub < pairs;
+            const int r = live ? nth_bit(amask, ri) : 0;
+            const float d = __shfl_sync(group, mine_du, r, width);
+            if (live) {
+                const int32_t t = t0 + ti;
+                const int32_t I = __ldg(g.colind + t);
+                const float* wt = g.w ? g.w + __ldg(g.voff + t) : nullptr;
+                const uint32_t bits = tile_row_of<K>(g.tiles, t, r);
+                if (wt && bits) wt += ones_before<K>(g.tiles, t, r);
+                relax_row(I, bits, d, wt);
+            }
+            ti += dt;
+            ri += dr;
+            if (ri >= na) {
+                ri -= na;
+                ++ti;
+            }
+        }
+        return;
+    }
+    du[sub] = mine_du;
+    __syncwarp(group);
+    // 2^lg lanes a tile, no more than it has active rows
+    auto log_up = [](int v) { return 32 - __clz(v - 1); };
+    const int lg = min(log_up(na), 31 - __clz(width) - log_up(min(nt, width)));
+    uint32_t mine_rows = amask;
+    if (lg > 0) {
+        mine_rows = 0u;
+        for (int i = sub & ((1 << lg) - 1); i < na; i += 1 << lg) mine_rows |= 1u << nth_bit(amask, i);
+    }
+    for (int32_t t = t0 + (sub >> lg); t < t1; t += width >> lg) {
+        const int32_t I = __ldg(g.colind + t);
+        const float* wt = g.w ? g.w + __ldg(g.voff + t) : nullptr;
+        if constexpr (K <= 8) {  // the tile is one word, a byte a row
+            using W = typename std::conditional<K == 4, uint32_t, unsigned long long>::type;
+            constexpr W ones = (W)0x0101010101010101ull;
+            const W w = __ldg(reinterpret_cast<const W*>(g.tiles) + t);
+            const W row_bytes = ((((mine_rows * ones) & (W)0x8040201008040201ull) + 0x7F * ones) >> 7) & ones;
+            W bits = w & (row_bytes * (W)0xFF);
             while (bits) {
-                int c[kBatch];
-                float cand[kBatch];
-                int old[kBatch];
 #pragma unroll
                 for (int q = 0; q < kBatch; ++q) {
                     c[q] = -1;
                     if (bits) {
-                        c[q] = __ffs(bits) - 1;
-                        bits &= bits - 1;
-                        cand[q] = d + (wt ? __ldg(wt + q) : 1.0f);
+                        const W low = bits & (~bits + 1);
+                        bits ^= low;
+                        const int at = sizeof(W) == 4 ? __ffs((int)low) - 1 : __ffsll((long long)low) - 1;
+                        const W below = w & (low - 1);
+                        c[q] = at & 7;
+                        cand[q] = du[at >> 3] +
+                                  (wt ? __ldg(wt + (sizeof(W) == 4 ? __popc((uint32_t)below) : __popcll(below))) : 1.0f);
                     }
                 }
-                if (wt) wt += kBatch;
-#pragma unroll
-                for (int q = 0; q < kBatch; ++q)
-                    if (c[q] >= 0)
-                        old[q] = atomicMin(reinterpret_cast<int*>(g.dist) + (int64_t)I * K + c[q],
-                                           __float_as_int(cand[q]));
-                uint32_t near_bits = 0u, far_bits = 0u;
-#pragma unroll
-                for (int q = 0; q < kBatch; ++q)
-                    if (c[q] >= 0 && cand[q] < __int_as_float(old[q])) {
-                        if (cand[q] >= th) {
-                            far_seen = fminf(far_seen, cand[q]);
-                            far_bits |= 1u << c[q];
-                        } else {
-                            near_bits |= 1u << c[q];
-                        }
-                    }
-                if (near_bits) mark_bits<K>(nxt, near_count, add_near, I, near_bits);
-                if (far_bits) mark_bits<K>(far, far_count, add_far, I, far_bits);
+                relax(I);
             }
-        }
-        ti += dt;
-        ri += dr;
-        if (ri >= na) {
-            ri -= na;
-            ++ti;
+        } else {
+            for (uint32_t rows = mine_rows & rows_with_bits<K>(g.tiles, t); rows; rows &= rows - 1) {
+                const int row = __ffs(rows) - 1;
+                relax_row(I, tile_row_of<K>(g.tiles, t, row), du[row],
+                          wt ? wt + ones_before<K>(g.tiles, t, row) : nullptr);
+            }
         }
     }
 }
@@ -263,6 +356,7 @@ __global__ void __launch_bounds__(kPushThreads) push_round_kernel(PushGraph g, P
     __shared__ PushState me;
     __shared__ int32_t ncur, block_min;
     __shared__ Appends<kPushBuffer> add_near, add_far;
+    __shared__ float du[kPushThreads];
     if (threadIdx.x == 0) {
         PushState p = ctl->state[round & 1];
         const int32_t nn = ctl->near[(round + 3) & 3].v;
@@ -311,7 +405,7 @@ __global__ void __launch_bounds__(kPushThreads) push_round_kernel(PushGraph g, P
     float far_seen = INFINITY;
     for (int64_t e = (int64_t)blockIdx.x * kPushWarps + (threadIdx.x >> 5); e < ncur; e += warps)
         push_row<K>(g, cur, nxt, far, near_count, far_count, add_near, add_far, th, buckets, cur.list[e], 32, FULL, lane,
-                    far_seen);
+                    du + (threadIdx.x & ~31), far_seen);
     if (far_seen < INFINITY) atomicMin(&block_min, __float_as_int(far_seen));
     __syncthreads();
     const int m_near = min(add_near.n, kPushBuffer), m_far = min(add_far.n, kPushBuffer);
@@ -351,6 +445,8 @@ constexpr int kClusterRounds = 128;
 constexpr int kNearBuffer = 2048;
 constexpr int kFarBuffer = 2048;
 constexpr int kClusterAverage = 25;  // rows a block and round
+constexpr int kMeshTiles = 5;        // tiles a row of the grids that both limits were measured on
+constexpr int64_t kFewTiles = 128 * 1024;
 
 struct ClusterShared {
     PushState me;
@@ -359,6 +455,7 @@ struct ClusterShared {
     int32_t listed;                 // they are in the set's list in device memory
     int32_t stop;
     int32_t block_min;
+    float du[kClusterThreads];  // distances of the rows at work
     Appends<kNearBuffer> near[2];  // by the parity of the round that marks
     Appends<kFarBuffer> far;
 };
@@ -497,7 +594,7 @@ __global__ void __launch_bounds__(kClusterThreads) push_cluster_kernel(PushGraph
                 J = cluster.map_shared_rank(&sh, b)->near[q].row[e - sh.from[b]];
             }
             push_row<K>(g, cur, nxt, far, near_count, &ctl->far[sh.me.epoch].v, sh.near[q ^ 1], sh.far, sh.me.theta,
-                        buckets, J, width, group, sub, far_seen);
+                        buckets, J, width, group, sub, sh.du + threadIdx.x - sub, far_seen);
         }
         if (far_seen < INFINITY) atomicMin(&sh.block_min, __float_as_int(far_seen));
         cluster.sync();  // all marks are made
@@ -597,7 +694,8 @@ b2sr_status sssp_push(b2sr_matrix* hT, const float* w, int32_t src, float* dist,
     const int64_t cap = max_iters > 0 ? max_iters : (buckets ? 4 * (int64_t)n + 4 : (int64_t)n + 1);
     constexpr int kBatch = 32;  // launched rounds between two looks at the state
     const int64_t limit = ceil_div(cap + 1, kBatch) * kBatch;  // rounds with work: whole batches
-    const PushGraph g{hT->rowptr, hT->colind, hT->tiles, w ? hT->voff : nullptr, w, dist, n};
+    const PushGraph g{hT->rowptr, hT->colind, hT->tiles, w ? hT->voff : nullptr, w, dist, n,
+                      hT->nnz >= kPairEntries * hT->T};
     PushState now = {};
     auto look = [&]() -> b2sr_status {
         B2SR_CUDA_TRY(cudaMemcpyAsync(&now, &ctl->state[0], sizeof(now), cudaMemcpyDeviceToHost, s));
@@ -608,7 +706,12 @@ b2sr_status sssp_push(b2sr_matrix* hT, const float* w, int32_t src, float* dist,
         constexpr int K = decltype(kc)::value;
         int dev = -1;
         const int blocks = cudaGetDevice(&dev) == cudaSuccess ? push_cluster_blocks<K>(dev) : 0;
-        const int32_t most = blocks * kClusterWarps * (K <= 8 ? 4 : 32 / K) * 2;  // rows it serves in two turns
+        // both limits are in tile-rows of kMeshTiles tiles: a round's work is in its
+        // tiles, unless the graph has too few to matter
+        const double scale = hT->T <= kFewTiles ? 1.0 : std::max(1.0, (double)hT->T / ((double)kMeshTiles * ntr));
+        // rows it serves in two turns
+        const int32_t most = (int32_t)(blocks * kClusterWarps * (K <= 8 ? 4 : 32 / K) * 2 / scale);
+        const double average = blocks * kClusterAverage / scale;
         now.active = 1;
         for (bool few = blocks > 0; few && now.active;) {
             const int64_t rounds = now.rounds, worked = (int64_t)now.worked;
@@ -621,7 +724,7 @@ b2sr_status sssp_push(b2sr_matrix* hT, const float* w, int32_t src, float* dist,
             }
             B2SR_TRY(look());
             if (now.active && now.rounds >= limit) return fail(B2SR_ERR_NOT_CONVERGED, "exceeded max_iters rounds");
-            few = !now.busy && (int64_t)now.worked - worked <= (now.rounds - rounds) * blocks * kClusterAverage;
+            few = !now.busy && (double)((int64_t)now.worked - worked) <= (double)(now.rounds - rounds) * average;
         }
         if (!now.active) return B2SR_OK;
         int64_t replayed = 0;

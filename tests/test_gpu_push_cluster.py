@@ -1,6 +1,8 @@
 """Push SSSP where its rounds change hands: the thread-block cluster's launches
 of 128 rounds and the launched rounds it leaves a wide round or a wide search
 to.  Distances are the same as those of the SpMV SSSP, bit for bit."""
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -91,3 +93,63 @@ def test_last_allowed_round(B, shape, k):
         assert B.b2sr_sssp_push_rounds() == rounds
         with pytest.raises(Exception, match="max_iters"):
             B.b2sr_sssp_push(m, src, max_iters=rounds - 33)
+
+
+def _random(n, m, seed):
+    rng = np.random.default_rng(seed)
+    u, v = rng.integers(0, n, (2, m))
+    key = np.unique(np.minimum(u, v) * n + np.maximum(u, v))
+    key = key[key // n != key % n]
+    return n, key // n, key % n
+
+
+def _skewed(n, m, seed):
+    """A few vertices with most of the edges."""
+    rng = np.random.default_rng(seed)
+    u, v = (n * rng.random((2, m)) ** 4).astype(np.int64)
+    key = np.unique(np.minimum(u, v) * n + np.maximum(u, v))
+    key = key[key // n != key % n]
+    return n, key // n, key % n
+
+
+SKEWED = {"random": lambda: _random(20_001, 160_000, 1), "skewed": lambda: _skewed(30_003, 200_000, 2),
+          "dense": lambda: _random(700, 60_000, 3), "star": lambda: (9000, np.zeros(8999, np.int64), np.arange(1, 9000)),
+          "wide": lambda: _random(300_000, 900_000, 4)}
+
+
+@pytest.mark.parametrize("delta", [0.0, 20.0])
+@pytest.mark.parametrize("k", [4, 8, 16, 32])
+@pytest.mark.parametrize("shape", SKEWED)
+def test_irregular_graphs(B, shape, k, delta):
+    """Tile-rows of none to thousands of tiles, tiles of one entry and of many,
+    rounds with every row of a tile active."""
+    n, u, v = SKEWED[shape]()
+    rp, ci, nnz = _csr(n, u, v)
+    rows = np.repeat(np.arange(n), np.diff(to_np(rp)))
+    lo, hi = np.minimum(rows, to_np(ci)), np.maximum(rows, to_np(ci))
+    w = (1.0 + ((lo * 7919 + hi * 104729) % 997) / 32.0).astype(np.float32)
+    src = int(u[0])
+    with B.b2sr_from_csr(n, rp, ci, k) as m:
+        wb = B.b2sr_weights_from_csr(m, rp, ci, to_dev(w))
+        for weights in (wb, None):
+            want = to_np(B.b2sr_sssp(m, src, weights)).view(np.int32)
+            got = to_np(B.b2sr_sssp_push(m, src, weights, delta=delta)).view(np.int32)
+            np.testing.assert_array_equal(got, want)
+
+
+def test_rounds_of_full_tile_rows(B):
+    """A random graph of 2^15 vertices, k = 16, one entry a tile: 6.3 ms when every
+    (tile, active row) pair had a lane of 16 SMs; 1.1 ms."""
+    n, u, v = _random(1 << 15, 1 << 18, 5)
+    rp, ci, nnz = _csr(n, u, v)
+    w = torch.rand(nnz, device="cuda") * 99.0 + 1.0
+    best = 1e9
+    with B.b2sr_from_csr(n, rp, ci, 16) as m:
+        wb = B.b2sr_weights_from_csr(m, rp, ci, w)
+        for _ in range(6):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            B.b2sr_sssp_push(m, 0, wb)
+            torch.cuda.synchronize()
+            best = min(best, time.perf_counter() - t0)
+    assert best < 0.004
