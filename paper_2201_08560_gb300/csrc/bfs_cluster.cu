@@ -16,7 +16,12 @@
 //     the slice to every block.
 // All waits are cluster barriers of co-scheduled blocks.  A launch runs at most
 // kLaunchRounds rounds; a longer search keeps its two sets in device memory
-// between launches.
+// between launches, and goes on in launched rounds if the graph is large: the
+// cluster is 16 of 152 SMs, and a round of it takes about 2 us more for every
+// chunk that a warp holds, a launched round hardly more (random graphs of 256
+// vertices in a row, permuted ids, k = 8, us a search in the cluster / launched
+// after 64 rounds: 3 chunks a warp 2,341 / 3,002, 5 chunks 4,937 / 4,837, 6
+// chunks 4,221 / 3,749, 12 chunks 26,222 / 14,838, after 16 rounds 14,189).
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -33,7 +38,10 @@ constexpr int kClusterWarps = kClusterThreads / 32;
 constexpr int kClusterRuns = 16;              // chunks a warp holds at most
 constexpr int64_t kClusterMaxN = 256 * 1024;  // three bitsets of n bits a block
 constexpr int kMaxCluster = 16;
-constexpr int kLaunchRounds = 64;
+constexpr int kLaunchRounds = 64;             // multiples of the launched loop's four
+constexpr int kShortRuns = 8;                 // and where more than kShortRounds rounds do
+constexpr int kShortRounds = 16;
+constexpr int kLongRuns = 5;                  // chunks a warp holds where long searches stay here
 
 // dynamic shared memory of a block: frontier, visited and partial bitsets, and
 // each lane's first tile-row in each of its chunks
@@ -214,16 +222,12 @@ static int cluster_blocks(int device) {
 
 template <int K>
 static b2sr_status run_cluster(const b2sr_matrix* h, const SourceList& srcs, int nsrc, int32_t* levels,
-                               int64_t max_rounds, cudaStream_t s, bool* taken) {
+                               int64_t max_rounds, uint32_t* kept, int32_t* active, cudaStream_t s, bool* finished,
+                               int64_t* rounds_run) {
     const int blocks = cluster_blocks<K>(h->device);
     if (blocks == 0) return B2SR_OK;
     const int64_t runs = ceil_div(h->nchunks, (int64_t)blocks * kClusterWarps);
     if (runs > kClusterRuns) return B2SR_OK;
-    const int64_t words = ceil_div(h->n, 32);
-    DevBuf buf(s);
-    B2SR_TRY(buf.alloc((size_t)(2 * words + 1) * sizeof(uint32_t)));
-    uint32_t* kept = buf.as<uint32_t>();
-    int32_t* active = reinterpret_cast<int32_t*>(kept + 2 * words);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(blocks);
     cfg.blockDim = dim3(kClusterThreads);
@@ -235,30 +239,37 @@ static b2sr_status run_cluster(const b2sr_matrix* h, const SourceList& srcs, int
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    for (int64_t begin = 1;; begin += kLaunchRounds) {
-        const int rounds = (int)std::min<int64_t>(kLaunchRounds, max_rounds + 1 - begin);
+    const int64_t at_once = runs > kShortRuns ? kShortRounds : kLaunchRounds;
+    for (int64_t begin = 1;; begin += at_once) {
+        const int rounds = (int)std::min<int64_t>(at_once, max_rounds + 1 - begin);
         B2SR_CUDA_TRY(cudaLaunchKernelEx(&cfg, bfs_cluster_kernel<K>, (const int32_t*)h->rowptr,
                                          (const int32_t*)h->colind, (const uint8_t*)h->tiles, (int32_t)h->T, h->ntr, h->n,
                                          (int32_t)h->nchunks, srcs, nsrc, begin, rounds, levels, kept, active));
         B2SR_LAUNCH_CHECK("bfs_cluster_kernel");
-        *taken = true;
         int32_t more = 0;
         B2SR_CUDA_TRY(cudaMemcpyAsync(&more, active, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
         B2SR_CUDA_TRY(cudaStreamSynchronize(s));
-        if (!more) return B2SR_OK;
+        *rounds_run = begin + rounds - 1;
+        if (!more) {
+            *finished = true;
+            return B2SR_OK;
+        }
         if (begin + rounds > max_rounds) return fail(B2SR_ERR_NOT_CONVERGED, "exceeded max_iters rounds");
+        if (runs > kLongRuns) return B2SR_OK;
     }
 }
 
 b2sr_status bfs_cluster(const b2sr_matrix* h, const SourceList& srcs, int nsrc, int32_t* levels, int64_t max_rounds,
-                        cudaStream_t s, bool* taken) {
-    *taken = false;
+                        uint32_t* kept, int32_t* active, cudaStream_t s, bool* finished, int64_t* rounds_run) {
+    *finished = false;
+    *rounds_run = 0;
     int dev = -1;
     if (h->k > 8 || h->nchunks == 0 || h->n > kClusterMaxN || nsrc > kParamSources ||
         cudaGetDevice(&dev) != cudaSuccess || dev != h->device)
         return B2SR_OK;
-    if (h->k == 4) return run_cluster<4>(h, srcs, nsrc, levels, max_rounds, s, taken);
-    return run_cluster<8>(h, srcs, nsrc, levels, max_rounds, s, taken);
+    if (h->k == 4)
+        return run_cluster<4>(h, srcs, nsrc, levels, max_rounds, kept, active, s, finished, rounds_run);
+    return run_cluster<8>(h, srcs, nsrc, levels, max_rounds, kept, active, s, finished, rounds_run);
 }
 
 }  // namespace b2sr

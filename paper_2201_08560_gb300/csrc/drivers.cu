@@ -54,6 +54,13 @@ __global__ void bfs_seed_kernel(const int32_t* srcs, SourceList few, int nsrc, i
     }
 }
 
+// A search goes on after `rounds` rounds: its frontier and visited set are there.
+__global__ void bfs_resume_kernel(uint32_t* fb, int64_t words, LoopFlags* flags, int32_t rounds) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < words; i += (int64_t)gridDim.x * blockDim.x)
+        fb[i] = 0u;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *flags = LoopFlags{1, 0, rounds, 0u};
+}
+
 // visited |= next; levels[v] = level+1 for every new vertex; the frontier just
 // used is cleared for the next round's output; ends the round
 __global__ void bfs_update_kernel(const uint32_t* __restrict__ next, uint32_t* __restrict__ used,
@@ -83,28 +90,35 @@ b2sr_status bfs_sources(b2sr_matrix* h, const int32_t* srcs_host, int nsrc, int3
     const int32_t n = h->n;
     const int64_t words = ceil_div(n, 32);
     const int64_t cap = max_iters > 0 ? max_iters : (int64_t)n + 1;
-    bool done = false;
-    // the same round limit as below: whole batches of four
-    const b2sr_status small = bfs_cluster(h, source_list(srcs_host, nsrc), nsrc, levels, round_up(cap + 1, 4), s, &done);
-    if (done || small != B2SR_OK) return small;
     DevBuf buf(s);
     B2SR_TRY(buf.alloc(sizeof(LoopFlags) + 3 * words * sizeof(uint32_t) + (size_t)nsrc * sizeof(int32_t)));
     LoopFlags* flags = buf.as<LoopFlags>();
     uint32_t* fa = reinterpret_cast<uint32_t*>(flags + 1);
-    uint32_t* fb = fa + words;
-    uint32_t* vis = fb + words;
-    int32_t* dsrc = nullptr;
-    if (nsrc > kParamSources) {
-        dsrc = reinterpret_cast<int32_t*>(vis + words);
-        B2SR_CUDA_TRY(cudaMemcpyAsync(dsrc, srcs_host, nsrc * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+    uint32_t* vis = fa + words;
+    uint32_t* fb = vis + words;
+    // the round limit is whole batches of four
+    bool finished = false;
+    int64_t ran = 0;
+    B2SR_TRY(bfs_cluster(h, source_list(srcs_host, nsrc), nsrc, levels, round_up(cap + 1, 4), fa, &flags->active, s,
+                         &finished, &ran));
+    if (finished) return B2SR_OK;
+    if (ran > 0) {
+        bfs_resume_kernel<<<grid_for(words), 256, 0, s>>>(fb, words, flags, (int32_t)ran);
+        B2SR_LAUNCH_CHECK("bfs_resume_kernel");
+    } else {
+        int32_t* dsrc = nullptr;
+        if (nsrc > kParamSources) {
+            dsrc = reinterpret_cast<int32_t*>(fb + words);
+            B2SR_CUDA_TRY(cudaMemcpyAsync(dsrc, srcs_host, nsrc * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+        }
+        bfs_init_kernel<<<grid_for(std::max<int64_t>(n, words)), 256, 0, s>>>(levels, n, fa, fb, vis, words, flags);
+        B2SR_LAUNCH_CHECK("bfs_init_kernel");
+        bfs_seed_kernel<<<(unsigned)ceil_div(nsrc, 256), 256, 0, s>>>(dsrc, source_list(srcs_host, nsrc), nsrc, levels,
+                                                                    fa, vis);
+        B2SR_LAUNCH_CHECK("bfs_seed_kernel");
     }
-    bfs_init_kernel<<<grid_for(std::max<int64_t>(n, words)), 256, 0, s>>>(levels, n, fa, fb, vis, words, flags);
-    B2SR_LAUNCH_CHECK("bfs_init_kernel");
-    bfs_seed_kernel<<<(unsigned)ceil_div(nsrc, 256), 256, 0, s>>>(dsrc, source_list(srcs_host, nsrc), nsrc, levels, fa,
-                                                                vis);
-    B2SR_LAUNCH_CHECK("bfs_seed_kernel");
     int64_t rounds = 0;
-    return run_captured(s, 4, cap + 1, &flags->active,
+    return run_captured(s, 4, cap + 1 - ran, &flags->active,
                         [&](cudaStream_t cs, int r) -> b2sr_status {
                             uint32_t* f = (r & 1) ? fb : fa;
                             uint32_t* nx = (r & 1) ? fa : fb;

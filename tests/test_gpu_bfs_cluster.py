@@ -40,3 +40,32 @@ def test_levels(name, k):
             want = np.where(want < 0, np.iinfo(np.int32).max, want).min(axis=0)
             want[want == np.iinfo(np.int32).max] = -1
             np.testing.assert_array_equal(to_np(B.b2sr_bfs_sources(m, srcs)), want)
+
+
+def _row_of_blobs(n, blob, seed):
+    """Random graphs of `blob` vertices, six neighbours each, in a row; ids permuted."""
+    rng = np.random.default_rng(seed)
+    m = n // blob
+    base = np.repeat(np.arange(m) * blob, 3 * blob)
+    u, v = base + rng.integers(0, blob, base.size), base + rng.integers(0, blob, base.size)
+    first = np.arange(m - 1) * blob
+    p = rng.permutation(n)
+    return graphs.from_edges(n, p[np.concatenate([u, first])], p[np.concatenate([v, first + blob])])
+
+
+@pytest.mark.parametrize("k", [4, 8])
+@pytest.mark.parametrize("n,blob", [(1 << 17, 512), (3 << 16, 1024), (1 << 18, 4096)])
+def test_long_searches_of_large_graphs(n, blob, k):
+    """Six to twelve chunks a warp: the rounds after the first launch's are launched
+    one by one, with the same levels and the same limit."""
+    from paper_2201_08560_gb300 import binding as B
+    g = _row_of_blobs(n, blob, seed=n)
+    want = oracle.bfs(g, 3)
+    rounds = int(want.max()) + 1  # the last finds nothing
+    assert rounds > 68
+    with B.b2sr_from_csr(g.n, *csr_dev(g), k) as m:
+        np.testing.assert_array_equal(to_np(B.b2sr_bfs(m, 3)), want)
+        np.testing.assert_array_equal(to_np(B.b2sr_bfs(m, 3, max_iters=rounds - 1)), want)
+        for short in (15, 16, 63, 64, rounds - 5):
+            with pytest.raises(Exception, match="max_iters"):
+                B.b2sr_bfs(m, 3, max_iters=short)
