@@ -495,13 +495,13 @@ __global__ void build_rowptr_from_rows(const int32_t* __restrict__ tilerow, int6
 
 static MatView view(const b2sr_matrix* h) { return MatView{h->rowptr, h->colind, h->tiles, h->T, h->ntr}; }
 
-// Tiles a quarter full or more: the tile form counts such a mask faster than the
+// Tiles a third full or more: the tile form counts such a mask faster than the
 // row form, whose work goes with the entries; at k = 32 where bitmaps leave an SM
 // few blocks.  us, tiles / rows, triangles of 64-vertex cliques, n = 2^20: k = 4
 // 1,798 / 12,817, k = 8 1,461 / 12,951, k = 16 2,327 / 12,724, k = 32 4,783 /
 // 6,948; of 256-vertex cliques, n = 2^15: k = 8 365 / 722, k = 32 1,432 / 777.
 static bool full_tiles(const b2sr_matrix* h, int64_t nnz, int64_t T) {
-    return (h->k <= 16 || ceil_div(h->n, 32) * 4 > kOneLaunchBitmap) && 4 * nnz >= (int64_t)h->k * h->k * T;
+    return (h->k <= 16 || ceil_div(h->n, 32) * 4 > kOneLaunchBitmap) && 3 * nnz >= (int64_t)h->k * h->k * T;
 }
 
 // Row lists of a handle, owned by `buf`.
