@@ -152,6 +152,7 @@ struct b2sr_matrix {
     int32_t* split = nullptr;
     int64_t nsplit_short = 0;
     int64_t nsplit_long = 0;
+    int64_t most_tiles = 0;      // of a tile-row that spans chunks (0: none does)
     // lazily built, cached derived arrays (built under the handle's mutex)
     int32_t* voff = nullptr;     // [T+1] set bits before each tile (weights offsets)
     int32_t* outdeg = nullptr;   // [n] ones per column

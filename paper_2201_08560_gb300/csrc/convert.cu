@@ -1030,7 +1030,8 @@ static b2sr_status merge_pieces(int32_t n, const int32_t* rowptr, const int32_t*
 // The row R that chunk c begins inside, when R started in an earlier chunk
 // and ends in c, goes to the split list: rows over at most kSplitShort chunks
 // from the front, longer ones from the back (in no order: each is joined by
-// itself).  meta: first and last tile-row with tiles, short and long rows.
+// itself).  meta: first and last tile-row with tiles, short and long rows, tiles
+// of the longest of them.
 __global__ void schedule_kernel(const int32_t* __restrict__ rowptr, int32_t ntr, int64_t T, int64_t CT,
                                 int64_t nchunks, int32_t* __restrict__ chunk_row, int32_t* __restrict__ split,
                                 int32_t* __restrict__ meta) {
@@ -1045,6 +1046,7 @@ __global__ void schedule_kernel(const int32_t* __restrict__ rowptr, int32_t ntr,
         const int64_t ce = min(cs + CT, T);
         const int64_t rs = rowptr[R], re = rowptr[R + 1];
         if (rs >= cs || re > ce) continue;
+        atomicMax(meta + 4, (int32_t)(re - rs));
         const int64_t ca = rs / CT;
         const int64_t at = c - ca + 1 <= kSplitShort ? atomicAdd(meta + 2, 1) : nchunks - 1 - atomicAdd(meta + 3, 1);
         split[3 * at] = R;
@@ -1065,18 +1067,19 @@ b2sr_status build_schedule(b2sr_matrix* h, cudaStream_t s) {
     B2SR_TRY(dalloc(&h->chunk_row, h->nchunks + 1, s));
     B2SR_TRY(dalloc(&h->split, 3 * h->nchunks, s));
     DevBuf meta(s);
-    B2SR_TRY(meta.alloc(4 * sizeof(int32_t)));
-    B2SR_CUDA_TRY(cudaMemsetAsync(meta.p, 0, 4 * sizeof(int32_t), s));
+    B2SR_TRY(meta.alloc(5 * sizeof(int32_t)));
+    B2SR_CUDA_TRY(cudaMemsetAsync(meta.p, 0, 5 * sizeof(int32_t), s));
     schedule_kernel<<<grid_for(h->nchunks + 1), 256, 0, s>>>(h->rowptr, h->ntr, h->T, CT, h->nchunks, h->chunk_row,
                                                             h->split, meta.as<int32_t>());
     B2SR_LAUNCH_CHECK("schedule_kernel");
-    int32_t got[4] = {0, 0, 0, 0};
+    int32_t got[5] = {0, 0, 0, 0, 0};
     B2SR_CUDA_TRY(cudaMemcpyAsync(got, meta.p, sizeof(got), cudaMemcpyDeviceToHost, s));
     B2SR_CUDA_TRY(cudaStreamSynchronize(s));
     h->first_row = got[0];
     h->last_row = got[1];
     h->nsplit_short = got[2];
     h->nsplit_long = got[3];
+    h->most_tiles = got[4];
     return B2SR_OK;
 }
 

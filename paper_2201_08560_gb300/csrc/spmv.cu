@@ -916,7 +916,7 @@ __device__ __forceinline__ void load_lane_tiles(const SpmvGeom& g, int32_t tl, u
 
 // ---------------------------------------------------------------------------
 // chunk kernel for the bit-vector schemes at k = 16 and 32 and for the value
-// schemes that neither the small-tile kernel nor the staged one takes:
+// schemes that neither the small-tile, the row-lane nor the staged kernel takes:
 // registers hold the accumulators (static row indices)
 // ---------------------------------------------------------------------------
 template <int K, class SEM>
@@ -2274,6 +2274,10 @@ constexpr bool use_small() {
 //   weighted min-plus        377, 294 / 592, 657   860, 748 / 895, 1250    2358, 2873 / 1360, 2459
 // The bits before a row, which a weight's place needs, cost a scan of the
 // tile; at k = 8 a step of four tiles mostly holds fewer set bits than lanes.
+// A tile-row that holds a quarter of the matrix and more keeps the other kernels:
+// its tiles are full rows of one vertex, which one lane walks alone while 31
+// wait (star of 2^20 leaves, k = 32 / 16 / 64-lane OR at k = 8: 177 / 97 / 73 us,
+// 65 / 51 / 54 in the others).
 enum { kRowLanesNever, kRowLanesUnweighted, kRowLanesAlways };
 template <int K, class SEM>
 constexpr int row_lanes() {
@@ -2282,7 +2286,8 @@ constexpr int row_lanes() {
     else return K == 16 && SEM::kMayWeight ? kRowLanesUnweighted : kRowLanesAlways;
 }
 template <int K, class SEM>
-static bool use_row_lanes(const SEM& sem) {
+static bool use_row_lanes(const b2sr_matrix* h, const SEM& sem) {
+    if (4 * h->most_tiles > h->T) return false;
     if constexpr (row_lanes<K, SEM>() == kRowLanesUnweighted) return !sem.weighted;
     else return row_lanes<K, SEM>() == kRowLanesAlways;
 }
@@ -2362,7 +2367,7 @@ static b2sr_status launch_direct(const b2sr_matrix* h, const SEM& sem, Partials<
         }
     } else {
         if constexpr (row_lanes<K, SEM>() != kRowLanesNever) {
-            if (use_row_lanes<K>(sem)) {
+            if (use_row_lanes<K>(h, sem)) {
                 const unsigned grid =
                     (unsigned)std::min<int64_t>(ceil_div(h->nchunks, kSpmvWarps),
                                                 (int64_t)sm_count() * small_min_blocks<K, SEM, kRowLanes>());
@@ -2371,10 +2376,8 @@ static b2sr_status launch_direct(const b2sr_matrix* h, const SEM& sem, Partials<
                 return B2SR_OK;
             }
         }
-        if constexpr (row_lanes<K, SEM>() != kRowLanesAlways) {
-            spmv_chunks_kernel<K, SEM><<<(unsigned)ceil_div(h->nchunks, kSpmvWarps), kSpmvThreads, 0, s>>>(g, sem, part);
-            B2SR_LAUNCH_CHECK("spmv_chunks_kernel");
-        }
+        spmv_chunks_kernel<K, SEM><<<(unsigned)ceil_div(h->nchunks, kSpmvWarps), kSpmvThreads, 0, s>>>(g, sem, part);
+        B2SR_LAUNCH_CHECK("spmv_chunks_kernel");
     }
     return B2SR_OK;
 }
@@ -2392,7 +2395,7 @@ static b2sr_status run_chunks(const b2sr_matrix* h, const SEM& sem, cudaStream_t
     // AUTO: the small-tile and row-lane kernels where they serve
     if constexpr (SEM::kGather && K <= 16)
         staged = h->schedule == B2SR_SCHED_STAGED ||
-                 (h->schedule == B2SR_SCHED_AUTO && !(use_small<K, SEM>() || use_row_lanes<K>(sem)));
+                 (h->schedule == B2SR_SCHED_AUTO && !(use_small<K, SEM>() || use_row_lanes<K>(h, sem)));
     if constexpr (SEM::kGather && K <= 16) if (staged) {
         const int smem = kSpmvWarps * GatherLayout<K, SEM>::bytes;
         if (smem > 48 * 1024)
