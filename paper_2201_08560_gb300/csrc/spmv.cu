@@ -915,9 +915,10 @@ __device__ __forceinline__ void load_lane_tiles(const SpmvGeom& g, int32_t tl, u
 }
 
 // ---------------------------------------------------------------------------
-// chunk kernel for the bit-vector schemes at k = 16 and 32 and for the value
-// schemes that neither the small-tile, the row-lane nor the staged kernel takes:
-// registers hold the accumulators (static row indices)
+// chunk kernel for the bit-vector schemes at k = 16 and 32, for counts at k = 8
+// where rows are short, and for the value schemes that neither the small-tile,
+// the row-lane nor the staged kernel takes: registers hold the accumulators
+// (static row indices)
 // ---------------------------------------------------------------------------
 template <int K, class SEM>
 __global__ void __launch_bounds__(kSpmvThreads) spmv_chunks_kernel(SpmvGeom g, SEM sem,
@@ -2329,6 +2330,17 @@ static b2sr_status launch_direct(const b2sr_matrix* h, const SEM& sem, Partials<
             // few chunks to spread the copy over: R-MAT 20, k = 4 / k = 8, Boolean:
             // 75 / 74.7 us without, 68 / 72.5 with it; permuted ids 76 / 89 and 67 / 82.
             constexpr int threads = small_threads<K, SEM, kSmBitsShared>();
+            // Counts at k = 8 of a large matrix without a chunk inside one tile-row:
+            // the eight counts a row cost the walk more than the shared bitset saves
+            // (uniform random graph of 2^20 vertices, 127 tiles a row: 118 us, 108 in the
+            // general kernel; R-MAT 20: 142, 161).
+            if constexpr (K == 8 && SEM::NV == 8 && !NoInput<SEM>::value)
+                if (h->most_tiles <= chunk_tiles(K) && h->T >= h->ntr && h->nchunks >= 2048) {
+                    spmv_chunks_kernel<K, SEM>
+                        <<<(unsigned)ceil_div(h->nchunks, kSpmvWarps), kSpmvThreads, 0, s>>>(g, sem, part);
+                    B2SR_LAUNCH_CHECK("spmv_chunks_kernel");
+                    return B2SR_OK;
+                }
             if constexpr (!NoInput<SEM>::value)
                 if (h->nchunks >= (int64_t)sm_count() * (threads / 32) * 4 &&
                     ceil_div(h->n, 32) * 4 + threads / 32 * small_warp_smem<SEM>() <= kMaxBlockSmem)
