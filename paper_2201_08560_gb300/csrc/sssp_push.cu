@@ -345,12 +345,21 @@ __device__ __forceinline__ void push_row(const PushGraph& g, const PushSet& cur,
     }
 }
 
+// Resident blocks an SM, which are all that are launched: a round of many rows is
+// bound by the loads in flight, and one of few costs no more for the blocks that
+// leave at once.  Random graph of 2^20 vertices, us a search with 2 / 3 / 4 blocks:
+// k = 4 3,308 / 2,374 / 1,914, k = 16 4,040 / 2,965 / 2,522; grid of 2048 x 2048,
+// delta 400, k = 8 35,162 / 34,861 / 34,865, k = 32 44,525 / 44,534 / 46,648 (four
+// blocks spill there).
+template <int K>
+constexpr int push_blocks() { return K <= 8 ? 4 : 3; }
+
 // One round over the whole chip, a warp per active tile-row.  The roles of the
 // sets follow from the previous round: its near list is this round's active
 // set; when that is empty but far vertices wait, the threshold rises; when both
 // are empty the loop is done.
 template <int K>
-__global__ void __launch_bounds__(kPushThreads) push_round_kernel(PushGraph g, PushSet s0, PushSet s1, PushSet s2,
+__global__ void __launch_bounds__(kPushThreads, push_blocks<K>()) push_round_kernel(PushGraph g, PushSet s0, PushSet s1, PushSet s2,
                                                                   PushControl* ctl, int round, int buckets, float delta) {
     constexpr unsigned FULL = 0xffffffffu;
     __shared__ PushState me;
@@ -687,7 +696,6 @@ b2sr_status sssp_push(b2sr_matrix* hT, const float* w, int32_t src, float* dist,
     B2SR_CUDA_TRY(cudaMemsetAsync(base, 0, 3 * bw, s));
     push_init_kernel<<<grid_for(n), 256, 0, s>>>(dist, n, src, hT->k, set[0], ctl, buckets ? delta : INFINITY);
     B2SR_LAUNCH_CHECK("push_init_kernel");
-    const int grid = sm_count() * 2;  // warps stride over the active list
     // default round limit: without buckets at most n rounds improve anything;
     // with them every raise of the threshold settles at least one vertex and
     // costs a few rounds beyond the improving ones, so 4n covers both
@@ -727,6 +735,7 @@ b2sr_status sssp_push(b2sr_matrix* hT, const float* w, int32_t src, float* dist,
             few = !now.busy && (double)((int64_t)now.worked - worked) <= (double)(now.rounds - rounds) * average;
         }
         if (!now.active) return B2SR_OK;
+        const int grid = sm_count() * push_blocks<K>();  // warps stride over the active list
         int64_t replayed = 0;
         B2SR_TRY(run_captured(s, kBatch, limit + 1 - now.rounds, &ctl->state[0].active,
                               [&](cudaStream_t cs, int r) -> b2sr_status {
