@@ -577,7 +577,11 @@ extern "C" b2sr_status b2sr_tc(b2sr_handle h, int64_t* count, void* stream) {
     clear_error();
     B2SR_TRY(check_handle(h));
     if (!count) return fail(B2SR_ERR_INVALID_ARG, "count is NULL");
-    if (counts_by_rows(h)) return lower_count(h, count, to_stream(stream));
+    if (counts_by_rows(h)) {
+        const b2sr_status st = lower_count(h, count, to_stream(stream));
+        if (st != B2SR_ERR_OOM) return st;
+        clear_error();  // the tile form needs L alone
+    }
     b2sr_handle L = nullptr;
     B2SR_TRY(b2sr_lower(h, stream, &L));
     b2sr_status st = masked_count(L, L, L, count, to_stream(stream), nullptr);

@@ -554,14 +554,19 @@ static b2sr_status count_rows(int32_t n, RowLists a, RowLists b, RowLists m, int
         B2SR_LAUNCH_CHECK("masked_rows_kernel");
         return B2SR_OK;
     };
-    void* tok = timing_begin(s);
-    B2SR_TRY(count_runs(a, b, m, split));
+    // the other entries by column: cnt, off, colptr and cursor a column, row_of and
+    // the rows a slot
+    DevBuf cnt(s), off(s), cur(s), rows(s);
     if (split) {
-        DevBuf cnt(s), off(s), cur(s), rows(s);
         B2SR_TRY(cnt.alloc(((size_t)n + 1) * sizeof(int32_t)));
         B2SR_TRY(off.alloc(((size_t)n + 1) * sizeof(int64_t)));
         B2SR_TRY(cur.alloc(2 * ((size_t)n + 1) * sizeof(int32_t)));
         B2SR_TRY(rows.alloc(2 * (size_t)slots * sizeof(int32_t)));
+    }
+    void* tok = timing_begin(s);
+    auto count_all = [&]() -> b2sr_status {
+        B2SR_TRY(count_runs(a, b, m, split));
+        if (!split) return B2SR_OK;
         int32_t* colptr = cur.as<int32_t>();
         int32_t* cursor = colptr + n + 1;
         int32_t* row_of = rows.as<int32_t>() + slots;
@@ -574,11 +579,11 @@ static b2sr_status count_rows(int32_t n, RowLists a, RowLists b, RowLists m, int
         place_by_column_kernel<<<grid_wide(slots), 256, 0, s>>>(row_of, m.colind, (int32_t)slots, cursor,
                                                                rows.as<int32_t>());
         B2SR_LAUNCH_CHECK("place_by_column_kernel");
-        const RowLists mt{colptr, colptr + 1, rows.as<int32_t>()};
-        B2SR_TRY(count_runs(b, a, mt, 0));
-    }
+        return count_runs(b, a, RowLists{colptr, colptr + 1, rows.as<int32_t>()}, 0);
+    };
+    const b2sr_status st = count_all();
     timing_end(tok, "spgemm_masked", bytes, s);
-    return B2SR_OK;
+    return st;
 }
 
 static b2sr_status masked_count_rows(const b2sr_matrix* A, const b2sr_matrix* B, const b2sr_matrix* M,
@@ -634,8 +639,12 @@ b2sr_status masked_count(const b2sr_matrix* A, const b2sr_matrix* B, const b2sr_
     const double bytes = 3.0 * (4.0 * ((double)A->ntr + 1.0)) + ((double)A->T + B->T + M->T) * (4.0 + tile_bytes(A->k));
     const int64_t most = std::max(A->nnz, std::max(B->nnz, M->nnz));
     if (!pairs && most < (int64_t(1) << 31) - kRunEntries && 16 * M->T >= A->T + B->T &&
-        !full_tiles(A, A->nnz + B->nnz + M->nnz, A->T + B->T + M->T))
-        return masked_count_rows(A, B, M, out, s, bytes);
+        !full_tiles(A, A->nnz + B->nnz + M->nnz, A->T + B->T + M->T)) {
+        const b2sr_status st = masked_count_rows(A, B, M, out, s, bytes);
+        if (st != B2SR_ERR_OOM) return st;
+        clear_error();  // the tile form needs no memory
+        B2SR_CUDA_TRY(cudaMemsetAsync(count, 0, sizeof(int64_t), s));
+    }
     return with_tile(A->k, [&](auto kc) -> b2sr_status {
         constexpr int K = decltype(kc)::value;
         // runs of eight mask tiles a warp; the blocks are scheduled as SMs free
