@@ -144,25 +144,25 @@ struct LiveState {
     int32_t dense;
 };
 
-// The next frontiers of four rounds, written in turn: round r reads the one
-// before (the sources' in round 0 of all) and writes set[r & 3].
-constexpr int kFrontiers = 4;
-template <class W>
+// The next frontiers of N rounds, written in turn: round r reads the one before
+// (the sources' in round 0 of all) and writes set[r % N].  N is four, or two
+// where the device has no room for four.
+template <class W, int N>
 struct Frontiers {
-    W* set[kFrontiers];
+    W* set[N];
 };
 
 // Rows without tiles are written by no SpMM: they are zero from the start.
 // Unused lanes count as visited, so a vertex every source has reached is all
 // ones in the mask and the SpMM can skip its rows.
-template <class W>
-__global__ void msbfs_init_kernel(int32_t n, int nsrc, Frontiers<W> f, W* vis, uint8_t* live, int64_t live_bytes,
+template <class W, int N>
+__global__ void msbfs_init_kernel(int32_t n, int nsrc, Frontiers<W, N> f, W* vis, uint8_t* live, int64_t live_bytes,
                                   LiveState* state, LoopFlags* flags) {
     constexpr int BITS = 8 * (int)sizeof(W);
     const W unused = nsrc < BITS ? (W)~(((W)1 << nsrc) - (W)1) : (W)0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
 #pragma unroll
-        for (int q = 0; q < kFrontiers; ++q) f.set[q][i] = (W)0;
+        for (int q = 0; q < N; ++q) f.set[q][i] = (W)0;
         vis[i] = unused;
         if (i < live_bytes) live[i] = 0;  // a byte for 32 vertices, rounded up to 16
     }
@@ -231,25 +231,25 @@ __global__ void msbfs_update_kernel(const W* __restrict__ Y, W* __restrict__ vis
     }
 }
 
-// The levels of what the last four rounds (fewer in a search's last batch)
-// found.  After the first four every level is written, -1 where nothing was
+// The levels of what the last N rounds (fewer at a search's end) found.  After
+// the first N every level is written, -1 where nothing was
 // found, and the sources' 0; later ones only where a round found something, a
 // warp going through the lanes that any of its 32 vertices has.  The levels are
 // most of a search's output (R-MAT 22, 64 sources: 1.07 GB): filled with -1
 // first and written round by round they took 242 us and 113 us a round; here
 // the two launches of such a search take 284 us and a round's update 20.
-template <class W>
-__global__ void msbfs_levels_kernel(Frontiers<W> f, const W* __restrict__ vis, int32_t* __restrict__ levels, int32_t n,
+template <class W, int N>
+__global__ void msbfs_levels_kernel(Frontiers<W, N> f, const W* __restrict__ vis, int32_t* __restrict__ levels, int32_t n,
                                     int nsrc, const LoopFlags* flags) {
     const int done = flags->level;
-    const int base = (done - 1) & ~(kFrontiers - 1), run = done - base;
+    const int base = (done - 1) & ~(N - 1), run = done - base;
     const int lane = (int)lane_id();
     for (int64_t v0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) - lane; v0 < n;
          v0 += (int64_t)gridDim.x * blockDim.x) {  // warp-uniform
         const int64_t v = v0 + lane;
-        W b[kFrontiers];
+        W b[4] = {};
 #pragma unroll
-        for (int q = 0; q < kFrontiers; ++q) b[q] = v < n && q < run ? f.set[q][v] : (W)0;
+        for (int q = 0; q < N; ++q) b[q] = v < n && q < run ? f.set[q][v] : (W)0;
         const W found = b[0] | b[1] | b[2] | b[3], one = b[1] | b[3], two = b[2] | b[3];
         const W seen = base == 0 && v < n ? vis[v] : found;
 #pragma unroll
@@ -288,41 +288,45 @@ static b2sr_status spmm_lanes(b2sr_matrix* h, const uint32_t* X, uint32_t* Y, co
     return spmm32_dispatch(h, X, Y, M, 1, s, gate, edges, live);
 }
 
-template <class W>
+// no_room: the workspace could not be allocated (nothing was done).
+template <class W, int N>
 static b2sr_status bfs_multi_lanes(b2sr_matrix* h, const int32_t* srcs_host, int nsrc, int32_t* levels,
-                                   int max_iters, cudaStream_t s) {
+                                   int max_iters, cudaStream_t s, bool* no_room) {
     const int32_t n = h->n;
     DevBuf buf(s);
     const size_t vb = round_up((size_t)n * sizeof(W), 256);
     const size_t lb = round_up(ceil_div(n, 32), 16);
-    B2SR_TRY(buf.alloc((kFrontiers + 1) * vb + lb + sizeof(LoopFlags) + sizeof(LiveState)));
-    Frontiers<W> f;
-    for (int q = 0; q < kFrontiers; ++q) f.set[q] = reinterpret_cast<W*>(buf.as<char>() + q * vb);
-    W* vis = reinterpret_cast<W*>(buf.as<char>() + kFrontiers * vb);
-    uint8_t* live = reinterpret_cast<uint8_t*>(buf.as<char>() + (kFrontiers + 1) * vb);
+    const b2sr_status room = buf.alloc((N + 1) * vb + lb + sizeof(LoopFlags) + sizeof(LiveState));
+    *no_room = room == B2SR_ERR_OOM;
+    B2SR_TRY(room);
+    Frontiers<W, N> f;
+    for (int q = 0; q < N; ++q) f.set[q] = reinterpret_cast<W*>(buf.as<char>() + q * vb);
+    W* vis = reinterpret_cast<W*>(buf.as<char>() + N * vb);
+    uint8_t* live = reinterpret_cast<uint8_t*>(buf.as<char>() + (N + 1) * vb);
     LoopFlags* flags = reinterpret_cast<LoopFlags*>(live + lb);
     LiveState* state = reinterpret_cast<LiveState*>(flags + 1);
     const LiveColumns columns{reinterpret_cast<const uint32_t*>(live), &state->dense};
-    W* sources = f.set[kFrontiers - 1];
-    msbfs_init_kernel<W><<<grid_for(n), 256, 0, s>>>(n, nsrc, f, vis, live, (int64_t)lb, state, flags);
+    W* sources = f.set[N - 1];
+    msbfs_init_kernel<W, N><<<grid_for(n), 256, 0, s>>>(n, nsrc, f, vis, live, (int64_t)lb, state, flags);
     B2SR_LAUNCH_CHECK("msbfs_init_kernel");
     msbfs_seed_kernel<W><<<1, 64, 0, s>>>(source_list(srcs_host, nsrc), nsrc, sources, vis,
                                           reinterpret_cast<uint32_t*>(live));
     B2SR_LAUNCH_CHECK("msbfs_seed_kernel");
     const int64_t cap = max_iters > 0 ? max_iters : (int64_t)n + 1;
     int64_t rounds = 0;
-    return run_captured(s, kFrontiers, cap + 1, &flags->active,
+    return run_captured(s, 4, cap + 1, &flags->active,
                         [&](cudaStream_t cs, int r) -> b2sr_status {
-                            W* nxt = f.set[r];
+                            const int q = r % N;
+                            W* nxt = f.set[q];
                             // rows without tiles are zero in every set from the start, but for the
                             // last's, which may have sources there until a round has written it
-                            B2SR_TRY(spmm_lanes(h, f.set[(r + kFrontiers - 1) % kFrontiers], nxt, vis, cs,
-                                                &flags->active, r == kFrontiers - 1, columns));
+                            B2SR_TRY(spmm_lanes(h, f.set[(q + N - 1) % N], nxt, vis, cs, &flags->active, q == N - 1,
+                                                columns));
                             msbfs_update_kernel<W><<<grid_for(ceil_div(n, 4), 4), 256, 0, cs>>>(
                                 nxt, vis, n, reinterpret_cast<uint32_t*>(live), state, flags);
                             B2SR_LAUNCH_CHECK("msbfs_update_kernel");
-                            if (r < kFrontiers - 1) return B2SR_OK;
-                            msbfs_levels_kernel<W><<<grid_for(n), 256, 0, cs>>>(f, vis, levels, n, nsrc, flags);
+                            if (q < N - 1) return B2SR_OK;
+                            msbfs_levels_kernel<W, N><<<grid_for(n), 256, 0, cs>>>(f, vis, levels, n, nsrc, flags);
                             B2SR_LAUNCH_CHECK("msbfs_levels_kernel");
                             return B2SR_OK;
                         },
@@ -331,8 +335,17 @@ static b2sr_status bfs_multi_lanes(b2sr_matrix* h, const int32_t* srcs_host, int
 
 b2sr_status bfs_multi(b2sr_matrix* h, const int32_t* srcs_host, int nsrc, int32_t* levels, int max_iters,
                       cudaStream_t s) {
-    if (nsrc <= 32) return bfs_multi_lanes<uint32_t>(h, srcs_host, nsrc, levels, max_iters, s);
-    return bfs_multi_lanes<unsigned long long>(h, srcs_host, nsrc, levels, max_iters, s);
+    // five lane words a vertex; where they do not fit, three
+    auto search = [&](auto lane_word) -> b2sr_status {
+        using W = decltype(lane_word);
+        bool no_room = false;
+        const b2sr_status st = bfs_multi_lanes<W, 4>(h, srcs_host, nsrc, levels, max_iters, s, &no_room);
+        if (!no_room) return st;
+        clear_error();
+        return bfs_multi_lanes<W, 2>(h, srcs_host, nsrc, levels, max_iters, s, &no_room);
+    };
+    if (nsrc <= 32) return search(uint32_t(0));
+    return search(0ull);
 }
 
 // ---------------------------------------------------------------------------
