@@ -256,7 +256,7 @@ b2sr_status bfs_dirop(b2sr_matrix* h, b2sr_matrix* hT, int32_t src, int32_t* lev
                                                                                     cur, curl, f, vis, nx, ctl);
                                     B2SR_LAUNCH_CHECK("dirop_push_kernel");
                                     B2SR_TRY(spmv_dispatch(h, B2SR_BOOL_OR_AND, B2SR_VEC_BITS, f, B2SR_VEC_BITS, nx,
-                                                           vis, 1, nullptr, cs, pull_gate));
+                                                           vis, 1, nullptr, cs, pull_gate, false));
                                     dirop_update_kernel<KT><<<grid_for(words), 256, 0, cs>>>(nx, vis, levels, words, n,
                                                                                             h->outdeg, nxt,
                                                                                             hT->rowptr, nxtl, ctl);
