@@ -1290,13 +1290,14 @@ b2sr_status ensure_outdeg(b2sr_matrix* h, cudaStream_t s) {
 // ---------------------------------------------------------------------------
 // B2SR -> CSR
 // ---------------------------------------------------------------------------
-// Ones per row come from the row-count SpMV (spmv.cu) or csr_rows_kernel, which also leaves the partial counts of the tile-rows that
-// cross chunks; a scan makes them row pointers.  The columns are then written by
-// a warp per chunk of tiles, so a hub's row of 10^5 tiles is shared by many
-// warps.  An entry's place is its row's pointer, plus the row's ones in earlier
-// chunks (the partials), plus those in earlier tiles of the chunk.  At k = 4 and
-// 8 (and 16) a lane takes a tile, 32 tiles a step, and those are a carry from
-// earlier steps and a scan over the lanes that restarts at every tile-row.
+// Ones per row come from the row-count SpMV (spmv.cu) or csr_rows_kernel, which
+// also leaves the partial counts of the tile-rows that cross chunks; a scan makes
+// them row pointers.  The columns are then written by a warp per chunk of tiles,
+// so a hub's row of 10^5 tiles is shared by many warps.  An entry's place is its
+// row's pointer, plus the row's ones in earlier chunks (the partials), plus those
+// in earlier tiles of the chunk.  Here a lane takes a tile, 32 tiles a step, and
+// those are a carry from earlier steps and a scan over the lanes that restarts at
+// every tile-row.
 template <int K>
 __global__ void __launch_bounds__(256) csr_fill_kernel(const int32_t* __restrict__ trp,
                                                        const int32_t* __restrict__ tci,
@@ -1467,12 +1468,26 @@ __global__ void __launch_bounds__(256) csr_rows_kernel(const int32_t* __restrict
                         at = pb + (sub ? mine : theirs);
                     }
                     const int32_t j = __shfl_sync(FULL, j0, ua + sub);
-                    if (__any_sync(FULL, __popc(b[q]) > 8)) {  // row by row, a lane a column
-                        for (int i = row0; i < row1; ++i) {
+                    // rows of many entries, if they are most of the tile's or there are few: row
+                    // by row, a lane a column
+                    const uint32_t many = __ballot_sync(FULL, __popc(b[q]) > 8);
+                    uint32_t some = __ballot_sync(FULL, b[q] != 0u);  // rows with entries
+                    if constexpr (SUBS == 2) some = (some | (some >> 16)) & 0xFFFFu;
+                    if (many != 0u && (__popc(many) >= 8 || __popc(some) <= 4)) {
+                        auto write_row = [&](int i) {
                             const int from = sub * K + i;
                             const uint32_t w = __shfl_sync(FULL, b[q], from);
                             const int64_t pw = __shfl_sync(FULL, p, from);
                             if ((w >> r) & 1u) colind[pw + __popc(w & ((1u << r) - 1u))] = j + r;
+                        };
+                        if (__popc(some) <= 4) {
+                            for (; some; some &= some - 1u) {
+                                const int i = __ffs(some) - 1;
+                                if (i >= row0 && i < row1) write_row(i);
+                            }
+                        } else {
+#pragma unroll 8
+                            for (int i = row0; i < row1; ++i) write_row(i);
                         }
                     } else {
                         for (uint32_t w = r >= row0 && r < row1 ? b[q] : 0u; w; w &= w - 1)
@@ -1513,22 +1528,26 @@ b2sr_status extract_csr(const b2sr_matrix* h, int64_t* off, int32_t* rowptr, int
     int32_t* first = part.as<int32_t>();
     int32_t* last = first + np;
     B2SR_CUDA_TRY(cudaMemsetAsync(cnt.p, 0, ((size_t)n + 1) * sizeof(int32_t), s));  // rows without tiles stay 0
-    // a kernel over the chunks' rows at k = 32, and at k = 16 where tiles hold more
-    // than a few entries or hardly a tile-row has one.  us, rows / tiles: 1 bit a
-    // tile 1078 / 903, 2.2 529 / 438, 9.8 104 / 104, 43 150 / 156, 171 195 / 297,
-    // 256 151 / 227; 2,000 entries in 2^26 rows 563 / 26,784.
+    // k = 16 and 32: a kernel over the chunks' rows where tiles are an eighth full,
+    // hardly a tile-row has one, or, at k = 32, the chunks outnumber the warps.  us,
+    // rows / tiles: k = 16, 1 entry a tile 1078 / 903, 2.2 529 / 438, 9.8 104 / 104,
+    // 43 150 / 156, 171 195 / 297, 256 123 / 213; 2,000 entries in 2^26 rows 563 /
+    // 26,784; k = 32, 4,000 chunks and fewer 152 / 126, 8,000 218 / 254, 130,000
+    // 1,719 / 3,967.
+    const bool full = 8 * h->nnz >= (int64_t)h->k * h->k * h->T;
+    const bool wide = h->k >= 16 && h->nchunks > 0 &&
+                      (full || h->ntr > 32 * h->T || (h->k == 32 && h->nchunks >= 4096));
     auto wide_rows = [&](auto fill, const int64_t* row_start) -> b2sr_status {
         constexpr bool FILL = decltype(fill)::value;
         auto kernel = h->k == 16 ? csr_rows_kernel<16, FILL> : csr_rows_kernel<32, FILL>;
         // few chunks of full tiles (64 full tiles are 65,536 entries) are shared by four warps each
-        const unsigned share = FILL && h->nchunks <= (int64_t)sm_count() * 2 ? 4 : 1;
-        kernel<<<dim3((unsigned)ceil_div(h->nchunks, 8), share), 256, 0, s>>>(h->rowptr, h->colind, h->tiles, n, h->T, h->nchunks,
-                                                                h->chunk_row, row_start, cnt.as<int32_t>(), first, last,
-                                                                colind);
+        const unsigned share = FILL && full && h->nchunks <= (int64_t)sm_count() * 16 ? 4 : 1;
+        kernel<<<dim3((unsigned)ceil_div(h->nchunks, 8), share), 256, 0, s>>>(
+            h->rowptr, h->colind, h->tiles, n, h->T, h->nchunks, h->chunk_row, row_start, cnt.as<int32_t>(), first, last,
+            colind);
         B2SR_LAUNCH_CHECK("csr_rows_kernel");
         return B2SR_OK;
     };
-    const bool wide = h->nchunks > 0 && (h->k == 32 || (h->k == 16 && (h->nnz > 8 * h->T || h->ntr > 32 * h->T)));
     if (wide) B2SR_TRY(wide_rows(std::false_type(), nullptr));
     B2SR_TRY(row_counts(h, cnt.as<int32_t>(), first, last, wide, s));
     B2SR_TRY(exclusive_scan_i32_to_i64(cnt.as<int32_t>(), off, (int64_t)n + 1, s));
@@ -1536,11 +1555,13 @@ b2sr_status extract_csr(const b2sr_matrix* h, int64_t* off, int32_t* rowptr, int
     B2SR_LAUNCH_CHECK("rowptr_out_kernel");
     if (!colind || h->nchunks == 0) return B2SR_OK;
     if (wide) return wide_rows(std::true_type(), off);
-    auto kernel = h->k == 4 ? csr_fill_kernel<4> : (h->k == 8 ? csr_fill_kernel<8> : csr_fill_kernel<16>);
-    kernel<<<(unsigned)ceil_div(h->nchunks, 8), 256, 0, s>>>(h->rowptr, h->colind, h->tiles, h->T, h->nchunks,
-                                                            h->chunk_row, off, first, last, colind);
-    B2SR_LAUNCH_CHECK("csr_fill_kernel");
-    return B2SR_OK;
+    return with_tile(h->k, [&](auto kc) -> b2sr_status {
+        constexpr int K = decltype(kc)::value;
+        csr_fill_kernel<K><<<(unsigned)ceil_div(h->nchunks, 8), 256, 0, s>>>(
+            h->rowptr, h->colind, h->tiles, h->T, h->nchunks, h->chunk_row, off, first, last, colind);
+        B2SR_LAUNCH_CHECK("csr_fill_kernel");
+        return B2SR_OK;
+    });
 }
 
 // ---------------------------------------------------------------------------

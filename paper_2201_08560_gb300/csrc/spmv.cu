@@ -2468,8 +2468,7 @@ b2sr_status row_counts(const b2sr_matrix* h, int32_t* cnt, int32_t* first, int32
         sem.n = h->n;
         SpmvGeom g{h->rowptr, h->colind, h->tiles, h->chunk_row, h->T, h->nchunks, h->ntr, nullptr};
         const Partials<int32_t> part{first, last};
-        if constexpr (K <= 16)
-            if (!chunks_done && h->nchunks > 0) B2SR_TRY((launch_direct<K, SEM>(h, sem, part, s, g)));
+        if (!chunks_done && h->nchunks > 0) B2SR_TRY((launch_direct<K, SEM>(h, sem, part, s, g)));
         return launch_fixup<K, SEM>(h, sem, part, s, nullptr, false);
     });
 }
