@@ -596,7 +596,7 @@ __global__ void __launch_bounds__(kFillThreads, 4) fill_tiles_kernel(const uint6
 // the pieces 75 and moving the tiles together 80.
 constexpr int kWindow = 1024;
 constexpr int kPieceCap = 2048;
-constexpr int kPieceRows = 1024;
+constexpr int kPieceRows = 4096;
 constexpr int kSliceTarget = 1920;  // a slice is cut at a tile-column: up to k * k <= 64 entries more
 constexpr int kPieceThreads = 256;
 constexpr int kPieceItems = kPieceCap / kPieceThreads;

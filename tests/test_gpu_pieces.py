@@ -65,13 +65,13 @@ def test_pieces_give_the_arrays(name, k):
 
 
 @pytest.mark.parametrize("k", [4, 8])
-@pytest.mark.parametrize("tail", [0, 1, 1023, 1024, 1025, 5000])
+@pytest.mark.parametrize("tail", [0, 1, 4095, 4096, 4097, 20000])
 def test_stretches_of_empty_rows(k, tail):
-    """Runs of 1,022 to 3,073 empty tile-rows before, between and after single
+    """Runs of 4,094 to 12,289 empty tile-rows before, between and after single
     entries, a short dense part and a long row."""
     from paper_2201_08560_gb300 import binding as B
     at, rows, cols = 0, [], []
-    for gap in (1024, 0, 1022, 1023, 1025, 2047, 2048, 3073):
+    for gap in (4096, 0, 4094, 4095, 4097, 8191, 8192, 12289):
         at += gap * k
         rows += [at + k - 1]
         cols += [at // 2]
