@@ -55,7 +55,7 @@ __device__ __forceinline__ bool finish_round(LoopFlags* f, int any) {
 // ---------------------------------------------------------------------------
 // Runs rounds (body(stream, r) enqueues one; r counts from 0 within a batch of
 // `per_graph`) until *active reads 0, reading it after every batch.  Every
-// round must be gated on *active.  The first kEagerBatches batches are
+// round must be gated on *active.  The first `eager_batches` batches are
 // enqueued on the caller's stream; a loop that goes on longer captures a batch
 // into a CUDA graph on a private stream and replays it.  (Capture,
 // instantiation, the private stream and its pinned flag cost 200 to 250 us a
@@ -66,9 +66,9 @@ constexpr int kEagerBatches = 4;
 
 template <class Body>
 b2sr_status run_captured(cudaStream_t user, int per_graph, int64_t max_rounds, const int32_t* active,
-                                Body&& body, int64_t* rounds) {
+                                Body&& body, int64_t* rounds, int eager_batches = kEagerBatches) {
     *rounds = 0;
-    for (int batch = 0; batch < kEagerBatches; ++batch) {
+    for (int batch = 0; batch < eager_batches; ++batch) {
         for (int r = 0; r < per_graph; ++r) B2SR_TRY(body(user, r));
         *rounds += per_graph;
         int32_t got = 0;
