@@ -21,7 +21,8 @@
 // chunk that a warp holds, a launched round hardly more (random graphs of 256
 // vertices in a row, permuted ids, k = 8, us a search in the cluster / launched
 // after 64 rounds: 3 chunks a warp 2,341 / 3,002, 5 chunks 4,937 / 4,837, 6
-// chunks 4,221 / 3,749, 12 chunks 26,222 / 14,838, after 16 rounds 14,189).
+// chunks 4,221 / 3,749, 8 chunks 6,544 / 5,046, 12 chunks 26,222 / 14,838, after 16 rounds 14,189;
+// ring of twelve neighbours a vertex, 6 chunks: 42,641 / 49,234).
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -41,7 +42,7 @@ constexpr int kMaxCluster = 16;
 constexpr int kLaunchRounds = 64;             // multiples of the launched loop's four
 constexpr int kShortRuns = 8;                 // and where more than kShortRounds rounds do
 constexpr int kShortRounds = 16;
-constexpr int kLongRuns = 5;                  // chunks a warp holds where long searches stay here
+constexpr int kLongRuns = 6;                  // chunks a warp holds where long searches stay here
 
 // dynamic shared memory of a block: frontier, visited and partial bitsets, and
 // each lane's first tile-row in each of its chunks

@@ -54,9 +54,9 @@ def _row_of_blobs(n, blob, seed):
 
 
 @pytest.mark.parametrize("k", [4, 8])
-@pytest.mark.parametrize("n,blob", [(1 << 17, 512), (3 << 16, 1024), (1 << 18, 4096)])
+@pytest.mark.parametrize("n,blob", [(5 << 15, 640), (3 << 16, 1024), (1 << 18, 4096)])
 def test_long_searches_of_large_graphs(n, blob, k):
-    """Six to twelve chunks a warp: the rounds after the first launch's are launched
+    """Eight to twelve chunks a warp: the rounds after the first launch's are launched
     one by one, with the same levels and the same limit."""
     from paper_2201_08560_gb300 import binding as B
     g = _row_of_blobs(n, blob, seed=n)
