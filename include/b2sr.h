@@ -95,7 +95,8 @@ typedef enum {
  * segment of a tile in shared memory (Sec. IV); STAGED is that idea for a
  * gather per set bit, DIRECT reads the vector from global memory. */
 typedef enum {
-    B2SR_SCHED_AUTO = 0,   /* STAGED at k = 8 (except the 64-lane OR), for min-plus at k = 4 and, with weights, at k = 16; else DIRECT */
+    B2SR_SCHED_AUTO = 0,   /* STAGED at k = 8 (except the 64-lane OR), for min-plus at k = 4 and, with weights, at
+                              k = 16, and at k = 8 and 16 for a matrix that is mostly one tile-row; else DIRECT */
     B2SR_SCHED_STAGED = 1, /* set-bit gathers staged in shared memory (cp.async), then reduced */
     B2SR_SCHED_DIRECT = 2  /* each lane walks its tiles and loads x directly */
 } b2sr_schedule;
@@ -303,9 +304,10 @@ b2sr_status b2sr_spmm_f32x4(b2sr_handle h, const float* X, float* Y, const uint3
  * they call in, such as a host whose own allocator already holds the device's
  * free memory, or a service that must not allocate once it is running.
  * Computes exactly what b2sr_spmv computes for BOOL_OR_AND, BITS -> BITS
- * (same x, y, mask and mask_complement meaning), but keeps its scratch (the
- * partial rows of tile-rows that cross chunks) in a fixed 4 MiB array compiled
- * into the library.  It calls no cudaMalloc, cudaFree or allocating routine.
+ * (same x, y, mask and mask_complement meaning), but keeps its scratch (at k =
+ * 16 and 32, the partial rows of tile-rows that cross chunks; k = 4 and 8 need
+ * none) in a fixed 4 MiB array compiled into the library.  It calls no
+ * cudaMalloc, cudaFree or allocating routine.
  *  - A device gets its copy of the array when the CUDA runtime loads the
  *    library's SpMV code on it: with lazy module loading (the default since
  *    CUDA 12.2) that is the first SpMV launch or the first call of this
@@ -317,13 +319,14 @@ b2sr_status b2sr_spmm_f32x4(b2sr_handle h, const float* X, float* Y, const uint3
  *    the process, so do not call this function after cudaDeviceReset.
  *  - h must belong to the current device (else B2SR_ERR_INVALID_ARG): each
  *    device's call uses that device's copy.
- *  - Matrices needing more scratch than the array holds (more than 262,144
- *    chunks at k=8, or 524,288 at k=4/16/32; a chunk is 256 tiles at k=4/8,
- *    128 at k=16, 64 at k=32) are rejected
- *    with B2SR_ERR_INVALID_ARG and a message giving both sizes.
- *  - Every call uses the same array and leaves its contents behind.  Nothing
- *    in it needs clearing (each call writes every value it reads), but calls
- *    that run at the same time on the GPU (other streams, other threads)
+ *  - Matrices of more than 262,144 chunks at k=8, or 524,288 at k=4/16/32 (a
+ *    chunk is 256 tiles at k=4/8, 128 at k=16, 64 at k=32) are rejected with
+ *    B2SR_ERR_INVALID_ARG and a message giving the sizes: at k=16/32 that is
+ *    what the array holds; the limits at k=4/8 are those of the partial rows
+ *    that these sizes used to keep there.
+ *  - Every call at k=16/32 uses the same array and leaves its contents behind.
+ *    Nothing in it needs clearing (each call writes every value it reads), but
+ *    calls that run at the same time on the GPU (other streams, other threads)
  *    overwrite each other's scratch: serialise them. */
 b2sr_status b2sr_spmv_bool_noalloc(b2sr_handle h, const uint32_t* x, uint32_t* y, const uint32_t* mask,
                                    int mask_complement, void* stream);
@@ -337,7 +340,11 @@ b2sr_status b2sr_spmv_bool_noalloc(b2sr_handle h, const uint32_t* x, uint32_t* y
  * the reduction fused (Sec. V, TC).  Rows of B are used directly, as
  * Listing 2's popc(r0 & shfl(r1)) does, so triangle counting passes
  * A = B = M = L.  All three handles need the same n and tile_dim.
- *   count  device int64[1] (written, not accumulated). */
+ *   count  device int64[1] (written, not accumulated).
+ * Counts over the operands' rows, extracted into temporary memory (4 bytes an
+ * entry and up to 16 a vertex for each distinct operand, 8 more a mask entry
+ * from 2^21 mask entries), or over tiles where those are a third full, the mask
+ * has few, or that memory is not to be had. */
 b2sr_status b2sr_spgemm_masked_count(b2sr_handle A, b2sr_handle B, b2sr_handle M, int64_t* count,
                                      void* stream);
 
@@ -409,7 +416,7 @@ b2sr_status b2sr_autotune(int32_t n, const int32_t* rowptr, const int32_t* colin
 /* BFS levels from `src` (Sec. V BFS: Boolean semiring, the visited set as a
  * complemented mask).  levels device int32[n]: 0 at src, -1 if unreachable.
  * At most max_iters levels (<= 0: n); B2SR_ERR_NOT_CONVERGED if exceeded.
- * Synchronises `stream` once per four levels (see b2sr_bfs_sources). */
+ * Synchronises `stream` at most once per four levels (see b2sr_bfs_sources). */
 b2sr_status b2sr_bfs(b2sr_handle h, int32_t src, int32_t* levels, int max_iters, void* stream);
 
 /* BFS from a set of sources, all at level 0 (Sec. V BFS with the first
@@ -420,8 +427,11 @@ b2sr_status b2sr_bfs(b2sr_handle h, int32_t src, int32_t* levels, int max_iters,
  * no edge joins two graphs: one call runs every graph's BFS at once.
  *   srcs_host host int32[nsrc], nsrc >= 1, each in [0, n), repeats allowed
  *   levels    device int32[n]
- * Level rounds run as a CUDA graph of four gated rounds replayed until a
- * round finds no new vertex: one host synchronisation per four levels.
+ * Level rounds run in batches of four gated rounds, from the fifth batch on as a
+ * replayed CUDA graph, until a round finds no new vertex: one host
+ * synchronisation per four levels.  At k = 4 and 8 the first rounds of a graph of
+ * at most 262,144 vertices (all of a smaller one's) run 16 or 64 to a launch in
+ * one thread-block cluster.
  * B2SR_ERR_NOT_CONVERGED past max_iters levels (<= 0: n). */
 b2sr_status b2sr_bfs_sources(b2sr_handle h, const int32_t* srcs_host, int nsrc, int32_t* levels,
                              int max_iters, void* stream);
@@ -443,7 +453,8 @@ b2sr_status b2sr_bfs_diropt(b2sr_handle h, b2sr_handle hT, int32_t src, int32_t*
  * frontiers packed as one uint64 per vertex (b2sr_spmm_bits64), or, for at
  * most 32 sources, one uint32 (half the bytes per step; same levels).
  *   srcs_host host int32[nsrc], 1 <= nsrc <= 64
- *   levels    device int32[nsrc * n]: row s holds the levels of srcs_host[s] */
+ *   levels    device int32[nsrc * n]: row s holds the levels of srcs_host[s]
+ * Temporary memory: five words a vertex, three where five are not to be had. */
 b2sr_status b2sr_bfs_multi(b2sr_handle h, const int32_t* srcs_host, int nsrc, int32_t* levels,
                            int max_iters, void* stream);
 
@@ -451,8 +462,9 @@ b2sr_status b2sr_bfs_multi(b2sr_handle h, const int32_t* srcs_host, int nsrc, in
  * relaxation, d <- min(d, A min.+ d), until no distance changes (the fixed
  * point delta-stepping also reaches).  weights in set-bit order
  * (b2sr_weights_from_csr), non-negative, or NULL for unit weights.
- * dist device float[n]: 0 at src, +inf if unreachable.  Rounds run as a CUDA
- * graph of 16 gated rounds: one host synchronisation per 16 rounds. */
+ * dist device float[n]: 0 at src, +inf if unreachable.  Rounds run in batches of
+ * 16 gated rounds, from the fifth batch on as a replayed CUDA graph: one host
+ * synchronisation per 16 rounds. */
 b2sr_status b2sr_sssp(b2sr_handle h, const float* weights, int32_t src, float* dist, int max_iters,
                       void* stream);
 
@@ -474,9 +486,10 @@ b2sr_status b2sr_sssp(b2sr_handle h, const float* weights, int32_t src, float* d
  *              <= 0: every active vertex every round (Bellman-Ford frontier)
  * A round touches only the active tile-rows.  Distances are updated with
  * integer atomicMin on the float bits; the order of updates and delta change
- * the number of rounds, never the result (bit-exact).  Rounds run as a CUDA
- * graph of 32 gated rounds: one host synchronisation per 32 rounds, and one
- * more at the end to read the round count.
+ * the number of rounds, never the result (bit-exact).  Rounds of little work run
+ * in one thread-block cluster, up to 512 to a host synchronisation, the others in
+ * batches of 32 gated rounds, from the fifth batch on as a replayed CUDA graph,
+ * with one synchronisation a batch and one at the end to read the round count.
  * B2SR_ERR_NOT_CONVERGED past max_iters rounds (<= 0: n, or 4n + 4 with
  * delta > 0). */
 b2sr_status b2sr_sssp_push(b2sr_handle hT, const float* weights_t, int32_t src, float* dist, float delta,
@@ -515,7 +528,7 @@ b2sr_status b2sr_cc(b2sr_handle h, int32_t* labels, int max_iters, void* stream)
  *   priority device float[n], not NaN (+0 and -0 are equal)
  *   in_set   device int32[n]: 1 for members, 0 otherwise
  * Symmetric matrices (undirected graphs); self-loops are ignored.  Rounds run
- * as a CUDA graph of 4 gated rounds.  B2SR_ERR_INVALID_ARG for a NaN
+ * in batches of 4 gated rounds.  B2SR_ERR_INVALID_ARG for a NaN
  * priority; B2SR_ERR_NOT_CONVERGED if vertices are still undecided after
  * max_iters rounds (<= 0: n), checked every 4 rounds. */
 b2sr_status b2sr_mis(b2sr_handle h, const float* priority, int32_t* in_set, int max_iters, void* stream);
@@ -532,21 +545,22 @@ typedef enum {
  * larger key, else 1 + the largest colour among the neighbours that do; each
  * colour class is an independent set.  MAX_TIMES: round r gives colour r to
  * every uncoloured vertex whose key is the largest among itself and its
- * uncoloured neighbours (a max-times SpMV per round, 8 rounds per CUDA-graph
- * replay).  PUSH: cnt[v] = neighbours with a larger key, counted in one pass;
+ * uncoloured neighbours (a max-times SpMV per round, 8 rounds a batch).  PUSH: cnt[v] = neighbours with a larger key, counted in one pass;
  * the vertices coloured r push along their rows and a vertex whose count
  * reaches 0 takes colour r + 1 (the levels of a topological sort; each edge
- * read twice in all, 16 rounds per replay).
+ * read twice in all, 16 rounds a batch).
  *   priority device float[n], not NaN
  *   colors   device int32[n]
  * Symmetric matrices; self-loops are ignored.  B2SR_ERR_INVALID_ARG for a NaN
  * priority or an unknown method; B2SR_ERR_NOT_CONVERGED if vertices are still
- * uncoloured after max_iters rounds (<= 0: n), checked at each replay. */
+ * uncoloured after max_iters rounds (<= 0: n), checked after each batch. */
 b2sr_status b2sr_color(b2sr_handle h, const float* priority, int32_t* colors, b2sr_color_method method,
                        int max_iters, void* stream);
 
-/* Triangle count (Sec. V TC): sum(L .* (L L^T)) for L = b2sr_lower(h), by
- * b2sr_spgemm_masked_count.  Symmetric matrices.  count device int64[1]. */
+/* Triangle count (Sec. V TC): sum(L .* (L L^T)) for the strictly lower triangle
+ * L, counted over the matrix's own rows up to the diagonal, or, where tiles are a
+ * third full or the rows find no room, by b2sr_spgemm_masked_count of
+ * b2sr_lower(h).  Symmetric matrices.  count device int64[1]. */
 b2sr_status b2sr_tc(b2sr_handle h, int64_t* count, void* stream);
 
 /* ---------------------------------------------------------------------- */
@@ -563,8 +577,8 @@ int64_t b2sr_launch_count(void);
  * recorded under its family: "spmv_bool", "spmv_count", "spmv_plus",
  * "spmv_minplus", "spmv_min_i32", "spmv_max", "spmv_maxkey", "spmm_or64",
  * "spmm_or32" (the batched BFS with at most 32 sources), "spmm_plus4" or
- * "spgemm_masked" (the masked-count SpGEMM kernel; its bytes are the three
- * matrices' arrays). */
+ * "spgemm_masked" (the masked count's kernels, between the extraction of the rows
+ * and the result; its bytes are the three matrices' arrays). */
 void b2sr_timing_enable(int on);
 
 /* Timing read-out (no counterpart in the paper).

@@ -10,7 +10,7 @@
 // pulling when the frontier's out-edges exceed the unexplored edges / alpha,
 // and back to pushing when the frontier falls below n / beta.  The decision
 // is taken on the device before every level, and both directions are gated
-// on it, so the level loop stays a replayed CUDA graph with one host
+// on it, so the level loop runs in batches of gated rounds with one host
 // synchronisation per four levels.  Levels are the same in either direction
 // (bit-exact with b2sr_bfs).
 #include <algorithm>

@@ -3,13 +3,15 @@
 // graphs packed block-diagonally in one arena), multi-source BFS (64 frontiers
 // per machine word), SSSP (min-plus relaxation rounds), PageRank (plus-times
 // with the column-stochastic matrix), connected components (FastSV hooking
-// and shortcutting around the min step) and triangle counting (masked SpGEMM
-// on the lower triangle).
+// and shortcutting around the min step) and triangle counting (the masked
+// count over the rows up to the diagonal, or over the tiles of the lower
+// triangle).
 //
-// Level-synchronous loops are captured once as a CUDA graph of several rounds;
-// each round's kernels are gated on a device flag that the round's update
-// kernel clears when nothing changes, and the graph is replayed until the host
-// reads the flag as 0.  One host synchronisation covers several rounds.
+// Level-synchronous loops run in batches of several rounds, launched one by one
+// at first and as a replayed CUDA graph in a longer loop (captured.cuh); each
+// round's kernels are gated on a device flag that the round's update kernel
+// clears when nothing changes, until the host reads the flag as 0.  One host
+// synchronisation covers a batch.
 #include <algorithm>
 #include <climits>
 #include <vector>

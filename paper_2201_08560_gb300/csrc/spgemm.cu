@@ -1,7 +1,9 @@
 // B2SR SpGEMM: bmm_bin_bin_sum_masked (Table 3, Listing 2; the fused-sum
 // triangle-counting kernel of Sec. V) and the Boolean product C = A (x) B.
 //
-// Masked count: each warp takes a run of consecutive mask tiles (so their
+// Masked count, two forms with one result: over the operands' rows, extracted as
+// column lists (further down), and over tiles, where those are full, the mask has
+// few or the rows find no room.  Tile form: each warp takes a run of consecutive mask tiles (so their
 // tile-rows come from one search, then a walk of the row pointers); for a mask
 // tile (I, J) the tile-column lists of A's tile-row I and B's tile-row J are
 // intersected (binary search of the shorter list's entries in the longer one,

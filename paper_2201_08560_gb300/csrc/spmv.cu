@@ -6,17 +6,19 @@
 // graphs make any row mapping badly imbalanced (a scale-20 R-MAT tile-row can
 // hold 10^5 tiles), so the unit of work here is a fixed-size chunk of
 // consecutive tiles:
-//   * one warp per chunk of 32*P tiles; lane l owns P consecutive tiles and
-//     issues every load it needs up front (its tiles and tile columns as
-//     16-byte vectors, then the input segments or, for full-precision
-//     vectors, one 4/8-byte cp.async gather per set bit into shared memory),
-//     so each warp keeps several KB in flight;
-//   * the lane walks its tiles in order, accumulating the k row results of
-//     the current tile-row and storing every row that starts and ends inside
-//     the lane (and the identity for empty tile-rows it passes);
-//   * rows that cross lanes are joined with a warp segmented scan (shuffles,
-//     fixed order); rows that cross chunks leave per-chunk partials that a
-//     second kernel joins, one warp per row, in a fixed order.
+//   * one warp per chunk of 32*P tiles, and four kernels that walk it: the
+//     small-tile one (bits at k = 4 and 8, unweighted values at k = 4; a lane a
+//     run of tiles, whole input segments), the row-lane one (values at k = 16 and
+//     32, the 64-lane OR at k = 8; a lane a row of the tile), the staged one
+//     (values at k <= 16 under that schedule; one cp.async gather per set bit
+//     into shared memory) and the general one (the rest; registers hold a lane's
+//     k row results);
+//   * every load a lane needs is issued up front, so each warp keeps several KB
+//     in flight;
+//   * rows that cross lanes are joined by shuffles in a fixed order; rows that
+//     cross chunks leave per-chunk partials that a second kernel joins, one warp
+//     per row, in a fixed order (Boolean rows at k = 4 and 8 are ORed into the
+//     cleared output instead).
 // Every reduction order is fixed by the data, so floating-point results are
 // bitwise reproducible and independent of launch geometry and stream.
 #include <algorithm>
@@ -1039,7 +1041,7 @@ __global__ void __launch_bounds__(kSpmvThreads) spmv_chunks_kernel(SpmvGeom g, S
 // in us before / after (one gather per set bit, a row search and a row-pointer
 // walk per lane before): plus-times 173 / 118 (permuted ids 148 / 138), label
 // min 183 / 129 (154 / 144), 64-lane OR 238 / 176, four fp32 columns 312 / 224
-// (236 / 194); Boolean 86 / 64 at k = 4 and 99 / 64 at k = 8.  Warp
+// (236 / 194); Boolean 86 / 59 at k = 4 and 99 / 63 at k = 8.  Warp
 // instructions of the plus-times kernel: 98M / 59M.
 // ---------------------------------------------------------------------------
 // lane-word schemes
@@ -2616,7 +2618,8 @@ extern "C" b2sr_status b2sr_spmm_bits64(b2sr_handle h, const uint64_t* X, uint64
 // or a deployment that must not allocate once it is running (fixed-memory or
 // real-time services).  For them b2sr_spmv_bool_noalloc keeps the only scratch
 // the Boolean SpMV needs -- the per-chunk partial rows joined by the fixup
-// kernel -- in a fixed array compiled into this file.  A device holds its copy
+// kernel at k = 16 and 32; k = 4 and 8 OR into the output and need none -- in a
+// fixed array compiled into this file.  A device holds its copy
 // from the moment the runtime loads this file's device code on it (the first
 // SpMV launch or symbol lookup there, under lazy module loading) until the
 // process exits or the device is reset.
@@ -2661,7 +2664,7 @@ static b2sr_status run_spmv_bool_fixed(const b2sr_matrix* h, const SemBool<K>& s
                                               std::to_string(2 * half) + " scratch bytes, the fixed array holds " +
                                               std::to_string(kNoallocScratchBytes));
     SpmvGeom g{h->rowptr, h->colind, h->tiles, h->chunk_row, h->T, h->nchunks, h->ntr, nullptr};
-    if constexpr (OrsInto<SEM>::value) {  // needs no scratch: the limit is the entry point's
+    if constexpr (OrsInto<SEM>::value) {  // needs no scratch; the entry point's limit stays what it was
         B2SR_TRY(clear_bitset(h, y, s, nullptr));
         if (h->nchunks == 0) return B2SR_OK;
         return launch_direct<K, SEM>(h, sem, Partials<uint32_t>{nullptr, nullptr}, s, g);
