@@ -1035,6 +1035,7 @@ static b2sr_status merge_pieces(int32_t n, const int32_t* rowptr, const int32_t*
 __global__ void schedule_kernel(const int32_t* __restrict__ rowptr, int32_t ntr, int64_t T, int64_t CT,
                                 int64_t nchunks, int32_t* __restrict__ chunk_row, int32_t* __restrict__ split,
                                 int32_t* __restrict__ meta) {
+    int32_t most = 0;
     for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c <= nchunks;
          c += (int64_t)gridDim.x * blockDim.x) {
         const int64_t cs = min(c * CT, T - 1);
@@ -1046,13 +1047,15 @@ __global__ void schedule_kernel(const int32_t* __restrict__ rowptr, int32_t ntr,
         const int64_t ce = min(cs + CT, T);
         const int64_t rs = rowptr[R], re = rowptr[R + 1];
         if (rs >= cs || re > ce) continue;
-        atomicMax(meta + 4, (int32_t)(re - rs));
+        most = max(most, (int32_t)(re - rs));
         const int64_t ca = rs / CT;
         const int64_t at = c - ca + 1 <= kSplitShort ? atomicAdd(meta + 2, 1) : nchunks - 1 - atomicAdd(meta + 3, 1);
         split[3 * at] = R;
         split[3 * at + 1] = (int32_t)ca;
         split[3 * at + 2] = (int32_t)c;
     }
+    most = __reduce_max_sync(0xffffffffu, most);
+    if (lane_id() == 0 && most > 0) atomicMax(meta + 4, most);
 }
 
 b2sr_status build_schedule(b2sr_matrix* h, cudaStream_t s) {
